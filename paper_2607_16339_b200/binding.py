@@ -123,15 +123,30 @@ def load():
     return lib
 
 
+# Marshalling is part of every call: a small step takes the device little longer than the host needs to
+# enqueue it.  Pointers therefore go over as plain integers, and the current stream comes from torch's raw
+# accessor instead of a Stream object (0.3 us against 3 us).
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+def _current_stream():
+    """The current stream of the current device, as an integer; replaces itself on first use."""
+    global _current_stream
+    import torch
+    stream = torch.cuda.current_stream().cuda_stream       # (initialises CUDA)
+    raw, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+    if raw is not None and dev is not None and raw(dev()) == stream:
+        _current_stream = lambda: raw(dev())
+    else:
+        _current_stream = lambda: torch.cuda.current_stream().cuda_stream
+    return stream
 
 
 def _stream(stream):
     if stream is None:
-        import torch
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        return _current_stream()
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 
 def full_recompute_static(dtype, n_q_heads, n_kv_heads, head_dim, rope_theta, q_pre, k_pre, v_pre, out,
