@@ -1192,11 +1192,10 @@ lacache_status lacache_sample_block(lacache_ctx* c, const void* logits, int dtyp
   if (!logits || !conf || !token) return fail(c, LACACHE_ERR_INVALID_ARG, "NULL pointer");
   if (dtype != LACACHE_DTYPE_BF16 && dtype != LACACHE_DTYPE_FP32) return fail(c, LACACHE_ERR_INVALID_ARG, "dtype %d", dtype);
   if (vocab <= 0) return fail(c, LACACHE_ERR_INVALID_ARG, "vocab %d", vocab);
-  constexpr int MAX_SPLITS = 64;
   const int n = c->g.B * c->g.block_len;
   if (n > 65535) return fail(c, LACACHE_ERR_UNSUPPORTED, "%d block rows: the sampler's grid takes at most 65535", n);
   if (!c->sample_part) {
-    CU_TRY(c, dev_alloc(c, &c->sample_part, (size_t)n * MAX_SPLITS * 4));
+    CU_TRY(c, dev_alloc(c, &c->sample_part, (size_t)n * SAMPLE_MAX_SEGMENTS * 4));
     CU_TRY(c, dev_alloc(c, &c->sample_counters, (size_t)n, true));
   }
   SampleArgs a{};
@@ -1204,20 +1203,12 @@ lacache_status lacache_sample_block(lacache_ctx* c, const void* logits, int dtyp
   a.n_tokens = c->g.T; a.vocab = vocab;
   a.rows = c->d_blk_tok + (size_t)c->built_block * n;
   a.n_rows = n;
-  // as many CTAs as are resident at once (four per SM), each with at least 2048 entries, slices a
-  // multiple of 8 entries (rounded down: no second wave of a few stragglers)
-  int splits = std::max(1, std::min(MAX_SPLITS, 4 * c->num_sms / n));
-  splits = std::min(splits, std::max(1, vocab / 2048));
-  int slice = ((vocab + splits - 1) / splits + 7) / 8 * 8;
-  splits = (vocab + slice - 1) / slice;
-  a.splits = splits; a.slice = slice;
-  const size_t row_bytes = (size_t)vocab * elem_size(dtype);
-  a.vector_ok = (row_bytes % 16 == 0 && !misaligned(logits)) ? 1 : 0;
   a.part = c->sample_part; a.counters = c->sample_counters;
   a.conf = conf; a.token = token; a.lse = lse;
   a.status = c->d_status;
+  a.no_pdl = c->knobs.no_pdl ? 1 : 0;
   c->last_launches = 0;
-  CU_TRY(c, sample_rows(a, (cudaStream_t)stream));
+  CU_TRY(c, sample_rows(a, c->num_sms, (cudaStream_t)stream));
   c->last_launches++;
   return LACACHE_OK;
 }

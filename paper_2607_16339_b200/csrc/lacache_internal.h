@@ -148,13 +148,14 @@ struct SampleArgs {
   const void* logits; int dtype;   // [n_tokens, vocab], bf16 or fp32
   int n_tokens, vocab;
   const int32_t* rows; int n_rows; // the rows to sample (device)
-  int splits, slice;               // CTAs per row and vocabulary entries per CTA (splits * slice >= vocab)
-  int vector_ok;                   // rows start on 16-byte boundaries and `slice` is a multiple of the vector width
-  float* part; int* counters;      // [n_rows][splits][4] partial results, [n_rows] arrival counters (zero between launches)
+  int segments, quota;             // parts of a row and entries per part (set by the launcher)
+  int no_pdl;                      // host only: launch the ordinary way
+  float* part; int* counters;      // [n_rows][SAMPLE_MAX_SEGMENTS][4] partial results, [n_rows] arrival counters (zero between launches)
   float* conf; int32_t* token; float* lse;   // [n_rows]; lse may be null
   int32_t* status;
 };
-cudaError_t sample_rows(const SampleArgs& a, cudaStream_t s);
+constexpr int SAMPLE_MAX_SEGMENTS = 64;   // parts a row may be cut into
+cudaError_t sample_rows(const SampleArgs& a, int num_sms, cudaStream_t s);
 
 struct ExportArgs {
   RotBuffers rot; StateBuffers st;

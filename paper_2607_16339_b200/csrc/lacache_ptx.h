@@ -95,6 +95,11 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 // in the stream has completed and its writes are visible (returns at once when
 // the kernel was launched the ordinary way).
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Lets the kernel behind this one in the stream, if launched programmatically dependent, be scheduled once every
+// CTA of this grid has said so or has exited.  CTAs of that kernel which are small pile up on the SMs that fall
+// idle first, and run there when this grid is over: said at a CTA's start, that costs a long kernel's successor
+// more than the launch latency it hides; said when a CTA has requested its last loads, it does not.
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_commit(uint32_t bar) {

@@ -72,6 +72,20 @@ def test_block_rows_against_oracle(dtype, vocab):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("rows,vocab", [(192, 50021), (96, 4097), (320, 2055)])
+def test_many_rows_of_an_unaligned_vocabulary(rows, vocab):
+    """Rows that start anywhere in a 16-byte vector, cut into many segments and into one."""
+    wl = small_workload(name="samp-odd", prompt_lens=(5,) * (rows // 32), gen_len=32, block_len=32, steps=1, hq=2, hkv=2)
+    ctx, sch = _built_ctx(wl, 0)
+    g = torch.Generator(device="cuda").manual_seed(rows)
+    logits = (torch.randn(wl.total_tokens, vocab, generator=g, device="cuda") * 4).to(torch.bfloat16)
+    at = sch.block_rows(0)
+    logits[at[0], [0, vocab - 1]] = 30.0       # the maximum at both ends of the row
+    logits[at[1], :-1] = float("-inf")
+    _check(ctx, at, logits)
+    ctx.destroy()
+
+
 def test_full_size_block_and_vocabulary():
     """The headline configuration's block (32 rows) and the large-batch extension's (8192 rows) at a
     vocabulary of 126464 entries (bf16 logits of every token would not fit for the latter: its logits
