@@ -784,6 +784,7 @@ lacache_status rope_all(lacache_ctx* c, const void* q, const void* k, const void
   r.pos_of_tok = c->d_pos; r.cos_tab = c->d_cos; r.sin_tab = c->d_sin;
   r.dst = dst;
   r.in_dtype = c->cfg.dtype;
+  r.no_pdl = c->knobs.no_pdl ? 1 : 0;
   CU_TRY(c, rope_write(c->g, r, c->engine, s));
   c->last_launches++;
   return LACACHE_OK;
@@ -989,7 +990,7 @@ lacache_status lacache_build_advance(lacache_ctx* c, const void* q, const void* 
     r.row_cos = c->d_blk_cos + row0 * (c->g.d / 2);
     r.row_sin = c->d_blk_sin + row0 * (c->g.d / 2);
   }
-  r.pdl = 0;
+  r.no_pdl = c->knobs.no_pdl ? 1 : 0;
   r.dst = c->rot;
   r.in_dtype = c->cfg.dtype;
   CU_TRY(c, rope_write(c->g, r, c->engine, s));
@@ -1151,13 +1152,13 @@ lacache_status step_impl(lacache_ctx* c, const void* q, const void* k, const voi
     r.row_cos = c->d_blk_cos + row0 * (c->g.d / 2);
     r.row_sin = c->d_blk_sin + row0 * (c->g.d / 2);
   }
-  // may start while the previous step's attention kernel drains (it waits before its stores); when
-  // the kernel before it in the stream is the one that writes its inputs, it waits for that one first
+  // With the overlap on, the RoPE kernel reads its inputs while the previous step's attention kernel drains
+  // (it waits before its stores), unless a producer just ahead in the stream writes them.
   const bool overlap = c->step_overlap && !c->knobs.no_pdl && !c->knobs.no_step_overlap;
-  // (the first step after a build is launched the ordinary way: the build's cached state, which the
-  // attention kernel reads before it waits on anything, is then complete and flushed)
-  r.pdl = inputs_just_written ? 2 : ((overlap && c->steps_since_build > 0) ? 1 : 0);
-  r.no_pdl = (c->knobs.no_pdl || c->knobs.no_step_overlap) ? 1 : 0;
+  // (In the first step after a build it waits before anything else, and lets the attention kernel start only
+  // then: the build's cached state, which that kernel reads before it waits on anything, is then complete.)
+  r.early_inputs = (overlap && c->steps_since_build > 0 && !inputs_just_written) ? 1 : 0;
+  r.no_pdl = c->knobs.no_pdl ? 1 : 0;
   c->steps_since_build++;
   r.dst = c->rot;
   r.in_dtype = c->cfg.dtype;
@@ -1165,7 +1166,7 @@ lacache_status step_impl(lacache_ctx* c, const void* q, const void* k, const voi
     // Algorithm 1's reuse pass at tile granularity: ordinary launches, one pass of the build kernel over
     // key windows (rows of the overlapping tiles x all keys; every other row: cached state + the keys of
     // the overlapping tiles), normalised output instead of state
-    r.pdl = 0;
+    r.early_inputs = 0;
     CU_TRY(c, rope_write(c->g, r, c->engine, s));
     c->last_launches++;
     return run_window(c, c->tile_step[blk], blk, c->st, c->st, StateBuffers{}, s, out, lse);

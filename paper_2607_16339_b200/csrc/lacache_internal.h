@@ -90,16 +90,17 @@ struct RopeArgs {
   const int32_t* row_tok; const float* row_cos; const float* row_sin;  // [n_src_rows], [n_src_rows][d/2]
   RotBuffers dst;
   int in_dtype;
-  // launch programmatically dependent on the kernel before it in the stream.  1: that kernel is a
-  // step's attention kernel, which lets its successors start early; this kernel then waits before its
-  // first store.  2: that kernel writes this kernel's inputs; this kernel waits before anything else.
-  int pdl;
-  int no_pdl;   // host only: launch the ordinary way whatever `pdl` says (experiment knob)
+  // The launch is programmatically dependent on the kernel before it in the stream.  early_inputs: the inputs
+  // were complete before that kernel (a step's attention kernel) was enqueued, so this kernel reads them while
+  // it drains and waits for it only before its first store; else it waits before anything else, and only its
+  // launch overlaps the end of that kernel.
+  int early_inputs;
+  int no_pdl;   // host only: launch the ordinary way (experiment knob)
 };
 
 struct AttnArgs {
   int mode;
-  const WorkItem* items; int n_items;   // SIMT: all items; tcgen05: stream-role items
+  const WorkItem* items; int n_items;   // SIMT: all items (a step's block queries first); tcgen05: stream-role items
   // tcgen05 only: items of the merge role (fixed rows of a step), CTA split
   const WorkItem* items_merge; int n_items_merge;
   int n_ctas_stream; int n_ctas;

@@ -45,12 +45,10 @@ __device__ __forceinline__ void store8_f16(void* plane, size_t off, const float 
 // [Hq,Hq+Hkv) k heads, [Hq+Hkv,Hq+2Hkv) v heads.
 template <bool TC>
 __global__ void __launch_bounds__(256) rope_write_kernel(Geometry g, RopeArgs a) {
-  // the attention kernel that follows may be launched programmatically
-  // dependent: let it start its prologue now (it waits for this grid's writes
-  // before it touches them)
-  // (when the kernel before this one writes this kernel's inputs, they are complete only after the
-  // wait, and the attention kernel, which also reads them early, must not start before that)
-  if (a.pdl == 2) asm volatile("griddepcontrol.wait;" ::: "memory");
+  // This kernel and the attention kernel behind it are launched programmatically dependent.  The attention
+  // kernel reads this kernel's inputs, and state that the kernels ahead may have written, before it waits for
+  // this grid: it may start only once those are complete, hence the order of the wait and the trigger.
+  if (!a.early_inputs) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int chunks = g.d / 16;
   const int slots = g.Hq + 2 * g.Hkv;
@@ -230,20 +228,17 @@ cudaError_t rope_write(const Geometry& g, const RopeArgs& a, int engine, cudaStr
   long long total = (long long)a.n_src_rows * (g.Hq + 2 * g.Hkv) * (g.d / 16);
   if (total == 0) return cudaSuccess;
   unsigned blocks = (unsigned)((total + 255) / 256);
-  if (engine == LACACHE_ENGINE_TCGEN05) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
-    cfg.blockDim = dim3(256);
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = (a.pdl && !a.no_pdl) ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, rope_write_kernel<true>, g, a);
-  }
-  rope_write_kernel<false><<<blocks, 256, 0, s>>>(g, a);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(256);
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = a.no_pdl ? 0 : 1;
+  return engine == LACACHE_ENGINE_TCGEN05 ? cudaLaunchKernelEx(&cfg, rope_write_kernel<true>, g, a)
+                                          : cudaLaunchKernelEx(&cfg, rope_write_kernel<false>, g, a);
 }
 
 cudaError_t export_buffers(const Geometry& g, const ExportArgs& a, int engine, cudaStream_t s) {
