@@ -768,7 +768,7 @@ lacache_status run_attention(lacache_ctx* c, const AttnArgs& a, bool scratch, cu
     if (c->engine == LACACHE_ENGINE_TCGEN05)
       CU_TRY(c, launch_tc(c, a, scratch ? c->maps_scratch : c->maps, s));
     else
-      CU_TRY(c, simt_attention(c->g, a, s));
+      CU_TRY(c, simt_attention(c->g, a, c->num_sms, s));
     c->last_launches++;
   }
   if (c->ev_stop) CU_TRY(c, cudaEventRecord(c->ev_stop, s));
@@ -1171,10 +1171,18 @@ lacache_status step_impl(lacache_ctx* c, const void* q, const void* k, const voi
     c->last_launches++;
     return run_window(c, c->tile_step[blk], blk, c->st, c->st, StateBuffers{}, s, out, lse);
   }
-  CU_TRY(c, rope_write(c->g, r, c->engine, s));
-  c->last_launches++;
+  // (the fp32 engine's step kernel rotates the block's rows itself)
+  const bool self_rotating = c->engine == LACACHE_ENGINE_SIMT && !c->knobs.no_qcomp;
+  if (!self_rotating) {
+    CU_TRY(c, rope_write(c->g, r, c->engine, s));
+    c->last_launches++;
+  }
   AttnArgs a = attn_args(c, MODE_STEP, c->step_list[blk], blk, c->rot, out, lse);
   a.step_overlap = overlap ? 1 : 0;
+  if (c->engine == LACACHE_ENGINE_SIMT) {
+    a.n_split_items = c->g.B * ((c->g.block_len + SIMT_ROWS - 1) / SIMT_ROWS);
+    a.raw_bf16 = c->cfg.dtype == LACACHE_DTYPE_BF16 ? 1 : 0;
+  }
   if (!c->knobs.no_qcomp) {
     a.q_raw = q;
     a.k_raw = k;

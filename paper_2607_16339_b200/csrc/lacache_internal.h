@@ -118,6 +118,11 @@ struct AttnArgs {
   // likewise the block's pre-RoPE keys and values [B * block_len, Hkv, d]: the first unit of a
   // pipelined merge-role CTA rotates the block's keys / converts its values itself
   const void* k_raw; const void* v_raw;
+  // SIMT: with the three raw pointers set, a step's kernel rotates the block's rows itself and leaves them in
+  // the rotated cache (no RoPE kernel ahead of it); their element type is bf16 or fp32
+  int raw_bf16;
+  int n_split_items;         // SIMT step: the block-query items, first in the list (their key range may be cut over CTAs)
+  int split_ctas;            // SIMT: CTAs (one cluster) a cut unit takes; chosen by the launcher
   int step_overlap;          // step: let the next step's kernels be scheduled while this one drains
   const int32_t* cu;         // [B+1]
   const int32_t* blk_start;  // [B] absolute token index of the block's first row
@@ -181,7 +186,7 @@ cudaError_t merge_chunk_states(const Geometry& g, const ChunkMergeArgs& a, cudaS
 cudaError_t rope_write(const Geometry& g, const RopeArgs& a, int engine, cudaStream_t s);
 cudaError_t export_buffers(const Geometry& g, const ExportArgs& a, int engine, cudaStream_t s);
 
-cudaError_t simt_attention(const Geometry& g, const AttnArgs& a, cudaStream_t s);
+cudaError_t simt_attention(const Geometry& g, const AttnArgs& a, int num_sms, cudaStream_t s);
 cudaError_t simt_prepare();  // function attributes
 
 struct TcMaps;  // opaque set of TMA descriptors, defined in lacache_tc.cu

@@ -1,192 +1,531 @@
 // CUDA-core fp32 attention kernels (the fp32 dtype path, and any shape the
 // tcgen05 path does not cover).  One generic kernel runs every mode:
 //   build : fixed queries x fixed keys            -> cached (m, l, O~)
-//   step  : fixed queries x block keys, starting from the cached state
+//   step  : fixed queries x block keys, merged with the cached state
 //           (Algorithm 1 reuse pass); block queries x all keys
 //   full  : all queries x all keys (no cache)
 // following the online-softmax recurrence of Eq. 2-6 with key tiles of 32.
 //
-// Mapping: a CTA owns 32 query rows of one (sequence, q head); each of its 8
-// warps owns 4 rows.  Per key tile, lane j holds the score of key j for the
-// warp's 4 rows (dot product over d from shared memory), row max / sum are
-// warp shuffles, and for P.V lane c owns output features c, c+32, ...
+// Mapping: a CTA of 4 warps owns 32 query rows of one (sequence, q head), 8 rows a
+// warp, and walks key tiles of 32.  A unit with many keys is cut over the S <= 8
+// CTAs of a thread-block cluster, whose online-softmax states are merged through
+// distributed shared memory.  What bounds this kernel at the sizes it serves is
+// not arithmetic but too few warps, each waiting for its own shared-memory loads
+// (a small model has about as many row tiles as the GPU has SMs), and the last
+// CTAs of an uneven wave: hence small CTAs, four to an SM, and many of them.
+// Per tile, a warp computes its 8 x 32 scores with 4 rows x 2 keys per lane and
+// its 8 x d part of P.V with 8 rows x d/32 features per lane: 32 products per 6
+// to 8 shared-memory wavefronts, which keeps the FMA pipe and the shared-memory
+// pipe about equally busy (one key and one row at a time, as this kernel once
+// did, read 9 words per 4 products).  Values stream in while the scores are
+// computed and the next keys while P.V is (cp.async, one buffer of each).
+//
+// In a step the kernel rotates the block's rows itself, wherever it needs them,
+// and leaves them in the rotated cache: one launch, no kernel in front of it.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "lacache_internal.h"
+#include "lacache_ptx.h"
+#include "lacache_rope_math.h"
 
 namespace lacache {
 namespace {
 
-constexpr int KT = 32;    // keys per tile
-constexpr int RPW = 4;    // rows per warp
-constexpr int WARPS = 8;
+using namespace ptx;
 
-__device__ __forceinline__ float warp_max(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+constexpr int KT = 32;       // keys per tile
+constexpr int RPW = 8;       // rows per warp
+constexpr int WARPS = SIMT_ROWS / RPW;
+constexpr int THREADS = WARPS * 32;
+constexpr int MAX_SPLIT = 8;  // CTAs of a cluster (the portable limit)
+
+// Shared memory, in floats: queries [32][D + 4] and keys [32][D + 4] (rows 16 bytes apart in the banks:
+// lanes read rows), values [32][D], per warp probabilities [32 keys][8 rows].  After the last tile the keys'
+// place holds the CTA's partial O~ [32][D], ML the partial (m, l).
+template <int D>
+struct Smem {
+  static constexpr int QS = D + 4, KS = D + 4;
+  static constexpr int Q = 0;
+  static constexpr int K = Q + SIMT_ROWS * QS;
+  static constexpr int V = K + KT * KS;
+  static constexpr int P = V + KT * D;
+  static constexpr int ML = P + WARPS * KT * RPW;
+  static constexpr int TOTAL = ML + SIMT_ROWS * 2;
+  static constexpr size_t bytes = TOTAL * sizeof(float);
+};
+
+__device__ __forceinline__ void cp_async16(float* dst, const float* src, bool valid) {
+  const int n = valid ? 16 : 0;   // 0: zero-fill
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(n) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ float4 ld_cluster_v4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
   return v;
 }
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+__device__ __forceinline__ float2 ld_cluster_v2(uint32_t addr) {
+  float2 v;
+  asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
   return v;
+}
+// two fp32 products-and-sums in one instruction (the same roundings as two fmaf)
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ float4 load4(const void* base, size_t off, bool bf16) {
+  if (!bf16) return *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(base) + off);
+  const uint2 u = *reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(base) + off);
+  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.x));
+  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&u.y));
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+// features c .. c + 3 (x1) and their partners c + d/2 .. (x2) of a raw row, rotated with the RoPE kernel's own
+// roundings
+__device__ __forceinline__ void rotate4(float4 x1, float4 x2, float4 cs, float4 sn, float4& y1, float4& y2) {
+  auto lo = [](float p, float q, float co, float si) { return __fsub_rn(__fmul_rn(p, co), __fmul_rn(q, si)); };
+  auto hi = [](float p, float q, float co, float si) { return __fadd_rn(__fmul_rn(q, co), __fmul_rn(p, si)); };
+  y1 = make_float4(lo(x1.x, x2.x, cs.x, sn.x), lo(x1.y, x2.y, cs.y, sn.y), lo(x1.z, x2.z, cs.z, sn.z), lo(x1.w, x2.w, cs.w, sn.w));
+  y2 = make_float4(hi(x1.x, x2.x, cs.x, sn.x), hi(x1.y, x2.y, cs.y, sn.y), hi(x1.z, x2.z, cs.z, sn.z), hi(x1.w, x2.w, cs.w, sn.w));
 }
 
 template <int D>
-__global__ void __launch_bounds__(WARPS * 32) simt_attn_kernel(Geometry g, AttnArgs a) {
-  constexpr int DPL = D / 32;  // output features per lane
-  extern __shared__ float sm[];
-  float* Qs = sm;                         // [32][D]
-  float* Ks = Qs + SIMT_ROWS * D;         // [KT][D+1]
-  float* Vs = Ks + KT * (D + 1);          // [KT][D]
+__global__ void __launch_bounds__(THREADS, 3) simt_attn_kernel(const __grid_constant__ Geometry g,
+                                                              const __grid_constant__ AttnArgs a) {
+  using SM = Smem<D>;
+  constexpr int D4 = D / 4;          // 16-byte columns of a row
+  constexpr int DPL = D / 32;        // output features per lane (P.V)
+  extern __shared__ __align__(16) float sm[];
 
-  const WorkItem it = a.items[blockIdx.x];
+  // Launched programmatically dependent: nothing is touched before the grids ahead have completed, but this
+  // grid's launch overlaps their end.
+  grid_dependency_wait();
+
+  // the first n_split_items items are cut over the `split` CTAs of a cluster, the others take one CTA each
+  const int S = a.split_ctas;
+  int item = (int)blockIdx.x, part = 0, n_parts = 1;
+  if (item < a.n_split_items * S) {
+    part = item % S;
+    item /= S;
+    n_parts = S;
+  } else {
+    item -= a.n_split_items * (S - 1);
+    if (item >= a.n_items) return;   // (the last cluster's filling; its CTAs are not split)
+  }
+  const WorkItem it = a.items[item];
   const int h = blockIdx.y;
   const int kh = h / g.group;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int seq_start = a.cu[it.seq], seq_end = a.cu[it.seq + 1];
   const int bs = a.blk_start ? a.blk_start[it.seq] : 0;
   const int be = bs + g.block_len;
 
-  int k0, k1, x0 = 0, x1 = 0;
+  int k0 = it.seq_start, k1 = it.seq_end, x0 = 0, x1 = 0;
   bool from_state = false, to_state = false;
   if (a.mode == MODE_BUILD) {
-    k0 = seq_start; k1 = seq_end; x0 = bs; x1 = be; to_state = true;
+    x0 = bs; x1 = be; to_state = true;
   } else if (a.mode == MODE_STEP && it.kind == ITEM_ROWS) {
     k0 = bs; k1 = be; from_state = true;
-  } else {
-    k0 = seq_start; k1 = seq_end;
   }
+  const bool raw = a.k_raw != nullptr;                    // a step that rotates the block's rows here
+  const bool q_raw = raw && it.kind == ITEM_BLOCK_CHUNK;  // (these rows' queries are the block's)
+  const size_t blk_row0 = (size_t)it.seq * g.block_len;   // the sequence's first row of the block's inputs
 
-  const float* qr = reinterpret_cast<const float*>(a.rot.q_hi) + (size_t)h * g.Tp * D;
-  const float* kr = reinterpret_cast<const float*>(a.rot.k_hi) + (size_t)kh * g.Tp * D;
-  const float* vr = reinterpret_cast<const float*>(a.rot.v) + (size_t)kh * g.Tp * D;
+  float* const qr = reinterpret_cast<float*>(a.rot.q_hi) + (size_t)h * g.Tp * D;
+  float* const kr = reinterpret_cast<float*>(a.rot.k_hi) + (size_t)kh * g.Tp * D;
+  float* const vr = reinterpret_cast<float*>(a.rot.v) + (size_t)kh * g.Tp * D;
 
-  // stage the query rows
-  for (int i = threadIdx.x; i < SIMT_ROWS * (D / 4); i += blockDim.x) {
-    int r = i / (D / 4), c4 = i % (D / 4);
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (r < it.nrows) v = *reinterpret_cast<const float4*>(qr + (size_t)(it.row0 + r) * D + c4 * 4);
-    *reinterpret_cast<float4*>(Qs + r * D + c4 * 4) = v;
-  }
-
-  float m[RPW], l[RPW], o[RPW][DPL];
-#pragma unroll
-  for (int i = 0; i < RPW; ++i) {
-    int r = warp * RPW + i;
-    m[i] = -INFINITY;
-    l[i] = 0.f;
-#pragma unroll
-    for (int t = 0; t < DPL; ++t) o[i][t] = 0.f;
-    if (from_state && r < it.nrows) {
-      size_t row = (size_t)h * g.Tp + it.row0 + r;
-      m[i] = a.st.m[row];
-      l[i] = a.st.l[row];
-#pragma unroll
-      for (int t = 0; t < DPL; ++t) o[i][t] = a.st.o[row * D + lane + 32 * t];
+  // the key tiles of this CTA's part (a tile wholly inside the excluded block holds nothing)
+  const int n_tiles_all = (k1 - k0 + KT - 1) / KT;
+  const int t_begin = n_tiles_all * part / n_parts, t_end = n_tiles_all * (part + 1) / n_parts;
+  auto next_tile = [&](int t) {
+    for (; t < t_end; ++t) {
+      const int kt = k0 + t * KT;
+      if (!(x1 > x0 && kt >= x0 && min(kt + KT, k1) <= x1)) break;
     }
-  }
+    return t;
+  };
+  float* const Ks = sm + SM::K;
+  float* const Vs = sm + SM::V;
+  const bool writes_cache = q_raw && it.row0 == bs && h % g.group == 0;   // leaves the block's keys and values in the cache
 
-  for (int kt = k0; kt < k1; kt += KT) {
-    // a tile entirely inside the excluded range contributes nothing
-    if (kt >= x0 && min(kt + KT, k1) <= x1 && x1 > x0) continue;
-    __syncthreads();
-    for (int i = threadIdx.x; i < KT * (D / 4); i += blockDim.x) {
-      int r = i / (D / 4), c4 = i % (D / 4);
-      float4 kv = make_float4(0.f, 0.f, 0.f, 0.f), vv = kv;
-      if (kt + r < k1) {
-        kv = *reinterpret_cast<const float4*>(kr + (size_t)(kt + r) * D + c4 * 4);
-        vv = *reinterpret_cast<const float4*>(vr + (size_t)(kt + r) * D + c4 * 4);
+  // (a tile that holds block rows of a step: the loads of a batch of raw rows leave together, then they are
+  // rotated and stored)
+  auto load_keys = [&](int t) {
+    const int kt = k0 + t * KT;
+    constexpr int N = KT * (D4 / 2) / THREADS, BATCH = 2;
+    static_assert(N % BATCH == 0, "whole batches");
+    const bool mixed = raw && kt < be && kt + KT > bs;
+    if (!mixed && kt + KT <= k1) {   // the common tile: one address, constant offsets
+      const int r = threadIdx.x / (D4 / 2), c = (threadIdx.x % (D4 / 2)) * 4;
+      const float* src = kr + (size_t)(kt + r) * D + c;
+      float* dst = Ks + r * SM::KS + c;
+      constexpr int RS = THREADS / (D4 / 2);   // rows per pass of the CTA
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        cp_async16(dst + j * RS * SM::KS, src + j * RS * D, true);
+        cp_async16(dst + j * RS * SM::KS + D / 2, src + j * RS * D + D / 2, true);
       }
-      float* kd = Ks + r * (D + 1) + c4 * 4;
-      kd[0] = kv.x; kd[1] = kv.y; kd[2] = kv.z; kd[3] = kv.w;
-      *reinterpret_cast<float4*>(Vs + r * D + c4 * 4) = vv;
+      cp_async_commit();
+      return;
     }
-    __syncthreads();
-
-    const int key = kt + lane;
-    const bool valid = key < k1 && !(key >= x0 && key < x1);
-    float s[RPW];
+#pragma unroll 1
+    for (int b = 0; b < N; b += BATCH) {
+      float4 x1[BATCH], x2[BATCH], cs[BATCH], sn[BATCH];
+      if (mixed) {
 #pragma unroll
-    for (int i = 0; i < RPW; ++i) s[i] = 0.f;
-    const float* krow = Ks + lane * (D + 1);
-    const float* qw = Qs + warp * RPW * D;
-#pragma unroll 8
-    for (int c = 0; c < D; ++c) {
-      float kv = krow[c];
+        for (int j = 0; j < BATCH; ++j) {
+          const int i = threadIdx.x + (b + j) * THREADS, c = (i % (D4 / 2)) * 4, key = kt + i / (D4 / 2);
+          const size_t row = blk_row0 + (min(max(key, bs), be - 1) - bs);
+          x1[j] = load4(a.k_raw, (row * g.Hkv + kh) * D + c, a.raw_bf16);
+          x2[j] = load4(a.k_raw, (row * g.Hkv + kh) * D + c + D / 2, a.raw_bf16);
+          cs[j] = *reinterpret_cast<const float4*>(a.row_cos + row * (D / 2) + c);
+          sn[j] = *reinterpret_cast<const float4*>(a.row_sin + row * (D / 2) + c);
+        }
+      }
 #pragma unroll
-      for (int i = 0; i < RPW; ++i) s[i] = fmaf(qw[i * D + c], kv, s[i]);
-    }
-#pragma unroll
-    for (int i = 0; i < RPW; ++i) {
-      float sv = valid ? s[i] * g.scale_log2 : -INFINITY;
-      float m_new = fmaxf(m[i], warp_max(sv));
-      if (m_new == -INFINITY) continue;  // nothing seen yet (warp-uniform)
-      float alpha = (m[i] == -INFINITY) ? 0.f : exp2f(m[i] - m_new);
-      float p = valid ? exp2f(sv - m_new) : 0.f;
-      l[i] = l[i] * alpha + warp_sum(p);
-      m[i] = m_new;
-#pragma unroll
-      for (int t = 0; t < DPL; ++t) o[i][t] *= alpha;
-#pragma unroll 8
-      for (int j = 0; j < KT; ++j) {
-        float pj = __shfl_sync(0xffffffffu, p, j);
-#pragma unroll
-        for (int t = 0; t < DPL; ++t) o[i][t] = fmaf(pj, Vs[j * D + lane + 32 * t], o[i][t]);
+      for (int j = 0; j < BATCH; ++j) {
+        const int i = threadIdx.x + (b + j) * THREADS, r = i / (D4 / 2), c = (i % (D4 / 2)) * 4, key = kt + r;
+        float* dst = Ks + r * SM::KS + c;
+        if (mixed && key >= bs && key < be) {
+          float4 y1, y2;
+          rotate4(x1[j], x2[j], cs[j], sn[j], y1, y2);
+          *reinterpret_cast<float4*>(dst) = y1;
+          *reinterpret_cast<float4*>(dst + D / 2) = y2;
+          if (writes_cache) {
+            *reinterpret_cast<float4*>(kr + (size_t)key * D + c) = y1;
+            *reinterpret_cast<float4*>(kr + (size_t)key * D + c + D / 2) = y2;
+          }
+        } else {
+          const float* src = kr + (size_t)(key < k1 ? key : k0) * D + c;
+          cp_async16(dst, src, key < k1);
+          cp_async16(dst + D / 2, src + D / 2, key < k1);
+        }
       }
     }
-  }
+    cp_async_commit();
+  };
+  auto load_values = [&](int t) {
+    const int kt = k0 + t * KT;
+    constexpr int N = KT * D4 / THREADS, BATCH = 4;
+    static_assert(N % BATCH == 0, "whole batches");
+    const bool mixed = raw && kt < be && kt + KT > bs;
+    if (!mixed && kt + KT <= k1) {   // (a tile of values is one contiguous run)
+      const float* src = vr + (size_t)kt * D + threadIdx.x * 4;
+#pragma unroll
+      for (int j = 0; j < N; ++j) cp_async16(Vs + (threadIdx.x + j * THREADS) * 4, src + j * THREADS * 4, true);
+      cp_async_commit();
+      return;
+    }
+#pragma unroll 1
+    for (int b = 0; b < N; b += BATCH) {
+      float4 v[BATCH];
+      if (mixed) {
+#pragma unroll
+        for (int j = 0; j < BATCH; ++j) {
+          const int i = threadIdx.x + (b + j) * THREADS, c = (i % D4) * 4, key = kt + i / D4;
+          v[j] = load4(a.v_raw, ((blk_row0 + (min(max(key, bs), be - 1) - bs)) * g.Hkv + kh) * D + c, a.raw_bf16);
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < BATCH; ++j) {
+        const int i = threadIdx.x + (b + j) * THREADS, r = i / D4, c = (i % D4) * 4, key = kt + r;
+        if (mixed && key >= bs && key < be) {
+          *reinterpret_cast<float4*>(Vs + r * D + c) = v[j];
+          if (writes_cache) *reinterpret_cast<float4*>(vr + (size_t)key * D + c) = v[j];
+        } else {
+          cp_async16(Vs + r * D + c, vr + (size_t)(key < k1 ? key : k0) * D + c, key < k1);
+        }
+      }
+    }
+    cp_async_commit();
+  };
 
-  const float LN2 = 0.69314718055994530942f;
+  // the cached state merged at the end is asked into L2 now
+  if (from_state)
+    for (int i = threadIdx.x; i < it.nrows * (D / 32); i += THREADS)
+      prefetch_l2(a.st.o + ((size_t)h * g.Tp + it.row0 + i / (D / 32)) * D + (i % (D / 32)) * 32);
+  int t = next_tile(t_begin);
+  if (t < t_end) {
+    load_keys(t);
+    load_values(t);
+  }
+  // queries (rows past the tile's end are zero)
 #pragma unroll
-  for (int i = 0; i < RPW; ++i) {
-    int r = warp * RPW + i;
-    if (r >= it.nrows) continue;
-    int tok = it.row0 + r;
-    if (to_state) {
-      size_t row = (size_t)h * g.Tp + tok;
-      if (lane == 0) { a.st.m[row] = m[i]; a.st.l[row] = l[i]; }
-#pragma unroll
-      for (int t = 0; t < DPL; ++t) a.st.o[row * D + lane + 32 * t] = o[i][t];
-    } else {
-      float inv = 1.f / l[i];
-      size_t row = (size_t)tok * g.Hq + h;
-      if (a.out_bf16) {
-        __nv_bfloat16* ob = reinterpret_cast<__nv_bfloat16*>(a.out);
-#pragma unroll
-        for (int t = 0; t < DPL; ++t) ob[row * D + lane + 32 * t] = __float2bfloat16_rn(o[i][t] * inv);
+  for (int j = 0; j < SIMT_ROWS * (D4 / 2) / THREADS; ++j) {
+    const int i = threadIdx.x + j * THREADS, r = i / (D4 / 2), c = (i % (D4 / 2)) * 4;
+    float4 y1 = make_float4(0.f, 0.f, 0.f, 0.f), y2 = y1;
+    if (r < it.nrows) {
+      const size_t tok = (size_t)(it.row0 + r);
+      if (q_raw) {
+        const size_t row = blk_row0 + (it.row0 - bs) + r, off = (row * g.Hq + h) * D + c, tab = row * (D / 2) + c;
+        rotate4(load4(a.q_raw, off, a.raw_bf16), load4(a.q_raw, off + D / 2, a.raw_bf16),
+                *reinterpret_cast<const float4*>(a.row_cos + tab), *reinterpret_cast<const float4*>(a.row_sin + tab), y1, y2);
+        if (part == 0) {
+          *reinterpret_cast<float4*>(qr + tok * D + c) = y1;
+          *reinterpret_cast<float4*>(qr + tok * D + c + D / 2) = y2;
+        }
       } else {
-#pragma unroll
-        for (int t = 0; t < DPL; ++t) a.out[row * D + lane + 32 * t] = o[i][t] * inv;
+        y1 = *reinterpret_cast<const float4*>(qr + tok * D + c);
+        y2 = *reinterpret_cast<const float4*>(qr + tok * D + c + D / 2);
       }
-      if (a.lse && lane == 0) a.lse[row] = (m[i] + log2f(l[i])) * LN2;
+    }
+    *reinterpret_cast<float4*>(sm + SM::Q + r * SM::QS + c) = y1;
+    *reinterpret_cast<float4*>(sm + SM::Q + r * SM::QS + c + D / 2) = y2;
+  }
+  __syncthreads();   // the queries are in place
+
+  // scores: lane = keys kp and kp + 16 x rows 4 rh .. 4 rh + 3 of the warp's eight
+  const int kp = lane & 15, rh = lane >> 4;
+  float m[4], l[4];
+  uint64_t o[RPW / 2][DPL];   // O~ of rows 2 i and 2 i + 1 of the warp, feature DPL * lane + c
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { m[i] = -INFINITY; l[i] = 0.f; }
+#pragma unroll
+  for (int i = 0; i < RPW / 2; ++i)
+#pragma unroll
+    for (int c = 0; c < DPL; ++c) o[i][c] = 0ull;
+  const bool rows = warp * RPW < it.nrows;   // this warp has rows (the others only help loading)
+  float* const Pw = sm + SM::P + warp * KT * RPW;
+  const float* const qw = sm + SM::Q + (warp * RPW + 4 * rh) * SM::QS;
+
+  while (t < t_end) {
+    const int tn = next_tile(t + 1);
+    cp_async_wait<1>();        // this tile's keys
+    __syncthreads();
+    // (each score in two halves: the even and the odd features)
+    uint64_t s0[4] = {0ull, 0ull, 0ull, 0ull}, s1[4] = {0ull, 0ull, 0ull, 0ull};
+    if (rows) {
+      const float* ka = Ks + kp * SM::KS;
+      const float* kb = ka + 16 * SM::KS;
+#pragma unroll 4
+      for (int c = 0; c < D; c += 4) {
+        const ulonglong2 va = *reinterpret_cast<const ulonglong2*>(ka + c), vb = *reinterpret_cast<const ulonglong2*>(kb + c);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(qw + i * SM::QS + c);
+          s0[i] = fma2(q.x, va.x, s0[i]); s1[i] = fma2(q.x, vb.x, s1[i]);
+          s0[i] = fma2(q.y, va.y, s0[i]); s1[i] = fma2(q.y, vb.y, s1[i]);
+        }
+      }
+    }
+    cp_async_wait<0>();        // this tile's values
+    __syncthreads();            // (and every warp has read the keys)
+    if (tn < t_end) load_keys(tn);
+    if (rows) {
+      const int key0 = k0 + t * KT + kp, key1 = key0 + 16;
+      const bool ok0 = key0 < k1 && !(key0 >= x0 && key0 < x1), ok1 = key1 < k1 && !(key1 >= x0 && key1 < x1);
+      float alpha[4];
+      float4 p0, p1;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 h0 = unpack2(s0[i]), h1 = unpack2(s1[i]);
+        const float a0 = ok0 ? (h0.x + h0.y) * g.scale_log2 : -INFINITY, a1 = ok1 ? (h1.x + h1.y) * g.scale_log2 : -INFINITY;
+        float mx = fmaxf(a0, a1);
+#pragma unroll
+        for (int x = 8; x > 0; x >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, x));
+        const float m_new = fmaxf(m[i], mx);
+        const float m_use = m_new == -INFINITY ? 0.f : m_new;
+        alpha[i] = m[i] == -INFINITY ? 0.f : exp2f(m[i] - m_new);
+        m[i] = m_new;
+        const float e0 = ok0 ? exp2f(a0 - m_use) : 0.f, e1 = ok1 ? exp2f(a1 - m_use) : 0.f;
+        l[i] = l[i] * alpha[i] + (e0 + e1);
+        (&p0.x)[i] = e0;
+        (&p1.x)[i] = e1;
+      }
+      *reinterpret_cast<float4*>(Pw + kp * RPW + 4 * rh) = p0;
+      *reinterpret_cast<float4*>(Pw + (kp + 16) * RPW + 4 * rh) = p1;
+      if (__any_sync(0xffffffffu, alpha[0] != 1.f || alpha[1] != 1.f || alpha[2] != 1.f || alpha[3] != 1.f)) {
+#pragma unroll
+        for (int i = 0; i < RPW / 2; ++i) {
+          const int src = (i >> 1) * 16;   // the lanes of rows 0..3 / 4..7
+          const uint64_t al = pack2(__shfl_sync(0xffffffffu, alpha[(2 * i) & 3], src), __shfl_sync(0xffffffffu, alpha[(2 * i + 1) & 3], src));
+#pragma unroll
+          for (int c = 0; c < DPL; ++c) o[i][c] = mul2(o[i][c], al);
+        }
+      }
+      __syncwarp();
+      // O~ += P~ V: lane = features DPL * lane .. of the warp's eight rows
+      const float* vl = Vs + lane * DPL;
+#pragma unroll 4
+      for (int j = 0; j < KT; ++j) {
+        const ulonglong2 pa = *reinterpret_cast<const ulonglong2*>(Pw + j * RPW), pb = *reinterpret_cast<const ulonglong2*>(Pw + j * RPW + 4);
+        float v[DPL];
+        if (DPL == 4) *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(vl + j * D);
+        else *reinterpret_cast<float2*>(v) = *reinterpret_cast<const float2*>(vl + j * D);
+#pragma unroll
+        for (int c = 0; c < DPL; ++c) {
+          const uint64_t vv = pack2(v[c], v[c]);
+          o[0][c] = fma2(pa.x, vv, o[0][c]); o[1][c] = fma2(pa.y, vv, o[1][c]);
+          o[2][c] = fma2(pb.x, vv, o[2][c]); o[3][c] = fma2(pb.y, vv, o[3][c]);
+        }
+      }
+    }
+    __syncthreads();            // every warp has read the values
+    if (tn < t_end) load_values(tn);
+    t = tn;
+  }
+
+  grid_launch_dependents();
+  // this warp's partial state of its rows to shared memory (every warp has left the keys behind)
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int x = 8; x > 0; x >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], x);
+  if (rows) {
+#pragma unroll
+    for (int i = 0; i < RPW / 2; ++i) {
+      float* dst = Ks + (warp * RPW + 2 * i) * D + lane * DPL;
+      float2 h[DPL];
+#pragma unroll
+      for (int c = 0; c < DPL; ++c) h[c] = unpack2(o[i][c]);
+      if (DPL == 4) {
+        *reinterpret_cast<float4*>(dst) = make_float4(h[0].x, h[1].x, h[2 % DPL].x, h[3 % DPL].x);
+        *reinterpret_cast<float4*>(dst + D) = make_float4(h[0].y, h[1].y, h[2 % DPL].y, h[3 % DPL].y);
+      } else {
+        *reinterpret_cast<float2*>(dst) = make_float2(h[0].x, h[1].x);
+        *reinterpret_cast<float2*>(dst + D) = make_float2(h[0].y, h[1].y);
+      }
+    }
+    if (kp == 0) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<float2*>(sm + SM::ML + (warp * RPW + 4 * rh + i) * 2) = make_float2(m[i], l[i]);
     }
   }
+  // the partial states of a row -- one of every CTA of the cluster, and the cached state -- merged (Eq. 2-6),
+  // 16 bytes of a row per thread; a split unit's rows are dealt out over its CTAs
+  if (n_parts > 1) cluster_sync_all();
+  else __syncthreads();
+  const float LN2 = 0.69314718055994530942f;
+  const uint32_t sm_base = smem_u32(sm);
+  const int my_rows = (it.nrows - part + n_parts - 1) / n_parts;
+  for (int i = threadIdx.x; i < my_rows * D4; i += THREADS) {
+    const int r = part + (i / D4) * n_parts, c4 = i % D4;
+    const int tok = it.row0 + r;
+    const size_t srow = (size_t)h * g.Tp + tok;
+    float M = -INFINITY, L = 0.f;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (from_state) {
+      M = a.st.m[srow];
+      L = a.st.l[srow];
+      acc = *reinterpret_cast<const float4*>(a.st.o + srow * D + c4 * 4);
+    }
+    for (int p0 = 0; p0 < n_parts; p0 += 4) {
+      float2 ml[4];
+      float4 v[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {   // (the loads of four parts leave together)
+        const uint32_t base = n_parts > 1 ? mapa_shared(sm_base, (uint32_t)min(p0 + k, n_parts - 1)) : sm_base;
+        ml[k] = ld_cluster_v2(base + (SM::ML + r * 2) * 4);
+        v[k] = ld_cluster_v4(base + (SM::K + r * D + c4 * 4) * 4);
+      }
+      float Mn = M;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) Mn = fmaxf(Mn, ml[k].x);
+      const float w0 = M == -INFINITY ? 0.f : exp2f(M - Mn);
+      L *= w0; acc.x *= w0; acc.y *= w0; acc.z *= w0; acc.w *= w0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const float w = (p0 + k >= n_parts || ml[k].x == -INFINITY) ? 0.f : exp2f(ml[k].x - Mn);
+        L = fmaf(ml[k].y, w, L);
+        acc.x = fmaf(v[k].x, w, acc.x); acc.y = fmaf(v[k].y, w, acc.y);
+        acc.z = fmaf(v[k].z, w, acc.z); acc.w = fmaf(v[k].w, w, acc.w);
+      }
+      M = Mn;
+    }
+    if (to_state) {
+      if (c4 == 0) { a.st.m[srow] = M; a.st.l[srow] = L; }
+      *reinterpret_cast<float4*>(a.st.o + srow * D + c4 * 4) = acc;
+    } else {
+      const float inv = 1.f / L;
+      const size_t orow = (size_t)tok * g.Hq + h;
+      acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
+      if (a.out_bf16) {
+        const __nv_bfloat162 b0 = __floats2bfloat162_rn(acc.x, acc.y), b1 = __floats2bfloat162_rn(acc.z, acc.w);
+        uint2 u;
+        u.x = *reinterpret_cast<const uint32_t*>(&b0);
+        u.y = *reinterpret_cast<const uint32_t*>(&b1);
+        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.out) + orow * D + c4 * 4) = u;
+      } else {
+        *reinterpret_cast<float4*>(a.out + orow * D + c4 * 4) = acc;
+      }
+      if (a.lse && c4 == 0) a.lse[orow] = (M + log2f(L)) * LN2;
+    }
+  }
+  if (n_parts > 1) cluster_sync_all();   // the partner CTAs may still read this one's shared memory
 }
 
 template <int D>
-constexpr size_t simt_smem() {
-  return sizeof(float) * (SIMT_ROWS * D + KT * (D + 1) + KT * D);
+cudaError_t launch(const Geometry& g, const AttnArgs& a, int n_ctas, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)n_ctas, (unsigned)g.Hq);
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = Smem<D>::bytes;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  int n_attr = 0;
+  if (!a.no_pdl) {
+    attr[n_attr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n_attr++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (a.split_ctas > 1) {
+    attr[n_attr].id = cudaLaunchAttributeClusterDimension;
+    attr[n_attr].val.clusterDim.x = (unsigned)a.split_ctas;
+    attr[n_attr].val.clusterDim.y = 1;
+    attr[n_attr++].val.clusterDim.z = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = n_attr;
+  return cudaLaunchKernelEx(&cfg, simt_attn_kernel<D>, g, a);
 }
 
 }  // namespace
 
 cudaError_t simt_prepare() {
   cudaError_t e = cudaFuncSetAttribute(simt_attn_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)simt_smem<128>());
+                                       (int)Smem<128>::bytes);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(simt_attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)simt_smem<64>());
+                              (int)Smem<64>::bytes);
 }
 
-cudaError_t simt_attention(const Geometry& g, const AttnArgs& a, cudaStream_t s) {
+cudaError_t simt_attention(const Geometry& g, const AttnArgs& args, int num_sms, cudaStream_t s) {
+  AttnArgs a = args;
   if (a.n_items == 0) return cudaSuccess;
-  dim3 grid(a.n_items, g.Hq);
-  if (g.d == 128)
-    simt_attn_kernel<128><<<grid, WARPS * 32, simt_smem<128>(), s>>>(g, a);
-  else
-    simt_attn_kernel<64><<<grid, WARPS * 32, simt_smem<64>(), s>>>(g, a);
-  return cudaGetLastError();
+  // Units with the long key range: the block queries of a step (its first items), every unit otherwise.  They
+  // are cut into parts of at least two tiles; of one where even that leaves SMs without a CTA, because a
+  // part's chain of tiles is then all the launch takes.
+  const bool step = a.mode == MODE_STEP;
+  if (!step) a.n_split_items = a.n_items;
+  const int rest = a.n_items - a.n_split_items;
+  const int max_tiles = (g.maxN + KT - 1) / KT;
+  int S = std::min(MAX_SPLIT, std::max(1, max_tiles / 2));
+  if ((long long)(a.n_split_items * S + rest) * g.Hq < num_sms) S = std::min(MAX_SPLIT, max_tiles);
+  a.split_ctas = S;
+  const int n_ctas = a.n_split_items * S + (rest + S - 1) / S * S;
+  return g.d == 128 ? launch<128>(g, a, n_ctas, s) : launch<64>(g, a, n_ctas, s);
 }
 
 }  // namespace lacache

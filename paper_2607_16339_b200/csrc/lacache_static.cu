@@ -35,6 +35,7 @@ static __device__ __align__(256) float g_static_scratch[STATIC_WORDS];
 
 constexpr int MAX_DEVICES = 64;
 float* g_scratch_dev[MAX_DEVICES];  // device address of the array, per device (nullptr = not set up)
+int g_num_sms[MAX_DEVICES];
 // What the tables and metadata in a device's copy of the array were last filled for: a call with the same
 // (n_tokens, head_dim, rope_theta) finds them as it needs them and copies nothing.
 struct Filled { int n_tokens, head_dim; float theta; };
@@ -86,6 +87,8 @@ extern "C" lacache_status lacache_full_recompute_static(int dtype, int n_tokens,
     e = cudaGetSymbolAddress((void**)&p, g_static_scratch);
     if (e != cudaSuccess || !p) return fail(LACACHE_ERR_CUDA, cudaGetErrorString(e));
     e = simt_prepare();
+    if (e != cudaSuccess) return fail(LACACHE_ERR_CUDA, cudaGetErrorString(e));
+    e = cudaDeviceGetAttribute(&g_num_sms[dev], cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return fail(LACACHE_ERR_CUDA, cudaGetErrorString(e));
     g_scratch_dev[dev] = p;
   }
@@ -161,6 +164,6 @@ extern "C" lacache_status lacache_full_recompute_static(int dtype, int n_tokens,
   a.rot = r.dst;
   a.out = out;
   a.lse = lse;
-  if ((e = simt_attention(g, a, s)) != cudaSuccess) return fail(LACACHE_ERR_CUDA, cudaGetErrorString(e));
+  if ((e = simt_attention(g, a, g_num_sms[dev], s)) != cudaSuccess) return fail(LACACHE_ERR_CUDA, cudaGetErrorString(e));
   return LACACHE_OK;
 }
