@@ -1,0 +1,283 @@
+// Q/K/V projection of many tokens, Y = X^ W^T (token-wise producer, lacache_qkv.cu): a plain tensor-core GEMM, where
+// the stream-K kernel of lacache_qkv.cu, made for the few tokens of a block, is bound by what it moves through L2 (a
+// 128 x 256 tile per SM reads 48 KB per 512 cycles: 26 TB/s over 148 SMs) and by its element-wise stores.
+//
+// Pairs of CTAs (clusters of two, tcgen05 cta_group::2) compute tiles of 256 tokens x 256 features (two heads): each
+// CTA stages its 128 tokens and its 128 features of a 64-wide k chunk (32 KB), the pair's MMAs (M 256, N 256) read both
+// CTAs' operands, and each CTA's TMEM receives its 128 tokens x 256 features.  Two accumulators alternate, so that the
+// rows of one tile are stored while the next is computed.
+//   warp 0 (one lane)  producer of this CTA's operands; every load counts its bytes on the leader's barrier
+//   warp 1             (leader CTA, one elected lane) issues the pair's MMAs
+//   warps 2..5         epilogue: TMEM lane = token; bf16 rows through 4 KB of staging per warp, so that a store
+//                      instruction writes 128 contiguous bytes of each of four rows
+// Tiles are dealt out with the token tiles running fastest: the clusters at work share few feature tiles, and both
+// operands of what they share stay in L2.
+#include <cuda.h>
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+#include "lacache_internal.h"
+#include "lacache_proj.h"
+#include "lacache_ptx.h"
+
+namespace lacache {
+namespace {
+
+using namespace ptx;
+
+constexpr int HD = 128;                  // head_dim: features per head
+constexpr int BK = 64;                   // k chunk: one 128-byte swizzled row
+constexpr int THREADS = 192;
+constexpr uint32_t HALF = 128 * BK * 2;  // 16 KB: one operand of one CTA
+constexpr uint32_t STAGE = 2 * HALF;
+constexpr int STAGES = 6;
+constexpr uint32_t SM_ST = STAGES * STAGE;            // 4 x 4 KB of staging
+constexpr uint32_t SM_BAR = SM_ST + 4 * 4096;
+enum { B_FULL = 0, B_FREE = STAGES, B_ACC_FULL = 2 * STAGES, B_ACC_FREE = B_ACC_FULL + 2, N_BARS = B_ACC_FREE + 2 };
+constexpr uint32_t SM_TOTAL = SM_BAR + 8 * N_BARS + 16;
+static_assert(SM_TOTAL <= 232448, "exceeds the 227 KB per-CTA limit");
+enum { LOC_FULL = 111, LOC_FREE = 112, LOC_ACC_FULL = 113, LOC_ACC_FREE = 114 };
+
+struct Pc {
+  uint32_t base;
+  volatile int* abort_flag;
+  int32_t* status;
+  long long wait_cycles;
+  __device__ __forceinline__ uint32_t bar(int slot) const { return base + SM_BAR + 8u * slot; }
+};
+// (every barrier here is signalled by the other CTA too: acquire at cluster scope)
+__device__ __forceinline__ bool wait(const Pc& c, int slot, uint32_t parity, int loc) {
+  const uint32_t b = c.bar(slot);
+  if (mbar_try_acquire_cluster(b, parity)) return true;
+  const long long t0 = clock64();
+  for (;;) {
+    if (mbar_try_acquire_cluster(b, parity)) return true;
+    if (*c.abort_flag) return false;
+    if (clock64() - t0 > c.wait_cycles) {
+      *c.abort_flag = 1;
+      if (atomicCAS(c.status, 0, (int)LACACHE_ERR_TIMEOUT) == 0) {
+        c.status[1] = loc; c.status[2] = blockIdx.x; c.status[3] = threadIdx.x;
+      }
+      return false;
+    }
+  }
+}
+// a load into this CTA's shared memory that counts its bytes on a barrier of the pair's leader
+__device__ __forceinline__ void load_pair(uint32_t dst, const CUtensorMap* map, uint32_t cluster_bar, int c0, int c1) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.cta_group::2 [%0], [%1, {%3, %4}], [%2];"
+      ::"r"(dst), "l"(map), "r"(cluster_bar), "r"(c0), "r"(c1)
+      : "memory");
+}
+__device__ __forceinline__ void mma_pair(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+      ::"r"(d_tmem), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// one arrival on the barrier at this offset in both CTAs, when every MMA issued so far is complete
+__device__ __forceinline__ void commit_pair(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+               "h"((uint16_t)3)
+               : "memory");
+}
+
+struct Tile { int tt, nt; };   // token tile, pair of heads
+__device__ __forceinline__ Tile tile_of(const ProjArgs& a, int i) { return Tile{i % a.n_ttiles, i / a.n_ttiles}; }
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(THREADS, 1)
+proj_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant__ CUtensorMap x_map, const __grid_constant__ ProjArgs a) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
+  const uint32_t rank = cluster_ctarank();
+  Pc c;
+  c.base = smem_u32(smem_raw);
+  uint32_t* words = reinterpret_cast<uint32_t*>(smem_raw + SM_BAR + 8 * N_BARS);  // [0] tmem, [1] abort
+  c.abort_flag = reinterpret_cast<volatile int*>(words + 1);
+  c.status = a.status;
+  c.wait_cycles = a.wait_cycles;
+  if (tid == 0) {
+    prefetch_map(&w_map);
+    prefetch_map(&x_map);
+    for (int i = 0; i < N_BARS; ++i) mbar_init(c.bar(i), i >= B_ACC_FREE ? 8u : 1u);   // (8: the epilogue warps of both CTAs)
+    words[1] = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async_smem();
+  }
+  __syncwarp();
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(words)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();   // both CTAs' barriers and TMEM are ready
+  tc_fence_after();
+  const uint32_t tmem = words[0];
+  const int first = (int)blockIdx.x >> 1, stride = (int)gridDim.x >> 1;   // this pair's tiles
+
+  if (warp == 0) {
+    if (tid == 0) {
+      // the weights do not depend on the norm kernel ahead, which writes the operand rows: the first ring of them is
+      // requested before the wait
+      int early = 0;
+      if (first < a.n_tiles) {
+        const int head = tile_of(a, first).nt * 2 + (int)rank;
+        early = min(STAGES, a.kc);
+        for (int k = 0; k < early; ++k) {
+          if (rank == 0) mbar_expect_tx(c.bar(B_FULL + k), 2 * STAGE);   // both CTAs' operands
+          load_pair(c.base + k * STAGE + HALF, &w_map, mapa_shared(c.bar(B_FULL + k), 0), 0, (head * a.kc + k) * HD);
+        }
+      }
+      grid_dependency_wait();
+      int s = 0;
+      uint32_t ph = 0;
+      for (int i = first; i < a.n_tiles; i += stride) {
+        const Tile t = tile_of(a, i);
+        const int row = t.tt * 256 + (int)rank * 128, head = t.nt * 2 + (int)rank;
+        bool ok = true;
+        for (int k = 0; k < a.kc && ok; ++k) {
+          ok = wait(c, B_FREE + s, ph ^ 1u, LOC_FREE);
+          if (!ok) break;
+          const uint32_t dst = c.base + s * STAGE, lead = mapa_shared(c.bar(B_FULL + s), 0);
+          const bool have_w = i == first && k < early;
+          if (rank == 0 && !have_w) mbar_expect_tx(c.bar(B_FULL + s), 2 * STAGE);
+          load_pair(dst, &x_map, lead, k * BK, row);
+          if (!have_w) load_pair(dst + HALF, &w_map, lead, 0, (head * a.kc + k) * HD);  // (a head past the last: rows of zeros)
+          if (++s == STAGES) { s = 0; ph ^= 1u; }
+        }
+        if (!ok) break;
+      }
+      // every load of this CTA has been requested: the kernel behind may be scheduled (it waits for this grid)
+      asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    }
+  } else if (warp == 1) {
+    if (rank == 0) {
+      const uint32_t idesc = idesc_f16(1u /*bf16*/, 0u, 256, 256);
+      const bool leader = elect_one();
+      int s = 0, n = 0;
+      uint32_t ph = 0;
+      bool ok = true;
+      for (int i = first; i < a.n_tiles && ok; i += stride, ++n) {
+        const int buf = n & 1;
+        ok = wait(c, B_ACC_FREE + buf, ((uint32_t)(n >> 1) & 1u) ^ 1u, LOC_ACC_FREE);   // drained by both CTAs' epilogues
+        if (!ok) break;
+        tc_fence_after();
+        for (int k = 0; k < a.kc; ++k) {
+          ok = wait(c, B_FULL + s, ph, LOC_FULL);
+          if (!ok) break;
+          tc_fence_after();
+          const uint64_t ad = smem_desc(c.base + s * STAGE, 16, 1024), bd = smem_desc(c.base + s * STAGE + HALF, 16, 1024);
+          if (leader) {
+#pragma unroll
+            for (int ks = 0; ks < BK / 16; ++ks)
+              mma_pair(tmem + 256u * buf, ad + 2u * ks, bd + 2u * ks, idesc, (k > 0 || ks > 0) ? 1u : 0u);
+            commit_pair(c.bar(B_FREE + s));
+          }
+          if (++s == STAGES) { s = 0; ph ^= 1u; }
+        }
+        if (ok && leader) commit_pair(c.bar(B_ACC_FULL + buf));
+      }
+    }
+  } else {
+    const int quad = warp & 3;                     // the TMEM lanes this warp may read
+    uint8_t* const st = smem_raw + SM_ST + (warp - 2) * 4096;
+    int n = 0;
+    for (int i = first; i < a.n_tiles; i += stride, ++n) {
+      const Tile t = tile_of(a, i);
+      const int buf = n & 1;
+      if (!wait(c, B_ACC_FULL + buf, (uint32_t)(n >> 1) & 1u, LOC_ACC_FULL)) break;
+      tc_fence_after();
+      const int t0 = t.tt * 256 + (int)rank * 128 + quad * 32;   // the warp's first token
+      const int rows = min(a.n_tokens - t0, 32);
+      const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16) + 256u * buf;
+      if (n == 0) grid_dependency_wait();   // results may overwrite rows that a grid ahead in the stream still reads
+#pragma unroll 1
+      for (int cb = 0; cb < 4; ++cb) {             // 64 features: half a head
+        const int head = t.nt * 2 + (cb >> 1);
+        uint32_t r[64];
+        tmem_ld32(acc + 64 * cb, *reinterpret_cast<uint32_t(*)[32]>(r));
+        tmem_ld32(acc + 64 * cb + 32, *reinterpret_cast<uint32_t(*)[32]>(r + 32));
+        tmem_ld_wait();
+        if (cb == 3) {   // the accumulator may be overwritten
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(mapa_shared(c.bar(B_ACC_FREE + buf), 0));
+        }
+        if (rows <= 0 || head >= a.n_heads) continue;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          uint32_t p[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const __nv_bfloat162 b = __floats2bfloat162_rn(__uint_as_float(r[8 * j + 2 * e]), __uint_as_float(r[8 * j + 2 * e + 1]));
+            p[e] = *reinterpret_cast<const uint32_t*>(&b);
+          }
+          *reinterpret_cast<uint4*>(st + lane * 128 + ((j ^ (lane & 7)) << 4)) = make_uint4(p[0], p[1], p[2], p[3]);
+        }
+        __syncwarp();
+        __nv_bfloat16* dst;
+        int H, h;
+        if (head < a.Hq) { dst = a.q; H = a.Hq; h = head; }
+        else if (head < a.Hq + a.Hkv) { dst = a.k; H = a.Hkv; h = head - a.Hq; }
+        else { dst = a.v; H = a.Hkv; h = head - a.Hq - a.Hkv; }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const int rr = 4 * j + (lane >> 3), ch = lane & 7;
+          if (rr < rows) {
+            int tok = t0 + rr;
+            if (a.dst_rows) tok = __ldg(a.dst_rows + tok);
+            if (!a.dst_rows || (unsigned)tok < (unsigned)a.max_rows)   // (a row out of range is reported by the norm kernel)
+              *reinterpret_cast<uint4*>(dst + ((size_t)tok * H + h) * HD + 64 * (cb & 1) + 8 * ch) =
+                  *reinterpret_cast<const uint4*>(st + rr * 128 + ((ch ^ (rr & 7)) << 4));
+          }
+        }
+        __syncwarp();
+      }
+    }
+  }
+  __syncwarp();
+  grid_dependency_wait();   // this grid must not complete before the grids ahead of it have
+  if (*c.abort_flag) {
+    // a bounded wait ran out: what was issued before that gets a fixed 50 us to land
+    const long long t0 = clock64();
+    while (clock64() - t0 < 100000ll) {
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();       // neither CTA leaves while the other may still use its shared memory or TMEM
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+  }
+}
+
+}  // namespace
+
+cudaError_t proj_prepare() {
+  return cudaFuncSetAttribute(proj_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
+}
+
+cudaError_t proj_many(const CUtensorMap& w_map, const CUtensorMap& x_map, ProjArgs a, int num_sms, bool pdl, cudaStream_t s) {
+  a.n_heads = a.Hq + 2 * a.Hkv;
+  a.n_ttiles = (a.n_tokens + 255) / 256;
+  a.n_tiles = a.n_ttiles * ((a.n_heads + 1) / 2);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(2 * std::min(a.n_tiles, std::max(1, num_sms / 2))));
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = SM_TOTAL;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, proj_kernel, w_map, x_map, a);
+}
+
+}  // namespace lacache

@@ -33,6 +33,7 @@
 #include <new>
 
 #include "lacache_internal.h"
+#include "lacache_proj.h"
 #include "lacache_ptx.h"
 
 using namespace lacache;
@@ -57,7 +58,7 @@ struct lacache_qkv {
   const void* full_owner = nullptr;     // the context whose tokens q / k / v currently hold
   int full_tokens = 0;
   CUtensorMap w_map;
-  CUtensorMap x_map[4];                 // boxes of 32, 64, 128, 256 tokens
+  CUtensorMap x_map[3];                 // boxes of 32, 64, 128 tokens
   cudaEvent_t ev_start = nullptr, ev_stop = nullptr;
   int last_launches = 0;
   // experiment knobs, read from the environment once at create
@@ -74,7 +75,8 @@ using namespace ptx;
 
 constexpr int QD = 128;                 // head_dim = features per tile = MMA M
 constexpr int BK = 64;                  // k chunk: one 128-byte swizzled row of bf16
-constexpr int MAX_TN = 256;
+constexpr int MAX_TN = 64;               // tokens per tile (more tokens: lacache_proj.cu)
+constexpr int ROW_PAD = 256;             // the operand buffer's rows: whole tiles of lacache_proj.cu
 constexpr int G_THREADS = 192;
 constexpr int EPI_THREADS = 128;
 constexpr uint32_t A_BYTES = QD * BK * 2;
@@ -858,7 +860,7 @@ lacache_status lacache_qkv_create(const lacache_qkv_config* cfg, lacache_qkv** o
   p->cfg = *cfg;
   p->err[0] = 0;
   p->n_ftiles = cfg->n_q_heads + 2 * cfg->n_kv_heads;
-  p->tokens_pad = (cfg->max_tokens + MAX_TN - 1) / MAX_TN * MAX_TN;
+  p->tokens_pad = (cfg->max_tokens + ROW_PAD - 1) / ROW_PAD * ROW_PAD;
   lacache_status st = LACACHE_OK;
   auto attempt = [&]() -> lacache_status {
     p->no_pdl = getenv("LACACHE_NO_PDL") != nullptr;
@@ -893,8 +895,9 @@ lacache_status lacache_qkv_create(const lacache_qkv_config* cfg, lacache_qkv** o
     QCU_TRY(p, cudaDeviceSynchronize());
     // the packed copy as a matrix of 64 columns: a tile is 128 consecutive rows
     if (!make_bf16_map(p, &p->w_map, p->w_packed, w_rows * (cfg->d_model / BK), BK, QD)) return LACACHE_ERR_CUDA;
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < 3; ++i)
       if (!make_bf16_map(p, &p->x_map[i], p->xhat, p->tokens_pad, cfg->d_model, 32 << i)) return LACACHE_ERR_CUDA;
+    QCU_TRY(p, proj_prepare());
     QCU_TRY(p, cudaFuncSetAttribute(qkv_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMQ_TOTAL));
     QCU_TRY(p, cudaFuncSetAttribute(qkv_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMQ_TOTAL));
     return LACACHE_OK;
@@ -985,9 +988,34 @@ lacache_status project_impl(lacache_qkv* p, const int32_t* token_ids, const void
     p->last_launches++;
   }
 
+  // Many tokens, or a model of few heads, whose tiles the stream-K split would cut into many parts each, go to the
+  // pair-of-CTAs GEMM.  Measured with its norm kernel (us, stream-K / GEMM): 96 heads x 4096: 38 / 42 at 32 tokens,
+  // 42 / 42 at 64, 48 / 42 at 96, 785 / 437 at 6411; 36 heads x 3584: 28 / 32 at 32, 36 / 32 at 96; 16 heads x 2048
+  // (9 parts a tile): 26 / 24 at 32, 34 / 24 at 64.
+  if ((n_tokens > MAX_TN || p->num_sms > 8 * p->n_ftiles) && !without_norm) {
+    ProjArgs pa{};
+    pa.n_tokens = n_tokens;
+    pa.kc = p->cfg.d_model / BK;
+    pa.Hq = p->cfg.n_q_heads;
+    pa.Hkv = p->cfg.n_kv_heads;
+    pa.q = reinterpret_cast<__nv_bfloat16*>(q);
+    pa.k = reinterpret_cast<__nv_bfloat16*>(k);
+    pa.v = reinterpret_cast<__nv_bfloat16*>(v);
+    pa.dst_rows = dst_rows;
+    pa.max_rows = max_rows;
+    pa.status = p->status;
+    pa.wait_cycles = p->wait_cycles > 0 ? p->wait_cycles : Q_WAIT_CYCLES;
+    const bool timed = p->ev_start && p->ev_stop;   // (an event between the two kernels: an ordinary launch)
+    if (timed) QCU_TRY(p, cudaEventRecord(p->ev_start, s));
+    QCU_TRY(p, proj_many(p->w_map, p->x_map[2], pa, p->num_sms, !no_pdl && !timed, s));
+    if (timed) QCU_TRY(p, cudaEventRecord(p->ev_stop, s));
+    p->last_launches++;
+    return LACACHE_OK;
+  }
+
   GemmArgs ga{};
   int tn_idx = 0;
-  while (tn_idx < 3 && (32 << tn_idx) < n_tokens) ++tn_idx;
+  while (tn_idx < 1 && (32 << tn_idx) < n_tokens) ++tn_idx;
   ga.n_tokens = n_tokens;
   ga.tn = 32 << tn_idx;
   ga.n_ttiles = (n_tokens + ga.tn - 1) / ga.tn;
@@ -1011,7 +1039,7 @@ lacache_status project_impl(lacache_qkv* p, const int32_t* token_ids, const void
   ga.status = p->status;
   const int n_ctas = (int)std::min<long long>(p->num_sms, ga.total_chunks);
   ga.hp = 0;
-  if (ga.tn <= 64 && n_ctas > ga.n_tiles && n_ctas < 2 * ga.n_tiles && !p->plain_split) {
+  if (n_ctas > ga.n_tiles && n_ctas < 2 * ga.n_tiles && !p->plain_split) {
     // closers take `per_closer` chunks each, helpers about HEAD_START chunks fewer
     const int HEAD_START = 8;
     const int n_helpers = n_ctas - ga.n_tiles;
