@@ -642,6 +642,7 @@ __global__ void qkv_pack_w_kernel(const uint4* __restrict__ w, uint4* __restrict
 // ---------------------------------------------------------------------------------------------------
 constexpr int N_THREADS = 256;
 constexpr int N_MAX_CHUNKS = 4;   // 8-element chunks per thread: d_model <= 8192
+constexpr int N_CTAS_PER_SM = 4;
 
 struct NormArgs {
   const int32_t* ids;             // or null
@@ -652,14 +653,19 @@ struct NormArgs {
   __nv_bfloat16* h_out;           // [n][d_model] or null
   const int32_t* dst_rows;        // or null; checked against max_rows here
   int max_rows;
-  int* ready;                     // incremented once this row of X^ is complete and visible
+  int* ready;                     // incremented once a row of X^ is complete and visible (null: nobody counts)
+  int n_tokens;
   int early_inputs;               // the inputs were complete before the preceding grid started: read them at once
   int d_model, vocab;
   float eps;
   int32_t* status;
 };
 
-__global__ void __launch_bounds__(N_THREADS) qkv_norm_kernel(const NormArgs a) {
+// A CTA walks the tokens blockIdx.x, blockIdx.x + gridDim.x, ...; with more tokens than resident CTAs, the row of the
+// next token is on its way while this one is reduced, and its id while that row is asked for (one token per CTA, every
+// access of the chain id -> row -> sum -> store exposed: 40 us for 6411 rows of 4096).  NC: chunks per thread.
+template <int NC>
+__global__ void __launch_bounds__(N_THREADS, NC > 2 ? 2 : N_CTAS_PER_SM) qkv_norm_kernel(const __grid_constant__ NormArgs a) {
   // The projection kernel may be scheduled now: before it waits for this grid it only sets itself up
   // and starts fetching weights.  This kernel is itself launched programmatically dependent and waits,
   // before its first load, for everything enqueued ahead of it (whatever wrote the token ids or hidden
@@ -667,91 +673,95 @@ __global__ void __launch_bounds__(N_THREADS) qkv_norm_kernel(const NormArgs a) {
   // (A caller that vouches for inputs that were complete before the grid ahead was even enqueued gets
   // the wait at the end instead: this kernel then runs alongside that grid, and still does not complete
   // before it, which is what the projection kernel's wait relies on.  The operand rows X^ it writes are
-  // read by nothing but the projection kernel of this call.)
+  // read by nothing but the projection kernel of this call.  h_out, a caller's buffer, is not written that way.)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (!a.early_inputs) grid_dependency_wait();
-  __shared__ float red[N_THREADS / 32];
-  const int t = blockIdx.x;
+  __shared__ float red[2][N_THREADS / 32];
   const int tid = threadIdx.x;
-  const __nv_bfloat16* src;
-  bool valid = true;
-  if (a.dst_rows && tid == 0) {
-    const int row = a.dst_rows[t];
-    if ((unsigned)row >= (unsigned)a.max_rows && atomicCAS(a.status, 0, (int)LACACHE_ERR_INVALID_ARG) == 0) {
-      a.status[1] = QLOC_ROW;
-      a.status[2] = t;
-      a.status[3] = row;
-    }
-  }
-  if (a.ids) {
-    const int id = a.ids[t];
-    valid = id >= 0 && id < a.vocab;
-    if (!valid && tid == 0 && atomicCAS(a.status, 0, (int)LACACHE_ERR_INVALID_ARG) == 0) {
-      a.status[1] = QLOC_TOKEN_ID;
-      a.status[2] = t;
-      a.status[3] = id;
-    }
-    src = a.table + (size_t)(valid ? id : 0) * a.d_model;
-  } else {
-    src = a.hidden + (size_t)t * a.d_model;
-  }
   const int n_chunks = a.d_model / 8;
-  uint4 raw[N_MAX_CHUNKS];
-  float ss = 0.f;
+  uint4 wraw[NC];
 #pragma unroll
-  for (int i = 0; i < N_MAX_CHUNKS; ++i) {
-    const int ch = tid + i * N_THREADS;
-    raw[i] = make_uint4(0, 0, 0, 0);
-    if (ch < n_chunks && valid) raw[i] = __ldg(reinterpret_cast<const uint4*>(src) + ch);
-    const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&raw[i]);
+  for (int i = 0; i < NC; ++i)
+    wraw[i] = tid + i * N_THREADS < n_chunks ? __ldg(reinterpret_cast<const uint4*>(a.weight) + tid + i * N_THREADS) : make_uint4(0, 0, 0, 0);
+  auto load_id = [&](int t) { return (a.ids && t < a.n_tokens) ? __ldg(a.ids + t) : 0; };
+  auto load_row = [&](int t, int id, uint4 (&raw)[NC]) {
+    const bool ok = t < a.n_tokens && (!a.ids || (id >= 0 && id < a.vocab));
+    const __nv_bfloat16* src = a.ids ? a.table + (size_t)(ok ? id : 0) * a.d_model : a.hidden + (size_t)(ok ? t : 0) * a.d_model;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float2 x = __bfloat1622float2(p[e]);
-      ss = fmaf(x.x, x.x, ss);
-      ss = fmaf(x.y, x.y, ss);
+    for (int i = 0; i < NC; ++i) {
+      const int ch = tid + i * N_THREADS;
+      raw[i] = (ok && ch < n_chunks) ? __ldg(reinterpret_cast<const uint4*>(src) + ch) : make_uint4(0, 0, 0, 0);
     }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-  if ((tid & 31) == 0) red[tid >> 5] = ss;
-  __syncthreads();
-  float tot = 0.f;
-#pragma unroll
-  for (int i = 0; i < N_THREADS / 32; ++i) tot += red[i];
-  // an invalid token id (reported through the status word) yields a zero row
-  const float rinv = valid ? 1.0f / sqrtf(tot / (float)a.d_model + a.eps) : 0.f;
-#pragma unroll
-  for (int i = 0; i < N_MAX_CHUNKS; ++i) {
-    const int ch = tid + i * N_THREADS;
-    if (ch >= n_chunks) continue;
-    const uint4 wraw = __ldg(reinterpret_cast<const uint4*>(a.weight) + ch);
-    const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&raw[i]);
-    const __nv_bfloat162* w = reinterpret_cast<const __nv_bfloat162*>(&wraw);
-    uint4 o;
-    __nv_bfloat162* q = reinterpret_cast<__nv_bfloat162*>(&o);
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const float2 x = __bfloat1622float2(p[e]);
-      const float2 g = __bfloat1622float2(w[e]);
-      q[e] = __floats2bfloat162_rn(x.x * rinv * g.x, x.y * rinv * g.y);
-    }
-    reinterpret_cast<uint4*>(a.xhat + (size_t)t * a.d_model)[ch] = o;
-    if (a.h_out && !a.early_inputs) reinterpret_cast<uint4*>(a.h_out + (size_t)t * a.d_model)[ch] = raw[i];
-  }
-  // publish the row: every thread's stores, then one count
-  __threadfence();
-  __syncthreads();
-  if (tid == 0) atomicAdd(a.ready, 1);
-  if (a.early_inputs) {
-    grid_dependency_wait();
-    if (a.h_out) {   // a caller's buffer: not before the grids ahead are complete
-#pragma unroll
-      for (int i = 0; i < N_MAX_CHUNKS; ++i) {
-        const int ch = tid + i * N_THREADS;
-        if (ch < n_chunks) reinterpret_cast<uint4*>(a.h_out + (size_t)t * a.d_model)[ch] = raw[i];
+  };
+  int t = blockIdx.x;
+  int id = load_id(t), id_nx = load_id(t + gridDim.x);
+  uint4 raw[NC];
+  load_row(t, id, raw);
+  int buf = 0;
+  for (; t < a.n_tokens; t += gridDim.x, buf ^= 1) {
+    uint4 nx[NC];
+    load_row(t + gridDim.x, id_nx, nx);
+    const int id_nn = load_id(t + 2 * gridDim.x);
+    const bool valid = !a.ids || (id >= 0 && id < a.vocab);
+    if (tid == 0) {
+      if (a.dst_rows) {
+        const int row = a.dst_rows[t];
+        if ((unsigned)row >= (unsigned)a.max_rows && atomicCAS(a.status, 0, (int)LACACHE_ERR_INVALID_ARG) == 0) {
+          a.status[1] = QLOC_ROW; a.status[2] = t; a.status[3] = row;
+        }
+      }
+      if (!valid && atomicCAS(a.status, 0, (int)LACACHE_ERR_INVALID_ARG) == 0) {
+        a.status[1] = QLOC_TOKEN_ID; a.status[2] = t; a.status[3] = id;
       }
     }
+    float ss = 0.f;
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&raw[i]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 x = __bfloat1622float2(p[e]);
+        ss = fmaf(x.x, x.x, ss);
+        ss = fmaf(x.y, x.y, ss);
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    if ((tid & 31) == 0) red[buf][tid >> 5] = ss;
+    __syncthreads();
+    float tot = 0.f;
+#pragma unroll
+    for (int i = 0; i < N_THREADS / 32; ++i) tot += red[buf][i];
+    // an invalid token id (reported through the status word) yields a zero row
+    const float rinv = valid ? 1.0f / sqrtf(tot / (float)a.d_model + a.eps) : 0.f;
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      const int ch = tid + i * N_THREADS;
+      if (ch >= n_chunks) continue;
+      const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&raw[i]);
+      const __nv_bfloat162* w = reinterpret_cast<const __nv_bfloat162*>(&wraw[i]);
+      uint4 o;
+      __nv_bfloat162* q = reinterpret_cast<__nv_bfloat162*>(&o);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 x = __bfloat1622float2(p[e]);
+        const float2 g = __bfloat1622float2(w[e]);
+        q[e] = __floats2bfloat162_rn(x.x * rinv * g.x, x.y * rinv * g.y);
+      }
+      reinterpret_cast<uint4*>(a.xhat + (size_t)t * a.d_model)[ch] = o;
+      if (a.h_out) reinterpret_cast<uint4*>(a.h_out + (size_t)t * a.d_model)[ch] = raw[i];
+    }
+    if (a.ready) {   // publish the row: every thread's stores, then one count
+      __threadfence();
+      __syncthreads();
+      if (tid == 0) atomicAdd(a.ready, 1);
+    }
+#pragma unroll
+    for (int i = 0; i < NC; ++i) raw[i] = nx[i];
+    id = id_nx;
+    id_nx = id_nn;
   }
+  if (a.early_inputs) grid_dependency_wait();
 }
 
 // ---------------------------------------------------------------------------------------------------
@@ -962,6 +972,7 @@ lacache_status project_impl(lacache_qkv* p, const int32_t* token_ids, const void
   na.h_out = reinterpret_cast<__nv_bfloat16*>(h_out);
   na.dst_rows = dst_rows;
   na.max_rows = max_rows;
+  na.n_tokens = n_tokens;
   na.early_inputs = early_inputs ? 1 : 0;
   na.ready = p->ready;
   na.d_model = p->cfg.d_model;
@@ -972,19 +983,20 @@ lacache_status project_impl(lacache_qkv* p, const int32_t* token_ids, const void
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   const bool no_pdl = p->no_pdl;
+  const bool many = (n_tokens > MAX_TN || p->num_sms > 8 * p->n_ftiles) && !without_norm;
   if (!without_norm) {
+    if (many) na.ready = nullptr;   // (the GEMM waits for the whole norm grid)
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(n_tokens);
+    cfg.gridDim = dim3((unsigned)std::min(n_tokens, N_CTAS_PER_SM * p->num_sms));
     cfg.blockDim = dim3(N_THREADS);
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = no_pdl ? 0 : 1;
-    QCU_TRY(p, cudaLaunchKernelEx(&cfg, qkv_norm_kernel, na));
-  }
-  // the norm kernel is enqueued and will publish its n_tokens rows: only now does the count the
-  // projection waits for move (a failed launch above leaves counter and target in step)
-  if (!without_norm) {
-    p->ready_target += (unsigned)n_tokens;
+    const int nc = (p->cfg.d_model / 8 + N_THREADS - 1) / N_THREADS;
+    QCU_TRY(p, cudaLaunchKernelEx(&cfg, nc == 1 ? qkv_norm_kernel<1> : nc == 2 ? qkv_norm_kernel<2> : nc == 3 ? qkv_norm_kernel<3> : qkv_norm_kernel<4>, na));
+    // the norm kernel is enqueued and will publish its n_tokens rows: only now does the count the
+    // projection waits for move (a failed launch above leaves counter and target in step)
+    if (!many) p->ready_target += (unsigned)n_tokens;
     p->last_launches++;
   }
 
@@ -992,7 +1004,7 @@ lacache_status project_impl(lacache_qkv* p, const int32_t* token_ids, const void
   // pair-of-CTAs GEMM.  Measured with its norm kernel (us, stream-K / GEMM): 96 heads x 4096: 38 / 42 at 32 tokens,
   // 42 / 42 at 64, 48 / 42 at 96, 785 / 437 at 6411; 36 heads x 3584: 28 / 32 at 32, 36 / 32 at 96; 16 heads x 2048
   // (9 parts a tile): 26 / 24 at 32, 34 / 24 at 64.
-  if ((n_tokens > MAX_TN || p->num_sms > 8 * p->n_ftiles) && !without_norm) {
+  if (many) {
     ProjArgs pa{};
     pa.n_tokens = n_tokens;
     pa.kc = p->cfg.d_model / BK;
