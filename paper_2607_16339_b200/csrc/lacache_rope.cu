@@ -40,81 +40,95 @@ __device__ __forceinline__ void store8_f16(void* plane, size_t off, const float 
   *reinterpret_cast<uint4*>(reinterpret_cast<__half*>(plane) + off) = rope_half8(y);
 }
 
-// One thread: 8 features c0..c0+7 of the first half and their partners at
-// c0 + d/2 of one (source row, head slot).  Head slots: [0,Hq) q heads,
-// [Hq,Hq+Hkv) k heads, [Hq+Hkv,Hq+2Hkv) v heads.
-template <bool TC>
-__global__ void __launch_bounds__(256) rope_write_kernel(Geometry g, RopeArgs a) {
+// One thread: 8 features c0 .. c0 + 7 of the first half and their partners at c0 + d/2, of one source row and HPT
+// consecutive heads of one tensor; cos and sin are loaded once for all of them (with one head per thread they are two
+// thirds of what a thread loads).  d/16 threads cover a row, a warp 32 / (d/16) consecutive rows, so that both the HPT
+// heads it reads per row and the rows it writes per head are contiguous.  blockIdx.y: group of HPT heads -- q, then k,
+// then v.  HPT = 4 from 65536 (row, head) pairs on (157 MB of bf16 rows in, as much out: 71 us with one head per thread,
+// 55 us = 5.7 TB/s with four; two and eight the same within 4 %), else 1: a block's rows are too few to fill the GPU with more per thread.
+template <bool TC, int HPT>
+__global__ void __launch_bounds__(256, HPT > 1 ? 3 : 1) rope_write_kernel(const __grid_constant__ Geometry g, const __grid_constant__ RopeArgs a) {
   // This kernel and the attention kernel behind it are launched programmatically dependent.  The attention
   // kernel reads this kernel's inputs, and state that the kernels ahead may have written, before it waits for
   // this grid: it may start only once those are complete, hence the order of the wait and the trigger.
   if (!a.early_inputs) asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int chunks = g.d / 16;
-  const int slots = g.Hq + 2 * g.Hkv;
-  const long long total = (long long)a.n_src_rows * slots * chunks;
-  long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (idx >= total) return;
-  int chunk = (int)(idx % chunks);
-  long long t = idx / chunks;
-  int slot = (int)(t % slots);
-  int r = (int)(t / slots);
-  int tok = a.row_tok ? a.row_tok[r] : (a.blk_start ? a.blk_start[r / a.block_len] + r % a.block_len : r);
-  const int half = g.d / 2;
-  const int c0 = chunk * 8;
-
+  const int shift = g.d == 128 ? 3 : 2;   // d / 16 chunks per row
+  const int chunk = threadIdx.x & ((1 << shift) - 1);
+  const int r = (int)blockIdx.x * (256 >> shift) + (int)(threadIdx.x >> shift);
+  if (r >= a.n_src_rows) return;
+  const int half = g.d / 2, c0 = chunk * 8;
+  int grp = blockIdx.y;
+  const int gq = (g.Hq + HPT - 1) / HPT, gk = (g.Hkv + HPT - 1) / HPT;
   const void* src;
-  int H, h;
-  int which;  // 0 q, 1 k, 2 v
-  if (slot < g.Hq) { src = a.q; H = g.Hq; h = slot; which = 0; }
-  else if (slot < g.Hq + g.Hkv) { src = a.k; H = g.Hkv; h = slot - g.Hq; which = 1; }
-  else { src = a.v; H = g.Hkv; h = slot - g.Hq - g.Hkv; which = 2; }
+  int H, which;  // 0 q, 1 k, 2 v
+  if (grp < gq) { src = a.q; H = g.Hq; which = 0; }
+  else if (grp < gq + gk) { src = a.k; H = g.Hkv; which = 1; grp -= gq; }
+  else { src = a.v; H = g.Hkv; which = 2; grp -= gq + gk; }
+  const int h0 = grp * HPT;
+  const int tok = a.row_tok ? a.row_tok[r] : (a.blk_start ? a.blk_start[r / a.block_len] + r % a.block_len : r);
+  const bool bf16_in = a.in_dtype == LACACHE_DTYPE_BF16;
 
-  float x1[8], x2[8], y1[8], y2[8];
-  size_t soff = ((size_t)r * H + h) * g.d;
-  rope_load8(src, soff + c0, a.in_dtype == LACACHE_DTYPE_BF16, x1);
-  rope_load8(src, soff + c0 + half, a.in_dtype == LACACHE_DTYPE_BF16, x2);
+  // (the rows as they come: converted they would take twice the registers)
+  constexpr int NR = TC ? 1 : 2;   // 16-byte words of 8 features (the tcgen05 engine's inputs are bf16)
+  uint4 raw[HPT][2][NR];
+#pragma unroll
+  for (int i = 0; i < HPT; ++i) {
+    const size_t soff = ((size_t)r * H + min(h0 + i, H - 1)) * g.d + c0;
+#pragma unroll
+    for (int e = 0; e < 2; ++e) rope_fetch8<NR>(src, soff + e * half, TC || bf16_in, raw[i][e]);
+  }
+  float cs[8], sn[8];
   if (which < 2) {
     const float4 *cp, *sp;
     if (a.row_cos) {
       cp = reinterpret_cast<const float4*>(a.row_cos + (size_t)r * half + c0);
       sp = reinterpret_cast<const float4*>(a.row_sin + (size_t)r * half + c0);
     } else {
-      int pos = a.pos_of_tok[tok];
+      const int pos = a.pos_of_tok[tok];
       cp = reinterpret_cast<const float4*>(a.cos_tab + (size_t)pos * half + c0);
       sp = reinterpret_cast<const float4*>(a.sin_tab + (size_t)pos * half + c0);
     }
-    float4 ca = cp[0], cb = cp[1], sa = sp[0], sb = sp[1];
-    float cs[8] = {ca.x, ca.y, ca.z, ca.w, cb.x, cb.y, cb.z, cb.w};
-    float sn[8] = {sa.x, sa.y, sa.z, sa.w, sb.x, sb.y, sb.z, sb.w};
-    rope_rotate8(x1, x2, cs, sn, y1, y2);
-  } else {
-#pragma unroll
-    for (int i = 0; i < 8; ++i) { y1[i] = x1[i]; y2[i] = x2[i]; }
+    const float4 ca = cp[0], cb = cp[1], sa = sp[0], sb = sp[1];
+    cs[0] = ca.x; cs[1] = ca.y; cs[2] = ca.z; cs[3] = ca.w; cs[4] = cb.x; cs[5] = cb.y; cs[6] = cb.z; cs[7] = cb.w;
+    sn[0] = sa.x; sn[1] = sa.y; sn[2] = sa.z; sn[3] = sa.w; sn[4] = sb.x; sn[5] = sb.y; sn[6] = sb.z; sn[7] = sb.w;
   }
   // Everything above read only this call's inputs and constant tables.  The stores below overwrite
   // cache rows that the previous step's attention kernel may still be reading when this kernel was
   // launched programmatically dependent on it: wait for that grid first (returns at once otherwise).
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  size_t doff = ((size_t)h * g.Tp + tok) * g.d;
-  if (TC) {
-    // tcgen05 storage: [head][feature half][Tp][64] (d = 128), each half of a row one 128-byte line
-    const size_t o1 = ((size_t)(2 * h) * g.Tp + tok) * 64 + c0;
-    const size_t o2 = ((size_t)(2 * h + 1) * g.Tp + tok) * 64 + c0;
-    if (which == 0) {
-      store8_split(a.dst.q_hi, a.dst.q_lo, o1, y1, g.op_f16 != 0);
-      store8_split(a.dst.q_hi, a.dst.q_lo, o2, y2, g.op_f16 != 0);
-    } else if (which == 1) {
-      store8_split(a.dst.k_hi, a.dst.k_lo, o1, y1, g.op_f16 != 0);
-      store8_split(a.dst.k_hi, a.dst.k_lo, o2, y2, g.op_f16 != 0);
+#pragma unroll
+  for (int i = 0; i < HPT; ++i) {
+    const int h = h0 + i;
+    if (h >= H) break;
+    float x1[8], x2[8], y1[8], y2[8];
+    rope_unpack8<NR>(raw[i][0], TC || bf16_in, x1);
+    rope_unpack8<NR>(raw[i][1], TC || bf16_in, x2);
+    if (which < 2) {
+      rope_rotate8(x1, x2, cs, sn, y1, y2);
     } else {
-      store8_f16(a.dst.v, o1, y1);
-      store8_f16(a.dst.v, o2, y2);
+#pragma unroll
+      for (int e = 0; e < 8; ++e) { y1[e] = x1[e]; y2[e] = x2[e]; }
     }
-  } else {
-    void* plane = which == 0 ? a.dst.q_hi : (which == 1 ? a.dst.k_hi : a.dst.v);
-    store8_f32(plane, doff + c0, y1);
-    store8_f32(plane, doff + c0 + half, y2);
+    if (TC) {
+      // tcgen05 storage: [head][feature half][Tp][64] (d = 128), each half of a row one 128-byte line
+      const size_t o1 = ((size_t)(2 * h) * g.Tp + tok) * 64 + c0;
+      const size_t o2 = ((size_t)(2 * h + 1) * g.Tp + tok) * 64 + c0;
+      if (which == 2) {
+        store8_f16(a.dst.v, o1, y1);
+        store8_f16(a.dst.v, o2, y2);
+      } else {
+        void* const hi = which == 0 ? a.dst.q_hi : a.dst.k_hi;
+        void* const lo = which == 0 ? a.dst.q_lo : a.dst.k_lo;
+        store8_split(hi, lo, o1, y1, g.op_f16 != 0);
+        store8_split(hi, lo, o2, y2, g.op_f16 != 0);
+      }
+    } else {
+      void* const plane = which == 0 ? a.dst.q_hi : (which == 1 ? a.dst.k_hi : a.dst.v);
+      const size_t doff = ((size_t)h * g.Tp + tok) * g.d + c0;
+      store8_f32(plane, doff, y1);
+      store8_f32(plane, doff + half, y2);
+    }
   }
 }
 
@@ -224,12 +238,14 @@ cudaError_t merge_chunk_states(const Geometry& g, const ChunkMergeArgs& a, cudaS
   return cudaLaunchKernelEx(&cfg, merge_chunk_states_kernel, g, a);
 }
 
-cudaError_t rope_write(const Geometry& g, const RopeArgs& a, int engine, cudaStream_t s) {
-  long long total = (long long)a.n_src_rows * (g.Hq + 2 * g.Hkv) * (g.d / 16);
-  if (total == 0) return cudaSuccess;
-  unsigned blocks = (unsigned)((total + 255) / 256);
+template <bool TC>
+static cudaError_t rope_launch(const Geometry& g, const RopeArgs& a, cudaStream_t s) {
+  const bool many = (long long)a.n_src_rows * (g.Hq + 2 * g.Hkv) >= 65536;
+  const int hpt = many ? 4 : 1;
+  const int rows_per_cta = 256 / (g.d / 16);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(blocks);
+  cfg.gridDim = dim3((unsigned)((a.n_src_rows + rows_per_cta - 1) / rows_per_cta),
+                     (unsigned)((g.Hq + hpt - 1) / hpt + 2 * ((g.Hkv + hpt - 1) / hpt)));
   cfg.blockDim = dim3(256);
   cfg.stream = s;
   cudaLaunchAttribute attr[1];
@@ -237,8 +253,12 @@ cudaError_t rope_write(const Geometry& g, const RopeArgs& a, int engine, cudaStr
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = a.no_pdl ? 0 : 1;
-  return engine == LACACHE_ENGINE_TCGEN05 ? cudaLaunchKernelEx(&cfg, rope_write_kernel<true>, g, a)
-                                          : cudaLaunchKernelEx(&cfg, rope_write_kernel<false>, g, a);
+  return many ? cudaLaunchKernelEx(&cfg, rope_write_kernel<TC, 4>, g, a) : cudaLaunchKernelEx(&cfg, rope_write_kernel<TC, 1>, g, a);
+}
+
+cudaError_t rope_write(const Geometry& g, const RopeArgs& a, int engine, cudaStream_t s) {
+  if (a.n_src_rows == 0) return cudaSuccess;
+  return engine == LACACHE_ENGINE_TCGEN05 ? rope_launch<true>(g, a, s) : rope_launch<false>(g, a, s);
 }
 
 cudaError_t export_buffers(const Geometry& g, const ExportArgs& a, int engine, cudaStream_t s) {

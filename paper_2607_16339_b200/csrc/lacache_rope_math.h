@@ -8,11 +8,22 @@
 
 namespace lacache {
 
-// 8 consecutive source features starting at element offset elem_off
-__device__ __forceinline__ void rope_load8(const void* base, size_t elem_off, bool bf16_in, float (&x)[8]) {
+// 8 consecutive source features starting at element offset elem_off: fetched (N 16-byte words: fp32 takes two), and
+// converted to fp32
+template <int N>
+__device__ __forceinline__ void rope_fetch8(const void* base, size_t elem_off, bool bf16_in, uint4 (&w)[N]) {
   if (bf16_in) {
-    uint4 u = *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(base) + elem_off);
-    const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&u);
+    w[0] = *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(base) + elem_off);
+  } else {
+    const uint4* p = reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(base) + elem_off);
+#pragma unroll
+    for (int i = 0; i < N; ++i) w[i] = p[i];
+  }
+}
+template <int N>
+__device__ __forceinline__ void rope_unpack8(const uint4 (&w)[N], bool bf16_in, float (&x)[8]) {
+  if (bf16_in) {
+    const __nv_bfloat162* p = reinterpret_cast<const __nv_bfloat162*>(&w[0]);
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       float2 f = __bfloat1622float2(p[i]);
@@ -20,11 +31,15 @@ __device__ __forceinline__ void rope_load8(const void* base, size_t elem_off, bo
       x[2 * i + 1] = f.y;
     }
   } else {
-    const float4* p = reinterpret_cast<const float4*>(reinterpret_cast<const float*>(base) + elem_off);
-    float4 a = p[0], b = p[1];
-    x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w;
-    x[4] = b.x; x[5] = b.y; x[6] = b.z; x[7] = b.w;
+    const float* p = reinterpret_cast<const float*>(&w[0]);
+#pragma unroll
+    for (int i = 0; i < 4 * N; ++i) x[i] = p[i];
   }
+}
+__device__ __forceinline__ void rope_load8(const void* base, size_t elem_off, bool bf16_in, float (&x)[8]) {
+  uint4 w[2];
+  rope_fetch8<2>(base, elem_off, bf16_in, w);
+  rope_unpack8<2>(w, bf16_in, x);
 }
 
 // (x1, x2) = features (c, c + d/2) rotated by the angle whose cos / sin are given;
