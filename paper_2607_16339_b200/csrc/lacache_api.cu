@@ -49,7 +49,6 @@ struct lacache_ctx {
     bool no_deep = false;    // LACACHE_NO_DEEP: earlier merge variant
     bool no_qcomp = false;   // LACACHE_NO_QCOMP: no in-kernel rotation of first units
     bool no_pack = false;    // LACACHE_NO_PACK: no head packing of GQA block queries
-    bool no_staged_state = false;   // LACACHE_NO_STAGED_STATE: builds store the cached state from the row threads
     bool no_pair = false;    // LACACHE_NO_PAIR: no paired CTAs (thread-block clusters) for two-chunk block rows
     bool no_chunked_advance = false;  // LACACHE_NO_CHUNKED_ADVANCE: an advance computes the finished block's rows as key-window units
     bool verbose = false;    // LACACHE_VERBOSE: prints the step plan
@@ -202,7 +201,6 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
     k.no_qcomp = getenv("LACACHE_NO_QCOMP") != nullptr;
     k.no_pack = getenv("LACACHE_NO_PACK") != nullptr;
     k.no_pair = getenv("LACACHE_NO_PAIR") != nullptr;
-    k.no_staged_state = getenv("LACACHE_NO_STAGED_STATE") != nullptr;
     k.no_chunked_advance = getenv("LACACHE_NO_CHUNKED_ADVANCE") != nullptr;
     k.verbose = getenv("LACACHE_VERBOSE") != nullptr;
   }
@@ -281,6 +279,9 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
   c->g.op_f16 = (c->engine == LACACHE_ENGINE_TCGEN05 && cfg->precision_mode == LACACHE_PRECISION_FP16) ? 1 : 0;
   const int TC_KEYS = tc_keys(c->split);
   const int R = tc ? TC_ROWS : SIMT_ROWS;
+  // builds and full recomputes with one-plane operands run the row kernel: items of two row tiles, 128-key tiles
+  const bool rk = tc && !c->split;
+  const int RI = rk ? TC_ROW_ITEM : R, RI_KEYS = rk ? TC_ROW_KEYS : TC_KEYS;
   std::vector<WorkItem> items;
   // Block-query units: the keys of each (sequence, head) are cut into balanced
   // chunks of `tpc` tiles.  Unless the caller fixes it, pick the chunk size and
@@ -330,6 +331,13 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
     }
   }
   if (tpc <= 0) tpc = 2;
+  // the row kernel's items, the most work first: a CTA draws every n-th
+  auto longest_first = [&](int from) {
+    std::stable_sort(items.begin() + from, items.end(), [](const WorkItem& p, const WorkItem& q) {
+      const long long wp = (long long)((p.nrows + 127) / 128) * (p.seq_end - p.seq_start), wq = (long long)((q.nrows + 127) / 128) * (q.seq_end - q.seq_start);
+      return wp > wq;
+    });
+  };
   c->max_chunks = 1;
   for (int k = 0; k < g.n_blk; ++k) {
     int off = (int)items.size();
@@ -368,7 +376,18 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
       c->step_list.push_back({off, (int)items.size() - off});
       c->merge_list.push_back({0, 0});
     }
-    c->build_list.push_back({rows_off, (int)items.size() - rows_off});
+    if (!rk) {
+      c->build_list.push_back({rows_off, (int)items.size() - rows_off});
+      continue;
+    }
+    // the build's row tiles run straight through the block (its rows get a state too, which nothing reads: a
+    // tile more per sequence would cost more); a sequence without fixed rows has none
+    off = (int)items.size();
+    for (int b = 0; b < g.B; ++b)
+      if (c->cu[b + 1] - c->cu[b] > g.block_len)
+        add_row_tiles(items, b, c->cu[b], c->cu[b + 1], TC_ROW_ITEM, c->cu[b], c->cu[b + 1], c->blk_start_all[(size_t)k * g.B + b]);
+    longest_first(off);
+    c->build_list.push_back({off, (int)items.size() - off});
   }
   int inc_chunks = 1;
   c->adv_tab.assign((size_t)g.n_blk * g.B * 2, 0);
@@ -391,8 +410,8 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
     for (int b = 0; b < g.B; ++b) {
       const int cs = c->cu[b], ce = c->cu[b + 1], s0 = c->blk_start_all[(size_t)k * g.B + b], e0 = s0 + g.block_len;
       const int from = (int)items.size();
-      add_row_tiles(items, b, cs, s0, R, cs, ce, s0);
-      add_row_tiles(items, b, e0, ce, R, cs, ce, s0);
+      add_row_tiles(items, b, cs, s0, RI, cs, ce, s0);
+      add_row_tiles(items, b, e0, ce, RI, cs, ce, s0);
       window(from, cs, cs, s0, 0);
     }
     c->inc_prefix.push_back({off, (int)items.size() - off});
@@ -400,8 +419,8 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
     for (int b = 0; b < g.B; ++b) {
       const int cs = c->cu[b], ce = c->cu[b + 1], s0 = c->blk_start_all[(size_t)k * g.B + b], e0 = s0 + g.block_len;
       const int from = (int)items.size();
-      add_row_tiles(items, b, cs, s0, R, cs, ce, s0);
-      add_row_tiles(items, b, e0, ce, R, cs, ce, s0);
+      add_row_tiles(items, b, cs, s0, RI, cs, ce, s0);
+      add_row_tiles(items, b, e0, ce, RI, cs, ce, s0);
       window(from, e0, e0, ce, W_INIT);
     }
     c->inc_comb.push_back({off, (int)items.size() - off});
@@ -411,7 +430,7 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
       // its rows changed their queries: prefix state over every key before block k, from scratch
       const int cs = c->cu[b], ce = c->cu[b + 1], s0 = c->blk_start_all[(size_t)k * g.B + b];
       const int from = (int)items.size();
-      add_row_tiles(items, b, s0 - g.block_len, s0, R, cs, ce, s0);
+      add_row_tiles(items, b, s0 - g.block_len, s0, RI, cs, ce, s0);
       window(from, cs, cs, s0, 0);
     }
     c->inc_fresh.push_back({off, (int)items.size() - off});
@@ -450,12 +469,12 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
       // every other fixed row: old prefix state + the finished block's keys (exactly the first key
       // tile, which ends at s0) = new prefix state, stored; + the keys after block k = cached state
       int from = (int)items.size();
-      add_row_tiles(items, b, cs, sp, R, cs, ce, s0);
-      add_row_tiles(items, b, e0, ce, R, cs, ce, s0);
-      window(from, s0 - TC_KEYS, sp, ce > e0 ? ce : s0, W_INIT | W_SNAP | W_JUMP_BLOCK);
+      add_row_tiles(items, b, cs, sp, RI, cs, ce, s0);
+      add_row_tiles(items, b, e0, ce, RI, cs, ce, s0);
+      window(from, s0 - RI_KEYS, sp, ce > e0 ? ce : s0, W_INIT | W_SNAP | W_JUMP_BLOCK);
       // the finished block's rows: their new prefix state + the keys after block k
       from = (int)items.size();
-      add_row_tiles(items, b, sp, s0, R, cs, ce, s0);
+      add_row_tiles(items, b, sp, s0, RI, cs, ce, s0);
       window(from, e0, e0, ce, W_INIT);
     }
     c->inc_fused.push_back({off, (int)items.size() - off});
@@ -490,7 +509,7 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
           c->tile_hi_all[(size_t)k * g.B + b] = hi;
           size_t from = items.size();
           if (pass == 2) {   // the rows of the overlapping tiles x all keys: the longest units, so they go first
-            add_row_tiles(items, b, lo, hi, R, cs, ce, s0);
+            add_row_tiles(items, b, lo, hi, RI, cs, ce, s0);
             window(from, cs, cs, ce, W_OUT);
             from = items.size();
           }
@@ -498,8 +517,8 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
           // the second launch, one with nothing after them is complete after the first)
           if (pass == 0 && lo == cs) continue;
           if (pass == 1 && hi == ce) continue;
-          add_row_tiles(items, b, cs, lo, R, cs, ce, s0);
-          add_row_tiles(items, b, hi, ce, R, cs, ce, s0);
+          add_row_tiles(items, b, cs, lo, RI, cs, ce, s0);
+          add_row_tiles(items, b, hi, ce, RI, cs, ce, s0);
           if (pass == 0) window(from, cs, cs, lo, 0);
           else if (pass == 1) window(from, hi, hi, ce, lo > cs ? W_INIT : 0);
           else window(from, lo, lo, hi, W_INIT | W_OUT);
@@ -510,7 +529,8 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
   }
   {
     int off = (int)items.size();
-    for (int b = 0; b < g.B; ++b) add_row_tiles(items, b, c->cu[b], c->cu[b + 1], R, c->cu[b], c->cu[b + 1], 0);
+    for (int b = 0; b < g.B; ++b) add_row_tiles(items, b, c->cu[b], c->cu[b + 1], RI, c->cu[b], c->cu[b + 1], 0);
+    if (rk) longest_first(off);
     c->full_list = {off, (int)items.size() - off};
   }
   c->items_host = items;
@@ -518,6 +538,7 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
   // ---- device memory ----
   CU_TRY(c, simt_prepare());
   if (tc) CU_TRY(c, tc_prepare());
+  if (rk) CU_TRY(c, rows_prepare());
 
   CU_TRY(c, dev_alloc(c, &c->d_cu, g.B + 1));
   CU_TRY(c, cudaMemcpy(c->d_cu, c->cu.data(), sizeof(int32_t) * (g.B + 1), cudaMemcpyHostToDevice));
@@ -713,8 +734,6 @@ AttnArgs attn_args(lacache_ctx* c, int mode, lacache_ctx::ListRef list, int blk,
     } else {
       a.n_ctas_stream = (int)std::min<long long>(c->num_sms, units_stream);
       a.n_ctas = a.n_ctas_stream;
-      // (a plain build writes the cached state itself: the buffer the tensor map of the state describes)
-      a.st_tma = (mode == MODE_BUILD && !c->split && !c->knobs.no_staged_state) ? 1 : 0;
     }
   }
   return a;
@@ -723,11 +742,11 @@ AttnArgs attn_args(lacache_ctx* c, int mode, lacache_ctx::ListRef list, int blk,
 // one launch of the tcgen05 kernel; with a span ring set, the launch gets the ring's next slot
 cudaError_t launch_tc(lacache_ctx* c, AttnArgs a, const TcMaps* maps, cudaStream_t s) {
   if (c->span_ring) a.span = c->span_ring + 2 * (size_t)(c->span_next++ % (unsigned)c->span_slots);
-  return tc_attention(c->g, a, maps, s);
+  return (a.mode == MODE_STEP || a.split) ? tc_attention(c->g, a, maps, s) : row_attention(c->g, a, maps, s);
 }
 
 lacache_status run_attention(lacache_ctx* c, const AttnArgs& a, bool scratch, cudaStream_t s) {
-  if (c->engine == LACACHE_ENGINE_TCGEN05 && a.out) {
+  if (c->engine == LACACHE_ENGINE_TCGEN05 && a.mode == MODE_STEP && a.out) {   // (the other modes store rows directly)
     if (!tc_set_out(scratch ? c->maps_scratch : c->maps, c->g, a.out, a.out_bf16 != 0, c->err, sizeof(c->err))) return LACACHE_ERR_CUDA;
   }
   if (c->ev_start) CU_TRY(c, cudaEventRecord(c->ev_start, s));

@@ -139,8 +139,6 @@ struct AttnArgs {
   int32_t* status;
   int blk_to_state;          // block-row units write the merged state (m, l, O~) of their rows to `st` instead
                              // of normalised rows to `out` (first launch of an incremental advance)
-  int st_tma;                // build: `st.o` is the buffer the cached-state tensor map was encoded for, so full row tiles
-                             // may leave through bulk tensor stores (one-plane operands)
   int pair_chunks;           // host only: a step whose block-row units all have two key chunks, as pairs of CTAs
                              // (thread-block clusters of two) that merge through distributed shared memory
   int no_pdl;                // host only: launch the ordinary way (experiment knob)
@@ -192,6 +190,9 @@ cudaError_t simt_prepare();  // function attributes
 struct TcMaps;  // opaque set of TMA descriptors, defined in lacache_tc.cu
 cudaError_t tc_attention(const Geometry& g, const AttnArgs& a, const TcMaps* maps, cudaStream_t s);
 cudaError_t tc_prepare();
+// row tiles over long key ranges (build, full recompute, key windows) with one-plane operands: lacache_rows.cu
+cudaError_t row_attention(const Geometry& g, const AttnArgs& a, const TcMaps* maps, cudaStream_t s);
+cudaError_t rows_prepare();
 // builds TMA descriptors for a rotated buffer set; returns nullptr and fills
 // err on failure
 TcMaps* tc_make_maps(const Geometry& g, const RotBuffers& rot, float* state_o, bool split, char* err, int errlen);
@@ -220,6 +221,8 @@ constexpr int TC_ROWS = 128;     // query rows per tcgen05 work item
 constexpr int TC_KEYS_SPLIT = 96;
 constexpr int TC_KEYS_PLAIN = 128;
 inline int tc_keys(bool split) { return split ? TC_KEYS_SPLIT : TC_KEYS_PLAIN; }
+constexpr int TC_ROW_KEYS = 128;   // keys per tile of the row kernel (lacache_rows.cu)
+constexpr int TC_ROW_ITEM = 256;   // query rows per item of the row kernel (two tiles)
 constexpr int TC_MAX_BLOCK = 64;
 constexpr int TC_DEEP_MAX_UNITS = 512;  // units per CTA the pipelined merge role can tabulate // largest block length the tcgen05 merge role handles
 

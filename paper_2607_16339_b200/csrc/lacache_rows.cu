@@ -1,0 +1,666 @@
+// tcgen05 attention of fixed row tiles over long key ranges (bf16 inputs, head_dim 128, one plane per rotated operand):
+// the cache build, the full recompute and the builds over key windows.  (The block queries of a step and the merge of
+// fixed rows with the block's keys are lacache_tc.cu, and so are these builds with split planes, whose operands leave
+// shared memory for one stage of keys only: 90 us against its 84 at 1536 tokens x 32 heads.)
+//
+// One persistent CTA per SM.  A unit is up to 256 query rows of one head, as two 128-row tiles A and B that share
+// every key / value tile.  What bounds a single tile is the chain scores -> softmax -> P~V of one key tile after the
+// other, in which the tensor cores and the exponential unit take turns; with two tiles one works for A while the
+// other works for B.
+//   warps 0..3   row threads of tile A, warps 4..7 of tile B: thread = query row = TMEM lane
+//   warp 8       TMA producer (one lane)
+//   warp 9       issues the score products S = Q' K'^T of both tiles, warp 10 the products O~ += P~ V
+// TMEM (512 columns): ONE score tile S (128) that A and B use in turn, their fp16 probabilities P~ (64 each) and their
+// O~ (128 each, accumulated over a unit's key tiles, rescaled in place when a row outgrows its reference).  A row
+// thread takes its 128 scores into registers at once and S is free again, so that the next scores of its tile are
+// computed while it still forms the probabilities of this one.  (With a score tile each, P~ written over S for want of
+// columns, the scores of key tile j + 1 had to wait for the products of tile j.)  Probabilities go over in halves of 64
+// keys: the products of the first half run while the row threads work on the second.
+// A row thread's time per key tile is what the kernel is bound by (two warps per scheduler, each a serial chain): the
+// exponentials of the first half are therefore formed with the reference exponent as it stands, beside the row's maximum,
+// and again only when the maximum asks for another one; the sums of the rounded probabilities come after the hand-over.
+//
+// Shared memory: two Q' tiles, two stages of keys (two 16 KB boxes of 64 features) and of values (two boxes of 64 keys).
+//
+// Arithmetic as in lacache_tc.cu: integer reference exponent, moved only when the row's maximum outgrows it by more
+// than RESCALE_SLACK; P~ rounded to fp16, the normaliser sums the rounded values.
+#include <algorithm>
+
+#include "lacache_internal.h"
+#include "lacache_ptx.h"
+#include "lacache_tc_util.h"
+
+namespace lacache {
+namespace {
+
+using namespace tcu;
+
+constexpr int ROW_THREADS = 256;
+constexpr int THREADS = 384;      // (warp 11 idles: register splits work on groups of four warps)
+constexpr int LAUNCH_REGS = 168, ROW_REGS = 216, ISSUER_REGS = 72;
+static_assert(ROW_THREADS * ROW_REGS + (THREADS - ROW_THREADS) * ISSUER_REGS <= THREADS * LAUNCH_REGS, "more registers than the block has");
+constexpr int KT = TC_ROW_KEYS;   // keys per tile
+constexpr int W_PRODUCER = 8, W_SCORES = 9, W_PRODUCTS = 10;   // the warps with another role
+
+struct RowMaps {
+  CUtensorMap q;      // box {64, 128 rows, 2 halves, 1 head, planes}: a whole Q' tile
+  CUtensorMap k_box;  // box {64, 128 rows, 1, 1, 1}
+  CUtensorMap v64;    // box {64, 64 rows, 2 halves, 1}
+};
+
+constexpr uint32_t BOX = 16384;
+constexpr int STAGES = 2;
+constexpr uint32_t Q_TILE = 32768;
+constexpr uint32_t SM_K = 2 * Q_TILE;
+constexpr uint32_t SM_V = SM_K + 2 * STAGES * BOX;
+constexpr uint32_t SM_ST = SM_V + 2 * STAGES * BOX;   // 4 KB of staging per row warp
+constexpr uint32_t SM_BARS = SM_ST + 8 * 4096;
+
+enum {
+  B_Q_FULL = 0, B_Q_FREE = 2,     // per tile
+  B_K_FULL = 4, B_K_FREE = 8,     // per box slot
+  B_V_FULL = 12, B_V_FREE = 16,   // per box slot
+  B_S_FULL = 20,                  // per tile
+  B_P_RDY = 22,                   // per tile and half: 2 * tile + half
+  B_PV_DONE = 26, B_O_FREE = 28,  // per tile
+  B_S_FREE = 30,
+  B_DONE = 31, N_BARS = 32
+};
+constexpr uint32_t SM_TOTAL = SM_BARS + 8 * N_BARS + 16;
+static_assert(SM_TOTAL <= 232448, "exceeds the 227 KB per-CTA limit");
+constexpr uint32_t TM_S = 0;
+__device__ constexpr uint32_t TM_P(int x) { return 128u + 64u * x; }
+__device__ constexpr uint32_t TM_O(int x) { return 256u + 128u * x; }
+
+struct Unit {
+  int row0, nrows, h, kh;
+  int key_base, n_tiles;  // key tile t holds keys key_base + 128 t ... (or see base1)
+  int k0, k1, x0, x1;     // valid keys [k0, k1) minus [x0, x1)
+  int base1;              // >= 0: tiles after the first are counted from this token
+  bool init, snap, out;   // start from a stored state; store the state after the first tile; write normalised rows
+  __device__ __forceinline__ int tiles() const { return nrows > BM ? 2 : 1; }
+  __device__ __forceinline__ int key_row(int t) const { return (base1 >= 0 && t > 0) ? base1 + (t - 1) * KT : key_base + t * KT; }
+};
+
+// units are head-minor (unit u = item u / Hq of head u % Hq): neighbours share keys in L2
+template <bool WINDOW>
+__device__ __forceinline__ Unit decode(const Geometry& g, const AttnArgs& a, int u) {
+  const WorkItem it = load_item(a.items + u / g.Hq);
+  Unit un;
+  un.h = u % g.Hq;
+  un.kh = un.h / g.group;
+  un.row0 = it.row0;
+  un.nrows = it.nrows;
+  un.key_base = un.k0 = it.seq_start;
+  un.k1 = it.seq_end;
+  un.x0 = un.x1 = 0;
+  un.base1 = -1;
+  un.init = un.snap = false;
+  un.out = a.mode == MODE_FULL;
+  un.n_tiles = (it.seq_end - it.seq_start + KT - 1) / KT;
+  if (WINDOW) {
+    un.key_base = it.pad;
+    un.k0 = it.kt0;
+    un.k1 = it.kt1;
+    un.n_tiles = it.kt1 > it.pad ? (it.kt1 - it.pad + KT - 1) / KT : 0;
+    if (it.chunk & 4) { un.x0 = it.blk_start; un.x1 = it.blk_start + g.block_len; }
+    if (it.chunk & 8) {   // the first tile ends where the block starts; the others start right after the block
+      un.base1 = it.blk_start + g.block_len;
+      un.n_tiles = 1 + (it.kt1 > un.base1 ? (it.kt1 - un.base1 + KT - 1) / KT : 0);
+    }
+    un.init = it.chunk & 1;
+    un.snap = (it.chunk >> 1) & 1;
+    un.out = (it.chunk & 16) != 0;
+  } else if (a.mode == MODE_BUILD) {
+    un.x0 = it.blk_start;
+    un.x1 = it.blk_start + g.block_len;
+  }
+  return un;
+}
+
+// ---- producer -----------------------------------------------------------------------------------------------
+// Three cursors -- Q' tiles, key boxes, value boxes -- and whichever has a free slot issues its load.
+template <bool WINDOW>
+__device__ void row_producer(const Cta& c, const RowMaps& maps, const Geometry& g, const AttnArgs& a, int first,
+                             int stride, int n_units) {
+  grid_dependency_wait();   // every operand is written by the kernels ahead
+  struct Cursor { int u, t, part, n; Unit un; bool live; };   // n: units (Q') or tiles (keys, values) so far
+  auto load_unit = [&](Cursor& k) {
+    for (; k.u < n_units; k.u += stride) {
+      k.un = decode<WINDOW>(g, a, k.u);
+      if (k.un.n_tiles > 0) return;
+    }
+    k.live = false;
+  };
+  Cursor q{first, 0, 0, 0, Unit{}, true};
+  load_unit(q);
+  Cursor k = q, v = q;
+  int nq0 = 0, nq1 = 0;   // Q' tiles loaded, per tile slot
+  long long t_idle = 0;
+  while (q.live || k.live || v.live) {
+    bool did = false;
+    if (q.live) {
+      const int x = q.part;
+      const int n = x ? nq1 : nq0;
+      if (n == 0 || mbar_test(c.bar(B_Q_FREE + x), (n - 1) & 1)) {
+        mbar_expect_tx(c.bar(B_Q_FULL + x), Q_TILE);
+        tma_load_5d(c.base + x * Q_TILE, &maps.q, c.bar(B_Q_FULL + x), 0, q.un.row0 + BM * x, 0, q.un.h, 0);
+        if (x) ++nq1; else ++nq0;
+        if (++q.part == q.un.tiles()) { q.part = 0; q.u += stride; load_unit(q); }
+        did = true;
+      }
+    }
+    if (k.live) {
+      const int slot = (k.n % STAGES) * 2 + k.part, use = k.n / STAGES;
+      if (use == 0 || mbar_test(c.bar(B_K_FREE + slot), (use - 1) & 1)) {
+        mbar_expect_tx(c.bar(B_K_FULL + slot), BOX);
+        tma_load_5d(c.base + SM_K + slot * BOX, &maps.k_box, c.bar(B_K_FULL + slot), 0, k.un.key_row(k.t),
+                    k.part, k.un.kh, 0);
+        if (++k.part == 2) {
+          k.part = 0;
+          ++k.n;
+          if (++k.t == k.un.n_tiles) { k.t = 0; k.u += stride; load_unit(k); }
+        }
+        did = true;
+      }
+    }
+    if (v.live) {
+      const int slot = (v.n % STAGES) * 2 + v.part, use = v.n / STAGES;
+      if (use == 0 || mbar_test(c.bar(B_V_FREE + slot), (use - 1) & 1)) {
+        mbar_expect_tx(c.bar(B_V_FULL + slot), BOX);
+        tma_load_4d(c.base + SM_V + slot * BOX, &maps.v64, c.bar(B_V_FULL + slot), 0, v.un.key_row(v.t) + 64 * v.part, 0, v.un.kh);
+        if (++v.part == 2) {
+          v.part = 0;
+          ++v.n;
+          if (++v.t == v.un.n_tiles) { v.t = 0; v.u += stride; load_unit(v); }
+        }
+        did = true;
+      }
+    }
+    if (did) {
+      t_idle = 0;
+    } else {  // nothing free: bounded idle
+      if (t_idle == 0) t_idle = clock64();
+      if (*c.abort_flag) return;
+      if (clock64() - t_idle > WAIT_CYCLES) {
+        *c.abort_flag = 1;
+        if (atomicCAS(c.status, 0, (int)LACACHE_ERR_TIMEOUT) == 0) {
+          c.status[1] = LOC_WAIT_K; c.status[2] = blockIdx.x; c.status[3] = threadIdx.x;
+        }
+        return;
+      }
+    }
+  }
+}
+
+// ---- the two issuers ----------------------------------------------------------------------------------------
+// A whole warp walks each of these loops and one elected lane issues.
+template <bool WINDOW>
+__device__ void row_scores(const Cta& c, const Geometry& g, const AttnArgs& a, int first, int stride, int n_units) {
+  const uint32_t idesc = idesc_f16(g.op_f16 ? 0u : 1u, 0u, BM, KT);
+  const bool leader = elect_one();
+  int nu[2] = {0, 0};   // units so far, per tile slot
+  int ns = 0;           // score tiles so far (A's and B's take turns)
+  int kt = 0;           // key tiles so far
+  for (int u = first; u < n_units; u += stride) {
+    const Unit un = decode<WINDOW>(g, a, u);
+    const int nx = un.tiles();
+    for (int j = 0; j < un.n_tiles; ++j, ++kt) {
+      const int slot0 = (kt % STAGES) * 2;
+      const uint32_t kph = (uint32_t)(kt / STAGES) & 1u;
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        if (x >= nx) break;
+        if (j == 0 && !wait_bar(c, B_Q_FULL + x, nu[x] & 1, LOC_WAIT_Q)) return;
+        if (x == 0 && !wait_bar(c, B_K_FULL + slot0, kph, LOC_WAIT_K)) return;
+        if (ns > 0 && !wait_bar(c, B_S_FREE, (ns - 1) & 1, LOC_WAIT_S)) return;   // the scores before these have been taken
+        tc_fence_after();
+#pragma unroll
+        for (int b = 0; b < 2; ++b) {   // box b: features 64 b ...
+          if (x == 0 && b > 0) {
+            if (!wait_bar(c, B_K_FULL + slot0 + b, kph, LOC_WAIT_K)) return;
+            tc_fence_after();
+          }
+          const uint64_t kd = smem_desc(c.base + SM_K + (slot0 + b) * BOX, 16, 1024);
+          const uint64_t qd = smem_desc(c.base + x * Q_TILE + b * BOX, 16, 1024);
+          if (leader) {
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) mma_ss(c.tmem + TM_S, qd + 2u * ks, kd + 2u * ks, idesc, (b > 0 || ks > 0) ? 1u : 0u);
+            if (x == nx - 1) tc_commit(c.bar(B_K_FREE + slot0 + b));
+          }
+        }
+        ++ns;
+        if (leader) {
+          tc_commit(c.bar(B_S_FULL + x));
+          if (j == un.n_tiles - 1) tc_commit(c.bar(B_Q_FREE + x));
+        }
+        if (j == un.n_tiles - 1) ++nu[x];
+      }
+    }
+  }
+}
+
+template <bool WINDOW>
+__device__ void row_products(const Cta& c, const Geometry& g, const AttnArgs& a, int first, int stride, int n_units) {
+  constexpr uint32_t idesc = idesc_f16(0u /*fp16*/, 1u, BM, D);
+  const bool leader = elect_one();
+  int nu[2] = {0, 0}, np[2] = {0, 0};   // units and tiles of products so far, per tile slot
+  int kt = 0;                           // key tiles so far
+  for (int u = first; u < n_units; u += stride) {
+    const Unit un = decode<WINDOW>(g, a, u);
+    const int nx = un.tiles();
+    for (int j = 0; j < un.n_tiles; ++j, ++kt) {
+      const int slot0 = (kt % STAGES) * 2;
+      const uint32_t vph = (uint32_t)(kt / STAGES) & 1u;
+#pragma unroll
+      for (int x = 0; x < 2; ++x) {
+        if (x >= nx) break;
+        // O~ of the unit before has been read by its row threads
+        if (j == 0 && nu[x] > 0 && !wait_bar(c, B_O_FREE + x, (nu[x] - 1) & 1, LOC_WAIT_O)) return;
+#pragma unroll
+        for (int hf = 0; hf < 2; ++hf) {
+          if (!wait_bar(c, B_P_RDY + 2 * x + hf, np[x] & 1, LOC_WAIT_S)) return;
+          if (x == 0 && !wait_bar(c, B_V_FULL + slot0 + hf, vph, LOC_WAIT_V)) return;
+          tc_fence_after();
+          // B = V, MN-major: 64 features contiguous, the next 64 features 8 KB on, 16 keys = 2 KB
+          const uint64_t vd = smem_desc(c.base + SM_V + (slot0 + hf) * BOX, 8192, 1024);
+          const uint32_t first_acc = (j == 0 && hf == 0 && !(WINDOW && un.init)) ? 0u : 1u;
+          if (leader) {
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks)
+              mma_ts(c.tmem + TM_O(x), c.tmem + TM_P(x) + 32 * hf + 8 * ks, vd + (uint64_t)(ks * 128), idesc, ks ? 1u : first_acc);
+            if (hf == 1) tc_commit(c.bar(B_PV_DONE + x));
+            if (x == nx - 1) tc_commit(c.bar(B_V_FREE + slot0 + hf));
+          }
+        }
+        ++np[x];
+        if (j == un.n_tiles - 1) ++nu[x];
+      }
+    }
+  }
+}
+
+// ---- row threads --------------------------------------------------------------------------------------------
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ float max3(float a, float b, float c) {
+  float m;
+  asm("max.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
+  return m;
+}
+__device__ __forceinline__ float add_half(float s, uint32_t h2, bool high) {   // s + one half of an fp16 pair
+  float r;
+  if (high) asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %1;\n\tadd.f32.f16 %0, hi, %2;\n\t}" : "=f"(r) : "r"(h2), "f"(s));
+  else asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %1;\n\tadd.f32.f16 %0, lo, %2;\n\t}" : "=f"(r) : "r"(h2), "f"(s));
+  return r;
+}
+__device__ __forceinline__ uint64_t span_bits(int lo, int hi) {   // bits [lo, hi) of 64
+  lo = max(lo, 0);
+  hi = min(hi, 64);
+  if (hi <= lo) return 0ull;
+  return (hi - lo == 64 ? ~0ull : ((1ull << (hi - lo)) - 1ull)) << lo;
+}
+
+// The O~ row of every thread of a warp, scaled by `mul`, to rows of global memory: state rows (fp32, `stride` D) or
+// output rows, through the warp's 4 KB of staging, 32 features at a time, so that a store instruction writes four rows'
+// 128 contiguous bytes (thread per row, it would touch 32 rows).  `rows`: how many of the warp's rows exist.  have_o: TMEM
+// holds O~ (else zeros).
+__device__ __forceinline__ void store_rows(const Cta& c, uint32_t o_tmem, bool have_o, float mul, float* dst32,
+                                           __nv_bfloat16* dst16, size_t stride, int rows) {
+  const int lane = threadIdx.x & 31;
+  uint8_t* const st = c.gen + SM_ST + (threadIdx.x >> 5) * 4096;
+#pragma unroll 1
+  for (int cb = 0; cb < 4; ++cb) {
+    uint32_t r[32];
+    if (have_o) {
+      tmem_ld32(o_tmem + 32 * cb, r);
+      tmem_ld_wait();
+#pragma unroll
+      for (int i = 0; i < 32; ++i) r[i] = __float_as_uint(__uint_as_float(r[i]) * mul);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 32; ++i) r[i] = 0u;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      *reinterpret_cast<uint4*>(st + lane * 128 + ((i ^ (lane & 7)) << 4)) = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int rr = 4 * i + (lane >> 3), ch = lane & 7;
+      if (rr < rows) {
+        const float4 v = *reinterpret_cast<const float4*>(st + rr * 128 + ((ch ^ (rr & 7)) << 4));
+        const size_t off = (size_t)rr * stride + 32 * cb + 4 * ch;
+        if (dst16) *reinterpret_cast<uint2*>(dst16 + off) = make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w));
+        else *reinterpret_cast<float4*>(dst32 + off) = v;
+      }
+    }
+    __syncwarp();
+  }
+}
+
+// wait_bar without a call: a row thread has most of its registers in use where it waits
+__device__ __forceinline__ bool wait_here(const Cta& c, int slot, uint32_t parity, int loc) {
+  const uint32_t bar = c.bar(slot);
+  if (mbar_try(bar, parity)) return true;
+  const long long t0 = clock64();
+  while (!mbar_try(bar, parity)) {
+    if (*c.abort_flag) return false;
+    if (clock64() - t0 > WAIT_CYCLES) {
+      *c.abort_flag = 1;
+      if (atomicCAS(c.status, 0, (int)LACACHE_ERR_TIMEOUT) == 0) {
+        c.status[1] = loc; c.status[2] = blockIdx.x; c.status[3] = threadIdx.x;
+      }
+      return false;
+    }
+  }
+  return true;
+}
+
+template <bool WINDOW>
+__device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, int first, int stride, int n_units) {
+  const float LN2 = 0.69314718055994530942f;
+  const int lane = threadIdx.x & 31;
+  const int x = threadIdx.x >> 7;                  // tile of this thread
+  const int quad = (threadIdx.x >> 5) & 3;
+  const int r = threadIdx.x & 127;                 // its row there = TMEM lane
+  const uint32_t tlane = c.tmem + ((uint32_t)(quad * 32) << 16);
+  const uint32_t s_tmem = tlane + TM_S, p_tmem = tlane + TM_P(x), o_tmem = tlane + TM_O(x);
+  int n = 0;                                       // key tiles of this tile slot so far
+  bool waited = false;                             // for the grids ahead
+  for (int u = first; u < n_units; u += stride) {
+    const Unit un = decode<WINDOW>(g, a, u);
+    const int n_rows = min(un.nrows - BM * x, BM);
+    if (n_rows <= 0) continue;                     // (a unit of one tile)
+    const int warp_rows = min(n_rows - 32 * quad, 32);   // rows of this warp (<= 0: none)
+    const bool valid = r < n_rows;
+    const int row = un.row0 + BM * x + r;
+    const size_t srow = (size_t)un.h * g.Tp + row;
+    float m_ref = -INFINITY, l = 0.f;
+    bool have_o = false;                           // O~ in TMEM holds something
+    if (WINDOW && un.init) {
+      if (!waited) { grid_dependency_wait(); waited = true; }
+      // The unit continues from a stored state of its rows.  Nobody else touches this tile's O~ between units (the
+      // previous unit's products are complete, and these threads have read its O~).
+      if (valid) { m_ref = a.init.m[srow]; l = a.init.l[srow]; }
+      if (un.n_tiles > 0) {
+#pragma unroll 1
+        for (int h2 = 0; h2 < 2; ++h2) {
+          uint32_t o[64];
+#pragma unroll
+          for (int i = 0; i < 64; ++i) o[i] = 0u;
+          if (valid) {   // (plain loads: the launch may update these rows in place)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) ld_global_v8(a.init.o + srow * D + 64 * h2 + 8 * i, o + 8 * i);
+          }
+          tmem_st32(o_tmem + 64 * h2, *reinterpret_cast<uint32_t(*)[32]>(o));
+          tmem_st32(o_tmem + 64 * h2 + 32, *reinterpret_cast<uint32_t(*)[32]>(o + 32));
+        }
+        tmem_st_wait();
+        have_o = true;
+      }
+    }
+
+    for (int j = 0; j < un.n_tiles; ++j, ++n) {
+      if (!wait_here(c, B_S_FULL + x, n & 1, LOC_WAIT_S)) return;
+      tc_fence_after();
+      if (WINDOW && un.snap && j == 1) {
+        // the state after the unit's first key tile
+        if (!wait_here(c, B_PV_DONE + x, (n - 1) & 1, LOC_WAIT_O)) return;
+        tc_fence_after();
+        if (!waited) { grid_dependency_wait(); waited = true; }
+        if (warp_rows > 0) {
+          store_rows(c, o_tmem, true, 1.f, a.snap.o + (srow - lane) * D, nullptr, D, warp_rows);
+          if (valid) { a.snap.m[srow] = m_ref; a.snap.l[srow] = l; }
+        }
+      }
+      if (warp_rows > 0) {
+        // The row's 128 scores come out of TMEM once, every load in flight before the one wait.
+        uint32_t s[KT];
+#pragma unroll
+        for (int i = 0; i < KT; i += 32) tmem_ld32(s_tmem + i, *reinterpret_cast<uint32_t(*)[32]>(s + i));
+        tmem_ld_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(c.bar(B_S_FREE));
+        const int tile_lo = un.key_row(j);
+        if (tile_lo < un.k0 || tile_lo + KT > un.k1 || (un.x0 < tile_lo + KT && un.x1 > tile_lo)) {
+          // columns that take no part: -inf (the same for every row)
+#pragma unroll
+          for (int hf = 0; hf < 2; ++hf) {
+            const int lo = tile_lo + 64 * hf;
+            const uint64_t bits = span_bits(un.k0 - lo, un.k1 - lo) & ~(un.x1 > un.x0 ? span_bits(un.x0 - lo, un.x1 - lo) : 0ull);
+#pragma unroll
+            for (int i = 0; i < 64; ++i) s[64 * hf + i] = ((bits >> i) & 1ull) ? s[64 * hf + i] : 0xff800000u;
+          }
+        }
+        // P~ = 2^(S c - m) of the columns 64 hf ..., rounded to fp16
+        uint32_t p[32];
+        auto probabilities = [&](int hf) {
+          const float m_use = (m_ref == -INFINITY) ? 0.f : m_ref;
+          const uint64_t nm = pack2(-m_use, -m_use), sc = pack2(g.scale_log2, g.scale_log2);
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            const int k = 64 * hf + 2 * i;
+            const uint64_t e = fma2(pack2(__uint_as_float(s[k]), __uint_as_float(s[k + 1])), sc, nm);
+            float e0, e1;
+            asm("mov.b64 {%0, %1}, %2;" : "=f"(e0), "=f"(e1) : "l"(e));
+            const __half2 h = __floats2half2_rn(ex2(e0), ex2(e1));
+            p[i] = *reinterpret_cast<const uint32_t*>(&h);
+          }
+        };
+        probabilities(0);   // (with the reference as it stands: it rarely moves)
+        float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+        for (int i = 0; i < KT; i += 8) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) mx[k] = max3(mx[k], __uint_as_float(s[i + 2 * k]), __uint_as_float(s[i + 2 * k + 1]));
+        }
+        const float cand = ceilf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * g.scale_log2);
+        float m_new = m_ref;
+        if (m_ref == -INFINITY || cand > m_ref + RESCALE_SLACK) m_new = fmaxf(m_ref, cand);
+        // the previous tile's products are complete: P~ may be overwritten, O~ rescaled
+        if (n > 0) {
+          if (!wait_here(c, B_PV_DONE + x, (n - 1) & 1, LOC_WAIT_O)) return;
+          tc_fence_after();
+        }
+        if (__any_sync(0xffffffffu, m_new != m_ref)) {
+          const float alpha = (m_new == m_ref) ? 1.f : (m_ref == -INFINITY ? 0.f : ex2(m_ref - m_new));
+          l *= alpha;
+          m_ref = m_new;
+          if (have_o) {
+#pragma unroll 1
+            for (int cb = 0; cb < 8; ++cb) {
+              uint32_t o[16];
+              tmem_ld16(o_tmem + 16 * cb, o);
+              tmem_ld_wait();
+#pragma unroll
+              for (int i = 0; i < 16; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+              tmem_st16(o_tmem + 16 * cb, o);
+            }
+          }
+          probabilities(0);
+        }
+        // (the normaliser sums the rounded probabilities)
+        float l0 = 0.f, l1 = 0.f, l2 = 0.f, l3 = 0.f;
+        auto sums = [&]() {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            if (i & 1) { l2 = add_half(l2, p[i], false); l3 = add_half(l3, p[i], true); }
+            else { l0 = add_half(l0, p[i], false); l1 = add_half(l1, p[i], true); }
+          }
+        };
+        tmem_st32(p_tmem, p);
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(c.bar(B_P_RDY + 2 * x));
+        sums();
+        probabilities(1);
+        tmem_st32(p_tmem + 32, p);
+        tmem_st_wait();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(c.bar(B_P_RDY + 2 * x + 1));
+        sums();
+        l += (l0 + l1) + (l2 + l3);
+        have_o = true;
+      } else {   // a warp without rows keeps the barriers' counts (and stays in step: no arrival a phase ahead)
+        if (lane == 0) mbar_arrive(c.bar(B_S_FREE));
+        if (n > 0 && !wait_here(c, B_PV_DONE + x, (n - 1) & 1, LOC_WAIT_O)) return;
+        if (lane == 0) {
+          mbar_arrive(c.bar(B_P_RDY + 2 * x));
+          mbar_arrive(c.bar(B_P_RDY + 2 * x + 1));
+        }
+      }
+    }
+
+    // ---- epilogue ----
+    if (!waited) { grid_dependency_wait(); waited = true; }   // no global store before the grids ahead are complete
+    if (un.n_tiles > 0) {
+      if (!wait_here(c, B_PV_DONE + x, (n - 1) & 1, LOC_WAIT_O)) return;
+      tc_fence_after();
+    }
+    if (warp_rows > 0) {
+      if (un.out) {
+        const size_t orow = (size_t)row * g.Hq + un.h, wrow = (size_t)(row - lane) * g.Hq + un.h;
+        float* d32 = a.out_bf16 ? nullptr : a.out + wrow * D;
+        __nv_bfloat16* d16 = a.out_bf16 ? reinterpret_cast<__nv_bfloat16*>(a.out) + wrow * D : nullptr;
+        store_rows(c, o_tmem, have_o, 1.f / l, d32, d16, (size_t)g.Hq * D, warp_rows);
+        if (valid && a.lse) a.lse[orow] = (m_ref + log2f(l)) * LN2;
+      } else if (WINDOW && un.init && un.n_tiles == 0) {
+        // no keys: the state the unit starts from
+        if (valid && a.init.o != a.st.o) {
+          for (int i = 0; i < 16; ++i) {
+            uint32_t o[8];
+            ld_global_v8(a.init.o + srow * D + 8 * i, o);
+            st_global_v8(a.st.o + srow * D + 8 * i, o);
+          }
+          a.st.m[srow] = m_ref;
+          a.st.l[srow] = l;
+        }
+      } else {
+        store_rows(c, o_tmem, have_o, 1.f, a.st.o + (srow - lane) * D, nullptr, D, warp_rows);
+        if (valid) { a.st.m[srow] = m_ref; a.st.l[srow] = l; }
+        if (WINDOW && un.snap && un.n_tiles == 1) {   // a single key tile: the state after it is the final one as well
+          store_rows(c, o_tmem, have_o, 1.f, a.snap.o + (srow - lane) * D, nullptr, D, warp_rows);
+          if (valid) { a.snap.m[srow] = m_ref; a.snap.l[srow] = l; }
+        }
+      }
+    }
+    if (un.n_tiles > 0) {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(c.bar(B_O_FREE + x));
+    }
+  }
+}
+
+template <bool WINDOW>
+__global__ void __launch_bounds__(THREADS, 1)
+row_attn_kernel(const __grid_constant__ RowMaps maps, const __grid_constant__ Geometry g, const __grid_constant__ AttnArgs a) {
+  extern __shared__ __align__(1024) uint8_t smem_raw[];
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (uniform over the warp)
+  if (a.span != nullptr && tid == 0) atomicMin(a.span, global_timer_ns());   // first CTA entry of this launch
+  Cta c;
+  c.base = smem_u32(smem_raw);
+  c.gen = smem_raw;
+  c.bar0 = c.base + SM_BARS;
+  uint32_t* words = reinterpret_cast<uint32_t*>(smem_raw + SM_BARS + 8 * N_BARS);  // [0] tmem, [1] abort
+  c.abort_flag = reinterpret_cast<volatile int*>(words + 1);
+  c.flag = nullptr;
+  c.status = a.status;
+  if ((c.base & 1023u) != 0) {  // swizzled tiles need a 1024-byte aligned base
+    if (tid == 0 && atomicCAS(a.status, 0, (int)LACACHE_ERR_CUDA) == 0) a.status[1] = LOC_SMEM_ALIGN;
+    return;
+  }
+  const int first = blockIdx.x, stride = gridDim.x, n_units = a.n_items * g.Hq;
+  if (tid == W_PRODUCER * 32) {
+    prefetch_map(&maps.q); prefetch_map(&maps.k_box); prefetch_map(&maps.v64);
+    for (int i = 0; i < N_BARS; ++i) {
+      uint32_t count = 1;
+      if ((i >= B_P_RDY && i < B_PV_DONE) || (i >= B_O_FREE && i <= B_S_FREE)) count = 4;   // the four warps of a tile
+      if (i == B_DONE) count = THREADS;
+      mbar_init(c.bar(i), count);
+    }
+    words[1] = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    fence_async_smem();
+  }
+  __syncwarp();
+  if (warp == W_SCORES) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(words)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  c.tmem = words[0];
+
+  if (warp < ROW_THREADS / 32) {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(ROW_REGS));
+    row_threads<WINDOW>(c, g, a, first, stride, n_units);
+  } else {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(ISSUER_REGS));
+    if (warp == W_SCORES) row_scores<WINDOW>(c, g, a, first, stride, n_units);
+    else if (warp == W_PRODUCTS) row_products<WINDOW>(c, g, a, first, stride, n_units);
+    else if (tid == W_PRODUCER * 32) row_producer<WINDOW>(c, maps, g, a, first, stride, n_units);
+  }
+  __syncwarp();
+
+  if (*c.abort_flag) {
+    // A bounded wait ran out and the roles have returned where they stood: copies and products issued before that
+    // get a fixed 50 us to land before shared memory and TMEM are given up.
+    const long long t0 = clock64();
+    while (clock64() - t0 < 100000ll) {
+    }
+  }
+  tc_fence_before();
+  mbar_arrive(c.bar(B_DONE));
+  if (warp == W_SCORES) {  // the warp that allocated frees TMEM once every thread is past its last access
+    wait_bar(c, B_DONE, 0, LOC_WAIT_O);
+    __syncwarp();
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(c.tmem), "r"(512) : "memory");
+    if (a.span != nullptr && (tid & 31) == 0) atomicMax(a.span + 1, global_timer_ns());   // last CTA exit
+  }
+}
+
+const void* row_kernel(bool window) { return window ? (const void*)row_attn_kernel<true> : (const void*)row_attn_kernel<false>; }
+
+}  // namespace
+
+cudaError_t rows_prepare() {
+  for (int i = 0; i < 2; ++i) {
+    cudaError_t e = cudaFuncSetAttribute(row_kernel(i != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
+}
+
+cudaError_t row_attention(const Geometry& g, const AttnArgs& a, const TcMaps* maps, cudaStream_t s) {
+  if (a.n_ctas <= 0 || a.n_items <= 0) return cudaSuccess;
+  RowMaps rm{maps->q, maps->k_box, maps->v64};
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(a.n_ctas);
+  cfg.blockDim = dim3(THREADS);
+  cfg.dynamicSmemBytes = SM_TOTAL;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];   // set-up overlaps the end of the kernel ahead
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = a.no_pdl ? 0 : 1;
+  void* params[3] = {&rm, const_cast<Geometry*>(&g), const_cast<AttnArgs*>(&a)};
+  return cudaLaunchKernelExC(&cfg, row_kernel(a.window), params);
+}
+
+}  // namespace lacache

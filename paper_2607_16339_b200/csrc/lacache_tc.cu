@@ -39,36 +39,14 @@
 #include "lacache_internal.h"
 #include "lacache_ptx.h"
 #include "lacache_rope_math.h"
+#include "lacache_tc_util.h"
 
 namespace lacache {
 
-struct TcMaps {
-  // rotated Q' / K': 5-D views {64 features, Tp rows, 2 feature halves, heads, 2 planes (hi, lo)} of the
-  // split-bf16 storage [plane][head][half][Tp][64]; one box = both planes and both halves of `rows` rows
-  // of one head, laid out in shared memory as [plane][half][rows][64] (128-byte swizzle)
-  alignas(64) CUtensorMap q;       // box 128 rows
-  alignas(64) CUtensorMap q64;     // box 64 rows (block queries)
-  // block queries of `pack` heads of one KV group side by side: dimensions ordered {64, rows, heads, halves,
-  // planes}, box {64, pack_rows, pack, 2, 2}: lands as [plane][half][head][row][64], i.e. one 128-row tile
-  alignas(64) CUtensorMap q_pack;
-  alignas(64) CUtensorMap k;       // box TC_KEYS rows (stream role)
-  alignas(64) CUtensorMap k64;     // box 64 rows (the block's keys, merge role)
-  alignas(64) CUtensorMap k32;     // box 32 rows (the block's keys, pipelined merge role)
-  // V: 4-D views {64, Tp, 2 halves, heads} of the fp16 storage [head][half][Tp][64]
-  alignas(64) CUtensorMap v;
-  alignas(64) CUtensorMap v64;
-  alignas(64) CUtensorMap v32;
-  alignas(64) CUtensorMap st_o;    // cached O~ [Hq][Tp][128] fp32, box 32 cols x 128 rows
-  alignas(64) CUtensorMap out;     // caller's out [T][Hq][128] fp32, box 32 cols x 1 head x 128 rows
-  alignas(64) CUtensorMap out_sub[4];  // the same with boxes of 64, 32, 16 and 8 rows (clipped row tiles)
-  const void* out_ptr;             // the buffer `out` was encoded for
-};
-
 namespace {
 
-constexpr int D = 128;
-constexpr int BM = TC_ROWS;   // 128 query rows (TMEM lanes)
-constexpr float RESCALE_SLACK = 3.f;
+using namespace tcu;
+
 constexpr int ROW_WARPS = 8;
 constexpr int ROW_THREADS = ROW_WARPS * 32;
 constexpr int THREADS = 64 + ROW_THREADS + 32;   // warp 0: TMA producer, warp 1: MMA issuer, warps 2-9: row threads,
@@ -109,11 +87,6 @@ constexpr uint32_t STAGE_ROW = 512;
 constexpr uint32_t SM_RX = Tile<false>::SM_V + 2 * Tile<false>::V_STAGE;
 constexpr uint32_t SM_RX_ML = SM_RX + 32 * STAGE_ROW;
 static_assert(SM_RX_ML + 32 * 8 <= SM_XCH, "no room for the partner's partial state");
-// build, one-plane operands: staging of a unit's cached O~ tile for bulk tensor stores, four swizzled boxes of
-// 32 features x 128 rows -- two in the upper half of the Q region (a one-plane Q tile needs the lower half),
-// two in the 32 KB behind the value stages
-__host__ __device__ constexpr uint32_t st_box(int cb) { return cb < 2 ? SM_Q + 32768u + (uint32_t)cb * 16384u : SM_RX + (uint32_t)(cb - 2) * 16384u; }
-static_assert(SM_RX + 2 * 16384u <= SM_XCH, "no room for the state staging tile");
 // merge role: the 96 KB after Q hold 2 stages of the block's keys {K hi, K lo, V} of 64
 // rows, then the staging tile of the cached O~ / the output
 constexpr uint32_t SM_KV = SM_K;
@@ -153,15 +126,9 @@ enum {
   BAR_PAIR,  // 4 barriers: the two warps that share a TMEM lane quadrant
   N_BARS = BAR_PAIR + 4,
   BAR_RX = BAR_IO_FULL,  // stream role of a paired step (it has no staging-tile barriers): the partner's partial state has arrived
-  // stream role of a build with one-plane operands: a unit's state tile is staged / its bulk store has read the staging
-  BAR_ST_RDY = BAR_OUT_RDY, BAR_ST_FREE = BAR_IO_FREE
 };
 
 enum { EPI_STATE = 0, EPI_OUT = 1, EPI_PARTIAL = 2, EPI_SEND = 3 };   // SEND: the partial state goes to the partner CTA
-
-constexpr long long WAIT_CYCLES = 4000000000ll;  // ~2 s
-
-using namespace ptx;
 
 // both planes and both feature halves of `rows` rows of head h, starting at row `row`
 __device__ __forceinline__ void load_qk_box(uint32_t dst, const CUtensorMap* map, uint32_t bar, int row, int h) {
@@ -170,98 +137,6 @@ __device__ __forceinline__ void load_qk_box(uint32_t dst, const CUtensorMap* map
 __device__ __forceinline__ void load_v_box(uint32_t dst, const CUtensorMap* map, uint32_t bar, int row, int h) {
   tma_load_4d(dst, map, bar, 0, row, 0, h);
 }
-// one 32-byte store of 8 words (the address is 32-byte aligned)
-__device__ __forceinline__ void st_global_v8(void* dst, const uint32_t* r) {
-  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(r[0]), "r"(r[1]), "r"(r[2]),
-               "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
-               : "memory");
-}
-// one 32-byte load of 8 words (the address is 32-byte aligned)
-__device__ __forceinline__ void ld_global_v8(const void* src, uint32_t* r) {
-  asm volatile("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ unsigned long long global_timer_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ float ex2(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-
-// p rounded to 11 significant bits (what fp16 keeps) with plain fp32 arithmetic
-// (Veltkamp split), so the fp16 conversion that follows is exact and the
-// normaliser can sum the very values the MMA multiplies without converting back.
-__device__ __forceinline__ float round_to_half_bits(float p) {
-  float c = __fmul_rn(p, 8193.0f);
-  return __fsub_rn(c, __fsub_rn(c, p));
-}
-// four consecutive output elements at element offset `off` of `out` (fp32, or bf16 when the context's
-// out_dtype says so)
-__device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
-  __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<uint32_t*>(&h);
-}
-__device__ __forceinline__ void store_out4(const AttnArgs& a, size_t off, float4 v) {
-  if (a.out_bf16) {
-    *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.out) + off) =
-        make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w));
-  } else {
-    *reinterpret_cast<float4*>(a.out + off) = v;
-  }
-}
-__device__ __forceinline__ WorkItem load_item(const WorkItem* p) {
-  const int4* q = reinterpret_cast<const int4*>(p);
-  int4 a = __ldg(q), b = __ldg(q + 1), c = __ldg(q + 2);
-  WorkItem w;
-  w.kind = a.x; w.seq = a.y; w.row0 = a.z; w.nrows = a.w;
-  w.chunk = b.x; w.kt0 = b.y; w.kt1 = b.z; w.pad = b.w;
-  w.seq_start = c.x; w.seq_end = c.y; w.blk_start = c.z; w.pad2 = c.w;
-  return w;
-}
-
-
-
-struct Cta {
-  uint32_t base;            // shared-space address of the region
-  uint8_t* gen;             // generic pointer to the same region
-  uint32_t tmem;            // TMEM base address
-  volatile int* abort_flag;
-  volatile uint32_t* flag;  // scratch word for CTA-wide decisions
-  int32_t* status;
-  __device__ __forceinline__ uint32_t bar(int slot) const { return base + SM_BAR + 8u * slot; }
-};
-
-// Bounded wait on phase `parity`; false if it ran out or the CTA is unwinding.
-__device__ __noinline__ bool wait_slow(const Cta& c, uint32_t bar, uint32_t parity, int loc) {
-  long long t0 = clock64();
-  for (;;) {
-#pragma unroll 1
-    for (int i = 0; i < 32; ++i)
-      if (mbar_try(bar, parity)) return true;
-    if (*c.abort_flag) return false;
-    if (clock64() - t0 > WAIT_CYCLES) {
-      *c.abort_flag = 1;
-      if (atomicCAS(c.status, 0, (int)LACACHE_ERR_TIMEOUT) == 0) {
-        c.status[1] = loc;
-        c.status[2] = blockIdx.x;
-        c.status[3] = threadIdx.x;
-      }
-      return false;
-    }
-  }
-}
-__device__ __forceinline__ bool wait_bar(const Cta& c, int slot, uint32_t parity, int loc) {
-  uint32_t b = c.bar(slot);
-  if (mbar_try(b, parity)) return true;
-  return wait_slow(c, b, parity, loc);
-}
-
 // One unit of work of the stream role, decoded identically by every warp role.
 // What the stream role's templates are instantiated for: a build or a full recompute; a step; a build
 // over key windows (units may start from a stored state and store a snapshot: the incremental rebuild).
@@ -505,12 +380,6 @@ __device__ void stream_producer(const Cta& c, const TcMaps& maps, const Geometry
   // that overlap the block -- so tiles of fixed tokens are requested at once and
   // the wait comes only when nothing else can be issued.
   bool dep_done = false;
-  // build with one-plane operands: full row tiles leave as bulk tensor stores from a staging tile the row
-  // threads fill (units in the order of the Q loads; at most two are between their Q load and their store)
-  constexpr bool STAGED = KIND == KIND_BUILD && !SPLIT;
-  int st_slot0 = 0, st_slot1 = 0;   // row0 | head << 24 of the (at most two) units between their Q load and their store
-  int st_head = 0, st_tail = 0;
-  bool st_pending = false;
   const bool q_computed = STEP && a.q_raw != nullptr;
   auto tile_depends = [&](const TileCursor& cu) {
     if (!STEP) return true;
@@ -518,22 +387,8 @@ __device__ void stream_producer(const Cta& c, const TcMaps& maps, const Geometry
     return krow < cu.it.blk_start + g.block_len && krow + BN > cu.it.blk_start;
   };
   long long t_idle = 0;
-  while (cq.valid || ck.valid || cv.valid || (STAGED && (st_head < st_tail || st_pending))) {
+  while (cq.valid || ck.valid || cv.valid) {
     bool did = false, blocked_on_dep = false;
-    if (STAGED && st_head < st_tail && mbar_test(c.bar(BAR_ST_RDY), st_head & 1)) {
-      // (dep_done: the unit's Q tile was loaded after the wait for the preceding grids, so no store precedes it)
-      const int sv = (st_head & 1) ? st_slot1 : st_slot0;
-      if (sv >= 0) {
-#pragma unroll
-        for (int cb = 0; cb < 4; ++cb) tma_store_3d(&maps.st_o, c.base + st_box(cb), 32 * cb, sv & 0xFFFFFF, sv >> 24);
-        bulk_commit();
-        st_pending = true;
-      } else {
-        mbar_arrive(c.bar(BAR_ST_FREE));
-      }
-      ++st_head;
-      did = true;
-    }
     if (cq.valid) {  // a unit without key tiles still needs its Q load (the MMA thread waits for it)
       if (cq.uu == 0 && q_computed) {
         // the row threads rotate this tile from the raw queries: nothing to load,
@@ -547,11 +402,6 @@ __device__ void stream_producer(const Cta& c, const TcMaps& maps, const Geometry
         blocked_on_dep = true;
       } else if (cq.uu == 0 || mbar_test(c.bar(BAR_Q_FREE), (cq.uu - 1) & 1)) {
         load_q_tile<SPLIT>(c, maps, cq.un.q_rows, cq.un.row0, cq.un.h, cq.un.rh != 0);
-        if (STAGED && a.st_tma && cq.un.epi == EPI_STATE) {
-          const int sv = cq.un.row0 | (cq.un.h << 24) | (cq.un.nrows == BM ? 0 : (int)0x80000000u);   // (top bit: a clipped tile, nothing staged)
-          if (st_tail & 1) st_slot1 = sv; else st_slot0 = sv;
-          ++st_tail;
-        }
         cq.q_done = true;
         cq.t = cq.un.t1;
         cursor_advance<PACKED, KIND, SPLIT>(g, a, cq, stride, n_units);
@@ -593,12 +443,6 @@ __device__ void stream_producer(const Cta& c, const TcMaps& maps, const Geometry
       dep_done = true;
       did = true;
     }
-    if (STAGED && !did && st_pending) {   // nothing else to issue: the last store has read its staging tile by now
-      bulk_wait_read();
-      mbar_arrive(c.bar(BAR_ST_FREE));
-      st_pending = false;
-      did = true;
-    }
     if (did) {
       t_idle = 0;
     } else {  // nothing free: bounded idle
@@ -613,7 +457,6 @@ __device__ void stream_producer(const Cta& c, const TcMaps& maps, const Geometry
       }
     }
   }
-  if (STAGED) bulk_wait_read();  // shared memory stays valid until the last store has read it
   // (a CTA without units never touches memory the RoPE kernel writes)
 }
 
@@ -1258,47 +1101,6 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
       if (!epi_sync(c, epi_phase)) return;  // the flag may be rewritten
       if (un.q_rows == BM && threadIdx.x == 64) mbar_arrive(c.bar(BAR_Q_FREE));
       continue;
-    }
-    if (KIND == KIND_BUILD && !SPLIT && un.epi == EPI_STATE && a.st_tma) {
-      // Build with one-plane operands: the state of a full row tile goes to a staging tile (four swizzled
-      // boxes outside the Q tile and the key / value stages) and leaves as bulk tensor stores issued by the
-      // producer thread, so these threads are back at the next unit's tiles after 16 shared-memory stores
-      // each instead of eight 32-byte global stores that touch 32 different lines per warp instruction.
-      // Every unit takes part in the hand-over (a clipped tile stores the old way and hands over nothing),
-      // so the barriers' phases follow the unit count.
-      if (uu >= 1 && !wait_bar(c, BAR_ST_FREE, (uu - 1) & 1, LOC_WAIT_O)) return;  // the previous store has read the tile
-      if (un.nrows == BM) {
-        if (threadIdx.x == 64) mbar_arrive(c.bar(BAR_Q_FREE));
-#pragma unroll 1
-        for (int cb = 0; cb < 4; ++cb) {     // sixteen features at a time: half a box row
-          uint32_t rr[16];
-          if (!first_tile) {
-            tmem_ld16(tlane + TS_O + 64 * half + 16 * cb, rr);
-            tmem_ld_wait();
-          } else {
-#pragma unroll
-            for (int j = 0; j < 16; ++j) rr[j] = 0u;
-          }
-          uint8_t* const sb = c.gen + st_box(2 * half + (cb >> 1)) + r * 128;
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const int ch = 4 * (cb & 1) + i;
-            *reinterpret_cast<float4*>(sb + ((ch ^ (r & 7)) << 4)) =
-                make_float4(__uint_as_float(rr[4 * i]), __uint_as_float(rr[4 * i + 1]), __uint_as_float(rr[4 * i + 2]),
-                            __uint_as_float(rr[4 * i + 3]));
-          }
-        }
-        if (half == 0) {
-          const size_t srow = (size_t)un.h * g.Tp + row;
-          a.st.m[srow] = m_ref; a.st.l[srow] = l_run;
-        }
-        fence_async_smem();   // the bulk stores read the tile through the async proxy
-        mbar_arrive(c.bar(BAR_ST_RDY));
-        tc_fence_before();
-        mbar_arrive(c.bar(BAR_O_FREE));  // the next unit may overwrite O~
-        continue;
-      }
-      mbar_arrive(c.bar(BAR_ST_RDY));   // (nothing staged: the producer answers at once)
     }
     if (un.epi == EPI_STATE && un.q_rows == BM) {
       // Cached state of a build unit, straight from TMEM to global memory (each thread 256
@@ -1982,6 +1784,7 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
   Cta c;
   c.base = smem_u32(smem_raw);
   c.gen = smem_raw;
+  c.bar0 = c.base + SM_BAR;
   uint32_t* words = reinterpret_cast<uint32_t*>(smem_raw + SM_BAR + 8 * N_BARS);  // [0] tmem, [1] abort, [2] flag
   c.abort_flag = reinterpret_cast<volatile int*>(words + 1);
   c.flag = reinterpret_cast<volatile uint32_t*>(words + 2);
@@ -2145,13 +1948,14 @@ bool make_f32_map(CUtensorMap* m, void* base, cuuint64_t d1, cuuint64_t d2, cuui
 // Split-bf16 planes [plane][H][2][Tp][64] (hi plane at `base`, lo plane `plane_elems` further) as a 5-D
 // tensor; fp16 values [H][2][Tp][64] as a 4-D tensor.  Box: `box_rows` rows of one head, both feature
 // halves (and both planes).
-bool make_qk_map(CUtensorMap* m, void* base, int H, int Tp, int box_rows, int planes, char* err, int errlen) {
+bool make_qk_map(CUtensorMap* m, void* base, int H, int Tp, int box_rows, int planes, char* err, int errlen,
+                 bool single = false) {   // single: a box holds one feature half of one plane
   EncodeTiledFn enc = get_encode();
   if (!enc) { snprintf(err, errlen, "cuTensorMapEncodeTiled entry point not found"); return false; }
   // (with one plane the last dimension has extent 1: the same instruction loads half as much)
   cuuint64_t dims[5] = {64, (cuuint64_t)Tp, 2, (cuuint64_t)H, (cuuint64_t)planes};
   cuuint64_t strides[4] = {128, (cuuint64_t)Tp * 128, (cuuint64_t)Tp * 256, (cuuint64_t)H * Tp * 256};
-  cuuint32_t box[5] = {64, (cuuint32_t)box_rows, 2, 1, (cuuint32_t)planes};
+  cuuint32_t box[5] = {64, (cuuint32_t)box_rows, single ? 1u : 2u, 1, single ? 1u : (cuuint32_t)planes};
   cuuint32_t estr[5] = {1, 1, 1, 1, 1};
   CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, base, dims, strides, box, estr,
                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -2191,16 +1995,17 @@ bool make_v_map(CUtensorMap* m, void* base, int H, int Tp, int box_rows, char* e
 }  // namespace
 
 namespace {
-// thirteen instantiations: {split planes, one plane per operand} x {build / full recompute; build over key windows; the
-// step of an MHA and of a GQA model, each with either variant of the merge role}
+// {build / full recompute; build over key windows; the step of an MHA and of a GQA model, each with either variant of
+// the merge role; the paired step}.  One-plane builds run lacache_rows.cu, and the paired step exists for one-plane
+// operands only: null where there is none.
 template <bool SPLIT>
 const void* const* kernel_table() {
-  // (the paired step exists for one-plane operands only: with split planes the entry repeats the ordinary step)
   static const void* const t[7] = {
-      (const void*)tc_attn_kernel<false, KIND_BUILD, false, SPLIT>, (const void*)tc_attn_kernel<false, KIND_WINDOW, false, SPLIT>,
+      SPLIT ? (const void*)tc_attn_kernel<false, KIND_BUILD, false, true> : nullptr,
+      SPLIT ? (const void*)tc_attn_kernel<false, KIND_WINDOW, false, true> : nullptr,
       (const void*)tc_attn_kernel<false, KIND_STEP, false, SPLIT>,  (const void*)tc_attn_kernel<false, KIND_STEP, true, SPLIT>,
       (const void*)tc_attn_kernel<true, KIND_STEP, false, SPLIT>,   (const void*)tc_attn_kernel<true, KIND_STEP, true, SPLIT>,
-      (const void*)tc_attn_kernel<false, SPLIT ? KIND_STEP : KIND_STEP2, true, SPLIT>};
+      SPLIT ? nullptr : (const void*)tc_attn_kernel<false, KIND_STEP2, true, false>};
   return t;
 }
 }  // namespace
@@ -2209,6 +2014,7 @@ cudaError_t tc_prepare() {
   for (int split = 0; split < 2; ++split) {
     const void* const* t = split ? kernel_table<true>() : kernel_table<false>();
     for (int i = 0; i < 7; ++i) {
+      if (!t[i]) continue;
       cudaError_t e = cudaFuncSetAttribute(t[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
       if (e != cudaSuccess) return e;
     }
@@ -2242,6 +2048,7 @@ TcMaps* tc_make_maps(const Geometry& g, const RotBuffers& rot, float* state_o, b
             make_qk_map(&m->k, rot.k_hi, g.Hkv, g.Tp, bn, planes, err, errlen) &&
             make_qk_map(&m->k64, rot.k_hi, g.Hkv, g.Tp, 64, planes, err, errlen) &&
             make_qk_map(&m->k32, rot.k_hi, g.Hkv, g.Tp, 32, planes, err, errlen) &&
+            make_qk_map(&m->k_box, rot.k_hi, g.Hkv, g.Tp, TC_ROW_KEYS, planes, err, errlen, true) &&
             make_v_map(&m->v, rot.v, g.Hkv, g.Tp, bn, err, errlen) &&
             make_v_map(&m->v64, rot.v, g.Hkv, g.Tp, 64, err, errlen) &&
             make_v_map(&m->v32, rot.v, g.Hkv, g.Tp, 32, err, errlen) &&
