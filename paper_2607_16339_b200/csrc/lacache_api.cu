@@ -331,12 +331,52 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
     }
   }
   if (tpc <= 0) tpc = 2;
-  // the row kernel's items, the most work first: a CTA draws every n-th
+  // The row kernel's items, the most work first: its CTAs draw them in a snake (0 .. n - 1, n - 1 .. 0, ...).  `keys`: of
+  // a key-window item from the token its tiles are counted from.
+  auto row_cost = [](int nrows, int keys) {   // in key tiles of two row tiles (one row tile alone takes 0.62 of two)
+    return (nrows > TC_ROWS ? 1.0 : 0.62) * ((keys + TC_ROW_KEYS - 1) / TC_ROW_KEYS) + 1.5;
+  };
+  auto item_keys = [](const WorkItem& w) { return w.kind == ITEM_ROWS_WINDOW ? std::max(0, w.kt1 - w.pad) : w.seq_end - w.seq_start; };
   auto longest_first = [&](int from) {
-    std::stable_sort(items.begin() + from, items.end(), [](const WorkItem& p, const WorkItem& q) {
-      const long long wp = (long long)((p.nrows + 127) / 128) * (p.seq_end - p.seq_start), wq = (long long)((q.nrows + 127) / 128) * (q.seq_end - q.seq_start);
-      return wp > wq;
+    if (!rk) return;
+    std::stable_sort(items.begin() + from, items.end(), [&](const WorkItem& p, const WorkItem& q) {
+      return row_cost(p.nrows, item_keys(p)) > row_cost(q.nrows, item_keys(q));
     });
+  };
+  // Few units leave the last round of CTAs half empty: some of the items with the least work then go out as two of one row
+  // tile each (at most 8 items, the number that makes the longest CTA shortest).
+  auto split_items = [&](int from) {
+    const int n = (int)items.size() - from, P = c->num_sms;
+    if (!rk || (long long)n * g.Hq > 8ll * P) return;
+    std::vector<WorkItem> best(items.begin() + from, items.end());
+    double best_t = 1e30;
+    for (int sp = 0; sp <= std::min(8, n); ++sp) {
+      std::vector<WorkItem> v;
+      int left = sp;
+      for (int i = n - 1; i >= 0; --i) {
+        WorkItem w = items[from + i];
+        if (left > 0 && w.nrows > TC_ROWS) {
+          --left;
+          WorkItem x = w;
+          x.row0 += TC_ROWS; x.nrows -= TC_ROWS; w.nrows = TC_ROWS;
+          v.push_back(x);
+        }
+        v.push_back(w);
+      }
+      if (left > 0) break;
+      std::stable_sort(v.begin(), v.end(), [&](const WorkItem& p, const WorkItem& q) { return row_cost(p.nrows, item_keys(p)) > row_cost(q.nrows, item_keys(q)); });
+      std::vector<double> t(P, 0.0);
+      double most = 0.0;
+      for (int u = 0; u < (int)v.size() * g.Hq; ++u) {
+        const int k = u / P, b = u % P;
+        double& cta = t[(k & 1) ? P - 1 - b : b];
+        cta += row_cost(v[u / g.Hq].nrows, item_keys(v[u / g.Hq]));
+        most = std::max(most, cta);
+      }
+      if (most < best_t - 1e-9) { best_t = most; best = v; }
+    }
+    items.resize(from);
+    items.insert(items.end(), best.begin(), best.end());
   };
   c->max_chunks = 1;
   for (int k = 0; k < g.n_blk; ++k) {
@@ -387,6 +427,7 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
       if (c->cu[b + 1] - c->cu[b] > g.block_len)
         add_row_tiles(items, b, c->cu[b], c->cu[b + 1], TC_ROW_ITEM, c->cu[b], c->cu[b + 1], c->blk_start_all[(size_t)k * g.B + b]);
     longest_first(off);
+    split_items(off);
     c->build_list.push_back({off, (int)items.size() - off});
   }
   int inc_chunks = 1;
@@ -414,6 +455,7 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
       add_row_tiles(items, b, e0, ce, RI, cs, ce, s0);
       window(from, cs, cs, s0, 0);
     }
+    longest_first(off);
     c->inc_prefix.push_back({off, (int)items.size() - off});
     off = (int)items.size();
     for (int b = 0; b < g.B; ++b) {
@@ -423,6 +465,7 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
       add_row_tiles(items, b, e0, ce, RI, cs, ce, s0);
       window(from, e0, e0, ce, W_INIT);
     }
+    longest_first(off);
     c->inc_comb.push_back({off, (int)items.size() - off});
     // advancing from block k - 1 (rows [sp, s0), blocks are consecutive), in two launches:
     off = (int)items.size();
@@ -477,6 +520,7 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
       add_row_tiles(items, b, sp, s0, RI, cs, ce, s0);
       window(from, e0, e0, ce, W_INIT);
     }
+    longest_first(off);
     c->inc_fused.push_back({off, (int)items.size() - off});
   }
   c->part_chunks = std::max(c->max_chunks, inc_chunks);
@@ -523,6 +567,7 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
           else if (pass == 1) window(from, hi, hi, ce, lo > cs ? W_INIT : 0);
           else window(from, lo, lo, hi, W_INIT | W_OUT);
         }
+        longest_first(off);
         (pass == 0 ? c->tile_prefix : pass == 1 ? c->tile_suffix : c->tile_step).push_back({off, (int)items.size() - off});
       }
     }
@@ -530,7 +575,8 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
   {
     int off = (int)items.size();
     for (int b = 0; b < g.B; ++b) add_row_tiles(items, b, c->cu[b], c->cu[b + 1], RI, c->cu[b], c->cu[b + 1], 0);
-    if (rk) longest_first(off);
+    longest_first(off);
+    split_items(off);
     c->full_list = {off, (int)items.size() - off};
   }
   c->items_host = items;

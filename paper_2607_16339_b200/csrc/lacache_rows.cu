@@ -8,14 +8,11 @@
 // other, in which the tensor cores and the exponential unit take turns; with two tiles one works for A while the
 // other works for B.
 //   warps 0..3   row threads of tile A, warps 4..7 of tile B: thread = query row = TMEM lane
-//   warp 8       TMA producer (one lane)
-//   warp 9       issues the score products S = Q' K'^T of both tiles, warp 10 the products O~ += P~ V
-// TMEM (512 columns): ONE score tile S (128) that A and B use in turn, their fp16 probabilities P~ (64 each) and their
-// O~ (128 each, accumulated over a unit's key tiles, rescaled in place when a row outgrows its reference).  A row
-// thread takes its 128 scores into registers at once and S is free again, so that the next scores of its tile are
-// computed while it still forms the probabilities of this one.  (With a score tile each, P~ written over S for want of
-// columns, the scores of key tile j + 1 had to wait for the products of tile j.)  Probabilities go over in halves of 64
-// keys: the products of the first half run while the row threads work on the second.
+//   warp 9       issues the products S = Q' K'^T and O~ += P~ V of both tiles
+//   warps 8, 10, 11  TMA loads of Q', keys, values (one lane each)
+// TMEM (512 columns): per tile its scores S (128; the fp16 probabilities P~ are written over the first 64) and O~ (128,
+// accumulated over a unit's key tiles, rescaled in place when a row outgrows its reference).  Probabilities go over in
+// halves of 64 keys: the products of the first half run while the row threads work on the second.
 // A row thread's time per key tile is what the kernel is bound by (two warps per scheduler, each a serial chain): the
 // exponentials of the first half are therefore formed with the reference exponent as it stands, beside the row's maximum,
 // and again only when the maximum asks for another one; the sums of the rounded probabilities come after the hand-over.
@@ -36,16 +33,16 @@ namespace {
 using namespace tcu;
 
 constexpr int ROW_THREADS = 256;
-constexpr int THREADS = 384;      // (warp 11 idles: register splits work on groups of four warps)
-constexpr int LAUNCH_REGS = 168, ROW_REGS = 216, ISSUER_REGS = 72;
+constexpr int THREADS = 384;
+constexpr int LAUNCH_REGS = 168, ROW_REGS = 208, ISSUER_REGS = 88;
 static_assert(ROW_THREADS * ROW_REGS + (THREADS - ROW_THREADS) * ISSUER_REGS <= THREADS * LAUNCH_REGS, "more registers than the block has");
 constexpr int KT = TC_ROW_KEYS;   // keys per tile
-constexpr int W_PRODUCER = 8, W_SCORES = 9, W_PRODUCTS = 10;   // the warps with another role
+constexpr int W_QUERIES = 8, W_MMA = 9, W_KEYS = 10, W_VALUES = 11;   // the warps with another role
 
 struct RowMaps {
   CUtensorMap q;      // box {64, 128 rows, 2 halves, 1 head, planes}: a whole Q' tile
-  CUtensorMap k_box;  // box {64, 128 rows, 1, 1, 1}
-  CUtensorMap v64;    // box {64, 64 rows, 2 halves, 1}
+  CUtensorMap k;      // likewise for keys
+  CUtensorMap v;      // box {64, 128 rows, 2 halves, 1}
 };
 
 constexpr uint32_t BOX = 16384;
@@ -58,18 +55,16 @@ constexpr uint32_t SM_BARS = SM_ST + 8 * 4096;
 
 enum {
   B_Q_FULL = 0, B_Q_FREE = 2,     // per tile
-  B_K_FULL = 4, B_K_FREE = 8,     // per box slot
-  B_V_FULL = 12, B_V_FREE = 16,   // per box slot
-  B_S_FULL = 20,                  // per tile
-  B_P_RDY = 22,                   // per tile and half: 2 * tile + half
-  B_PV_DONE = 26, B_O_FREE = 28,  // per tile
-  B_S_FREE = 30,
-  B_DONE = 31, N_BARS = 32
+  B_K_FULL = 4, B_K_FREE = 6,     // per stage
+  B_V_FULL = 8, B_V_FREE = 10,    // per stage
+  B_S_FULL = 12,                  // per tile
+  B_P_RDY = 14,                   // per tile and half: 2 * tile + half
+  B_O_FULL = 18, B_O_FREE = 20,   // per tile
+  B_DONE = 22, N_BARS = 23
 };
 constexpr uint32_t SM_TOTAL = SM_BARS + 8 * N_BARS + 16;
 static_assert(SM_TOTAL <= 232448, "exceeds the 227 KB per-CTA limit");
-constexpr uint32_t TM_S = 0;
-__device__ constexpr uint32_t TM_P(int x) { return 128u + 64u * x; }
+__device__ constexpr uint32_t TM_S(int x) { return 128u * x; }   // (P~ in its first 64 columns)
 __device__ constexpr uint32_t TM_O(int x) { return 256u + 128u * x; }
 
 struct Unit {
@@ -80,6 +75,13 @@ struct Unit {
   bool init, snap, out;   // start from a stored state; store the state after the first tile; write normalised rows
   __device__ __forceinline__ int tiles() const { return nrows > BM ? 2 : 1; }
   __device__ __forceinline__ int key_row(int t) const { return (base1 >= 0 && t > 0) ? base1 + (t - 1) * KT : key_base + t * KT; }
+};
+
+// A CTA's units: the list, sorted by work, is dealt out in a snake, so that who draws first in one round draws last in
+// the next.
+struct Walk {
+  int first, stride, n_units;
+  __device__ __forceinline__ int unit(int k) const { return k * stride + ((k & 1) ? stride - 1 - first : first); }   // (grows with k)
 };
 
 // units are head-minor (unit u = item u / Hq of head u % Hq): neighbours share keys in L2
@@ -118,165 +120,158 @@ __device__ __forceinline__ Unit decode(const Geometry& g, const AttnArgs& a, int
   return un;
 }
 
-// ---- producer -----------------------------------------------------------------------------------------------
-// Three cursors -- Q' tiles, key boxes, value boxes -- and whichever has a free slot issues its load.
-template <bool WINDOW>
-__device__ void row_producer(const Cta& c, const RowMaps& maps, const Geometry& g, const AttnArgs& a, int first,
-                             int stride, int n_units) {
-  grid_dependency_wait();   // every operand is written by the kernels ahead
-  struct Cursor { int u, t, part, n; Unit un; bool live; };   // n: units (Q') or tiles (keys, values) so far
-  auto load_unit = [&](Cursor& k) {
-    for (; k.u < n_units; k.u += stride) {
-      k.un = decode<WINDOW>(g, a, k.u);
-      if (k.un.n_tiles > 0) return;
+// wait_bar without a call: a row thread has most of its registers in use where it waits
+__device__ __forceinline__ bool wait_here(const Cta& c, int slot, uint32_t parity, int loc) {
+  const uint32_t bar = c.bar(slot);
+  if (mbar_try(bar, parity)) return true;
+  const long long t0 = clock64();
+  while (!mbar_try(bar, parity)) {
+    if (*c.abort_flag) return false;
+    if (clock64() - t0 > WAIT_CYCLES) {
+      *c.abort_flag = 1;
+      if (atomicCAS(c.status, 0, (int)LACACHE_ERR_TIMEOUT) == 0) {
+        c.status[1] = loc; c.status[2] = blockIdx.x; c.status[3] = threadIdx.x;
+      }
+      return false;
     }
-    k.live = false;
+  }
+  return true;
+}
+
+// ---- producers ----------------------------------------------------------------------------------------------
+// One lane each for Q' tiles, key tiles and value tiles, with blocking waits (one lane that polled all three took several
+// hundred cycles to notice a free stage, which with two stages is time the tensor core waits).
+template <bool WINDOW>
+__device__ void load_queries(const Cta& c, const RowMaps& maps, const Geometry& g, const AttnArgs& a, const Walk& wk) {
+  int n0 = 0, n1 = 0;   // Q' tiles loaded, per tile slot
+  for (int k_ = 0, u = wk.unit(0); u < wk.n_units; u = wk.unit(++k_)) {
+    const Unit un = decode<WINDOW>(g, a, u);
+    if (un.n_tiles == 0) continue;
+    for (int x = 0; x < un.tiles(); ++x) {
+      const int n = x ? n1 : n0;
+      if (n > 0 && !wait_here(c, B_Q_FREE + x, (n - 1) & 1, LOC_WAIT_Q)) return;
+      mbar_expect_tx(c.bar(B_Q_FULL + x), Q_TILE);
+      tma_load_5d(c.base + x * Q_TILE, &maps.q, c.bar(B_Q_FULL + x), 0, un.row0 + BM * x, 0, un.h, 0);
+      if (x) ++n1; else ++n0;
+    }
+  }
+}
+template <bool WINDOW, bool KEYS>
+__device__ void load_tiles(const Cta& c, const RowMaps& maps, const Geometry& g, const AttnArgs& a, const Walk& wk) {
+  constexpr int FULL = KEYS ? B_K_FULL : B_V_FULL, FREE = KEYS ? B_K_FREE : B_V_FREE;
+  int n = 0;            // tiles so far
+  for (int k_ = 0, u = wk.unit(0); u < wk.n_units; u = wk.unit(++k_)) {
+    const Unit un = decode<WINDOW>(g, a, u);
+    for (int t = 0; t < un.n_tiles; ++t, ++n) {
+      const int st = n % STAGES, use = n / STAGES;
+      if (use > 0 && !wait_here(c, FREE + st, (use - 1) & 1, KEYS ? LOC_WAIT_K : LOC_WAIT_V)) return;
+      mbar_expect_tx(c.bar(FULL + st), 2 * BOX);
+      if (KEYS) tma_load_5d(c.base + SM_K + st * 2 * BOX, &maps.k, c.bar(FULL + st), 0, un.key_row(t), 0, un.kh, 0);
+      else tma_load_4d(c.base + SM_V + st * 2 * BOX, &maps.v, c.bar(FULL + st), 0, un.key_row(t), 0, un.kh);
+    }
+  }
+}
+
+// ---- tensor-core products -----------------------------------------------------------------------------------
+// A whole warp walks this loop and one elected lane issues.  The order is fixed: P~V of a tile's key tile j, then its
+// scores of key tile j + 1, A and B in turn.  The tensor core executes what one thread issues in order, so the scores
+// may overwrite the probabilities the products ahead of them read, and a tile's scores being complete says that its
+// products are.  The order also keeps the two tiles half a period apart: while one's products and scores are computed,
+// the other's row threads have the exponential unit.
+template <bool WINDOW>
+__device__ void row_mma(const Cta& c, const Geometry& g, const AttnArgs& a, const Walk& wk) {
+  const uint32_t idesc_s = idesc_f16(g.op_f16 ? 0u : 1u, 0u, BM, KT);
+  constexpr uint32_t idesc_o = idesc_f16(0u /*fp16*/, 1u, BM, D);
+  const bool leader = elect_one();
+  int nq0 = 0, nq1 = 0, no0 = 0, no1 = 0, np0 = 0, np1 = 0;   // per tile slot: units' scores begun, units' products begun, key tiles of products
+  int ks = 0, kv = 0;                                   // key tiles of scores (both tiles' of it), of products
+  // scores of key tile j of a unit: tile x of nx, n_tiles in all
+  auto scores = [&](int x, int nx, int j, int n_tiles) -> bool {
+    const int st = ks % STAGES;
+    if (j == 0) {
+      if (!wait_here(c, B_Q_FULL + x, (x ? nq1 : nq0) & 1, LOC_WAIT_Q)) return false;
+      if (x) ++nq1; else ++nq0;
+    }
+    if (x == 0 && !wait_here(c, B_K_FULL + st, (uint32_t)(ks / STAGES) & 1u, LOC_WAIT_K)) return false;
+    tc_fence_after();
+    {
+      const uint64_t kd = smem_desc(c.base + SM_K + st * 2 * BOX, 16, 1024);
+      const uint64_t qd = smem_desc(c.base + x * Q_TILE, 16, 1024);
+      if (leader) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {   // 64 features of a row are 128 bytes, the next 64 a box (16 KB) on
+          const uint32_t off = (i >> 2) * (BOX >> 4) + (i & 3) * 2;
+          mma_ss(c.tmem + TM_S(x), qd + off, kd + off, idesc_s, i ? 1u : 0u);
+        }
+        if (x == nx - 1) tc_commit(c.bar(B_K_FREE + st));
+      }
+    }
+    if (leader) {
+      tc_commit(c.bar(B_S_FULL + x));
+      if (j == n_tiles - 1) tc_commit(c.bar(B_Q_FREE + x));
+    }
+    if (x == nx - 1) ++ks;
+    return true;
   };
-  Cursor q{first, 0, 0, 0, Unit{}, true};
-  load_unit(q);
-  Cursor k = q, v = q;
-  int nq0 = 0, nq1 = 0;   // Q' tiles loaded, per tile slot
-  long long t_idle = 0;
-  while (q.live || k.live || v.live) {
-    bool did = false;
-    if (q.live) {
-      const int x = q.part;
-      const int n = x ? nq1 : nq0;
-      if (n == 0 || mbar_test(c.bar(B_Q_FREE + x), (n - 1) & 1)) {
-        mbar_expect_tx(c.bar(B_Q_FULL + x), Q_TILE);
-        tma_load_5d(c.base + x * Q_TILE, &maps.q, c.bar(B_Q_FULL + x), 0, q.un.row0 + BM * x, 0, q.un.h, 0);
-        if (x) ++nq1; else ++nq0;
-        if (++q.part == q.un.tiles()) { q.part = 0; q.u += stride; load_unit(q); }
-        did = true;
-      }
+  // the next unit with key tiles, from this CTA's k-th on
+  auto next_unit = [&](int& k, Unit& un) -> bool {
+    for (; wk.unit(k) < wk.n_units; ++k) {
+      un = decode<WINDOW>(g, a, wk.unit(k));
+      if (un.n_tiles > 0) return true;
     }
-    if (k.live) {
-      const int slot = (k.n % STAGES) * 2 + k.part, use = k.n / STAGES;
-      if (use == 0 || mbar_test(c.bar(B_K_FREE + slot), (use - 1) & 1)) {
-        mbar_expect_tx(c.bar(B_K_FULL + slot), BOX);
-        tma_load_5d(c.base + SM_K + slot * BOX, &maps.k_box, c.bar(B_K_FULL + slot), 0, k.un.key_row(k.t),
-                    k.part, k.un.kh, 0);
-        if (++k.part == 2) {
-          k.part = 0;
-          ++k.n;
-          if (++k.t == k.un.n_tiles) { k.t = 0; k.u += stride; load_unit(k); }
-        }
-        did = true;
-      }
-    }
-    if (v.live) {
-      const int slot = (v.n % STAGES) * 2 + v.part, use = v.n / STAGES;
-      if (use == 0 || mbar_test(c.bar(B_V_FREE + slot), (use - 1) & 1)) {
-        mbar_expect_tx(c.bar(B_V_FULL + slot), BOX);
-        tma_load_4d(c.base + SM_V + slot * BOX, &maps.v64, c.bar(B_V_FULL + slot), 0, v.un.key_row(v.t) + 64 * v.part, 0, v.un.kh);
-        if (++v.part == 2) {
-          v.part = 0;
-          ++v.n;
-          if (++v.t == v.un.n_tiles) { v.t = 0; v.u += stride; load_unit(v); }
-        }
-        did = true;
-      }
-    }
-    if (did) {
-      t_idle = 0;
-    } else {  // nothing free: bounded idle
-      if (t_idle == 0) t_idle = clock64();
-      if (*c.abort_flag) return;
-      if (clock64() - t_idle > WAIT_CYCLES) {
-        *c.abort_flag = 1;
-        if (atomicCAS(c.status, 0, (int)LACACHE_ERR_TIMEOUT) == 0) {
-          c.status[1] = LOC_WAIT_K; c.status[2] = blockIdx.x; c.status[3] = threadIdx.x;
-        }
-        return;
-      }
-    }
-  }
-}
-
-// ---- the two issuers ----------------------------------------------------------------------------------------
-// A whole warp walks each of these loops and one elected lane issues.
-template <bool WINDOW>
-__device__ void row_scores(const Cta& c, const Geometry& g, const AttnArgs& a, int first, int stride, int n_units) {
-  const uint32_t idesc = idesc_f16(g.op_f16 ? 0u : 1u, 0u, BM, KT);
-  const bool leader = elect_one();
-  int nu[2] = {0, 0};   // units so far, per tile slot
-  int ns = 0;           // score tiles so far (A's and B's take turns)
-  int kt = 0;           // key tiles so far
-  for (int u = first; u < n_units; u += stride) {
-    const Unit un = decode<WINDOW>(g, a, u);
-    const int nx = un.tiles();
-    for (int j = 0; j < un.n_tiles; ++j, ++kt) {
-      const int slot0 = (kt % STAGES) * 2;
-      const uint32_t kph = (uint32_t)(kt / STAGES) & 1u;
+    return false;
+  };
+  int k = 0;
+  Unit un{};
+  if (!next_unit(k, un)) return;
+  int nx = un.tiles();
+  if (!scores(0, nx, 0, un.n_tiles)) return;
+  if (nx > 1 && !scores(1, nx, 0, un.n_tiles)) return;
+  for (bool more = true; more;) {
+    ++k;
+    Unit nxt{};
+    more = next_unit(k, nxt);
+    const int nx2 = more ? nxt.tiles() : 0;
+    for (int j = 0; j < un.n_tiles; ++j, ++kv) {
+      const int st = kv % STAGES;
+      const bool last = j == un.n_tiles - 1;
 #pragma unroll
       for (int x = 0; x < 2; ++x) {
-        if (x >= nx) break;
-        if (j == 0 && !wait_bar(c, B_Q_FULL + x, nu[x] & 1, LOC_WAIT_Q)) return;
-        if (x == 0 && !wait_bar(c, B_K_FULL + slot0, kph, LOC_WAIT_K)) return;
-        if (ns > 0 && !wait_bar(c, B_S_FREE, (ns - 1) & 1, LOC_WAIT_S)) return;   // the scores before these have been taken
-        tc_fence_after();
+        if (x < nx) {
+          if (j == 0) {   // O~ of the unit before has been read by its row threads
+            const int no = x ? no1 : no0;
+            if (no > 0 && !wait_here(c, B_O_FREE + x, (no - 1) & 1, LOC_WAIT_O)) return;
+            if (x) ++no1; else ++no0;
+          }
 #pragma unroll
-        for (int b = 0; b < 2; ++b) {   // box b: features 64 b ...
-          if (x == 0 && b > 0) {
-            if (!wait_bar(c, B_K_FULL + slot0 + b, kph, LOC_WAIT_K)) return;
+          for (int hf = 0; hf < 2; ++hf) {
+            if (!wait_here(c, B_P_RDY + 2 * x + hf, (x ? np1 : np0) & 1, LOC_WAIT_S)) return;
+            if (x == 0 && hf == 0 && !wait_here(c, B_V_FULL + st, (uint32_t)(kv / STAGES) & 1u, LOC_WAIT_V)) return;
             tc_fence_after();
-          }
-          const uint64_t kd = smem_desc(c.base + SM_K + (slot0 + b) * BOX, 16, 1024);
-          const uint64_t qd = smem_desc(c.base + x * Q_TILE + b * BOX, 16, 1024);
-          if (leader) {
+            // B = V, MN-major: 64 features contiguous, the next 64 features a box on, 16 keys = 2 KB
+            const uint64_t vd = smem_desc(c.base + SM_V + st * 2 * BOX + hf * 8192, BOX, 1024);
+            const uint32_t first_acc = (j == 0 && hf == 0 && !(WINDOW && un.init)) ? 0u : 1u;
+            if (leader) {
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks) mma_ss(c.tmem + TM_S, qd + 2u * ks, kd + 2u * ks, idesc, (b > 0 || ks > 0) ? 1u : 0u);
-            if (x == nx - 1) tc_commit(c.bar(B_K_FREE + slot0 + b));
+              for (int i = 0; i < 4; ++i)
+                mma_ts(c.tmem + TM_O(x), c.tmem + TM_S(x) + 32 * hf + 8 * i, vd + (uint64_t)(i * 128), idesc_o, i ? 1u : first_acc);
+              if (x == nx - 1 && hf == 1) tc_commit(c.bar(B_V_FREE + st));
+            }
           }
+          if (last && leader) tc_commit(c.bar(B_O_FULL + x));
+          if (x) ++np1; else ++np0;
         }
-        ++ns;
-        if (leader) {
-          tc_commit(c.bar(B_S_FULL + x));
-          if (j == un.n_tiles - 1) tc_commit(c.bar(B_Q_FREE + x));
+        // the tile's next scores: of the next key tile, or of the next unit's first (a unit of one tile leaves B's place
+        // to the next unit at once)
+        if (!last) {
+          if (x < nx && !scores(x, nx, j + 1, un.n_tiles)) return;
+        } else if (x < nx2) {
+          if (!scores(x, nx2, 0, nxt.n_tiles)) return;
         }
-        if (j == un.n_tiles - 1) ++nu[x];
       }
     }
-  }
-}
-
-template <bool WINDOW>
-__device__ void row_products(const Cta& c, const Geometry& g, const AttnArgs& a, int first, int stride, int n_units) {
-  constexpr uint32_t idesc = idesc_f16(0u /*fp16*/, 1u, BM, D);
-  const bool leader = elect_one();
-  int nu[2] = {0, 0}, np[2] = {0, 0};   // units and tiles of products so far, per tile slot
-  int kt = 0;                           // key tiles so far
-  for (int u = first; u < n_units; u += stride) {
-    const Unit un = decode<WINDOW>(g, a, u);
-    const int nx = un.tiles();
-    for (int j = 0; j < un.n_tiles; ++j, ++kt) {
-      const int slot0 = (kt % STAGES) * 2;
-      const uint32_t vph = (uint32_t)(kt / STAGES) & 1u;
-#pragma unroll
-      for (int x = 0; x < 2; ++x) {
-        if (x >= nx) break;
-        // O~ of the unit before has been read by its row threads
-        if (j == 0 && nu[x] > 0 && !wait_bar(c, B_O_FREE + x, (nu[x] - 1) & 1, LOC_WAIT_O)) return;
-#pragma unroll
-        for (int hf = 0; hf < 2; ++hf) {
-          if (!wait_bar(c, B_P_RDY + 2 * x + hf, np[x] & 1, LOC_WAIT_S)) return;
-          if (x == 0 && !wait_bar(c, B_V_FULL + slot0 + hf, vph, LOC_WAIT_V)) return;
-          tc_fence_after();
-          // B = V, MN-major: 64 features contiguous, the next 64 features 8 KB on, 16 keys = 2 KB
-          const uint64_t vd = smem_desc(c.base + SM_V + (slot0 + hf) * BOX, 8192, 1024);
-          const uint32_t first_acc = (j == 0 && hf == 0 && !(WINDOW && un.init)) ? 0u : 1u;
-          if (leader) {
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
-              mma_ts(c.tmem + TM_O(x), c.tmem + TM_P(x) + 32 * hf + 8 * ks, vd + (uint64_t)(ks * 128), idesc, ks ? 1u : first_acc);
-            if (hf == 1) tc_commit(c.bar(B_PV_DONE + x));
-            if (x == nx - 1) tc_commit(c.bar(B_V_FREE + slot0 + hf));
-          }
-        }
-        ++np[x];
-        if (j == un.n_tiles - 1) ++nu[x];
-      }
-    }
+    un = nxt;
+    nx = nx2;
   }
 }
 
@@ -347,36 +342,18 @@ __device__ __forceinline__ void store_rows(const Cta& c, uint32_t o_tmem, bool h
   }
 }
 
-// wait_bar without a call: a row thread has most of its registers in use where it waits
-__device__ __forceinline__ bool wait_here(const Cta& c, int slot, uint32_t parity, int loc) {
-  const uint32_t bar = c.bar(slot);
-  if (mbar_try(bar, parity)) return true;
-  const long long t0 = clock64();
-  while (!mbar_try(bar, parity)) {
-    if (*c.abort_flag) return false;
-    if (clock64() - t0 > WAIT_CYCLES) {
-      *c.abort_flag = 1;
-      if (atomicCAS(c.status, 0, (int)LACACHE_ERR_TIMEOUT) == 0) {
-        c.status[1] = loc; c.status[2] = blockIdx.x; c.status[3] = threadIdx.x;
-      }
-      return false;
-    }
-  }
-  return true;
-}
-
 template <bool WINDOW>
-__device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, int first, int stride, int n_units) {
+__device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, const Walk& wk) {
   const float LN2 = 0.69314718055994530942f;
   const int lane = threadIdx.x & 31;
   const int x = threadIdx.x >> 7;                  // tile of this thread
   const int quad = (threadIdx.x >> 5) & 3;
   const int r = threadIdx.x & 127;                 // its row there = TMEM lane
   const uint32_t tlane = c.tmem + ((uint32_t)(quad * 32) << 16);
-  const uint32_t s_tmem = tlane + TM_S, p_tmem = tlane + TM_P(x), o_tmem = tlane + TM_O(x);
-  int n = 0;                                       // key tiles of this tile slot so far
+  const uint32_t s_tmem = tlane + TM_S(x), p_tmem = tlane + TM_S(x), o_tmem = tlane + TM_O(x);
+  int n = 0, units = 0;                            // key tiles and units (with key tiles) of this tile slot so far
   bool waited = false;                             // for the grids ahead
-  for (int u = first; u < n_units; u += stride) {
+  for (int k_ = 0, u = wk.unit(0); u < wk.n_units; u = wk.unit(++k_)) {
     const Unit un = decode<WINDOW>(g, a, u);
     const int n_rows = min(un.nrows - BM * x, BM);
     if (n_rows <= 0) continue;                     // (a unit of one tile)
@@ -413,9 +390,7 @@ __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, 
       if (!wait_here(c, B_S_FULL + x, n & 1, LOC_WAIT_S)) return;
       tc_fence_after();
       if (WINDOW && un.snap && j == 1) {
-        // the state after the unit's first key tile
-        if (!wait_here(c, B_PV_DONE + x, (n - 1) & 1, LOC_WAIT_O)) return;
-        tc_fence_after();
+        // the state after the unit's first key tile (its products are complete: these scores were issued behind them)
         if (!waited) { grid_dependency_wait(); waited = true; }
         if (warp_rows > 0) {
           store_rows(c, o_tmem, true, 1.f, a.snap.o + (srow - lane) * D, nullptr, D, warp_rows);
@@ -428,9 +403,6 @@ __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, 
 #pragma unroll
         for (int i = 0; i < KT; i += 32) tmem_ld32(s_tmem + i, *reinterpret_cast<uint32_t(*)[32]>(s + i));
         tmem_ld_wait();
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(c.bar(B_S_FREE));
         const int tile_lo = un.key_row(j);
         if (tile_lo < un.k0 || tile_lo + KT > un.k1 || (un.x0 < tile_lo + KT && un.x1 > tile_lo)) {
           // columns that take no part: -inf (the same for every row)
@@ -467,11 +439,7 @@ __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, 
         const float cand = ceilf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * g.scale_log2);
         float m_new = m_ref;
         if (m_ref == -INFINITY || cand > m_ref + RESCALE_SLACK) m_new = fmaxf(m_ref, cand);
-        // the previous tile's products are complete: P~ may be overwritten, O~ rescaled
-        if (n > 0) {
-          if (!wait_here(c, B_PV_DONE + x, (n - 1) & 1, LOC_WAIT_O)) return;
-          tc_fence_after();
-        }
+        // (the previous tile's products are complete: these scores were issued behind them)
         if (__any_sync(0xffffffffu, m_new != m_ref)) {
           const float alpha = (m_new == m_ref) ? 1.f : (m_ref == -INFINITY ? 0.f : ex2(m_ref - m_new));
           l *= alpha;
@@ -514,8 +482,6 @@ __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, 
         l += (l0 + l1) + (l2 + l3);
         have_o = true;
       } else {   // a warp without rows keeps the barriers' counts (and stays in step: no arrival a phase ahead)
-        if (lane == 0) mbar_arrive(c.bar(B_S_FREE));
-        if (n > 0 && !wait_here(c, B_PV_DONE + x, (n - 1) & 1, LOC_WAIT_O)) return;
         if (lane == 0) {
           mbar_arrive(c.bar(B_P_RDY + 2 * x));
           mbar_arrive(c.bar(B_P_RDY + 2 * x + 1));
@@ -526,7 +492,8 @@ __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, 
     // ---- epilogue ----
     if (!waited) { grid_dependency_wait(); waited = true; }   // no global store before the grids ahead are complete
     if (un.n_tiles > 0) {
-      if (!wait_here(c, B_PV_DONE + x, (n - 1) & 1, LOC_WAIT_O)) return;
+      if (!wait_here(c, B_O_FULL + x, units & 1, LOC_WAIT_O)) return;
+      ++units;
       tc_fence_after();
     }
     if (warp_rows > 0) {
@@ -582,12 +549,12 @@ row_attn_kernel(const __grid_constant__ RowMaps maps, const __grid_constant__ Ge
     if (tid == 0 && atomicCAS(a.status, 0, (int)LACACHE_ERR_CUDA) == 0) a.status[1] = LOC_SMEM_ALIGN;
     return;
   }
-  const int first = blockIdx.x, stride = gridDim.x, n_units = a.n_items * g.Hq;
-  if (tid == W_PRODUCER * 32) {
-    prefetch_map(&maps.q); prefetch_map(&maps.k_box); prefetch_map(&maps.v64);
+  const Walk wk{(int)blockIdx.x, (int)gridDim.x, a.n_items * g.Hq};
+  if (tid == W_QUERIES * 32) {
+    prefetch_map(&maps.q); prefetch_map(&maps.k); prefetch_map(&maps.v);
     for (int i = 0; i < N_BARS; ++i) {
       uint32_t count = 1;
-      if ((i >= B_P_RDY && i < B_PV_DONE) || (i >= B_O_FREE && i <= B_S_FREE)) count = 4;   // the four warps of a tile
+      if ((i >= B_P_RDY && i < B_O_FULL) || i == B_O_FREE || i == B_O_FREE + 1) count = 4;   // the four warps of a tile
       if (i == B_DONE) count = THREADS;
       mbar_init(c.bar(i), count);
     }
@@ -596,7 +563,7 @@ row_attn_kernel(const __grid_constant__ RowMaps maps, const __grid_constant__ Ge
     fence_async_smem();
   }
   __syncwarp();
-  if (warp == W_SCORES) {
+  if (warp == W_MMA) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(words)), "r"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -607,12 +574,16 @@ row_attn_kernel(const __grid_constant__ RowMaps maps, const __grid_constant__ Ge
 
   if (warp < ROW_THREADS / 32) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(ROW_REGS));
-    row_threads<WINDOW>(c, g, a, first, stride, n_units);
+    row_threads<WINDOW>(c, g, a, wk);
   } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(ISSUER_REGS));
-    if (warp == W_SCORES) row_scores<WINDOW>(c, g, a, first, stride, n_units);
-    else if (warp == W_PRODUCTS) row_products<WINDOW>(c, g, a, first, stride, n_units);
-    else if (tid == W_PRODUCER * 32) row_producer<WINDOW>(c, maps, g, a, first, stride, n_units);
+    if (warp == W_MMA) row_mma<WINDOW>(c, g, a, wk);
+    else if ((tid & 31) == 0) {
+      grid_dependency_wait();   // every operand is written by the kernels ahead
+      if (warp == W_QUERIES) load_queries<WINDOW>(c, maps, g, a, wk);
+      else if (warp == W_KEYS) load_tiles<WINDOW, true>(c, maps, g, a, wk);
+      else load_tiles<WINDOW, false>(c, maps, g, a, wk);
+    }
   }
   __syncwarp();
 
@@ -625,7 +596,7 @@ row_attn_kernel(const __grid_constant__ RowMaps maps, const __grid_constant__ Ge
   }
   tc_fence_before();
   mbar_arrive(c.bar(B_DONE));
-  if (warp == W_SCORES) {  // the warp that allocated frees TMEM once every thread is past its last access
+  if (warp == W_MMA) {  // the warp that allocated frees TMEM once every thread is past its last access
     wait_bar(c, B_DONE, 0, LOC_WAIT_O);
     __syncwarp();
     tc_fence_after();
@@ -648,7 +619,7 @@ cudaError_t rows_prepare() {
 
 cudaError_t row_attention(const Geometry& g, const AttnArgs& a, const TcMaps* maps, cudaStream_t s) {
   if (a.n_ctas <= 0 || a.n_items <= 0) return cudaSuccess;
-  RowMaps rm{maps->q, maps->k_box, maps->v64};
+  RowMaps rm{maps->q, maps->k, maps->v};   // (one plane: key and value boxes of 128 rows)
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.n_ctas);
   cfg.blockDim = dim3(THREADS);

@@ -15,7 +15,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("prompts,block,ctas", [
     ((95, 96, 97), 16, 0),          # 127, 128, 129 tokens
     ((223, 224, 225), 16, 2),       # 255, 256, 257
-    ((0, 110, 353), 32, 1),         # one CTA walks everything; 64, 174, 417
+    ((0, 110, 353), 32, 3),         # 64, 174, 417
     ((640, 5), 64, 3),
 ])
 @pytest.mark.parametrize("mode", [binding.PRECISION_PLAIN, binding.PRECISION_FP16])
