@@ -280,7 +280,7 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
   const int TC_KEYS = tc_keys(c->split);
   const int R = tc ? TC_ROWS : SIMT_ROWS;
   // builds and full recomputes with one-plane operands run the row kernel: items of two row tiles, 128-key tiles
-  const bool rk = tc && !c->split;
+  const bool rk = tc;
   const int RI = rk ? TC_ROW_ITEM : R, RI_KEYS = rk ? TC_ROW_KEYS : TC_KEYS;
   std::vector<WorkItem> items;
   // Block-query units: the keys of each (sequence, head) are cut into balanced
@@ -788,7 +788,7 @@ AttnArgs attn_args(lacache_ctx* c, int mode, lacache_ctx::ListRef list, int blk,
 // one launch of the tcgen05 kernel; with a span ring set, the launch gets the ring's next slot
 cudaError_t launch_tc(lacache_ctx* c, AttnArgs a, const TcMaps* maps, cudaStream_t s) {
   if (c->span_ring) a.span = c->span_ring + 2 * (size_t)(c->span_next++ % (unsigned)c->span_slots);
-  return (a.mode == MODE_STEP || a.split) ? tc_attention(c->g, a, maps, s) : row_attention(c->g, a, maps, s);
+  return a.mode == MODE_STEP ? tc_attention(c->g, a, maps, s) : row_attention(c->g, a, maps, s);
 }
 
 lacache_status run_attention(lacache_ctx* c, const AttnArgs& a, bool scratch, cudaStream_t s) {

@@ -41,26 +41,32 @@ constexpr int W_QUERIES = 8, W_MMA = 9, W_KEYS = 10, W_VALUES = 11;   // the war
 
 struct RowMaps {
   CUtensorMap q;      // box {64, 128 rows, 2 halves, 1 head, planes}: a whole Q' tile
-  CUtensorMap k;      // likewise for keys
+  CUtensorMap k;      // one plane: likewise for keys; split planes: box {64, 128 rows, 1, 1, 1}
   CUtensorMap v;      // box {64, 128 rows, 2 halves, 1}
 };
 
 constexpr uint32_t BOX = 16384;
-constexpr int STAGES = 2;
-constexpr uint32_t Q_TILE = 32768;
-constexpr uint32_t SM_K = 2 * Q_TILE;
-constexpr uint32_t SM_V = SM_K + 2 * STAGES * BOX;
-constexpr uint32_t SM_ST = SM_V + 2 * STAGES * BOX;   // 4 KB of staging per row warp
-constexpr uint32_t SM_BARS = SM_ST + 8 * 4096;
+template <bool SPLIT>
+struct Lay {
+  static constexpr int STAGES = SPLIT ? 1 : 2;                 // key tiles and value tiles in shared memory
+  static constexpr int PIECES = SPLIT ? 4 : 1;                 // loads of a key tile: {features} x {hi, lo} boxes, or all of it
+  static constexpr uint32_t Q_TILE = SPLIT ? 65536 : 32768;    // [plane][64 features][row]
+  static constexpr uint32_t K_TILE = Q_TILE;
+  static constexpr uint32_t SM_K = 2 * Q_TILE;
+  static constexpr uint32_t SM_V = SM_K + STAGES * K_TILE;
+  static constexpr uint32_t SM_ST = SM_V + 2 * STAGES * BOX;   // one plane: 4 KB of staging per row warp
+};
+constexpr uint32_t SM_BARS = 229376;
+static_assert(Lay<false>::SM_ST + 8 * 4096 <= SM_BARS && Lay<true>::SM_ST <= SM_BARS, "shared memory overruns");
 
 enum {
   B_Q_FULL = 0, B_Q_FREE = 2,     // per tile
-  B_K_FULL = 4, B_K_FREE = 6,     // per stage
-  B_V_FULL = 8, B_V_FREE = 10,    // per stage
-  B_S_FULL = 12,                  // per tile
-  B_P_RDY = 14,                   // per tile and half: 2 * tile + half
-  B_O_FULL = 18, B_O_FREE = 20,   // per tile
-  B_DONE = 22, N_BARS = 23
+  B_K_FULL = 4, B_K_FREE = 8,     // per stage, or piece of the one stage
+  B_V_FULL = 12, B_V_FREE = 14,   // per stage
+  B_S_FULL = 16,                  // per tile
+  B_P_RDY = 18,                   // per tile and half: 2 * tile + half
+  B_O_FULL = 22, B_O_FREE = 24,   // per tile
+  B_DONE = 26, N_BARS = 27
 };
 constexpr uint32_t SM_TOTAL = SM_BARS + 8 * N_BARS + 16;
 static_assert(SM_TOTAL <= 232448, "exceeds the 227 KB per-CTA limit");
@@ -141,7 +147,7 @@ __device__ __forceinline__ bool wait_here(const Cta& c, int slot, uint32_t parit
 // ---- producers ----------------------------------------------------------------------------------------------
 // One lane each for Q' tiles, key tiles and value tiles, with blocking waits (one lane that polled all three took several
 // hundred cycles to notice a free stage, which with two stages is time the tensor core waits).
-template <bool WINDOW>
+template <bool SPLIT, bool WINDOW>
 __device__ void load_queries(const Cta& c, const RowMaps& maps, const Geometry& g, const AttnArgs& a, const Walk& wk) {
   int n0 = 0, n1 = 0;   // Q' tiles loaded, per tile slot
   for (int k_ = 0, u = wk.unit(0); u < wk.n_units; u = wk.unit(++k_)) {
@@ -150,24 +156,35 @@ __device__ void load_queries(const Cta& c, const RowMaps& maps, const Geometry& 
     for (int x = 0; x < un.tiles(); ++x) {
       const int n = x ? n1 : n0;
       if (n > 0 && !wait_here(c, B_Q_FREE + x, (n - 1) & 1, LOC_WAIT_Q)) return;
-      mbar_expect_tx(c.bar(B_Q_FULL + x), Q_TILE);
-      tma_load_5d(c.base + x * Q_TILE, &maps.q, c.bar(B_Q_FULL + x), 0, un.row0 + BM * x, 0, un.h, 0);
+      mbar_expect_tx(c.bar(B_Q_FULL + x), Lay<SPLIT>::Q_TILE);
+      tma_load_5d(c.base + x * Lay<SPLIT>::Q_TILE, &maps.q, c.bar(B_Q_FULL + x), 0, un.row0 + BM * x, 0, un.h, 0);
       if (x) ++n1; else ++n0;
     }
   }
 }
-template <bool WINDOW, bool KEYS>
+template <bool SPLIT, bool WINDOW, bool KEYS>
 __device__ void load_tiles(const Cta& c, const RowMaps& maps, const Geometry& g, const AttnArgs& a, const Walk& wk) {
-  constexpr int FULL = KEYS ? B_K_FULL : B_V_FULL, FREE = KEYS ? B_K_FREE : B_V_FREE;
+  using L = Lay<SPLIT>;
   int n = 0;            // tiles so far
   for (int k_ = 0, u = wk.unit(0); u < wk.n_units; u = wk.unit(++k_)) {
     const Unit un = decode<WINDOW>(g, a, u);
     for (int t = 0; t < un.n_tiles; ++t, ++n) {
-      const int st = n % STAGES, use = n / STAGES;
-      if (use > 0 && !wait_here(c, FREE + st, (use - 1) & 1, KEYS ? LOC_WAIT_K : LOC_WAIT_V)) return;
-      mbar_expect_tx(c.bar(FULL + st), 2 * BOX);
-      if (KEYS) tma_load_5d(c.base + SM_K + st * 2 * BOX, &maps.k, c.bar(FULL + st), 0, un.key_row(t), 0, un.kh, 0);
-      else tma_load_4d(c.base + SM_V + st * 2 * BOX, &maps.v, c.bar(FULL + st), 0, un.key_row(t), 0, un.kh);
+      const int st = n % L::STAGES, use = n / L::STAGES, row = un.key_row(t);
+      if (!KEYS) {
+        if (use > 0 && !wait_here(c, B_V_FREE + st, (use - 1) & 1, LOC_WAIT_V)) return;
+        mbar_expect_tx(c.bar(B_V_FULL + st), 2 * BOX);
+        tma_load_4d(c.base + L::SM_V + st * 2 * BOX, &maps.v, c.bar(B_V_FULL + st), 0, row, 0, un.kh);
+      } else if (!SPLIT) {
+        if (use > 0 && !wait_here(c, B_K_FREE + st, (use - 1) & 1, LOC_WAIT_K)) return;
+        mbar_expect_tx(c.bar(B_K_FULL + st), 2 * BOX);
+        tma_load_5d(c.base + L::SM_K + st * L::K_TILE, &maps.k, c.bar(B_K_FULL + st), 0, row, 0, un.kh, 0);
+      } else {
+        for (int b = 0; b < L::PIECES; ++b) {   // refilled box by box, as the scores of the second tile leave them
+          if (use > 0 && !wait_here(c, B_K_FREE + b, (use - 1) & 1, LOC_WAIT_K)) return;
+          mbar_expect_tx(c.bar(B_K_FULL + b), BOX);
+          tma_load_5d(c.base + L::SM_K + b * BOX, &maps.k, c.bar(B_K_FULL + b), 0, row, b >> 1, un.kh, b & 1);
+        }
+      }
     }
   }
 }
@@ -178,25 +195,27 @@ __device__ void load_tiles(const Cta& c, const RowMaps& maps, const Geometry& g,
 // may overwrite the probabilities the products ahead of them read, and a tile's scores being complete says that its
 // products are.  The order also keeps the two tiles half a period apart: while one's products and scores are computed,
 // the other's row threads have the exponential unit.
-template <bool WINDOW>
+template <bool SPLIT, bool WINDOW>
 __device__ void row_mma(const Cta& c, const Geometry& g, const AttnArgs& a, const Walk& wk) {
-  const uint32_t idesc_s = idesc_f16(g.op_f16 ? 0u : 1u, 0u, BM, KT);
+  using L = Lay<SPLIT>;
+  const uint32_t idesc_s = idesc_f16((!SPLIT && g.op_f16) ? 0u : 1u, 0u, BM, KT);
   constexpr uint32_t idesc_o = idesc_f16(0u /*fp16*/, 1u, BM, D);
   const bool leader = elect_one();
   int nq0 = 0, nq1 = 0, no0 = 0, no1 = 0, np0 = 0, np1 = 0;   // per tile slot: units' scores begun, units' products begun, key tiles of products
   int ks = 0, kv = 0;                                   // key tiles of scores (both tiles' of it), of products
   // scores of key tile j of a unit: tile x of nx, n_tiles in all
   auto scores = [&](int x, int nx, int j, int n_tiles) -> bool {
-    const int st = ks % STAGES;
+    const int st = ks % L::STAGES;
+    const uint32_t kph = (uint32_t)(ks / L::STAGES) & 1u;
     if (j == 0) {
       if (!wait_here(c, B_Q_FULL + x, (x ? nq1 : nq0) & 1, LOC_WAIT_Q)) return false;
       if (x) ++nq1; else ++nq0;
     }
-    if (x == 0 && !wait_here(c, B_K_FULL + st, (uint32_t)(ks / STAGES) & 1u, LOC_WAIT_K)) return false;
-    tc_fence_after();
-    {
-      const uint64_t kd = smem_desc(c.base + SM_K + st * 2 * BOX, 16, 1024);
-      const uint64_t qd = smem_desc(c.base + x * Q_TILE, 16, 1024);
+    if (!SPLIT) {
+      if (x == 0 && !wait_here(c, B_K_FULL + st, kph, LOC_WAIT_K)) return false;
+      tc_fence_after();
+      const uint64_t kd = smem_desc(c.base + L::SM_K + st * L::K_TILE, 16, 1024);
+      const uint64_t qd = smem_desc(c.base + x * L::Q_TILE, 16, 1024);
       if (leader) {
 #pragma unroll
         for (int i = 0; i < 8; ++i) {   // 64 features of a row are 128 bytes, the next 64 a box (16 KB) on
@@ -204,6 +223,27 @@ __device__ void row_mma(const Cta& c, const Geometry& g, const AttnArgs& a, cons
           mma_ss(c.tmem + TM_S(x), qd + off, kd + off, idesc_s, i ? 1u : 0u);
         }
         if (x == nx - 1) tc_commit(c.bar(B_K_FREE + st));
+      }
+    } else {
+      tc_fence_after();
+#pragma unroll
+      for (int b = 0; b < L::PIECES; ++b) {   // piece b: features f, plane p of the keys: Q hi . K p, and Q lo . K hi
+        const int f = b >> 1, p = b & 1;
+        if (x == 0) {
+          if (!wait_here(c, B_K_FULL + b, kph, LOC_WAIT_K)) return false;
+          tc_fence_after();
+        }
+        const uint64_t kd = smem_desc(c.base + L::SM_K + b * BOX, 16, 1024);
+        const uint64_t qh = smem_desc(c.base + x * L::Q_TILE + f * BOX, 16, 1024), ql = qh + (2 * BOX >> 4);
+        if (leader) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) mma_ss(c.tmem + TM_S(x), qh + 2u * i, kd + 2u * i, idesc_s, (b > 0 || i > 0) ? 1u : 0u);
+          if (p == 0) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) mma_ss(c.tmem + TM_S(x), ql + 2u * i, kd + 2u * i, idesc_s, 1u);
+          }
+          if (x == nx - 1) tc_commit(c.bar(B_K_FREE + b));
+        }
       }
     }
     if (leader) {
@@ -233,7 +273,7 @@ __device__ void row_mma(const Cta& c, const Geometry& g, const AttnArgs& a, cons
     more = next_unit(k, nxt);
     const int nx2 = more ? nxt.tiles() : 0;
     for (int j = 0; j < un.n_tiles; ++j, ++kv) {
-      const int st = kv % STAGES;
+      const int st = kv % L::STAGES;
       const bool last = j == un.n_tiles - 1;
 #pragma unroll
       for (int x = 0; x < 2; ++x) {
@@ -246,10 +286,10 @@ __device__ void row_mma(const Cta& c, const Geometry& g, const AttnArgs& a, cons
 #pragma unroll
           for (int hf = 0; hf < 2; ++hf) {
             if (!wait_here(c, B_P_RDY + 2 * x + hf, (x ? np1 : np0) & 1, LOC_WAIT_S)) return;
-            if (x == 0 && hf == 0 && !wait_here(c, B_V_FULL + st, (uint32_t)(kv / STAGES) & 1u, LOC_WAIT_V)) return;
+            if (x == 0 && hf == 0 && !wait_here(c, B_V_FULL + st, (uint32_t)(kv / L::STAGES) & 1u, LOC_WAIT_V)) return;
             tc_fence_after();
             // B = V, MN-major: 64 features contiguous, the next 64 features a box on, 16 keys = 2 KB
-            const uint64_t vd = smem_desc(c.base + SM_V + st * 2 * BOX + hf * 8192, BOX, 1024);
+            const uint64_t vd = smem_desc(c.base + L::SM_V + st * 2 * BOX + hf * 8192, BOX, 1024);
             const uint32_t first_acc = (j == 0 && hf == 0 && !(WINDOW && un.init)) ? 0u : 1u;
             if (leader) {
 #pragma unroll
@@ -306,12 +346,13 @@ __device__ __forceinline__ uint64_t span_bits(int lo, int hi) {   // bits [lo, h
 
 // The O~ row of every thread of a warp, scaled by `mul`, to rows of global memory: state rows (fp32, `stride` D) or
 // output rows, through the warp's 4 KB of staging, 32 features at a time, so that a store instruction writes four rows'
-// 128 contiguous bytes (thread per row, it would touch 32 rows).  `rows`: how many of the warp's rows exist.  have_o: TMEM
+// 128 contiguous bytes (thread per row, it would touch 32 rows; split planes leave no room for the staging).  `rows`: how many of the warp's rows exist.  have_o: TMEM
 // holds O~ (else zeros).
+template <bool SPLIT>
 __device__ __forceinline__ void store_rows(const Cta& c, uint32_t o_tmem, bool have_o, float mul, float* dst32,
                                            __nv_bfloat16* dst16, size_t stride, int rows) {
   const int lane = threadIdx.x & 31;
-  uint8_t* const st = c.gen + SM_ST + (threadIdx.x >> 5) * 4096;
+  uint8_t* const st = c.gen + Lay<SPLIT>::SM_ST + (threadIdx.x >> 5) * 4096;
 #pragma unroll 1
   for (int cb = 0; cb < 4; ++cb) {
     uint32_t r[32];
@@ -323,6 +364,27 @@ __device__ __forceinline__ void store_rows(const Cta& c, uint32_t o_tmem, bool h
     } else {
 #pragma unroll
       for (int i = 0; i < 32; ++i) r[i] = 0u;
+    }
+    if (SPLIT) {
+      if (lane < rows) {
+        const size_t off = (size_t)lane * stride + 32 * cb;
+        if (dst16) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            uint32_t p[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) p[e] = pack_bf16x2(__uint_as_float(r[8 * i + 2 * e]), __uint_as_float(r[8 * i + 2 * e + 1]));
+            *reinterpret_cast<uint4*>(dst16 + off + 8 * i) = make_uint4(p[0], p[1], p[2], p[3]);
+          }
+        } else if (stride == D) {   // state rows: 32-byte aligned
+#pragma unroll
+          for (int i = 0; i < 4; ++i) st_global_v8(dst32 + off + 8 * i, r + 8 * i);
+        } else {
+#pragma unroll
+          for (int i = 0; i < 8; ++i) *reinterpret_cast<uint4*>(dst32 + off + 4 * i) = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+        }
+      }
+      continue;
     }
 #pragma unroll
     for (int i = 0; i < 8; ++i)
@@ -342,7 +404,7 @@ __device__ __forceinline__ void store_rows(const Cta& c, uint32_t o_tmem, bool h
   }
 }
 
-template <bool WINDOW>
+template <bool SPLIT, bool WINDOW>
 __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, const Walk& wk) {
   const float LN2 = 0.69314718055994530942f;
   const int lane = threadIdx.x & 31;
@@ -393,7 +455,7 @@ __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, 
         // the state after the unit's first key tile (its products are complete: these scores were issued behind them)
         if (!waited) { grid_dependency_wait(); waited = true; }
         if (warp_rows > 0) {
-          store_rows(c, o_tmem, true, 1.f, a.snap.o + (srow - lane) * D, nullptr, D, warp_rows);
+          store_rows<SPLIT>(c, o_tmem, true, 1.f, a.snap.o + (srow - lane) * D, nullptr, D, warp_rows);
           if (valid) { a.snap.m[srow] = m_ref; a.snap.l[srow] = l; }
         }
       }
@@ -501,7 +563,7 @@ __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, 
         const size_t orow = (size_t)row * g.Hq + un.h, wrow = (size_t)(row - lane) * g.Hq + un.h;
         float* d32 = a.out_bf16 ? nullptr : a.out + wrow * D;
         __nv_bfloat16* d16 = a.out_bf16 ? reinterpret_cast<__nv_bfloat16*>(a.out) + wrow * D : nullptr;
-        store_rows(c, o_tmem, have_o, 1.f / l, d32, d16, (size_t)g.Hq * D, warp_rows);
+        store_rows<SPLIT>(c, o_tmem, have_o, 1.f / l, d32, d16, (size_t)g.Hq * D, warp_rows);
         if (valid && a.lse) a.lse[orow] = (m_ref + log2f(l)) * LN2;
       } else if (WINDOW && un.init && un.n_tiles == 0) {
         // no keys: the state the unit starts from
@@ -515,10 +577,10 @@ __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, 
           a.st.l[srow] = l;
         }
       } else {
-        store_rows(c, o_tmem, have_o, 1.f, a.st.o + (srow - lane) * D, nullptr, D, warp_rows);
+        store_rows<SPLIT>(c, o_tmem, have_o, 1.f, a.st.o + (srow - lane) * D, nullptr, D, warp_rows);
         if (valid) { a.st.m[srow] = m_ref; a.st.l[srow] = l; }
         if (WINDOW && un.snap && un.n_tiles == 1) {   // a single key tile: the state after it is the final one as well
-          store_rows(c, o_tmem, have_o, 1.f, a.snap.o + (srow - lane) * D, nullptr, D, warp_rows);
+          store_rows<SPLIT>(c, o_tmem, have_o, 1.f, a.snap.o + (srow - lane) * D, nullptr, D, warp_rows);
           if (valid) { a.snap.m[srow] = m_ref; a.snap.l[srow] = l; }
         }
       }
@@ -531,7 +593,7 @@ __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, 
   }
 }
 
-template <bool WINDOW>
+template <bool SPLIT, bool WINDOW>
 __global__ void __launch_bounds__(THREADS, 1)
 row_attn_kernel(const __grid_constant__ RowMaps maps, const __grid_constant__ Geometry g, const __grid_constant__ AttnArgs a) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -574,15 +636,15 @@ row_attn_kernel(const __grid_constant__ RowMaps maps, const __grid_constant__ Ge
 
   if (warp < ROW_THREADS / 32) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(ROW_REGS));
-    row_threads<WINDOW>(c, g, a, wk);
+    row_threads<SPLIT, WINDOW>(c, g, a, wk);
   } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(ISSUER_REGS));
-    if (warp == W_MMA) row_mma<WINDOW>(c, g, a, wk);
+    if (warp == W_MMA) row_mma<SPLIT, WINDOW>(c, g, a, wk);
     else if ((tid & 31) == 0) {
       grid_dependency_wait();   // every operand is written by the kernels ahead
-      if (warp == W_QUERIES) load_queries<WINDOW>(c, maps, g, a, wk);
-      else if (warp == W_KEYS) load_tiles<WINDOW, true>(c, maps, g, a, wk);
-      else load_tiles<WINDOW, false>(c, maps, g, a, wk);
+      if (warp == W_QUERIES) load_queries<SPLIT, WINDOW>(c, maps, g, a, wk);
+      else if (warp == W_KEYS) load_tiles<SPLIT, WINDOW, true>(c, maps, g, a, wk);
+      else load_tiles<SPLIT, WINDOW, false>(c, maps, g, a, wk);
     }
   }
   __syncwarp();
@@ -605,13 +667,16 @@ row_attn_kernel(const __grid_constant__ RowMaps maps, const __grid_constant__ Ge
   }
 }
 
-const void* row_kernel(bool window) { return window ? (const void*)row_attn_kernel<true> : (const void*)row_attn_kernel<false>; }
+const void* row_kernel(bool split, bool window) {
+  if (split) return window ? (const void*)row_attn_kernel<true, true> : (const void*)row_attn_kernel<true, false>;
+  return window ? (const void*)row_attn_kernel<false, true> : (const void*)row_attn_kernel<false, false>;
+}
 
 }  // namespace
 
 cudaError_t rows_prepare() {
-  for (int i = 0; i < 2; ++i) {
-    cudaError_t e = cudaFuncSetAttribute(row_kernel(i != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
+  for (int i = 0; i < 4; ++i) {
+    cudaError_t e = cudaFuncSetAttribute(row_kernel(i & 1, i & 2), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -619,7 +684,7 @@ cudaError_t rows_prepare() {
 
 cudaError_t row_attention(const Geometry& g, const AttnArgs& a, const TcMaps* maps, cudaStream_t s) {
   if (a.n_ctas <= 0 || a.n_items <= 0) return cudaSuccess;
-  RowMaps rm{maps->q, maps->k, maps->v};   // (one plane: key and value boxes of 128 rows)
+  RowMaps rm{maps->q, a.split ? maps->k_box : maps->k_rows, maps->v_rows};
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.n_ctas);
   cfg.blockDim = dim3(THREADS);
@@ -631,7 +696,7 @@ cudaError_t row_attention(const Geometry& g, const AttnArgs& a, const TcMaps* ma
   cfg.attrs = attr;
   cfg.numAttrs = a.no_pdl ? 0 : 1;
   void* params[3] = {&rm, const_cast<Geometry*>(&g), const_cast<AttnArgs*>(&a)};
-  return cudaLaunchKernelExC(&cfg, row_kernel(a.window), params);
+  return cudaLaunchKernelExC(&cfg, row_kernel(a.split, a.window), params);
 }
 
 }  // namespace lacache

@@ -274,16 +274,19 @@ __device__ __forceinline__ void issue_s_mma(uint32_t q_base, uint32_t q_box, uin
   const uint64_t kd[2] = {smem_desc(k_hi, 16, 1024), smem_desc(k_lo, 16, 1024)};
   const uint32_t qb16 = q_box >> 4, kb16 = k_box >> 4;
   uint32_t acc = 0;
+  // per half of the features: hi.hi [, lo.hi, hi.lo] -- the order of the row kernel (lacache_rows.cu): the scores of
+  // a query and a key are the same bits wherever they are computed
 #pragma unroll
-  for (int term = 0; term < (SPLIT ? 3 : 1); ++term) {   // hi.hi [+ hi.lo + lo.hi]
-    const uint64_t qa = qd[term == 2 ? 1 : 0];
-    const uint64_t ka = kd[term == 1 ? 1 : 0];
+  for (int f = 0; f < 2; ++f) {
 #pragma unroll
-    for (int ks = 0; ks < D / 16; ++ks) {
-      const uint32_t qoff = (ks >> 2) * qb16 + (ks & 3) * 2;
-      const uint32_t koff = (ks >> 2) * kb16 + (ks & 3) * 2;
-      mma_ss(s_tmem, qa + qoff, ka + koff, idesc, acc);
-      acc = 1;
+    for (int term = 0; term < (SPLIT ? 3 : 1); ++term) {
+      const uint64_t qa = qd[term == 1 ? 1 : 0] + f * qb16;
+      const uint64_t ka = kd[term == 2 ? 1 : 0] + f * kb16;
+#pragma unroll
+      for (int ks = 0; ks < 4; ++ks) {
+        mma_ss(s_tmem, qa + 2 * ks, ka + 2 * ks, idesc, acc);
+        acc = 1;
+      }
     }
   }
 }
@@ -2048,7 +2051,9 @@ TcMaps* tc_make_maps(const Geometry& g, const RotBuffers& rot, float* state_o, b
             make_qk_map(&m->k, rot.k_hi, g.Hkv, g.Tp, bn, planes, err, errlen) &&
             make_qk_map(&m->k64, rot.k_hi, g.Hkv, g.Tp, 64, planes, err, errlen) &&
             make_qk_map(&m->k32, rot.k_hi, g.Hkv, g.Tp, 32, planes, err, errlen) &&
+            make_qk_map(&m->k_rows, rot.k_hi, g.Hkv, g.Tp, TC_ROW_KEYS, planes, err, errlen) &&
             make_qk_map(&m->k_box, rot.k_hi, g.Hkv, g.Tp, TC_ROW_KEYS, planes, err, errlen, true) &&
+            make_v_map(&m->v_rows, rot.v, g.Hkv, g.Tp, TC_ROW_KEYS, err, errlen) &&
             make_v_map(&m->v, rot.v, g.Hkv, g.Tp, bn, err, errlen) &&
             make_v_map(&m->v64, rot.v, g.Hkv, g.Tp, 64, err, errlen) &&
             make_v_map(&m->v32, rot.v, g.Hkv, g.Tp, 32, err, errlen) &&

@@ -26,7 +26,8 @@ struct TcMaps {
   alignas(64) CUtensorMap v;
   alignas(64) CUtensorMap v64;
   alignas(64) CUtensorMap v32;
-  alignas(64) CUtensorMap k_box;   // one plane, one feature half, 128 rows (row kernel)
+  // row kernel: boxes of 128 keys, whole or (k_box) one plane and one feature half
+  alignas(64) CUtensorMap k_rows, v_rows, k_box;
   alignas(64) CUtensorMap st_o;    // cached O~ [Hq][Tp][128] fp32, box 32 cols x 128 rows
   alignas(64) CUtensorMap out;     // caller's out [T][Hq][128] fp32, box 32 cols x 1 head x 128 rows
   alignas(64) CUtensorMap out_sub[4];  // the same with boxes of 64, 32, 16 and 8 rows (clipped row tiles)
