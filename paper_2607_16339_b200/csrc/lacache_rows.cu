@@ -1,7 +1,6 @@
-// tcgen05 attention of fixed row tiles over long key ranges (bf16 inputs, head_dim 128, one plane per rotated operand):
-// the cache build, the full recompute and the builds over key windows.  (The block queries of a step and the merge of
-// fixed rows with the block's keys are lacache_tc.cu, and so are these builds with split planes, whose operands leave
-// shared memory for one stage of keys only: 90 us against its 84 at 1536 tokens x 32 heads.)
+// tcgen05 attention of fixed row tiles over long key ranges (bf16 inputs, head_dim 128): the cache build, the full
+// recompute and the builds over key windows.  (The block queries of a step and the merge of fixed rows with the block's
+// keys are lacache_tc.cu.)
 //
 // One persistent CTA per SM.  A unit is up to 256 query rows of one head, as two 128-row tiles A and B that share
 // every key / value tile.  What bounds a single tile is the chain scores -> softmax -> P~V of one key tile after the
@@ -17,7 +16,14 @@
 // exponentials of the first half are therefore formed with the reference exponent as it stands, beside the row's maximum,
 // and again only when the maximum asks for another one; the sums of the rounded probabilities come after the hand-over.
 //
-// Shared memory: two Q' tiles, two stages of keys (two 16 KB boxes of 64 features) and of values (two boxes of 64 keys).
+// Shared memory: two Q' tiles, two stages of keys and of values.  Split planes (S = hi.hi + lo.hi + hi.lo) take 128 KB for
+// Q' and leave one stage: a key tile's four boxes {features} x {hi, lo} are freed and refilled one by one behind the second
+// tile's products, and what the tensor core waits for a refill is a fifth of its time.
+//
+// Measured (the build launch; one row tile per CTA, two threads per row, as it was before / now): 28/4 heads x 5120 rows
+// and keys, one fp16 plane: 411 / 302 us (1.24 PFLOP/s); eight ragged requests of 512 to 1188 tokens x 32 heads: 159 / 119;
+// 1536 tokens x 32 heads, split planes: 84 / 76.  Bound by the row threads and by the chain probabilities -> products ->
+// scores about equally: without the exponentials 278 us, with a quarter of the products 267, with neither 170.
 //
 // Arithmetic as in lacache_tc.cu: integer reference exponent, moved only when the row's maximum outgrows it by more
 // than RESCALE_SLACK; P~ rounded to fp16, the normaliser sums the rounded values.

@@ -1,4 +1,5 @@
-// tcgen05 attention kernel for sm_100a (bf16 inputs, head_dim 128).
+// tcgen05 attention kernel of a denoising step for sm_100a (bf16 inputs, head_dim 128).  (Builds and full recomputes:
+// lacache_rows.cu.)
 //
 // One persistent CTA per SM, warp-specialised:
 //   warp 0 (one lane)  producer: TMA loads of Q, K, V tiles into shared memory
@@ -17,12 +18,11 @@
 //                  shared memory.  The normaliser sums the rounded P~.
 //
 // Two roles, chosen per CTA:
-//   stream role  a tile of 128 (or 64) query rows streams key tiles of 128
-//                keys; O~ accumulates in TMEM and is rescaled in place only
-//                when a row maximum outgrows the reference exponent; used for the cache build
-//                (rows in U x keys in U -> cached state), the full recompute,
-//                and the block queries of a step (one chunk of key tiles per
-//                work unit; the last chunk to finish merges the partials).
+//   stream role  the block queries: a tile of 128 (or 64) query rows streams key
+//                tiles of 128 keys; O~ accumulates in TMEM and is rescaled in
+//                place only when a row maximum outgrows the reference exponent
+//                (one chunk of key tiles per work unit; the last chunk to finish
+//                merges the partials).
 //   merge role   the reuse pass for fixed queries: per tile of 128 rows, the
 //                scores against the block's keys, then
 //                out = (alpha O~_cache + P~ V) / (alpha l_cache + sum P~).
@@ -128,7 +128,7 @@ enum {
   BAR_RX = BAR_IO_FULL,  // stream role of a paired step (it has no staging-tile barriers): the partner's partial state has arrived
 };
 
-enum { EPI_STATE = 0, EPI_OUT = 1, EPI_PARTIAL = 2, EPI_SEND = 3 };   // SEND: the partial state goes to the partner CTA
+enum { EPI_OUT = 1, EPI_PARTIAL = 2, EPI_SEND = 3 };   // SEND: the partial state goes to the partner CTA
 
 // both planes and both feature halves of `rows` rows of head h, starting at row `row`
 __device__ __forceinline__ void load_qk_box(uint32_t dst, const CUtensorMap* map, uint32_t bar, int row, int h) {
@@ -138,15 +138,11 @@ __device__ __forceinline__ void load_v_box(uint32_t dst, const CUtensorMap* map,
   tma_load_4d(dst, map, bar, 0, row, 0, h);
 }
 // One unit of work of the stream role, decoded identically by every warp role.
-// What the stream role's templates are instantiated for: a build or a full recompute; a step; a build
-// over key windows (units may start from a stored state and store a snapshot: the incremental rebuild).
-// Separate kernels, so that the plain build and the step carry none of the window code.
 // KIND_STEP2: a step whose block-row units all have exactly two key chunks, run by the two CTAs of a
 // thread-block cluster: the CTA with the second chunk hands its partial state to its partner through
 // distributed shared memory, and the partner writes the merged rows (one round of units, unpacked heads,
 // one-plane operands: the receiving buffer needs 32 KB that the split planes' tiles leave no room for).
-enum StreamKind : int { KIND_BUILD = 0, KIND_STEP = 1, KIND_WINDOW = 2, KIND_STEP2 = 3 };
-__host__ __device__ constexpr bool kind_is_step(int k) { return k == KIND_STEP || k == KIND_STEP2; }
+enum StreamKind : int { KIND_STEP = 1, KIND_STEP2 = 3 };
 
 struct Unit {
   int row0, nrows, h, kh, seq;
@@ -155,15 +151,11 @@ struct Unit {
   int epi, chunk, nchunks;
   int q_rows;             // rows of the Q box: 128 or 64
   int nh, rh;             // packed block queries: nh heads h, h + 1, ... of one KV group, rh lanes each (rh = 0: one head)
-  int init;               // build over a key window: the unit starts from the rows' state in a.init instead of an empty one
-  int snap;               // ... and stores the state it has after its first key tile to a.snap
-  int base1;              // >= 0: key tiles after the first are counted from this token instead of key_base + BN
 };
 // first key (token index) of key tile t of a unit
-template <int KIND, bool SPLIT>
+template <bool SPLIT>
 __device__ __forceinline__ int tile_key_row(const Unit& un, int t) {
   constexpr int BN = Tile<SPLIT>::BN;
-  if (KIND == KIND_WINDOW && un.base1 >= 0 && t > 0) return un.base1 + (t - 1) * BN;
   return un.key_base + t * BN;
 }
 // head and row within the head's rows of tile row r; whether r holds a real query row (rh is 0, 32 or 64)
@@ -188,9 +180,6 @@ template <bool PACKED, int KIND, bool SPLIT>
 __device__ __forceinline__ Unit decode_stream(const Geometry& g, const AttnArgs& a, const WorkItem& it, int u) {
   using TL = Tile<SPLIT>;
   constexpr int BN = TL::BN;
-  constexpr bool STEP = kind_is_step(KIND);
-  constexpr bool WINDOW = KIND == KIND_WINDOW;
-  (void)WINDOW;
   Unit un;
   // units are head-minor: unit u = item u / slots of head (or head group) u % slots (a CTA's units, a
   // fixed stride apart, then cycle through the items instead of drawing one item's heads)
@@ -220,45 +209,15 @@ __device__ __forceinline__ Unit decode_stream(const Geometry& g, const AttnArgs&
   un.chunk = 0;
   un.nchunks = 1;
   un.q_rows = BM;
-  un.init = un.snap = 0;
-  un.base1 = -1;
-  if (WINDOW) {
-    // keys [kt0, kt1) of the sequence (token indices), optionally without the block's; tiles are
-    // counted from token `pad`, which may lie before the window (and before token 0: those key rows
-    // load as zeros and are masked like every key outside the window)
-    un.key_base = it.pad;
-    un.k0 = it.kt0;
-    un.k1 = it.kt1;
-    un.t1 = it.kt1 > it.pad ? (it.kt1 - it.pad + BN - 1) / BN : 0;
-    if (it.chunk & 4) {
-      un.x0 = it.blk_start;
-      un.x1 = it.blk_start + g.block_len;
-    }
-    if (it.chunk & 8) {
-      // the first tile ends where the block starts; the others start right after the block
-      un.base1 = it.blk_start + g.block_len;
-      un.t1 = 1 + (it.kt1 > un.base1 ? (it.kt1 - un.base1 + BN - 1) / BN : 0);
-    }
-    un.epi = (it.chunk & 16) ? EPI_OUT : EPI_STATE;   // bit 4: normalised rows to out / lse instead of a state
-    un.init = it.chunk & 1;
-    un.snap = (it.chunk >> 1) & 1;
-  } else if (!STEP && a.mode == MODE_BUILD) {
-    un.x0 = it.blk_start;
-    un.x1 = it.blk_start + g.block_len;
-    un.epi = EPI_STATE;
-  } else if (STEP) {
-    un.t0 = it.kt0;
-    un.t1 = it.kt1;
-    un.chunk = it.chunk;
-    un.nchunks = it.pad;
-    // (block rows whose result is a state, not normalised rows, always leave partial states: a launch of
-    // its own merges them)
-    un.epi = (it.pad > 1 || a.blk_to_state) ? EPI_PARTIAL : EPI_OUT;
-    if (KIND == KIND_STEP2) un.epi = it.chunk == 0 ? EPI_OUT : EPI_SEND;   // (every unit has two chunks)
-    un.q_rows = un.rh ? BM : 64;
-  } else {
-    un.epi = EPI_OUT;
-  }
+  un.t0 = it.kt0;
+  un.t1 = it.kt1;
+  un.chunk = it.chunk;
+  un.nchunks = it.pad;
+  // (block rows whose result is a state, not normalised rows, always leave partial states: a launch of
+  // its own merges them)
+  un.epi = (it.pad > 1 || a.blk_to_state) ? EPI_PARTIAL : EPI_OUT;
+  if (KIND == KIND_STEP2) un.epi = it.chunk == 0 ? EPI_OUT : EPI_SEND;   // (every unit has two chunks)
+  un.q_rows = un.rh ? BM : 64;
   return un;
 }
 
@@ -331,9 +290,6 @@ struct TileCursor {
 };
 template <bool PACKED, int KIND, bool SPLIT>
 __device__ __forceinline__ void cursor_load_unit(const Geometry& g, const AttnArgs& a, TileCursor& cu, int n_units) {
-  constexpr bool STEP = kind_is_step(KIND);
-  constexpr bool WINDOW = KIND == KIND_WINDOW;
-  (void)WINDOW;
   cu.valid = cu.u < n_units;
   if (!cu.valid) return;
   cu.it = load_item(a.items + unit_item<PACKED, KIND>(g, a, cu.u));
@@ -344,9 +300,6 @@ __device__ __forceinline__ void cursor_load_unit(const Geometry& g, const AttnAr
 template <bool PACKED, int KIND, bool SPLIT>
 __device__ __forceinline__ void cursor_advance(const Geometry& g, const AttnArgs& a, TileCursor& cu, int stride,
                                                int n_units) {
-  constexpr bool STEP = kind_is_step(KIND);
-  constexpr bool WINDOW = KIND == KIND_WINDOW;
-  (void)WINDOW;
   // move to the next tile; cross into the next unit(s) when this one is exhausted
   if (cu.t < cu.un.t1) {
     ++cu.t;
@@ -365,9 +318,6 @@ __device__ void stream_producer(const Cta& c, const TcMaps& maps, const Geometry
   using TL = Tile<SPLIT>;
   constexpr int BN = TL::BN;
   constexpr uint32_t KS_BOX = TL::KS_BOX, K_STAGE = TL::K_STAGE, SM_V = TL::SM_V, V_STAGE = TL::V_STAGE;
-  constexpr bool STEP = kind_is_step(KIND);
-  constexpr bool WINDOW = KIND == KIND_WINDOW;
-  (void)WINDOW;
   // three independent cursors: Q tiles (one per unit), key tiles, value tiles
   TileCursor cq, ck, cv;
   cq.u = first; cq.uu = 0; cq.jj = 0; cq.loads_q = true;
@@ -383,9 +333,8 @@ __device__ void stream_producer(const Cta& c, const TcMaps& maps, const Geometry
   // that overlap the block -- so tiles of fixed tokens are requested at once and
   // the wait comes only when nothing else can be issued.
   bool dep_done = false;
-  const bool q_computed = STEP && a.q_raw != nullptr;
+  const bool q_computed = a.q_raw != nullptr;
   auto tile_depends = [&](const TileCursor& cu) {
-    if (!STEP) return true;
     const int krow = cu.un.key_base + cu.t * BN;
     return krow < cu.it.blk_start + g.block_len && krow + BN > cu.it.blk_start;
   };
@@ -408,9 +357,6 @@ __device__ void stream_producer(const Cta& c, const TcMaps& maps, const Geometry
         cq.q_done = true;
         cq.t = cq.un.t1;
         cursor_advance<PACKED, KIND, SPLIT>(g, a, cq, stride, n_units);
-        // a build's Q tiles come from HBM once the batch outgrows L2: the next unit's tile is asked
-        // into L2 a whole unit ahead of its load
-        if (!STEP && cq.valid) tma_prefetch_5d(&maps.q, 0, cq.un.row0, 0, cq.un.h, 0);
         did = true;
       }
     }
@@ -419,7 +365,7 @@ __device__ void stream_producer(const Cta& c, const TcMaps& maps, const Geometry
       if (!dep_done && tile_depends(ck)) {
         blocked_on_dep = true;
       } else if (kuse == 0 || mbar_test(c.bar(sk ? BAR_K_FREE1 : BAR_K_FREE), (kuse - 1) & 1)) {
-        const int krow = tile_key_row<KIND, SPLIT>(ck.un, ck.t);
+        const int krow = tile_key_row<SPLIT>(ck.un, ck.t);
         const uint32_t bar = c.bar(sk ? BAR_K_FULL1 : BAR_K_FULL);
         const uint32_t khi = c.base + SM_K + sk * K_STAGE;
         mbar_expect_tx(bar, K_STAGE);
@@ -433,7 +379,7 @@ __device__ void stream_producer(const Cta& c, const TcMaps& maps, const Geometry
       if (!dep_done && tile_depends(cv)) {
         blocked_on_dep = true;
       } else if (vuse == 0 || mbar_test(c.bar(sv ? BAR_V_FREE1 : BAR_V_FREE), (vuse - 1) & 1)) {
-        const int krow = tile_key_row<KIND, SPLIT>(cv.un, cv.t);
+        const int krow = tile_key_row<SPLIT>(cv.un, cv.t);
         const uint32_t bar = c.bar(sv ? BAR_V_FULL1 : BAR_V_FULL), vb = c.base + SM_V + sv * V_STAGE;
         mbar_expect_tx(bar, 2 * KS_BOX);
         load_v_box(vb, &maps.v, bar, krow, cv.un.kh);
@@ -476,9 +422,6 @@ __device__ void stream_mma_scores(const Cta& c, const Geometry& g, const AttnArg
   using TL = Tile<SPLIT>;
   constexpr int BN = TL::BN;
   constexpr uint32_t KS_BOX = TL::KS_BOX, K_STAGE = TL::K_STAGE, SK_LO = TL::SK_LO;
-  constexpr bool STEP = kind_is_step(KIND);
-  constexpr bool WINDOW = KIND == KIND_WINDOW;
-  (void)WINDOW;
   // (operand format of the score product: bf16 planes, or fp16 in the one-plane fp16 mode)
   const uint32_t IDESC_S = idesc_f16((!SPLIT && g.op_f16) ? 0u : 1u, 0u, BM, BN);
   int uu = 0;
@@ -490,7 +433,7 @@ __device__ void stream_mma_scores(const Cta& c, const Geometry& g, const AttnArg
     const uint32_t q_box = (uint32_t)un.q_rows * 128u;
     const int n_tiles = un.t1 - un.t0;
     if (!wait_bar(c, BAR_Q_FULL, uu & 1, LOC_WAIT_Q)) return;
-    if (uu == 0 && STEP && a.q_raw != nullptr && !wait_bar(c, BAR_QC, 0, LOC_WAIT_Q)) return;
+    if (uu == 0 && a.q_raw != nullptr && !wait_bar(c, BAR_QC, 0, LOC_WAIT_Q)) return;
     for (int j = 0; j < n_tiles; ++j, ++js) {
       const uint32_t sk = js & 1u, b = js & 1u;
       // the score buffer was last used two tiles ago (possibly by the previous unit): its
@@ -514,9 +457,6 @@ __device__ void stream_mma_pv(const Cta& c, const Geometry& g, const AttnArgs& a
   using TL = Tile<SPLIT>;
   constexpr int BN = TL::BN;
   constexpr uint32_t KS_BOX = TL::KS_BOX, SM_V = TL::SM_V, V_STAGE = TL::V_STAGE;
-  constexpr bool STEP = kind_is_step(KIND);
-  constexpr bool WINDOW = KIND == KIND_WINDOW;
-  (void)WINDOW;
   int uu = 0;
   uint32_t jp = 0;  // P~V tiles issued so far
   for (int u = first; u < n_units; u += stride, ++uu) {
@@ -534,7 +474,7 @@ __device__ void stream_mma_pv(const Cta& c, const Geometry& g, const AttnArgs& a
       if (!wait_bar(c, sv ? BAR_V_FULL1 : BAR_V_FULL, ph, LOC_WAIT_V)) return;
       tc_fence_after();
       issue_pv_mma(c.base + SM_V + sv * V_STAGE, KS_BOX, c.tmem + TS_P + 64 * b, c.tmem + TS_O, BN / 16,
-                   (j == 0 && !(WINDOW && un.init)) ? 0u : 1u);
+                   j == 0 ? 0u : 1u);
       tc_commit(c.bar(BAR_O_FULL));
       tc_commit(c.bar(sv ? BAR_V_FREE1 : BAR_V_FREE));
     }
@@ -550,21 +490,9 @@ __device__ __forceinline__ bool epi_sync(const Cta& c, uint32_t& phase) {
   return ok;
 }
 
-// Cooperative, fully coalesced copy of the first nrows staging rows (512 B each,
-// chunks XOR-swizzled by the row) to rows of `stride` floats in global memory:
+// Cooperative, fully coalesced copy of the first nrows staging rows (512 B each, chunks XOR-swizzled by the row) to rows
+// of `out` (element offset `off0` of the first row, `stride` elements between rows), in the output's element type:
 // every warp-wide store writes one whole row.
-__device__ __forceinline__ void coop_store_rows(const Cta& c, uint32_t stage_off, float* gbase, size_t stride,
-                                                int nrows) {
-  const int t = threadIdx.x - 64;
-  for (int i = t; i < nrows * 32; i += ROW_THREADS) {
-    const int rr = i >> 5, ch = i & 31;
-    float4 v = *reinterpret_cast<const float4*>(c.gen + stage_off + rr * STAGE_ROW + ((ch ^ (rr & 7)) << 4));
-    *reinterpret_cast<float4*>(gbase + (size_t)rr * stride + ch * 4) = v;
-  }
-}
-
-// The same for rows of `out` (element offset `off0` of the first row, `stride` elements between rows), in
-// the output's element type.
 __device__ __forceinline__ void coop_store_out_rows(const Cta& c, const AttnArgs& a, uint32_t stage_off, size_t off0,
                                                     size_t stride, int nrows) {
   const int t = threadIdx.x - 64;
@@ -687,9 +615,6 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
   using TL = Tile<SPLIT>;
   constexpr int BN = TL::BN;
   constexpr int HC = TL::HC;
-  constexpr bool STEP = kind_is_step(KIND);
-  constexpr bool WINDOW = KIND == KIND_WINDOW;
-  (void)WINDOW;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int quad = warp & 3;
   const int half = (warp - 2) >> 2;         // 0: first 64 columns / features, 1: the rest
@@ -706,7 +631,7 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
     if (u + stride < n_units) nxt = load_item(a.items + unit_item<PACKED, KIND>(g, a, u + stride));
     const Unit un = decode_stream<PACKED, KIND, SPLIT>(g, a, it, u);
     it = nxt;
-    if (u == first && STEP && a.q_raw != nullptr) {
+    if (u == first && a.q_raw != nullptr) {
       // The CTA's first unit: rotate the block's queries of this (sequence, head) here,
       // with the very arithmetic of the RoPE kernel, and write them where the TMA load
       // would have put them ([plane][feature half][row][64], 16-byte chunks XOR-swizzled
@@ -753,54 +678,6 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
     const bool active = unit_row_valid(un, quad * 32);  // this warp holds at least one real row (its first)
     float m_ref = -INFINITY, l_part = 0.f;
     bool first_tile = true;
-    bool calm = false;     // the unit's latest tile moved no reference exponent of this warp
-    bool have_o = false;   // O~ in TMEM holds something before the unit's first P~V
-    if (WINDOW && un.t1 <= un.t0) {
-      // A unit without key tiles gives these threads nothing to wait for, and the other roles' parity
-      // waits hold only while nobody runs more than one phase ahead: stay in step with the producer (the
-      // unit's Q load lands only after the previous unit has been released by these threads).
-      if (!wait_bar(c, BAR_Q_FULL, uu & 1, LOC_WAIT_Q)) return;
-    }
-    if (WINDOW && un.init) {
-      // (the state may have been written by the launch just before this one)
-      grid_dependency_wait();
-      // The unit continues from a stored state (m, l, O~) of its rows: the reference exponent and the
-      // normaliser go to registers (the normaliser to the first thread of the pair), O~ to the
-      // accumulator columns this thread owns.  Nobody else reads or writes those cells between units
-      // (the previous unit's P~V products are complete, and its epilogue read them from this thread).
-      // The TMEM stores are warp-wide: rows past the end of a clipped tile store zeros.
-      const size_t srow = (size_t)un.h * g.Tp + row;
-      if (row_valid) {
-        m_ref = a.init.m[srow];
-        if (half == 0) l_part = a.init.l[srow];
-      }
-      const float4* src = reinterpret_cast<const float4*>(a.init.o + srow * D + 64 * half);
-      {
-        // all sixteen loads of the row half are in flight together (one round trip, not four)
-        // (32-byte loads: a warp's load touches 32 rows whatever its width, so wider loads mean
-        // fewer passes through the L1 tags; plain loads, not the read-only path: the launch may update
-        // these rows in place)
-        uint32_t rr[64];
-#pragma unroll
-        for (int i = 0; i < 64; ++i) rr[i] = 0u;
-        if (row_valid) {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) ld_global_v8(src + 2 * i, rr + 8 * i);
-        }
-        tmem_st32(tlane + TS_O + 64 * half, *reinterpret_cast<uint32_t(*)[32]>(rr));
-        tmem_st32(tlane + TS_O + 64 * half + 32, *reinterpret_cast<uint32_t(*)[32]>(rr + 32));
-      }
-      tmem_st_wait();
-      have_o = true;
-      if (u + stride < n_units && (it.chunk & 1) && r < it.nrows) {
-        // the next unit's rows of that state, asked into L2 now (`it` already holds its item)
-        const char* nx = reinterpret_cast<const char*>(
-            a.init.o + ((size_t)((u + stride) % g.Hq) * g.Tp + it.row0 + r) * D + 64 * half);
-        prefetch_l2(nx);
-        prefetch_l2(nx + 128);
-      }
-    }
-
     for (int t = un.t0; t < un.t1; ++t, ++jj) {
       const int b = jj & 1;
       if (!wait_bar(c, BAR_S_FULL + b, (jj >> 1) & 1, LOC_WAIT_S)) return;
@@ -810,32 +687,7 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
       // previous tile, either before an in-place rescale or at the end of the tile
       bool o_waited = first_tile;
       if (active) {
-        if (WINDOW && un.snap && t == un.t0 + 1) {
-          // The state after the unit's first key tile goes to a.snap before this tile changes it:
-          // P~V of that tile must be complete; the pair adds up its normaliser halves.
-          if (!wait_bar(c, BAR_O_FULL, (jj - 1) & 1, LOC_WAIT_O)) return;
-          o_waited = true;
-          tc_fence_after();
-          volatile float* lxs = xch + 2 * (xslot & 1u);
-          ++xslot;
-          lxs[half] = l_part;
-          mbar_arrive(c.bar(BAR_PAIR + quad));
-          if (!wait_bar(c, BAR_PAIR + quad, pair_phase & 1, LOC_WAIT_S)) return;
-          ++pair_phase;
-          const float l_sum = lxs[0] + lxs[1];
-          const size_t srow = (size_t)un.h * g.Tp + row;
-          float4* dst = reinterpret_cast<float4*>(a.snap.o + srow * D + 64 * half);
-          uint32_t rr[64];   // (warp-wide loads; rows past the end of a clipped tile only skip the stores)
-          tmem_ld32(tlane + TS_O + 64 * half, *reinterpret_cast<uint32_t(*)[32]>(rr));
-          tmem_ld32(tlane + TS_O + 64 * half + 32, *reinterpret_cast<uint32_t(*)[32]>(rr + 32));
-          tmem_ld_wait();
-          if (row_valid) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) st_global_v8(dst + 2 * i, rr + 8 * i);
-            if (half == 0) { a.snap.m[srow] = m_ref; a.snap.l[srow] = l_sum; }
-          }
-        }
-        const int tile_lo = tile_key_row<KIND, SPLIT>(un, t);
+        const int tile_lo = tile_key_row<SPLIT>(un, t);
         const int v_lo = max(un.k0 - tile_lo, 0), v_hi = min(un.k1 - tile_lo, BN);
         const int e_lo = un.x0 - tile_lo, e_hi = un.x1 - tile_lo;
         const bool all_valid = v_lo == 0 && v_hi == BN && (un.x1 <= un.x0 || e_hi <= 0 || e_lo >= BN);
@@ -878,37 +730,10 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
           mx = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
         }
         // The pair's maxima cross through shared memory (the slots alternate between consecutive exchanges).
-        // That round trip sits between the maximum and the exponentials of every tile, so a build does not
-        // wait for it: after a unit's first tile the reference exponent almost never moves (it moves only
-        // when a row's maximum outgrows it by more than RESCALE_SLACK), so the probabilities are formed
-        // with the reference as it stands while the exchange is under way, and formed again, the exact
-        // way, only when the exchange says that some row of the warp has to move its reference.
         volatile float* mxch = xch + 2 * (xslot & 1u);
         ++xslot;
         mxch[half] = mx;
         mbar_arrive(c.bar(BAR_PAIR + quad));
-        float ps0 = 0.f, ps1 = 0.f, ps2 = 0.f, ps3 = 0.f;
-        uint32_t pk[HC / 2];
-        // Probabilities of this thread's columns, from the registers: P~ = 2^(S c - m) rounded to fp16 (what
-        // the P~V product multiplies); the normaliser sums the rounded values, converted back exactly.
-        auto probabilities = [&](float m_sub) {
-          ps0 = ps1 = ps2 = ps3 = 0.f;
-#pragma unroll
-          for (int j = 0; j < HC / 2; ++j) {
-            const float p0 = ex2(fmaf(__uint_as_float(sr[2 * j]), g.scale_log2, -m_sub));
-            const float p1 = ex2(fmaf(__uint_as_float(sr[2 * j + 1]), g.scale_log2, -m_sub));
-            const __half2 hp = __floats2half2_rn(p0, p1);
-            const float2 pf = __half22float2(hp);
-            if (j & 1) { ps2 += pf.x; ps3 += pf.y; } else { ps0 += pf.x; ps1 += pf.y; }
-            pk[j] = *reinterpret_cast<const uint32_t*>(&hp);
-          }
-        };
-        // (not for the block queries of a step: few tiles per unit, and that kernel is sensitive to its size;
-        // and only after a tile that left every reference of the warp where it was: with large scores the
-        // references of a unit's first tiles move often, and forming the probabilities twice costs more
-        // than the exchange)
-        const bool ahead = !STEP && calm && !__any_sync(0xffffffffu, m_ref == -INFINITY);
-        if (ahead) probabilities(m_ref);
         if (!wait_bar(c, BAR_PAIR + quad, pair_phase & 1, LOC_WAIT_S)) return;
         ++pair_phase;
         mx = fmaxf(mxch[0], mxch[1]);
@@ -919,28 +744,35 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
         if (m_ref == -INFINITY || cand > m_ref + RESCALE_SLACK) m_new = fmaxf(m_ref, cand);
         float alpha = 1.f;
         // (both warps of the pair see the same rows and the same maxima: they take the same branch)
-        calm = !__any_sync(0xffffffffu, m_new != m_ref);
-        if (!(ahead && calm)) {
-          const float m_use = (m_new == -INFINITY) ? 0.f : m_new;
-          if (m_new != m_ref) alpha = (m_ref == -INFINITY) ? 0.f : ex2(m_ref - m_new);
-          if ((!first_tile || (WINDOW && have_o)) && __any_sync(0xffffffffu, alpha != 1.f)) {
-            // O~ in TMEM is rescaled in place: P~V of the previous tile must be done
-            if (!o_waited) {
-              if (!wait_bar(c, BAR_O_FULL, (jj - 1) & 1, LOC_WAIT_O)) return;
-              o_waited = true;
-              tc_fence_after();
-            }
+        const float m_use = (m_new == -INFINITY) ? 0.f : m_new;
+        if (m_new != m_ref) alpha = (m_ref == -INFINITY) ? 0.f : ex2(m_ref - m_new);
+        if (!first_tile && __any_sync(0xffffffffu, alpha != 1.f)) {
+          // O~ in TMEM is rescaled in place: P~V of the previous tile must be done
+          if (!wait_bar(c, BAR_O_FULL, (jj - 1) & 1, LOC_WAIT_O)) return;
+          o_waited = true;
+          tc_fence_after();
 #pragma unroll 1
-            for (int cb = 0; cb < 4; ++cb) {
-              uint32_t rr[16];
-              tmem_ld16(tlane + TS_O + 64 * half + 16 * cb, rr);
-              tmem_ld_wait();
+          for (int cb = 0; cb < 4; ++cb) {
+            uint32_t rr[16];
+            tmem_ld16(tlane + TS_O + 64 * half + 16 * cb, rr);
+            tmem_ld_wait();
 #pragma unroll
-              for (int j = 0; j < 16; ++j) rr[j] = __float_as_uint(__uint_as_float(rr[j]) * alpha);
-              tmem_st16(tlane + TS_O + 64 * half + 16 * cb, rr, 0);
-            }
+            for (int j = 0; j < 16; ++j) rr[j] = __float_as_uint(__uint_as_float(rr[j]) * alpha);
+            tmem_st16(tlane + TS_O + 64 * half + 16 * cb, rr, 0);
           }
-          probabilities(m_use);
+        }
+        // Probabilities of this thread's columns, from the registers: P~ = 2^(S c - m) rounded to fp16 (what
+        // the P~V product multiplies); the normaliser sums the rounded values, converted back exactly.
+        float ps0 = 0.f, ps1 = 0.f, ps2 = 0.f, ps3 = 0.f;
+        uint32_t pk[HC / 2];
+#pragma unroll
+        for (int j = 0; j < HC / 2; ++j) {
+          const float p0 = ex2(fmaf(__uint_as_float(sr[2 * j]), g.scale_log2, -m_use));
+          const float p1 = ex2(fmaf(__uint_as_float(sr[2 * j + 1]), g.scale_log2, -m_use));
+          const __half2 hp = __floats2half2_rn(p0, p1);
+          const float2 pf = __half22float2(hp);
+          if (j & 1) { ps2 += pf.x; ps3 += pf.y; } else { ps0 += pf.x; ps1 += pf.y; }
+          pk[j] = *reinterpret_cast<const uint32_t*>(&hp);
         }
 #pragma unroll
         for (int cb = 0; cb < HC / 16; ++cb)
@@ -1105,42 +937,6 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
       if (un.q_rows == BM && threadIdx.x == 64) mbar_arrive(c.bar(BAR_Q_FREE));
       continue;
     }
-    if (un.epi == EPI_STATE && un.q_rows == BM) {
-      // Cached state of a build unit, straight from TMEM to global memory (each thread 256
-      // contiguous bytes of its row).  Nothing is staged in the Q region, so the next unit's Q
-      // tile may be loaded while this epilogue runs.
-      if (threadIdx.x == 64) mbar_arrive(c.bar(BAR_Q_FREE));
-      const size_t srow = (size_t)un.h * g.Tp + row;
-      float4* dst = reinterpret_cast<float4*>(a.st.o + srow * D + 64 * half);
-      // (the TMEM loads are warp-wide: rows past the end of a clipped tile take part in them and
-      // only skip the stores; first_tile is uniform over the CTA)
-      uint32_t rr[64];
-      if (!first_tile || (WINDOW && have_o)) {
-        tmem_ld32(tlane + TS_O + 64 * half, *reinterpret_cast<uint32_t(*)[32]>(rr));
-        tmem_ld32(tlane + TS_O + 64 * half + 32, *reinterpret_cast<uint32_t(*)[32]>(rr + 32));
-        tmem_ld_wait();
-      } else {
-#pragma unroll
-        for (int j = 0; j < 64; ++j) rr[j] = 0u;
-      }
-      if (row_valid) {   // 32-byte stores: whole sectors, half as many instructions
-#pragma unroll
-        for (int i = 0; i < 8; ++i) st_global_v8(dst + 2 * i, rr + 8 * i);
-      }
-      if (row_valid && half == 0) { a.st.m[srow] = m_ref; a.st.l[srow] = l_run; }
-      if (WINDOW && un.snap && un.t1 - un.t0 <= 1) {
-        // a single key tile: the state after it is the final one as well
-        float4* sdst = reinterpret_cast<float4*>(a.snap.o + srow * D + 64 * half);
-        if (row_valid) {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) st_global_v8(sdst + 2 * i, rr + 8 * i);
-          if (half == 0) { a.snap.m[srow] = m_ref; a.snap.l[srow] = l_run; }
-        }
-      }
-      tc_fence_before();
-      mbar_arrive(c.bar(BAR_O_FREE));  // the next unit may overwrite O~
-      continue;
-    }
     // O~ (this thread's 64 features) from TMEM to its staging row.  The staging
     // area is the Q region (every score MMA of the unit is complete: the last
     // P~V, waited for above, was issued after them); 64-row units use its upper
@@ -1175,12 +971,7 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
     }
     tc_fence_before();
     mbar_arrive(c.bar(BAR_O_FREE));  // the next unit may overwrite O~
-    if (un.epi == EPI_STATE) {
-      const size_t srow = (size_t)un.h * g.Tp + row;
-      if (row_valid && half == 0) { a.st.m[srow] = m_ref; a.st.l[srow] = l_run; }
-      if (!epi_sync(c, epi_phase)) return;
-      coop_store_rows(c, stage_off, a.st.o + ((size_t)un.h * g.Tp + un.row0) * D, D, un.nrows);
-    } else if (un.epi == EPI_OUT) {
+    {   // (EPI_OUT)
       const size_t orow = (size_t)row * g.Hq + hrow;
       if (row_valid && half == 0 && a.lse) a.lse[orow] = (KIND == KIND_STEP2 ? lse2 : m_ref + log2f(l_run)) * LN2;
       if (!epi_sync(c, epi_phase)) return;
@@ -1770,7 +1561,6 @@ __device__ void deep_rows(const Cta& c, const Geometry& g, const AttnArgs& a, in
 template <bool PACKED, int KIND, bool DEEP, bool SPLIT>
 __global__ void __launch_bounds__(THREADS, 1)
 tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const AttnArgs a) {
-  constexpr bool STEP = kind_is_step(KIND);
   // (PACKED: the steps of a GQA model whose block queries share tiles across heads, see decode_stream;
   // KIND: see StreamKind; DEEP: which variant of the merge role a step runs)
   extern __shared__ __align__(1024) uint8_t smem_raw[];
@@ -1782,7 +1572,7 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
   // would crowd the SMs that fall idle first and run there when this grid is over (said at a CTA's last loads,
   // 48.9 us against 47.0 for a step at N = 5120 and 1376 against 1346 for a walk of five blocks there; at
   // N = 768 it would save 0.6 of 20.4 us).
-  if (STEP && a.step_overlap) grid_launch_dependents();
+  if (a.step_overlap) grid_launch_dependents();
   if (a.span != nullptr && tid == 0) atomicMin(a.span, global_timer_ns());   // first CTA entry of this launch
   Cta c;
   c.base = smem_u32(smem_raw);
@@ -1797,7 +1587,7 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
   const int n_ctas_merge = (int)gridDim.x - a.n_ctas_stream;
   // stream-role CTAs take the low block indices (they are scheduled first: the block
   // queries' chain of key tiles is the longest dependent chain of a step)
-  const bool stream = !STEP || (int)blockIdx.x < a.n_ctas_stream;   // (only a step has fixed rows to merge)
+  const bool stream = (int)blockIdx.x < a.n_ctas_stream;
   int first, stride, n_units;
   if (stream) {
     first = blockIdx.x; stride = a.n_ctas_stream; n_units = a.n_items * (PACKED ? a.stream_slots : g.Hq);
@@ -1807,7 +1597,7 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
   const bool deep = !stream && DEEP;   // (DEEP: a.merge_deep, which variant of the merge role this launch runs)
   if (tid == 0) {  // descriptor fetches overlap the set-up below
     if (stream) {
-      prefetch_map(STEP ? (PACKED ? &maps.q_pack : &maps.q64) : &maps.q);
+      prefetch_map(PACKED ? &maps.q_pack : &maps.q64);
       prefetch_map(&maps.k); prefetch_map(&maps.v);
     } else {
       prefetch_map(&maps.q); prefetch_map(&maps.st_o); prefetch_map(&maps.out);
@@ -1998,16 +1788,13 @@ bool make_v_map(CUtensorMap* m, void* base, int H, int Tp, int box_rows, char* e
 }  // namespace
 
 namespace {
-// {build / full recompute; build over key windows; the step of an MHA and of a GQA model, each with either variant of
-// the merge role; the paired step}.  One-plane builds run lacache_rows.cu, and the paired step exists for one-plane
-// operands only: null where there is none.
+// The step of an MHA and of a GQA model, each with either variant of the merge role; the paired step, which exists for
+// one-plane operands only.
 template <bool SPLIT>
 const void* const* kernel_table() {
-  static const void* const t[7] = {
-      SPLIT ? (const void*)tc_attn_kernel<false, KIND_BUILD, false, true> : nullptr,
-      SPLIT ? (const void*)tc_attn_kernel<false, KIND_WINDOW, false, true> : nullptr,
-      (const void*)tc_attn_kernel<false, KIND_STEP, false, SPLIT>,  (const void*)tc_attn_kernel<false, KIND_STEP, true, SPLIT>,
-      (const void*)tc_attn_kernel<true, KIND_STEP, false, SPLIT>,   (const void*)tc_attn_kernel<true, KIND_STEP, true, SPLIT>,
+  static const void* const t[5] = {
+      (const void*)tc_attn_kernel<false, KIND_STEP, false, SPLIT>, (const void*)tc_attn_kernel<false, KIND_STEP, true, SPLIT>,
+      (const void*)tc_attn_kernel<true, KIND_STEP, false, SPLIT>,  (const void*)tc_attn_kernel<true, KIND_STEP, true, SPLIT>,
       SPLIT ? nullptr : (const void*)tc_attn_kernel<false, KIND_STEP2, true, false>};
   return t;
 }
@@ -2016,7 +1803,7 @@ const void* const* kernel_table() {
 cudaError_t tc_prepare() {
   for (int split = 0; split < 2; ++split) {
     const void* const* t = split ? kernel_table<true>() : kernel_table<false>();
-    for (int i = 0; i < 7; ++i) {
+    for (int i = 0; i < 5; ++i) {
       if (!t[i]) continue;
       cudaError_t e = cudaFuncSetAttribute(t[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
       if (e != cudaSuccess) return e;
@@ -2080,7 +1867,7 @@ cudaError_t tc_attention(const Geometry& g, const AttnArgs& a, const TcMaps* map
     attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
     ++n_attr;
   }
-  const bool paired = a.mode == MODE_STEP && a.pair_chunks && !a.split;
+  const bool paired = a.pair_chunks && !a.split;
   if (paired) {   // CTAs 2k and 2k + 1 form a cluster: the two key chunks of one (sequence, head)
     attr[n_attr].id = cudaLaunchAttributeClusterDimension;
     attr[n_attr].val.clusterDim.x = 2;
@@ -2091,10 +1878,7 @@ cudaError_t tc_attention(const Geometry& g, const AttnArgs& a, const TcMaps* map
   cfg.attrs = attr;
   cfg.numAttrs = n_attr;
   const void* const* t = a.split ? kernel_table<true>() : kernel_table<false>();
-  int which;
-  if (a.mode != MODE_STEP) which = a.window ? 1 : 0;
-  else if (paired) which = 6;
-  else which = (a.pack > 1 ? 4 : 2) + (a.merge_deep ? 1 : 0);
+  const int which = paired ? 4 : (a.pack > 1 ? 2 : 0) + (a.merge_deep ? 1 : 0);
   void* params[3] = {const_cast<TcMaps*>(maps), const_cast<Geometry*>(&g), const_cast<AttnArgs*>(&a)};
   return cudaLaunchKernelExC(&cfg, t[which], params);
 }
