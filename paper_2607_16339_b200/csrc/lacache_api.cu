@@ -46,7 +46,6 @@ struct lacache_ctx {
     int deep_units = TC_DEEP_MAX_UNITS;  // LACACHE_DEEP_UNITS: units per CTA one launch of the pipelined merge variant takes
     bool no_pdl = false;     // LACACHE_NO_PDL: plain stream-ordered launches
     bool no_step_overlap = false;  // LACACHE_NO_STEP_OVERLAP
-    bool no_deep = false;    // LACACHE_NO_DEEP: earlier merge variant
     bool no_qcomp = false;   // LACACHE_NO_QCOMP: no in-kernel rotation of first units
     bool no_pack = false;    // LACACHE_NO_PACK: no head packing of GQA block queries
     bool no_pair = false;    // LACACHE_NO_PAIR: no paired CTAs (thread-block clusters) for two-chunk block rows
@@ -197,7 +196,6 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
     k.deep_units = std::max(1, std::min(geti("LACACHE_DEEP_UNITS", TC_DEEP_MAX_UNITS), (int)TC_DEEP_MAX_UNITS));
     k.no_pdl = getenv("LACACHE_NO_PDL") != nullptr;
     k.no_step_overlap = getenv("LACACHE_NO_STEP_OVERLAP") != nullptr;
-    k.no_deep = getenv("LACACHE_NO_DEEP") != nullptr;
     k.no_qcomp = getenv("LACACHE_NO_QCOMP") != nullptr;
     k.no_pack = getenv("LACACHE_NO_PACK") != nullptr;
     k.no_pair = getenv("LACACHE_NO_PAIR") != nullptr;
@@ -324,7 +322,7 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
         double ts = ceil(units_s / ns) * (3.0 + 1.6 * eff_tiles + merge_cost);
         // (a CTA with many merge units runs in the HBM-saturated regime, where a unit costs more)
         const double per_cta = ceil(units_m / (sms - ns));
-        double tm = 4.0 + per_cta * ((g.block_len <= 32 && per_cta <= 8) ? 2.6 : 3.4);
+        double tm = 4.0 + per_cta * (((g.block_len <= 32 || !c->split) && per_cta <= 8) ? 2.6 : 3.4);
         double t = std::max(ts, tm);
         if (t < best - 1e-9) { best = t; tpc = cand; }
       }
@@ -717,7 +715,7 @@ AttnArgs attn_args(lacache_ctx* c, int mode, lacache_ctx::ListRef list, int blk,
       a.n_items_merge = ml.n;
       long long units_merge = (long long)ml.n * Hq;
       int total = (int)std::min<long long>(c->num_sms, units_stream + units_merge);
-      const bool deep_ok = c->g.block_len <= 32 && !c->knobs.no_deep;
+      const bool deep_ok = c->g.block_len <= 32 || !c->split;   // (which variant of the merge role the step runs)
       const int deep_cap = deep_unit_cap(c);
       if (c->step_plan.empty()) c->step_plan.resize(c->g.n_blk);
       lacache_ctx::StepPlan& plan = c->step_plan[blk];
@@ -740,7 +738,7 @@ AttnArgs attn_args(lacache_ctx* c, int mode, lacache_ctx::ListRef list, int blk,
           rest = (double)units_merge - (double)deep_cap * (total - cand);
           per_cta = deep_cap;
         }
-        double tm = 4.0 + per_cta * ((c->g.block_len <= 32 && per_cta <= 8) ? 2.6 : 3.4);
+        double tm = 4.0 + per_cta * ((deep_ok && per_cta <= 8) ? 2.6 : 3.4);
         double t = std::max(ts, tm) + (rest > 0 ? 4.0 + ceil(rest / c->num_sms) * 3.4 : 0.0);
         if (t < best - 1e-9) { best = t; ns = cand; }
       }

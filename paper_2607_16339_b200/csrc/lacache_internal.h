@@ -108,7 +108,7 @@ struct AttnArgs {
   // block rows of `pack` query heads of one KV group share a 128-row tile (they read the same keys and
   // values): units then count (KV head, group of `pack` heads) pairs, each head taking `pack_rows` lanes.
   int stream_slots; int pack; int pack_rows;
-  int merge_deep;            // merge role runs its pipelined variant (block_len <= 32, bounded units per CTA)
+  int merge_deep;            // merge role runs its pipelined variant (block_len <= 32 or one-plane operands; bounded units per CTA)
   int split_merge;           // host only: more merge units per CTA than the pipelined variant tabulates, so the
                              // fixed rows of the step go out in several launches of that variant
   // step only: the block's pre-RoPE queries [B * block_len, Hq, d] and the cos/sin rows of

@@ -1254,7 +1254,7 @@ __device__ void merge_rows(const Cta& c, const TcMaps& maps, const Geometry& g, 
 
 // ===========================================================================
 // ===========================================================================
-// merge role, pipelined variant for block_len <= 32.  The block's keys and
+// merge role, pipelined variant.  For block_len <= 32 the block's keys and
 // values need only 24 KB, which leaves room for two staging tiles of cached
 // O~: the tile of unit u + 1 streams in while unit u is combined and while the
 // output of unit u - 1 streams out, so a CTA keeps ~190 KB of loads and stores
@@ -1265,29 +1265,38 @@ __device__ void merge_rows(const Cta& c, const TcMaps& maps, const Geometry& g, 
 // ===========================================================================
 constexpr uint32_t DM_IO = 65536;                      // two staging tiles of 4 boxes (64 KB each)
 constexpr uint32_t DM_IO_TILE = 4 * IO_BOX;
-constexpr uint32_t DM_KBOX = 32 * 128;                 // one [32 rows][64 cols] 16-bit box
-constexpr uint32_t DM_K = DM_IO + 2 * DM_IO_TILE;      // K hi (2 boxes), K lo (2 boxes)
-constexpr uint32_t DM_V = DM_K + 4 * DM_KBOX;          // V (2 boxes)
-constexpr uint32_t DM_TAB = DM_V + 2 * DM_KBOX;        // unit table: {row0, nrows, blk_start, head}
-constexpr int DM_MAX_UNITS = (int)((SM_XCH - DM_TAB) / 16);
-static_assert(DM_TAB % 16 == 0 && DM_MAX_UNITS >= TC_DEEP_MAX_UNITS, "unit table");
+// Where the block's keys and values and the unit table ({row0, nrows, blk_start, head}) are.  WIDE (block_len 33 .. 64,
+// one-plane operands): the keys and values of 64 rows take 32 KB, which the staging tiles leave no room for behind them,
+// but a one-plane Q' tile leaves the upper half of its region.
+template <bool SPLIT, bool WIDE>
+struct Deep {
+  static_assert(!(SPLIT && WIDE), "split planes leave no room for 64 rows");
+  static constexpr uint32_t BOX = (WIDE ? 64 : 32) * 128;                // one [rows][64 cols] 16-bit box
+  static constexpr uint32_t K = WIDE ? 32768 : DM_IO + 2 * DM_IO_TILE;   // K hi (2 boxes) [, K lo (2 boxes)]
+  static constexpr uint32_t V = K + (WIDE ? 2 : 4) * BOX;                // V (2 boxes)
+  static constexpr uint32_t TAB = WIDE ? DM_IO + 2 * DM_IO_TILE : V + 2 * BOX;
+  static_assert(TAB % 16 == 0 && (SM_XCH - TAB) / 16 >= TC_DEEP_MAX_UNITS, "unit table");
+  static_assert(!WIDE || V + 2 * BOX <= DM_IO, "the Q' region's upper half");
+};
 
 struct DUnit { int row0, nrows, blk_start, h, seq; };
+template <bool SPLIT, bool WIDE>
 __device__ __forceinline__ DUnit deep_unit(const Cta& c, int i) {
-  const int4 v = *reinterpret_cast<const int4*>(c.gen + DM_TAB + 16 * i);
+  const int4 v = *reinterpret_cast<const int4*>(c.gen + Deep<SPLIT, WIDE>::TAB + 16 * i);
   return DUnit{v.x, v.y, v.z, v.w & 0xFFFF, v.w >> 16};
 }
 
-template <bool SPLIT>
+template <bool SPLIT, bool WIDE>
 __device__ void deep_producer(const Cta& c, const TcMaps& maps, const Geometry& g, int n_my, bool kv_computed,
                               bool out_bf16) {
+  using DL = Deep<SPLIT, WIDE>;
   if (n_my == 0) return;
   auto load_q = [&](int i) {
-    const DUnit un = deep_unit(c, i);
+    const DUnit un = deep_unit<SPLIT, WIDE>(c, i);
     load_q_tile<SPLIT>(c, maps, BM, un.row0, un.h);
   };
   auto load_io = [&](int i) {
-    const DUnit un = deep_unit(c, i);
+    const DUnit un = deep_unit<SPLIT, WIDE>(c, i);
     const uint32_t bar = c.bar((i & 1) ? BAR_IO_FULL1 : BAR_IO_FULL);
     const uint32_t dst = c.base + DM_IO + (i & 1) * DM_IO_TILE;
     mbar_expect_tx(bar, DM_IO_TILE);
@@ -1295,18 +1304,18 @@ __device__ void deep_producer(const Cta& c, const TcMaps& maps, const Geometry& 
     for (int cb = 0; cb < 4; ++cb) tma_load_3d(dst + cb * IO_BOX, &maps.st_o, bar, 32 * cb, un.row0, un.h);
   };
   auto load_k = [&](int i) {
-    const DUnit un = deep_unit(c, i);
-    const uint32_t bar = c.bar(BAR_KV_FULL), kb = c.base + DM_K;
+    const DUnit un = deep_unit<SPLIT, WIDE>(c, i);
+    const uint32_t bar = c.bar(BAR_KV_FULL), kb = c.base + DL::K;
     const int kh = un.h / g.group;
-    mbar_expect_tx(bar, (SPLIT ? 4 : 2) * DM_KBOX);
-    load_qk_box(kb, &maps.k32, bar, un.blk_start, kh);
+    mbar_expect_tx(bar, (SPLIT ? 4 : 2) * DL::BOX);
+    load_qk_box(kb, WIDE ? &maps.k64 : &maps.k32, bar, un.blk_start, kh);
   };
   auto load_v = [&](int i) {
-    const DUnit un = deep_unit(c, i);
-    const uint32_t bar = c.bar(BAR_KV_FULL1), vb = c.base + DM_V;
+    const DUnit un = deep_unit<SPLIT, WIDE>(c, i);
+    const uint32_t bar = c.bar(BAR_KV_FULL1), vb = c.base + DL::V;
     const int kh = un.h / g.group;
-    mbar_expect_tx(bar, 2 * DM_KBOX);
-    load_v_box(vb, &maps.v32, bar, un.blk_start, kh);
+    mbar_expect_tx(bar, 2 * DL::BOX);
+    load_v_box(vb, WIDE ? &maps.v64 : &maps.v32, bar, un.blk_start, kh);
   };
   // Q' and cached O~ of fixed rows do not depend on the RoPE kernel launched
   // just before this one; the block's keys and values do
@@ -1342,7 +1351,7 @@ __device__ void deep_producer(const Cta& c, const TcMaps& maps, const Geometry& 
       load_v(vu); ++vu; did = true;
     }
     if (mbar_test(c.bar((su & 1) ? BAR_OUT_RDY1 : BAR_OUT_RDY), (su >> 1) & 1)) {
-      const DUnit un = deep_unit(c, su);
+      const DUnit un = deep_unit<SPLIT, WIDE>(c, su);
       if (!dep_done) { grid_dependency_wait(); dep_done = true; }  // no store before the preceding grids are complete
       if (store_out_tile(maps, c.base + DM_IO + (su & 1) * DM_IO_TILE, un.h, un.row0, un.nrows, out_bf16) > 0) {
         bulk_commit();
@@ -1375,17 +1384,18 @@ __device__ void deep_producer(const Cta& c, const TcMaps& maps, const Geometry& 
   bulk_wait_read();  // shared memory stays valid until the last store has read it
 }
 
-template <bool SPLIT>
+template <bool SPLIT, bool WIDE>
 __device__ void deep_mma(const Cta& c, const Geometry& g, int n_my, bool kv_computed) {
+  using DL = Deep<SPLIT, WIDE>;
   if (n_my == 0) return;
   const int n_s = (g.block_len + 15) & ~15;
   const uint32_t idesc_s = idesc_f16((!SPLIT && g.op_f16) ? 0u : 1u, 0u, BM, (uint32_t)n_s);
-  const uint32_t kb = c.base + DM_K;
+  const uint32_t kb = c.base + DL::K;
   if (!wait_bar(c, BAR_Q_FULL, 0, LOC_WAIT_Q)) return;
   if (!wait_bar(c, BAR_KV_FULL, 0, LOC_WAIT_K)) return;
   if (kv_computed && !wait_bar(c, BAR_QC, 0, LOC_WAIT_K)) return;  // keys and values written by the row threads
   tc_fence_after();
-  issue_s_mma<SPLIT>(c.base + SM_Q, BM * 128u, kb, kb + 2 * DM_KBOX, DM_KBOX, c.tmem + TM_S, idesc_s);
+  issue_s_mma<SPLIT>(c.base + SM_Q, BM * 128u, kb, kb + 2 * DL::BOX, DL::BOX, c.tmem + TM_S, idesc_s);
   tc_commit(c.bar(BAR_S_FULL));
   tc_commit(c.bar(BAR_Q_FREE));
   tc_commit(c.bar(BAR_KV_FREE));
@@ -1395,7 +1405,7 @@ __device__ void deep_mma(const Cta& c, const Geometry& g, int n_my, bool kv_comp
     if (k >= 1 && !wait_bar(c, BAR_O_FREE + b, (k - 1) & 1, LOC_WAIT_O)) return;
     if (!wait_bar(c, BAR_KV_FULL1, uu & 1, LOC_WAIT_V)) return;
     tc_fence_after();
-    issue_pv_mma(c.base + DM_V, DM_KBOX, c.tmem + TM_P + 32 * b, c.tmem + TM_O + 128 * b, n_s / 16, 0u);
+    issue_pv_mma(c.base + DL::V, DL::BOX, c.tmem + TM_P + 32 * b, c.tmem + TM_O + 128 * b, n_s / 16, 0u);
     tc_commit(c.bar(BAR_O_FULL + b));
     tc_commit(c.bar(BAR_KV_FREE1));
     if (uu + 1 < n_my) {  // scores of the next unit as soon as its tiles land
@@ -1403,7 +1413,7 @@ __device__ void deep_mma(const Cta& c, const Geometry& g, int n_my, bool kv_comp
       if (!wait_bar(c, BAR_Q_FULL, (uu + 1) & 1, LOC_WAIT_Q)) return;
       if (!wait_bar(c, BAR_KV_FULL, (uu + 1) & 1, LOC_WAIT_K)) return;
       tc_fence_after();
-      issue_s_mma<SPLIT>(c.base + SM_Q, BM * 128u, kb, kb + 2 * DM_KBOX, DM_KBOX, c.tmem + TM_S + 64 * bn, idesc_s);
+      issue_s_mma<SPLIT>(c.base + SM_Q, BM * 128u, kb, kb + 2 * DL::BOX, DL::BOX, c.tmem + TM_S + 64 * bn, idesc_s);
       tc_commit(c.bar(BAR_S_FULL + bn));
       tc_commit(c.bar(BAR_Q_FREE));
       tc_commit(c.bar(BAR_KV_FREE));
@@ -1411,8 +1421,9 @@ __device__ void deep_mma(const Cta& c, const Geometry& g, int n_my, bool kv_comp
   }
 }
 
-template <bool SPLIT>
+template <bool SPLIT, bool WIDE>
 __device__ void deep_rows(const Cta& c, const Geometry& g, const AttnArgs& a, int n_my) {
+  using DL = Deep<SPLIT, WIDE>;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int quad = warp & 3;
   const int half = (warp - 2) >> 2;
@@ -1424,7 +1435,7 @@ __device__ void deep_rows(const Cta& c, const Geometry& g, const AttnArgs& a, in
   // the cached (m, l) of a unit's rows are fetched one unit ahead
   float m_nx = -INFINITY, l_nx = 0.f;
   if (n_my > 0) {
-    const DUnit un = deep_unit(c, 0);
+    const DUnit un = deep_unit<SPLIT, WIDE>(c, 0);
     if (r < un.nrows) {
       const size_t srow = (size_t)un.h * g.Tp + un.row0 + r;
       m_nx = __ldg(a.st.m + srow);
@@ -1436,7 +1447,7 @@ __device__ void deep_rows(const Cta& c, const Geometry& g, const AttnArgs& a, in
     // computed here with the RoPE kernel's own arithmetic and written where the TMA loads
     // would have put them ([plane][feature half][row][64], 16-byte chunks XOR-swizzled by
     // the row), so the unit does not wait for that kernel.
-    const DUnit un = deep_unit(c, 0);
+    const DUnit un = deep_unit<SPLIT, WIDE>(c, 0);
     const int kh = un.h / g.group;
     const int tq = threadIdx.x - 64;
     for (int i = tq; i < L * 8; i += ROW_THREADS) {
@@ -1460,44 +1471,44 @@ __device__ void deep_rows(const Cta& c, const Geometry& g, const AttnArgs& a, in
         rope_split8(y1, h1, l1);
         rope_split8(y2, h2, l2);
       }
-      uint8_t* const k0 = c.gen + DM_K + ki * 128 + ((ch ^ (ki & 7)) << 4);
+      uint8_t* const k0 = c.gen + DL::K + ki * 128 + ((ch ^ (ki & 7)) << 4);
       *reinterpret_cast<uint4*>(k0) = h1;
-      *reinterpret_cast<uint4*>(k0 + DM_KBOX) = h2;
+      *reinterpret_cast<uint4*>(k0 + DL::BOX) = h2;
       if (SPLIT) {
-        *reinterpret_cast<uint4*>(k0 + 2 * DM_KBOX) = l1;
-        *reinterpret_cast<uint4*>(k0 + 3 * DM_KBOX) = l2;
+        *reinterpret_cast<uint4*>(k0 + 2 * DL::BOX) = l1;
+        *reinterpret_cast<uint4*>(k0 + 3 * DL::BOX) = l2;
       }
       // values: the same two 8-feature chunks of row ki, unrotated
       float v1[8], v2[8];
       rope_load8(a.v_raw, soff + c0, true, v1);
       rope_load8(a.v_raw, soff + c0 + D / 2, true, v2);
-      uint8_t* const v0 = c.gen + DM_V + ki * 128 + ((ch ^ (ki & 7)) << 4);
+      uint8_t* const v0 = c.gen + DL::V + ki * 128 + ((ch ^ (ki & 7)) << 4);
       *reinterpret_cast<uint4*>(v0) = rope_half8(v1);
-      *reinterpret_cast<uint4*>(v0 + DM_KBOX) = rope_half8(v2);
+      *reinterpret_cast<uint4*>(v0 + DL::BOX) = rope_half8(v2);
     }
-    // rows [L, 32) of the boxes (block_len < 32) are never multiplied by a non-zero P~
+    // rows [L, 32) of the boxes ([L, 64) of wide ones) are never multiplied by a non-zero P~
     // but must not hold NaN or Inf patterns: clear them
-    for (int i = tq + L * 8; i < 32 * 8; i += ROW_THREADS) {
+    for (int i = tq + L * 8; i < (WIDE ? 64 : 32) * 8; i += ROW_THREADS) {
       const int ki = i >> 3, ch = i & 7;
       const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-      uint8_t* const k0 = c.gen + DM_K + ki * 128 + ((ch ^ (ki & 7)) << 4);
-      *reinterpret_cast<uint4*>(k0) = z; *reinterpret_cast<uint4*>(k0 + DM_KBOX) = z;
-      if (SPLIT) { *reinterpret_cast<uint4*>(k0 + 2 * DM_KBOX) = z; *reinterpret_cast<uint4*>(k0 + 3 * DM_KBOX) = z; }
-      uint8_t* const v0 = c.gen + DM_V + ki * 128 + ((ch ^ (ki & 7)) << 4);
-      *reinterpret_cast<uint4*>(v0) = z; *reinterpret_cast<uint4*>(v0 + DM_KBOX) = z;
+      uint8_t* const k0 = c.gen + DL::K + ki * 128 + ((ch ^ (ki & 7)) << 4);
+      *reinterpret_cast<uint4*>(k0) = z; *reinterpret_cast<uint4*>(k0 + DL::BOX) = z;
+      if (SPLIT) { *reinterpret_cast<uint4*>(k0 + 2 * DL::BOX) = z; *reinterpret_cast<uint4*>(k0 + 3 * DL::BOX) = z; }
+      uint8_t* const v0 = c.gen + DL::V + ki * 128 + ((ch ^ (ki & 7)) << 4);
+      *reinterpret_cast<uint4*>(v0) = z; *reinterpret_cast<uint4*>(v0 + DL::BOX) = z;
     }
     fence_async_smem();  // the MMAs read shared memory through the async proxy
     mbar_arrive(c.bar(BAR_QC));
   }
   for (int uu = 0; uu < n_my; ++uu) {
-    const DUnit un = deep_unit(c, uu);
+    const DUnit un = deep_unit<SPLIT, WIDE>(c, uu);
     const int b = uu & 1, par = (uu >> 1) & 1;
     const int row = un.row0 + r;
     const bool row_valid = r < un.nrows;
     const float m_c = m_nx, l_c = l_nx;
     m_nx = -INFINITY; l_nx = 0.f;
     if (uu + 1 < n_my) {
-      const DUnit nx = deep_unit(c, uu + 1);
+      const DUnit nx = deep_unit<SPLIT, WIDE>(c, uu + 1);
       if (r < nx.nrows) {
         const size_t srow = (size_t)nx.h * g.Tp + nx.row0 + r;
         m_nx = __ldg(a.st.m + srow);
@@ -1513,10 +1524,17 @@ __device__ void deep_rows(const Cta& c, const Geometry& g, const AttnArgs& a, in
     float mx = -INFINITY;
     uint32_t s0[32];
     tmem_ld32(tlane + TM_S + 64 * b, s0);
+    uint32_t s1[WIDE ? 32 : 1];   // (wide: columns 32 .. 63)
+    if constexpr (WIDE) tmem_ld32(tlane + TM_S + 64 * b + 32, s1);
     tmem_ld_wait();
 #pragma unroll
     for (int j = 0; j < 32; ++j)
       if (j < L) mx = fmaxf(mx, __uint_as_float(s0[j]));
+    if constexpr (WIDE) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j)
+        if (32 + j < L) mx = fmaxf(mx, __uint_as_float(s1[j]));
+    }
     const float m_new = fmaxf(m_c, ceilf(mx * g.scale_log2));
     const float alpha = (m_c == -INFINITY) ? 0.f : ex2(m_c - m_new);
     float psum = 0.f;
@@ -1531,6 +1549,17 @@ __device__ void deep_rows(const Cta& c, const Geometry& g, const AttnArgs& a, in
         pk[j] = *reinterpret_cast<uint32_t*>(&hp);
       }
       if (half == 0) tmem_st16(tlane + TM_P + 32 * b, pk);
+      if constexpr (WIDE) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          float p0 = (32 + 2 * j < L) ? round_to_half_bits(ex2(fmaf(__uint_as_float(s1[2 * j]), g.scale_log2, -m_new))) : 0.f;
+          float p1 = (33 + 2 * j < L) ? round_to_half_bits(ex2(fmaf(__uint_as_float(s1[2 * j + 1]), g.scale_log2, -m_new))) : 0.f;
+          psum += p0 + p1;
+          __half2 hp = __floats2half2_rn(p0, p1);
+          pk[j] = *reinterpret_cast<uint32_t*>(&hp);
+        }
+        if (half == 1) tmem_st16(tlane + TM_P + 32 * b + 16, pk);
+      }
     }
     tmem_st_wait();
     tc_fence_before();
@@ -1558,11 +1587,14 @@ __device__ void deep_rows(const Cta& c, const Geometry& g, const AttnArgs& a, in
   }
 }
 
-template <bool PACKED, int KIND, bool DEEP, bool SPLIT>
+template <bool PACKED, int KIND, int DEEP, bool SPLIT>
 __global__ void __launch_bounds__(THREADS, 1)
 tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const AttnArgs a) {
   // (PACKED: the steps of a GQA model whose block queries share tiles across heads, see decode_stream;
-  // KIND: see StreamKind; DEEP: which variant of the merge role a step runs)
+  // KIND: see StreamKind; DEEP: which variant of the merge role a step runs -- 0: one staging tile, 1: pipelined, 2: pipelined,
+  // for blocks of 33 .. 64 rows)
+  constexpr bool WIDE = DEEP == 2;
+  using DL = Deep<SPLIT && !WIDE, WIDE>;
   extern __shared__ __align__(1024) uint8_t smem_raw[];
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
@@ -1594,14 +1626,14 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
   } else {
     first = blockIdx.x - a.n_ctas_stream; stride = n_ctas_merge; n_units = a.n_items_merge * g.Hq;
   }
-  const bool deep = !stream && DEEP;   // (DEEP: a.merge_deep, which variant of the merge role this launch runs)
+  const bool deep = !stream && DEEP != 0;   // (DEEP: a.merge_deep, which variant of the merge role this launch runs)
   if (tid == 0) {  // descriptor fetches overlap the set-up below
     if (stream) {
       prefetch_map(PACKED ? &maps.q_pack : &maps.q64);
       prefetch_map(&maps.k); prefetch_map(&maps.v);
     } else {
       prefetch_map(&maps.q); prefetch_map(&maps.st_o); prefetch_map(&maps.out);
-      prefetch_map(deep ? &maps.k32 : &maps.k64); prefetch_map(deep ? &maps.v32 : &maps.v64);
+      prefetch_map(deep && !WIDE ? &maps.k32 : &maps.k64); prefetch_map(deep && !WIDE ? &maps.v32 : &maps.v64);
     }
   }
   const int n_my = first < n_units ? (n_units - first + stride - 1) / stride : 0;
@@ -1640,7 +1672,7 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
       // units are head-minor (unit u = row tile u / Hq of head u % Hq): a CTA's units, a
       // fixed stride apart, then cycle through the row tiles, clipped ones included
       const WorkItem w = load_item(a.items_merge + u / g.Hq);
-      *reinterpret_cast<int4*>(smem_raw + DM_TAB + 16 * i) = make_int4(w.row0, w.nrows, w.blk_start, (u % g.Hq) | (w.seq << 16));
+      *reinterpret_cast<int4*>(smem_raw + DL::TAB + 16 * i) = make_int4(w.row0, w.nrows, w.blk_start, (u % g.Hq) | (w.seq << 16));
     }
   }
   __syncwarp();
@@ -1662,21 +1694,21 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
     if (stream) {
       if (tid == 0) stream_producer<PACKED, KIND, SPLIT>(c, maps, g, a, first, stride, n_units, it0);
     } else if (deep) {
-      if (tid == 0) deep_producer<SPLIT>(c, maps, g, n_my, a.k_raw != nullptr, a.out_bf16 != 0);
+      if (tid == 0) deep_producer<SPLIT, WIDE>(c, maps, g, n_my, a.k_raw != nullptr, a.out_bf16 != 0);
     } else {
       if (tid == 0) merge_producer<SPLIT>(c, maps, g, a, first, stride, n_units, it0);
     }
   } else if (warp == 1) {
     if (tid == 32) {
       if (stream) stream_mma_scores<PACKED, KIND, SPLIT>(c, g, a, first, stride, n_units, it0);
-      else if (deep) deep_mma<SPLIT>(c, g, n_my, a.k_raw != nullptr);
+      else if (deep) deep_mma<SPLIT, WIDE>(c, g, n_my, a.k_raw != nullptr);
       else merge_mma<SPLIT>(c, g, a, first, stride, n_units);
     }
   } else if (warp == 10) {
     if (tid == 320 && stream) stream_mma_pv<PACKED, KIND, SPLIT>(c, g, a, first, stride, n_units, it0);
   } else {
     if (stream) stream_rows<PACKED, KIND, SPLIT>(c, g, a, first, stride, n_units, it0);
-    else if (deep) deep_rows<SPLIT>(c, g, a, n_my);
+    else if (deep) deep_rows<SPLIT, WIDE>(c, g, a, n_my);
     else merge_rows(c, maps, g, a, first, stride, n_units, it0);
     bulk_wait_read();
   }
@@ -1788,14 +1820,15 @@ bool make_v_map(CUtensorMap* m, void* base, int H, int Tp, int box_rows, char* e
 }  // namespace
 
 namespace {
-// The step of an MHA and of a GQA model, each with either variant of the merge role; the paired step, which exists for
-// one-plane operands only.
+// The step of an MHA and of a GQA model, each for blocks of more than 32 rows (the pipelined merge role for wide blocks, with
+// split planes the one with a single staging tile) and of up to 32; the paired step, which exists for one-plane operands
+// only.
 template <bool SPLIT>
 const void* const* kernel_table() {
   static const void* const t[5] = {
-      (const void*)tc_attn_kernel<false, KIND_STEP, false, SPLIT>, (const void*)tc_attn_kernel<false, KIND_STEP, true, SPLIT>,
-      (const void*)tc_attn_kernel<true, KIND_STEP, false, SPLIT>,  (const void*)tc_attn_kernel<true, KIND_STEP, true, SPLIT>,
-      SPLIT ? nullptr : (const void*)tc_attn_kernel<false, KIND_STEP2, true, false>};
+      (const void*)tc_attn_kernel<false, KIND_STEP, SPLIT ? 0 : 2, SPLIT>, (const void*)tc_attn_kernel<false, KIND_STEP, 1, SPLIT>,
+      (const void*)tc_attn_kernel<true, KIND_STEP, SPLIT ? 0 : 2, SPLIT>,  (const void*)tc_attn_kernel<true, KIND_STEP, 1, SPLIT>,
+      SPLIT ? nullptr : (const void*)tc_attn_kernel<false, KIND_STEP2, 1, false>};
   return t;
 }
 }  // namespace
@@ -1878,7 +1911,7 @@ cudaError_t tc_attention(const Geometry& g, const AttnArgs& a, const TcMaps* map
   cfg.attrs = attr;
   cfg.numAttrs = n_attr;
   const void* const* t = a.split ? kernel_table<true>() : kernel_table<false>();
-  const int which = paired ? 4 : (a.pack > 1 ? 2 : 0) + (a.merge_deep ? 1 : 0);
+  const int which = paired ? 4 : (a.pack > 1 ? 2 : 0) + (g.block_len <= 32 ? 1 : 0);
   void* params[3] = {const_cast<TcMaps*>(maps), const_cast<Geometry*>(&g), const_cast<AttnArgs*>(&a)};
   return cudaLaunchKernelExC(&cfg, t[which], params);
 }
