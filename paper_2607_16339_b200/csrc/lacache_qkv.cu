@@ -202,15 +202,31 @@ __device__ __forceinline__ Work my_work(const GemmArgs& a) {
   return w;
 }
 
-// destination of feature tile ft, input token t: a row of q, k or v (null: the row is dropped)
-__device__ __forceinline__ __nv_bfloat16* out_row(const GemmArgs& a, int ft, int t) {
+// Row 0 of feature tile ft's head in q, k or v, and the elements between two rows of it.
+struct Dest { __nv_bfloat16* p; uint32_t stride; };
+__device__ __forceinline__ Dest dest_of(const GemmArgs& a, int ft) {
+  if (ft < a.Hq) return {a.q + (size_t)ft * QD, (uint32_t)(a.Hq * QD)};
+  if (ft < a.Hq + a.Hkv) return {a.k + (size_t)(ft - a.Hq) * QD, (uint32_t)(a.Hkv * QD)};
+  return {a.v + (size_t)(ft - a.Hq - a.Hkv) * QD, (uint32_t)(a.Hkv * QD)};
+}
+// output row of input token t (-1: there is none)
+__device__ __forceinline__ int out_row(const GemmArgs& a, int t) {
+  if (t >= a.n_tokens) return -1;
   if (a.dst_rows) {
     t = __ldg(a.dst_rows + t);
-    if ((unsigned)t >= (unsigned)a.max_rows) return nullptr;   // reported by the norm kernel
+    if ((unsigned)t >= (unsigned)a.max_rows) return -1;   // reported by the norm kernel
   }
-  if (ft < a.Hq) return a.q + ((size_t)t * a.Hq + ft) * QD;
-  if (ft < a.Hq + a.Hkv) return a.k + ((size_t)t * a.Hkv + (ft - a.Hq)) * QD;
-  return a.v + ((size_t)t * a.Hkv + (ft - a.Hq - a.Hkv)) * QD;
+  return t;
+}
+// Feature f of 32 tokens (lane i of the warp holds the row of the i-th, -1: not stored) as bf16.  Unrolled over
+// registers by 32, this runs once per kernel from a cold instruction cache: its length is its time (2.5 us with the
+// row looked up and the address built inside, per token).
+__device__ __forceinline__ void store_feature(const Dest& d, int f, int lane_row, const float (&v)[32]) {
+#pragma unroll
+  for (int i = 0; i < 32; ++i) {
+    const int row = __shfl_sync(0xffffffffu, lane_row, i);
+    if (row >= 0) d.p[(size_t)row * d.stride + f] = __float2bfloat16_rn(v[i]);
+  }
 }
 
 // Walks this CTA's chunks in order without divisions: ring stage and phase, tile coordinates, chunk.
@@ -332,6 +348,22 @@ __device__ __forceinline__ void closer_epilogue(const QCta& c, const GemmArgs& a
   const int ft = tile / a.n_ttiles, tt = tile % a.n_ttiles;
   const int t0 = tt * a.tn;
   const int nt = min(a.tn, a.n_tokens - t0);
+  // the helpers whose ranges touch the first hp chunks of this tile, in ascending order (at most three:
+  // a helper's range is at least hp long); looked up before the wait below, not
+  // behind it: its divisions cost a microsecond at the kernel's end
+  const Sharing sh = sharing(a);
+  const long long x_lo = (long long)tile * sh.kce;
+  const int j_lo = cta_of(sh, x_lo), j_hi = cta_of(sh, x_lo + sh.kce - 1);
+  const float *p0 = nullptr, *p1 = nullptr, *p2 = nullptr;
+  int n_parts = 0;
+  for (int j = j_lo; j <= j_hi; ++j) {
+    const long long s0 = range_start(sh, j), s1 = range_start(sh, j + 1);
+    if (s1 <= s0) continue;
+    const int slot = tile - (int)(s0 / sh.kce);    // the ordinal of this tile among the helper's segments
+    const float* p = a.ws + ((size_t)(sh.first_cta + j) * WS_SLOTS + slot) * (size_t)(MAX_TN * QD) + f;
+    if (n_parts == 0) p0 = p; else if (n_parts == 1) p1 = p; else p2 = p;
+    ++n_parts;
+  }
   // Every helper part of the tile has been published once the tile's counter shows all hp chunks.  The
   // counter is looked at only after this launch's operand rows are complete: every earlier launch of the
   // handle (whose closer may not have reset the counter yet) is then over.
@@ -359,22 +391,9 @@ __device__ __forceinline__ void closer_epilogue(const QCta& c, const GemmArgs& a
   asm volatile("bar.sync 1, 128;" ::: "memory");
   if (*flag == 0) return;
   __threadfence();
-  // the helpers whose ranges touch the first hp chunks of this tile, in ascending order (at most three:
-  // a helper's range is at least hp long)
-  const Sharing sh = sharing(a);
-  const long long x_lo = (long long)tile * sh.kce;
-  const int j_lo = cta_of(sh, x_lo), j_hi = cta_of(sh, x_lo + sh.kce - 1);
-  const float *p0 = nullptr, *p1 = nullptr, *p2 = nullptr;
-  int n_parts = 0;
-  for (int j = j_lo; j <= j_hi; ++j) {
-    const long long s0 = range_start(sh, j), s1 = range_start(sh, j + 1);
-    if (s1 <= s0) continue;
-    const int slot = tile - (int)(s0 / sh.kce);    // the ordinal of this tile among the helper's segments
-    const float* p = a.ws + ((size_t)(sh.first_cta + j) * WS_SLOTS + slot) * (size_t)(MAX_TN * QD) + f;
-    if (n_parts == 0) p0 = p; else if (n_parts == 1) p1 = p; else p2 = p;
-    ++n_parts;
-  }
+  const Dest dst = dest_of(a, ft);
   for (int g = 0; g * 32 < nt; ++g) {
+    const int lane_row = out_row(a, t0 + g * 32 + (tid & 31));
     float pre0[32], pre1[32], pre2[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) {
@@ -385,25 +404,17 @@ __device__ __forceinline__ void closer_epilogue(const QCta& c, const GemmArgs& a
       pre2[i] = (t < nt && n_parts > 2) ? __ldcg(p2 + o) : 0.f;
     }
     if (g == 0) {
+      grid_dependency_wait();   // results may overwrite rows that a grid ahead in the stream still reads
       if (!q_wait(c, QB_ACC_FULL, 0, QLOC_WAIT_ACC_FULL)) return;
       tc_fence_after();
-      grid_dependency_wait();   // results may overwrite rows that a grid ahead in the stream still reads
     }
     uint32_t r[32];
     tmem_ld32(tmem + lane_off + (uint32_t)(g * 32), r);
     tmem_ld_wait();
+    float sum[32];
 #pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      const int t = g * 32 + i;
-      float sum = 0.f + pre0[i];
-      if (n_parts > 1) sum += pre1[i];
-      if (n_parts > 2) sum += pre2[i];
-      sum += __uint_as_float(r[i]);
-      if (t < nt) {
-        __nv_bfloat16* dst = out_row(a, ft, t0 + t);
-        if (dst) dst[f] = __float2bfloat16_rn(sum);
-      }
-    }
+    for (int i = 0; i < 32; ++i) sum[i] = ((0.f + pre0[i]) + pre1[i]) + pre2[i] + __uint_as_float(r[i]);
+    store_feature(dst, f, lane_row, sum);
   }
   tc_fence_before();
   mbar_arrive(c.bar(QB_ACC_FREE));
@@ -440,14 +451,10 @@ __device__ __forceinline__ void gemm_epilogue(const QCta& c, const GemmArgs& a, 
       tmem_ld_wait();
       if (whole) {
         grid_dependency_wait();   // results may overwrite rows that a grid ahead in the stream still reads
+        float v[32];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const int t = g * 32 + i;
-          if (t < nt) {
-            __nv_bfloat16* dst = out_row(a, ft, t0 + t);
-            if (dst) dst[f] = __float2bfloat16_rn(__uint_as_float(r[i]));
-          }
-        }
+        for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
+        store_feature(dest_of(a, ft), f, out_row(a, t0 + g * 32 + (tid & 31)), v);
       } else {
 #pragma unroll
         for (int i = 0; i < 32; ++i) {
@@ -491,6 +498,7 @@ __device__ __forceinline__ void gemm_epilogue(const QCta& c, const GemmArgs& a, 
           ++n_parts;
         }
         const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        const Dest dst = dest_of(a, ft);
         for (int tb = 0; tb < nt; tb += 32) {
           float4 acc[8];
           if (n_parts <= 3) {
@@ -537,8 +545,8 @@ __device__ __forceinline__ void gemm_epilogue(const QCta& c, const GemmArgs& a, 
               uint2 o;
               o.x = *reinterpret_cast<uint32_t*>(&lo);
               o.y = *reinterpret_cast<uint32_t*>(&hi);
-              __nv_bfloat16* dst = out_row(a, ft, t0 + t);
-              if (dst) *reinterpret_cast<uint2*>(dst + f4) = o;
+              const int row = out_row(a, t0 + t);
+              if (row >= 0) *reinterpret_cast<uint2*>(dst.p + (size_t)row * dst.stride + f4) = o;
             }
           }
         }
@@ -1052,10 +1060,13 @@ lacache_status project_impl(lacache_qkv* p, const int32_t* token_ids, const void
   const int n_ctas = (int)std::min<long long>(p->num_sms, ga.total_chunks);
   ga.hp = 0;
   if (n_ctas > ga.n_tiles && n_ctas < 2 * ga.n_tiles && !p->plain_split) {
-    // closers take `per_closer` chunks each, helpers about HEAD_START chunks fewer
-    const int HEAD_START = 8;
+    // closers take `per_closer` chunks each, helpers about 7/16 of a tile's chunks fewer: a helper's parts have to be
+    // published and counted before a closer may fetch them, and a closer's loads speed up once the helpers are through
+    // (the weights' stream as a whole is what is limited).  96 heads x 4096, 32 tokens, the whole step from token ids:
+    // 48.8 us at 8 chunks, 48.5 at 16, 48.1 at 24, 47.9 at 28, 47.8 at 32, 47.9 at 40.
+    const int head_start = ga.kc * 7 / 16;
     const int n_helpers = n_ctas - ga.n_tiles;
-    const long long num = ga.total_chunks + (long long)n_helpers * HEAD_START;
+    const long long num = ga.total_chunks + (long long)n_helpers * head_start;
     const int per_closer = (int)((num + n_ctas - 1) / n_ctas);
     const int hp = ga.kc - per_closer;
     if (hp >= 1 && (long long)ga.n_tiles * hp >= n_helpers) ga.hp = hp;
