@@ -115,9 +115,7 @@ struct AttnArgs {
   // those tokens [B * block_len][d/2]; a CTA's first block-query unit rotates its Q tile
   // from these itself and so does not have to wait for the RoPE kernel
   const void* q_raw; const float* row_cos; const float* row_sin;   // (bf16: the tcgen05 engine takes bf16 inputs only)
-  // likewise the block's pre-RoPE keys and values [B * block_len, Hkv, d]: the first unit of a
-  // pipelined merge-role CTA rotates the block's keys / converts its values itself
-  const void* k_raw; const void* v_raw;
+  const void* k_raw; const void* v_raw;   // likewise the block's pre-RoPE keys and values [B * block_len, Hkv, d] (SIMT)
   // SIMT: with the three raw pointers set, a step's kernel rotates the block's rows itself and leaves them in
   // the rotated cache (no RoPE kernel ahead of it); their element type is bf16 or fp32
   int raw_bf16;

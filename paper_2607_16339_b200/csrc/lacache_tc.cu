@@ -1287,8 +1287,7 @@ __device__ __forceinline__ DUnit deep_unit(const Cta& c, int i) {
 }
 
 template <bool SPLIT, bool WIDE>
-__device__ void deep_producer(const Cta& c, const TcMaps& maps, const Geometry& g, int n_my, bool kv_computed,
-                              bool out_bf16) {
+__device__ void deep_producer(const Cta& c, const TcMaps& maps, const Geometry& g, int n_my, bool out_bf16) {
   using DL = Deep<SPLIT, WIDE>;
   if (n_my == 0) return;
   auto load_q = [&](int i) {
@@ -1320,39 +1319,23 @@ __device__ void deep_producer(const Cta& c, const TcMaps& maps, const Geometry& 
   // Q' and cached O~ of fixed rows do not depend on the RoPE kernel launched
   // just before this one; the block's keys and values do
   // (the second unit's cached-O~ tile is requested once the first Q' tile has landed, not with it: at the start
-  // of a step every CTA's requests queue in front of HBM, and the tile that is needed last gives way)
+  // of a step every CTA's requests queue in front of HBM, and the tile that is needed last gives way).
+  // Waiting for the RoPE kernel costs less than rotating the first unit's keys here would (20.2 us against 20.5 for a
+  // step at 32 heads, N = 768, 80.5 against 81.5 for eight such sequences): that code ran once, at 4 us of instruction
+  // fetches behind the bulk loads.
   load_q(0);
   load_io(0);
-  bool dep_done = false;
   bool q0_landed = false;   // (latched: the barrier's parity comes round again)
-  if (kv_computed) {
-    // the row threads rotate / convert the block's keys and values of the first unit
-    // from the raw inputs (plain arrivals keep the barriers' phase counts in step)
-    mbar_arrive(c.bar(BAR_KV_FULL));
-    mbar_arrive(c.bar(BAR_KV_FULL1));
-  } else {
-    grid_dependency_wait();
-    dep_done = true;
-    load_k(0);
-    load_v(0);
-  }
+  grid_dependency_wait();
+  load_k(0);
+  load_v(0);
   int qu = 1, ku = 1, vu = 1, iu = 1, su = 0;
   bool pending_read = false;  // an output store may still be reading its staging tile
   long long t_idle = 0;
   while (su < n_my) {
     bool did = false;
-    if (qu < n_my && mbar_test(c.bar(BAR_Q_FREE), (qu - 1) & 1)) { load_q(qu); ++qu; did = true; }
-    if (ku < n_my && mbar_test(c.bar(BAR_KV_FREE), (ku - 1) & 1)) {
-      if (!dep_done) { grid_dependency_wait(); dep_done = true; }  // long over by now
-      load_k(ku); ++ku; did = true;
-    }
-    if (vu < n_my && mbar_test(c.bar(BAR_KV_FREE1), (vu - 1) & 1)) {
-      if (!dep_done) { grid_dependency_wait(); dep_done = true; }
-      load_v(vu); ++vu; did = true;
-    }
     if (mbar_test(c.bar((su & 1) ? BAR_OUT_RDY1 : BAR_OUT_RDY), (su >> 1) & 1)) {
       const DUnit un = deep_unit<SPLIT, WIDE>(c, su);
-      if (!dep_done) { grid_dependency_wait(); dep_done = true; }  // no store before the preceding grids are complete
       if (store_out_tile(maps, c.base + DM_IO + (su & 1) * DM_IO_TILE, un.h, un.row0, un.nrows, out_bf16) > 0) {
         bulk_commit();
         pending_read = true;
@@ -1360,6 +1343,12 @@ __device__ void deep_producer(const Cta& c, const TcMaps& maps, const Geometry& 
       ++su;
       did = true;
     }
+    if (qu < n_my && mbar_test(c.bar(BAR_Q_FREE), (qu - 1) & 1)) {
+      load_q(qu); ++qu; did = true;
+      q0_landed = true;   // (its scores are done; the test below may come too late to see that phase of the barrier)
+    }
+    if (ku < n_my && mbar_test(c.bar(BAR_KV_FREE), (ku - 1) & 1)) { load_k(ku); ++ku; did = true; }
+    if (vu < n_my && mbar_test(c.bar(BAR_KV_FREE1), (vu - 1) & 1)) { load_v(vu); ++vu; did = true; }
     if (!q0_landed && mbar_test(c.bar(BAR_Q_FULL), 0)) q0_landed = true;
     if (!did && iu < n_my && su > iu - 2 && q0_landed) {  // the tile of unit iu - 2 has been handed to its store
       if (pending_read) { bulk_wait_read(); pending_read = false; }
@@ -1385,7 +1374,7 @@ __device__ void deep_producer(const Cta& c, const TcMaps& maps, const Geometry& 
 }
 
 template <bool SPLIT, bool WIDE>
-__device__ void deep_mma(const Cta& c, const Geometry& g, int n_my, bool kv_computed) {
+__device__ void deep_mma(const Cta& c, const Geometry& g, int n_my) {
   using DL = Deep<SPLIT, WIDE>;
   if (n_my == 0) return;
   const int n_s = (g.block_len + 15) & ~15;
@@ -1393,7 +1382,6 @@ __device__ void deep_mma(const Cta& c, const Geometry& g, int n_my, bool kv_comp
   const uint32_t kb = c.base + DL::K;
   if (!wait_bar(c, BAR_Q_FULL, 0, LOC_WAIT_Q)) return;
   if (!wait_bar(c, BAR_KV_FULL, 0, LOC_WAIT_K)) return;
-  if (kv_computed && !wait_bar(c, BAR_QC, 0, LOC_WAIT_K)) return;  // keys and values written by the row threads
   tc_fence_after();
   issue_s_mma<SPLIT>(c.base + SM_Q, BM * 128u, kb, kb + 2 * DL::BOX, DL::BOX, c.tmem + TM_S, idesc_s);
   tc_commit(c.bar(BAR_S_FULL));
@@ -1441,64 +1429,6 @@ __device__ void deep_rows(const Cta& c, const Geometry& g, const AttnArgs& a, in
       m_nx = __ldg(a.st.m + srow);
       l_nx = __ldg(a.st.l + srow);
     }
-  }
-  if (n_my > 0 && a.k_raw != nullptr) {
-    // First unit: the block's keys (rotated, split bf16) and values (fp16) of this head,
-    // computed here with the RoPE kernel's own arithmetic and written where the TMA loads
-    // would have put them ([plane][feature half][row][64], 16-byte chunks XOR-swizzled by
-    // the row), so the unit does not wait for that kernel.
-    const DUnit un = deep_unit<SPLIT, WIDE>(c, 0);
-    const int kh = un.h / g.group;
-    const int tq = threadIdx.x - 64;
-    for (int i = tq; i < L * 8; i += ROW_THREADS) {
-      const int ki = i >> 3, ch = i & 7, c0 = ch * 8;
-      const size_t src = (size_t)un.seq * L + ki;
-      const size_t soff = (src * g.Hkv + kh) * D;
-      float x1[8], x2[8], cs[8], sn[8], y1[8], y2[8];
-      rope_load8(a.k_raw, soff + c0, true, x1);
-      rope_load8(a.k_raw, soff + c0 + D / 2, true, x2);
-      const float4* cp = reinterpret_cast<const float4*>(a.row_cos + src * (D / 2) + c0);
-      const float4* sp = reinterpret_cast<const float4*>(a.row_sin + src * (D / 2) + c0);
-      const float4 ca = cp[0], cb = cp[1], sa = sp[0], sb = sp[1];
-      cs[0] = ca.x; cs[1] = ca.y; cs[2] = ca.z; cs[3] = ca.w; cs[4] = cb.x; cs[5] = cb.y; cs[6] = cb.z; cs[7] = cb.w;
-      sn[0] = sa.x; sn[1] = sa.y; sn[2] = sa.z; sn[3] = sa.w; sn[4] = sb.x; sn[5] = sb.y; sn[6] = sb.z; sn[7] = sb.w;
-      rope_rotate8(x1, x2, cs, sn, y1, y2);
-      uint4 h1, l1, h2, l2;
-      if (!SPLIT && g.op_f16) {
-        h1 = rope_half8(y1);
-        h2 = rope_half8(y2);
-      } else {
-        rope_split8(y1, h1, l1);
-        rope_split8(y2, h2, l2);
-      }
-      uint8_t* const k0 = c.gen + DL::K + ki * 128 + ((ch ^ (ki & 7)) << 4);
-      *reinterpret_cast<uint4*>(k0) = h1;
-      *reinterpret_cast<uint4*>(k0 + DL::BOX) = h2;
-      if (SPLIT) {
-        *reinterpret_cast<uint4*>(k0 + 2 * DL::BOX) = l1;
-        *reinterpret_cast<uint4*>(k0 + 3 * DL::BOX) = l2;
-      }
-      // values: the same two 8-feature chunks of row ki, unrotated
-      float v1[8], v2[8];
-      rope_load8(a.v_raw, soff + c0, true, v1);
-      rope_load8(a.v_raw, soff + c0 + D / 2, true, v2);
-      uint8_t* const v0 = c.gen + DL::V + ki * 128 + ((ch ^ (ki & 7)) << 4);
-      *reinterpret_cast<uint4*>(v0) = rope_half8(v1);
-      *reinterpret_cast<uint4*>(v0 + DL::BOX) = rope_half8(v2);
-    }
-    // rows [L, 32) of the boxes ([L, 64) of wide ones) are never multiplied by a non-zero P~
-    // but must not hold NaN or Inf patterns: clear them
-    for (int i = tq + L * 8; i < (WIDE ? 64 : 32) * 8; i += ROW_THREADS) {
-      const int ki = i >> 3, ch = i & 7;
-      const uint4 z = make_uint4(0u, 0u, 0u, 0u);
-      uint8_t* const k0 = c.gen + DL::K + ki * 128 + ((ch ^ (ki & 7)) << 4);
-      *reinterpret_cast<uint4*>(k0) = z; *reinterpret_cast<uint4*>(k0 + DL::BOX) = z;
-      if (SPLIT) { *reinterpret_cast<uint4*>(k0 + 2 * DL::BOX) = z; *reinterpret_cast<uint4*>(k0 + 3 * DL::BOX) = z; }
-      uint8_t* const v0 = c.gen + DL::V + ki * 128 + ((ch ^ (ki & 7)) << 4);
-      *reinterpret_cast<uint4*>(v0) = z; *reinterpret_cast<uint4*>(v0 + DL::BOX) = z;
-    }
-    fence_async_smem();  // the MMAs read shared memory through the async proxy
-    mbar_arrive(c.bar(BAR_QC));
   }
   for (int uu = 0; uu < n_my; ++uu) {
     const DUnit un = deep_unit<SPLIT, WIDE>(c, uu);
@@ -1694,14 +1624,14 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
     if (stream) {
       if (tid == 0) stream_producer<PACKED, KIND, SPLIT>(c, maps, g, a, first, stride, n_units, it0);
     } else if (deep) {
-      if (tid == 0) deep_producer<SPLIT, WIDE>(c, maps, g, n_my, a.k_raw != nullptr, a.out_bf16 != 0);
+      if (tid == 0) deep_producer<SPLIT, WIDE>(c, maps, g, n_my, a.out_bf16 != 0);
     } else {
       if (tid == 0) merge_producer<SPLIT>(c, maps, g, a, first, stride, n_units, it0);
     }
   } else if (warp == 1) {
     if (tid == 32) {
       if (stream) stream_mma_scores<PACKED, KIND, SPLIT>(c, g, a, first, stride, n_units, it0);
-      else if (deep) deep_mma<SPLIT, WIDE>(c, g, n_my, a.k_raw != nullptr);
+      else if (deep) deep_mma<SPLIT, WIDE>(c, g, n_my);
       else merge_mma<SPLIT>(c, g, a, first, stride, n_units);
     }
   } else if (warp == 10) {
