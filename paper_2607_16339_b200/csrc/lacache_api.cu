@@ -759,6 +759,12 @@ AttnArgs attn_args(lacache_ctx* c, int mode, lacache_ctx::ListRef list, int blk,
         const long long per_cta = n_merge_ctas > 0 ? (units_merge + n_merge_ctas - 1) / n_merge_ctas : 0;
         a.merge_deep = (deep_ok && per_cta <= deep_cap) ? 1 : 0;
         a.split_merge = (deep_ok && per_cta > deep_cap) ? 1 : 0;
+        // A short step lets the kernels behind it be scheduled as SMs fall idle (they wait for it before anything else).
+        // Few tiles per CTA end together; with more, the kernels behind crowd the SMs that are idle first and run there.
+        // Steps of 32 heads with one plane: 17.1 -> 16.2 us at 768 tokens, 23.6 -> 22.8 at 1536; of 28/4 heads 31.0 -> 29.3
+        // at 1280 tokens (per_cta 3 to 5), but 31.1 -> 31.8 for four sequences (7) and 45 -> 49 at 5120 tokens.  Split planes
+        // lose 0.3 us; a step from token ids, behind which the projection's CTAs would wait on SMs, between -0.8 and 2.8.
+        a.step_overlap = (a.merge_deep && !c->split && c->g.block_len <= 32 && per_cta <= 5) ? 1 : 0;
       }
       // Two key chunks per (sequence, head), one round of block-row units, unpacked heads, one-plane operands:
       // the two chunks of a head run as a pair of CTAs that merge through distributed shared memory.
@@ -1241,7 +1247,7 @@ lacache_status step_impl(lacache_ctx* c, const void* q, const void* k, const voi
     c->last_launches++;
   }
   AttnArgs a = attn_args(c, MODE_STEP, c->step_list[blk], blk, c->rot, out, lse);
-  a.step_overlap = overlap ? 1 : 0;
+  a.step_overlap = (overlap || (a.step_overlap && !inputs_just_written)) ? 1 : 0;   // (the planner's rule: steps without a producer ahead)
   if (c->engine == LACACHE_ENGINE_SIMT) {
     a.n_split_items = c->g.B * ((c->g.block_len + SIMT_ROWS - 1) / SIMT_ROWS);
     a.raw_bf16 = c->cfg.dtype == LACACHE_DTYPE_BF16 ? 1 : 0;

@@ -1530,10 +1530,8 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
   const int warp = tid >> 5;
   // In a step with the overlap on, the kernels behind it may be scheduled as SMs free up from here on: they read,
   // before they wait for this grid, only state that stays fixed until the next build and inputs that were
-  // complete long before.  Otherwise this kernel lets its successor start when it ends: the successor's CTAs
-  // would crowd the SMs that fall idle first and run there when this grid is over (said at a CTA's last loads,
-  // 48.9 us against 47.0 for a step at N = 5120 and 1376 against 1346 for a walk of five blocks there; at
-  // N = 768 it would save 0.6 of 20.4 us).
+  // complete long before.  So they may in a short step without it, where they wait first (the planner's rule).  Otherwise
+  // this kernel lets its successor start when it ends.
   if (a.step_overlap) grid_launch_dependents();
   if (a.span != nullptr && tid == 0) atomicMin(a.span, global_timer_ns());   // first CTA entry of this launch
   Cta c;
