@@ -82,11 +82,15 @@ struct Tile {
 // Q region: in all of it for 128-row units (the next unit's Q load waits for the
 // epilogue), in its upper half for 64-row units (whose Q tile needs only the lower half).
 constexpr uint32_t STAGE_ROW = 512;
-// paired step, one-plane operands: where the partner CTA puts its partial state -- O~ of up to 32 rows in the
-// staging layout (512 bytes a row, 16-byte chunks XOR-swizzled by the row), then (m, l) per row
-constexpr uint32_t SM_RX = Tile<false>::SM_V + 2 * Tile<false>::V_STAGE;
-constexpr uint32_t SM_RX_ML = SM_RX + 32 * STAGE_ROW;
-static_assert(SM_RX_ML + 32 * 8 <= SM_XCH, "no room for the partner's partial state");
+// paired step: where the partner CTA puts its partial state -- O~ of up to 32 rows in the staging layout (512 bytes a row,
+// 16-byte chunks XOR-swizzled by the row) behind the value stages, (m, l) per row in the upper half of the Q region
+// behind the 32 rows staged there (with split planes the value stages leave the O~ rows and no more)
+template <bool SPLIT>
+struct Rx {
+  static constexpr uint32_t O = Tile<SPLIT>::SM_V + 2 * Tile<SPLIT>::V_STAGE;
+  static constexpr uint32_t ML = SM_Q + 32768 + 32 * STAGE_ROW;
+  static_assert(O + 32 * STAGE_ROW <= SM_XCH && ML + 32 * 8 <= SM_K, "no room for the partner's partial state");
+};
 // merge role: the 96 KB after Q hold 2 stages of the block's keys {K hi, K lo, V} of 64
 // rows, then the staging tile of the cached O~ / the output
 constexpr uint32_t SM_KV = SM_K;
@@ -812,7 +816,7 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
     float mul = (un.epi == EPI_OUT) ? 1.f / l_run : 1.f;
     float mul_rx = 0.f, lse2 = 0.f;   // paired step: weight of the partner's O~, merged log2 normaliser
     if (KIND == KIND_STEP2) {
-      const uint32_t rx_row = SM_RX + (uint32_t)r * STAGE_ROW;
+      const uint32_t rx_row = Rx<SPLIT>::O + (uint32_t)r * STAGE_ROW;
       if (un.epi == EPI_SEND) {
         // Second key chunk of its (sequence, head): O~ of the block's rows from TMEM into the partner CTA's
         // receiving buffer (the layout of a staging tile), m and l behind it, then one arrival per thread on
@@ -838,7 +842,7 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
             }
           }
         }
-        if (row_valid && half == 0) st_cluster_v2(mapa_shared(c.base + SM_RX_ML + (uint32_t)r * 8u, peer), m_ref, l_run);
+        if (row_valid && half == 0) st_cluster_v2(mapa_shared(c.base + Rx<SPLIT>::ML + (uint32_t)r * 8u, peer), m_ref, l_run);
         mbar_arrive_cluster(mapa_shared(c.bar(BAR_RX), peer));
         tc_fence_before();
         mbar_arrive(c.bar(BAR_O_FREE));  // (a paired step has one unit per CTA; kept for the barrier's phase count)
@@ -862,7 +866,7 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
       }
       float m2 = -INFINITY, l2 = 0.f;
       if (row_valid) {
-        const float2 ml = *reinterpret_cast<const float2*>(c.gen + SM_RX_ML + r * 8);
+        const float2 ml = *reinterpret_cast<const float2*>(c.gen + Rx<SPLIT>::ML + r * 8);
         m2 = ml.x; l2 = ml.y;
       }
       const float M = fmaxf(m_ref, m2);
@@ -942,7 +946,7 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
     // P~V, waited for above, was issued after them); 64-row units use its upper
     // half, which their Q tiles never touch.
     const uint32_t stage_off = SM_Q + (un.q_rows == BM ? 0u : 32768u);
-    const bool own_stage = un.q_rows == BM || r < 64;
+    const bool own_stage = un.q_rows == BM || r < (KIND == KIND_STEP2 ? 32 : 64);   // (paired: up to 32 rows, see Rx)
     uint8_t* const srow = c.gen + stage_off + r * STAGE_ROW;
 #pragma unroll 1
     for (int cb = 0; cb < 4; ++cb) {
@@ -961,7 +965,7 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
           float4 v = make_float4(__uint_as_float(rr[4 * i]) * mul, __uint_as_float(rr[4 * i + 1]) * mul,
                                  __uint_as_float(rr[4 * i + 2]) * mul, __uint_as_float(rr[4 * i + 3]) * mul);
           if (KIND == KIND_STEP2 && row_valid) {   // + the partner chunk's O~, weighted
-            const float4 p = *reinterpret_cast<const float4*>(c.gen + SM_RX + r * STAGE_ROW + ((ch ^ (r & 7)) << 4));
+            const float4 p = *reinterpret_cast<const float4*>(c.gen + Rx<SPLIT>::O + r * STAGE_ROW + ((ch ^ (r & 7)) << 4));
             v.x = fmaf(p.x, mul_rx, v.x); v.y = fmaf(p.y, mul_rx, v.y);
             v.z = fmaf(p.z, mul_rx, v.z); v.w = fmaf(p.w, mul_rx, v.w);
           }
@@ -1749,14 +1753,13 @@ bool make_v_map(CUtensorMap* m, void* base, int H, int Tp, int box_rows, char* e
 
 namespace {
 // The step of an MHA and of a GQA model, each for blocks of more than 32 rows (the pipelined merge role for wide blocks, with
-// split planes the one with a single staging tile) and of up to 32; the paired step, which exists for one-plane operands
-// only.
+// split planes the one with a single staging tile) and of up to 32; the paired step.
 template <bool SPLIT>
 const void* const* kernel_table() {
   static const void* const t[5] = {
       (const void*)tc_attn_kernel<false, KIND_STEP, SPLIT ? 0 : 2, SPLIT>, (const void*)tc_attn_kernel<false, KIND_STEP, 1, SPLIT>,
       (const void*)tc_attn_kernel<true, KIND_STEP, SPLIT ? 0 : 2, SPLIT>,  (const void*)tc_attn_kernel<true, KIND_STEP, 1, SPLIT>,
-      SPLIT ? nullptr : (const void*)tc_attn_kernel<false, KIND_STEP2, 1, false>};
+      (const void*)tc_attn_kernel<false, KIND_STEP2, 1, SPLIT>};
   return t;
 }
 }  // namespace
@@ -1765,7 +1768,6 @@ cudaError_t tc_prepare() {
   for (int split = 0; split < 2; ++split) {
     const void* const* t = split ? kernel_table<true>() : kernel_table<false>();
     for (int i = 0; i < 5; ++i) {
-      if (!t[i]) continue;
       cudaError_t e = cudaFuncSetAttribute(t[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
       if (e != cudaSuccess) return e;
     }
@@ -1828,7 +1830,7 @@ cudaError_t tc_attention(const Geometry& g, const AttnArgs& a, const TcMaps* map
     attr[n_attr].val.programmaticStreamSerializationAllowed = 1;
     ++n_attr;
   }
-  const bool paired = a.pair_chunks && !a.split;
+  const bool paired = a.pair_chunks != 0;
   if (paired) {   // CTAs 2k and 2k + 1 form a cluster: the two key chunks of one (sequence, head)
     attr[n_attr].id = cudaLaunchAttributeClusterDimension;
     attr[n_attr].val.clusterDim.x = 2;

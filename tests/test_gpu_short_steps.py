@@ -7,7 +7,8 @@ import torch
 from paper_2607_16339_b200 import binding
 from paper_2607_16339_b200.workloads import SyntheticSchedule, small_workload
 
-from lacache_testlib import make_ctx, new_outputs, to_dev
+from lacache_testlib import advance_to_block, make_ctx, new_outputs, to_dev
+from test_gpu_parity import _run_points
 
 pytestmark = pytest.mark.gpu
 MODES = {"plain": binding.PRECISION_PLAIN, "fp16": binding.PRECISION_FP16}
@@ -54,3 +55,29 @@ def test_steps_and_builds_in_stream_order(prompts, block, hq, hkv, mode):
         for i, ((o0, l0), (o1, l1)) in enumerate(zip(ref, run(False))):
             assert torch.equal(o0, o1) and torch.equal(l0, l1), "call %d" % i
     ctx.destroy()
+
+
+@pytest.mark.parametrize("block", [16, 32])
+def test_two_key_chunks_as_a_pair_of_ctas_with_split_planes(block, monkeypatch):
+    """The paired step with split planes, whose operand tiles leave the partner's state just room enough: against the
+    oracle, and against the same step with the pairing switched off."""
+    wl = small_workload(name="pair-split-%d" % block, prompt_lens=(100, 131, 90), gen_len=2 * block, block_len=block,
+                        steps=2, hq=4, hkv=4)
+    monkeypatch.setenv("LACACHE_STREAM_CTAS", str(wl.batch * 2 * wl.n_q_heads))   # (read when a context is created)
+    outs = []
+    for pair in (True, False):
+        if not pair:
+            monkeypatch.setenv("LACACHE_NO_PAIR", "1")
+        _run_points(wl, "tc", seed=12, sc_tiles_per_chunk=1)
+        sch = SyntheticSchedule(wl, seed=12)
+        ctx = make_ctx(wl, sc_tiles_per_chunk=1)
+        q, k, v = (to_dev(a, wl) for a in advance_to_block(sch, 1))
+        ctx.build(1, q, k, v)
+        out, lse = new_outputs(wl)
+        ctx.step(*(to_dev(a, wl) for a in sch.draw_step(1, 1)), out, lse)
+        torch.cuda.synchronize()
+        assert ctx.poll_status()[0] == 0
+        outs.append((out.clone(), lse.clone()))
+        ctx.destroy()
+    assert (outs[0][0] - outs[1][0]).abs().max().item() <= 1e-5
+    assert (outs[0][1] - outs[1][1]).abs().max().item() <= 1e-5
