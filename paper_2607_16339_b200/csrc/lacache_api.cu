@@ -768,7 +768,7 @@ AttnArgs attn_args(lacache_ctx* c, int mode, lacache_ctx::ListRef list, int blk,
       }
       // Two key chunks per (sequence, head), one round of block-row units, unpacked heads:
       // the two chunks of a head run as a pair of CTAs that merge through distributed shared memory.
-      if (a.pack == 1 && a.merge_deep && !a.split_merge && !c->knobs.no_pair && c->g.block_len <= 32 &&
+      if (a.pack == 1 && (a.merge_deep || a.split_merge) && !c->knobs.no_pair && c->g.block_len <= 32 &&
           units_stream == ns && (ns % 2) == 0 && (a.n_ctas % 2) == 0) {
         if (plan.pair < 0) {
           plan.pair = 1;
@@ -809,10 +809,11 @@ lacache_status run_attention(lacache_ctx* c, const AttnArgs& a, bool scratch, cu
     const int deep_cap = deep_unit_cap(c);
     AttnArgs b = a;
     b.merge_deep = 1;
-    const int m0 = a.n_ctas - a.n_ctas_stream;
+    const int m0 = a.pair_chunks ? (a.n_ctas - a.n_ctas_stream) & ~1 : a.n_ctas - a.n_ctas_stream;   // (pairs: an even grid)
     int done = std::min(a.n_items_merge, std::max(1, deep_cap * m0 / Hq));
     b.n_items_merge = done;
     b.n_ctas = a.n_ctas_stream + (int)std::min<long long>((long long)done * Hq, m0);
+    if (a.pair_chunks) b.n_ctas += b.n_ctas & 1;
     CU_TRY(c, launch_tc(c, b, maps, s));
     c->last_launches++;
     const int rest = a.n_items_merge - done;
@@ -823,6 +824,7 @@ lacache_status run_attention(lacache_ctx* c, const AttnArgs& a, bool scratch, cu
       while (done < a.n_items_merge) {
         AttnArgs m = a;
         m.merge_deep = 1;
+        m.pair_chunks = 0;
         m.n_items = 0;
         m.n_ctas_stream = 0;
         m.items_merge = a.items_merge + done;
