@@ -86,6 +86,43 @@ def test_many_rows_of_an_unaligned_vocabulary(rows, vocab):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("vocab", [7, 1000, 4099, 126464])
+def test_entries_masked_with_the_lowest_value_of_the_type(dtype, vocab):
+    """torch.finfo(dtype).min as a mask (finite, but its product with log2 e is not): whole batches of a lane, whole
+    segments and whole rows of it, before and behind the other entries; and the largest value as a logit."""
+    wl = small_workload(name="samp-min", prompt_lens=(21,), gen_len=32, block_len=16, steps=1, hq=2, hkv=2)
+    ctx, sch = _built_ctx(wl, 0)
+    g = torch.Generator(device="cuda").manual_seed(vocab)
+    logits = (torch.randn(wl.total_tokens, vocab, generator=g, device="cuda") * 4).to(dtype)
+    at, info = sch.block_rows(0), torch.finfo(dtype)
+    logits[at[0], : vocab // 2] = info.min
+    logits[at[1], vocab // 2:] = info.min
+    logits[at[2], ::2] = info.min
+    logits[at[3], : vocab - 1] = info.min          # one entry left, at the end
+    logits[at[4], 1:] = info.min                   # ... at the start
+    logits[at[5]] = info.min                       # none: uniform
+    logits[at[6]] = info.min
+    logits[at[6], ::3] = float("-inf")
+    logits[at[7], vocab // 3] = info.max
+    logits[at[8], vocab // 2:] = info.max
+    logits[at[9], 0] = info.max * 0.7              # two that differ, both beyond 2^127
+    logits[at[9], vocab - 1] = info.max * 0.8
+    logits[at[10], ::2] = info.min * 0.7
+    n = at.shape[0]
+    conf, lse = torch.empty(n, device="cuda"), torch.empty(n, device="cuda")
+    tok = torch.empty(n, device="cuda", dtype=torch.int32)
+    ctx.sample_block(logits, conf, tok, lse)
+    torch.cuda.synchronize()
+    assert ctx.poll_status()[0] == 0
+    ref_tok, ref_conf, ref_lse = sampler.block_confidence(logits.float().cpu().numpy().astype(np.float64), at)
+    assert np.array_equal(tok.cpu().numpy().astype(np.int64), ref_tok)
+    c, l = conf.cpu().numpy().astype(np.float64), lse.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(c - ref_conf) <= 2e-5 * ref_conf), (c, ref_conf)
+    assert np.all(np.abs(l - ref_lse) <= 2e-5 * np.maximum(1.0, np.abs(ref_lse))), (l, ref_lse)
+    ctx.destroy()
+
+
 def test_full_size_block_and_vocabulary():
     """The headline configuration's block (32 rows) and the large-batch extension's (8192 rows) at a
     vocabulary of 126464 entries (bf16 logits of every token would not fit for the latter: its logits
