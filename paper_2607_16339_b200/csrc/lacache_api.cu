@@ -580,9 +580,12 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
   c->items_host = items;
 
   // ---- device memory ----
-  CU_TRY(c, simt_prepare());
-  if (tc) CU_TRY(c, tc_prepare());
-  if (rk) CU_TRY(c, rows_prepare());
+  if (tc) {
+    CU_TRY(c, tc_prepare(c->split));
+    CU_TRY(c, rows_prepare(c->split));
+  } else {
+    CU_TRY(c, simt_prepare());
+  }
 
   CU_TRY(c, dev_alloc(c, &c->d_cu, g.B + 1));
   CU_TRY(c, cudaMemcpy(c->d_cu, c->cu.data(), sizeof(int32_t) * (g.B + 1), cudaMemcpyHostToDevice));

@@ -183,14 +183,14 @@ cudaError_t rope_write(const Geometry& g, const RopeArgs& a, int engine, cudaStr
 cudaError_t export_buffers(const Geometry& g, const ExportArgs& a, int engine, cudaStream_t s);
 
 cudaError_t simt_attention(const Geometry& g, const AttnArgs& a, int num_sms, cudaStream_t s);
-cudaError_t simt_prepare();  // function attributes
+cudaError_t simt_prepare();  // function attributes (the *_prepare functions: of the kernels a context of that kind may launch)
 
 struct TcMaps;  // opaque set of TMA descriptors, defined in lacache_tc.cu
 cudaError_t tc_attention(const Geometry& g, const AttnArgs& a, const TcMaps* maps, cudaStream_t s);
-cudaError_t tc_prepare();
+cudaError_t tc_prepare(bool split);
 // row tiles over long key ranges (build, full recompute, key windows) with one-plane operands: lacache_rows.cu
 cudaError_t row_attention(const Geometry& g, const AttnArgs& a, const TcMaps* maps, cudaStream_t s);
-cudaError_t rows_prepare();
+cudaError_t rows_prepare(bool split);
 // builds TMA descriptors for a rotated buffer set; returns nullptr and fills
 // err on failure
 TcMaps* tc_make_maps(const Geometry& g, const RotBuffers& rot, float* state_o, bool split, char* err, int errlen);

@@ -680,9 +680,9 @@ const void* row_kernel(bool split, bool window) {
 
 }  // namespace
 
-cudaError_t rows_prepare() {
-  for (int i = 0; i < 4; ++i) {
-    cudaError_t e = cudaFuncSetAttribute(row_kernel(i & 1, i & 2), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
+cudaError_t rows_prepare(bool split) {
+  for (int i = 0; i < 2; ++i) {
+    cudaError_t e = cudaFuncSetAttribute(row_kernel(split, i != 0), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
