@@ -12,8 +12,10 @@
 #include <vector>
 
 #include "lacache_internal.h"
+#include "lacache_plan.h"
 
 using namespace lacache;
+using namespace lacache::plan;
 
 struct lacache_ctx {
   lacache_config cfg;
@@ -143,23 +145,6 @@ cudaError_t dev_alloc(lacache_ctx* c, T** p, size_t n_elems, bool zero = false) 
   return cudaSuccess;
 }
 
-// Tiles of `rows_per_item` query rows over [lo, hi) of one sequence.
-void add_row_tiles(std::vector<WorkItem>& v, int seq, int lo, int hi, int rows_per_item, int seq_start,
-                   int seq_end, int blk_start, int kind = ITEM_ROWS) {
-  for (int r = lo; r < hi; r += rows_per_item) {
-    WorkItem w{};
-    w.kind = kind;
-    w.seq = seq;
-    w.row0 = r;
-    w.nrows = std::min(rows_per_item, hi - r);
-    w.pad = 1;
-    w.seq_start = seq_start;
-    w.seq_end = seq_end;
-    w.blk_start = blk_start;
-    v.push_back(w);
-  }
-}
-
 lacache_status alloc_rot(lacache_ctx* c, RotBuffers* r) {
   const Geometry& g = c->g;
   size_t nq = (size_t)g.Hq * g.Tp * g.d, nk = (size_t)g.Hkv * g.Tp * g.d;
@@ -277,9 +262,8 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
   c->g.op_f16 = (c->engine == LACACHE_ENGINE_TCGEN05 && cfg->precision_mode == LACACHE_PRECISION_FP16) ? 1 : 0;
   const int TC_KEYS = tc_keys(c->split);
   const int R = tc ? TC_ROWS : SIMT_ROWS;
-  // builds and full recomputes with one-plane operands run the row kernel: items of two row tiles, 128-key tiles
-  const bool rk = tc;
-  const int RI = rk ? TC_ROW_ITEM : R, RI_KEYS = rk ? TC_ROW_KEYS : TC_KEYS;
+  // builds, full recomputes and key windows run the row kernel: items of two row tiles, 128-key tiles
+  const int RI = tc ? TC_ROW_ITEM : R, RI_KEYS = tc ? TC_ROW_KEYS : TC_KEYS;
   std::vector<WorkItem> items;
   // Block-query units: the keys of each (sequence, head) are cut into balanced
   // chunks of `tpc` tiles.  Unless the caller fixes it, pick the chunk size and
@@ -329,52 +313,8 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
     }
   }
   if (tpc <= 0) tpc = 2;
-  // The row kernel's items, the most work first: its CTAs draw them in a snake (0 .. n - 1, n - 1 .. 0, ...).  `keys`: of
-  // a key-window item from the token its tiles are counted from.
-  auto row_cost = [](int nrows, int keys) {   // in key tiles of two row tiles (one row tile alone takes 0.62 of two)
-    return (nrows > TC_ROWS ? 1.0 : 0.62) * ((keys + TC_ROW_KEYS - 1) / TC_ROW_KEYS) + 1.5;
-  };
-  auto item_keys = [](const WorkItem& w) { return w.kind == ITEM_ROWS_WINDOW ? std::max(0, w.kt1 - w.pad) : w.seq_end - w.seq_start; };
   auto longest_first = [&](int from) {
-    if (!rk) return;
-    std::stable_sort(items.begin() + from, items.end(), [&](const WorkItem& p, const WorkItem& q) {
-      return row_cost(p.nrows, item_keys(p)) > row_cost(q.nrows, item_keys(q));
-    });
-  };
-  // Few units leave the last round of CTAs half empty: some of the items with the least work then go out as two of one row
-  // tile each (at most 8 items, the number that makes the longest CTA shortest).
-  auto split_items = [&](int from) {
-    const int n = (int)items.size() - from, P = c->num_sms;
-    if (!rk || (long long)n * g.Hq > 8ll * P) return;
-    std::vector<WorkItem> best(items.begin() + from, items.end());
-    double best_t = 1e30;
-    for (int sp = 0; sp <= std::min(8, n); ++sp) {
-      std::vector<WorkItem> v;
-      int left = sp;
-      for (int i = n - 1; i >= 0; --i) {
-        WorkItem w = items[from + i];
-        if (left > 0 && w.nrows > TC_ROWS) {
-          --left;
-          WorkItem x = w;
-          x.row0 += TC_ROWS; x.nrows -= TC_ROWS; w.nrows = TC_ROWS;
-          v.push_back(x);
-        }
-        v.push_back(w);
-      }
-      if (left > 0) break;
-      std::stable_sort(v.begin(), v.end(), [&](const WorkItem& p, const WorkItem& q) { return row_cost(p.nrows, item_keys(p)) > row_cost(q.nrows, item_keys(q)); });
-      std::vector<double> t(P, 0.0);
-      double most = 0.0;
-      for (int u = 0; u < (int)v.size() * g.Hq; ++u) {
-        const int k = u / P, b = u % P;
-        double& cta = t[(k & 1) ? P - 1 - b : b];
-        cta += row_cost(v[u / g.Hq].nrows, item_keys(v[u / g.Hq]));
-        most = std::max(most, cta);
-      }
-      if (most < best_t - 1e-9) { best_t = most; best = v; }
-    }
-    items.resize(from);
-    items.insert(items.end(), best.begin(), best.end());
+    if (tc) sort_longest_first(items, from);
   };
   c->max_chunks = 1;
   for (int k = 0; k < g.n_blk; ++k) {
@@ -413,21 +353,12 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
     } else {
       c->step_list.push_back({off, (int)items.size() - off});
       c->merge_list.push_back({0, 0});
-    }
-    if (!rk) {
       c->build_list.push_back({rows_off, (int)items.size() - rows_off});
-      continue;
     }
-    // the build's row tiles run straight through the block (its rows get a state too, which nothing reads: a
-    // tile more per sequence would cost more); a sequence without fixed rows has none
-    off = (int)items.size();
-    for (int b = 0; b < g.B; ++b)
-      if (c->cu[b + 1] - c->cu[b] > g.block_len)
-        add_row_tiles(items, b, c->cu[b], c->cu[b + 1], TC_ROW_ITEM, c->cu[b], c->cu[b + 1], c->blk_start_all[(size_t)k * g.B + b]);
-    longest_first(off);
-    split_items(off);
-    c->build_list.push_back({off, (int)items.size() - off});
   }
+  if (tc)
+    for (const Range& r : add_build_lists(items, c->cu.data(), g.B, g.block_len, c->blk_start_all.data(), g.n_blk, g.Hq, c->num_sms))
+      c->build_list.push_back({r.off, r.n});
   int inc_chunks = 1;
   c->adv_tab.assign((size_t)g.n_blk * g.B * 2, 0);
   for (int k = 0; k < g.n_blk && tc; ++k) {
@@ -574,7 +505,7 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
     int off = (int)items.size();
     for (int b = 0; b < g.B; ++b) add_row_tiles(items, b, c->cu[b], c->cu[b + 1], RI, c->cu[b], c->cu[b + 1], 0);
     longest_first(off);
-    split_items(off);
+    if (tc) split_items(items, off, g.Hq, c->num_sms);
     c->full_list = {off, (int)items.size() - off};
   }
   c->items_host = items;

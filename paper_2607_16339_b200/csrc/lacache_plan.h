@@ -1,0 +1,100 @@
+// Work lists of the row kernel (lacache_rows.cu), planned on the host when a context is created.  Host code only.
+#pragma once
+#include <algorithm>
+#include <vector>
+
+#include "lacache_internal.h"
+
+namespace lacache {
+namespace plan {
+
+// Tiles of `rows_per_item` query rows over [lo, hi) of one sequence.
+inline void add_row_tiles(std::vector<WorkItem>& v, int seq, int lo, int hi, int rows_per_item, int seq_start,
+                          int seq_end, int blk_start, int kind = ITEM_ROWS) {
+  for (int r = lo; r < hi; r += rows_per_item) {
+    WorkItem w{};
+    w.kind = kind;
+    w.seq = seq;
+    w.row0 = r;
+    w.nrows = std::min(rows_per_item, hi - r);
+    w.pad = 1;
+    w.seq_start = seq_start;
+    w.seq_end = seq_end;
+    w.blk_start = blk_start;
+    v.push_back(w);
+  }
+}
+
+// An item's work in key tiles of two row tiles (one row tile alone takes 0.62 of two).
+inline double row_cost(const WorkItem& w) {
+  // (of a key-window item: from the token its tiles are counted from)
+  const int keys = w.kind == ITEM_ROWS_WINDOW ? std::max(0, w.kt1 - w.pad) : w.seq_end - w.seq_start;
+  return (w.nrows > TC_ROWS ? 1.0 : 0.62) * ((keys + TC_ROW_KEYS - 1) / TC_ROW_KEYS) + 1.5;
+}
+// The items from `from` on, the most work first: the row kernel's CTAs draw them in a snake (0 .. n - 1, n - 1 .. 0, ...).
+inline void sort_longest_first(std::vector<WorkItem>& items, size_t from) {
+  std::stable_sort(items.begin() + from, items.end(), [](const WorkItem& p, const WorkItem& q) { return row_cost(p) > row_cost(q); });
+}
+
+// Few units leave the last round of CTAs half empty: some of the items with the least work (of those from `from` on, sorted)
+// then go out as two of one row tile each -- at most 8 items, the number that makes the longest CTA shortest.
+inline void split_items(std::vector<WorkItem>& items, size_t from, int heads, int num_sms) {
+  const int n = (int)(items.size() - from), P = num_sms;
+  if ((long long)n * heads > 8ll * P) return;
+  std::vector<WorkItem> best(items.begin() + from, items.end());
+  double best_t = 1e30;
+  for (int sp = 0; sp <= std::min(8, n); ++sp) {
+    std::vector<WorkItem> v;
+    int left = sp;
+    for (int i = n - 1; i >= 0; --i) {
+      WorkItem w = items[from + i];
+      if (left > 0 && w.nrows > TC_ROWS) {
+        --left;
+        WorkItem x = w;
+        x.row0 += TC_ROWS; x.nrows -= TC_ROWS; w.nrows = TC_ROWS;
+        v.push_back(x);
+      }
+      v.push_back(w);
+    }
+    if (left > 0) break;
+    sort_longest_first(v, 0);
+    std::vector<double> t(P, 0.0);
+    double most = 0.0;
+    for (int u = 0; u < (int)v.size() * heads; ++u) {
+      const int k = u / P, b = u % P;
+      double& cta = t[(k & 1) ? P - 1 - b : b];
+      cta += row_cost(v[u / heads]);
+      most = std::max(most, cta);
+    }
+    if (most < best_t - 1e-9) { best_t = most; best = v; }
+  }
+  items.resize(from);
+  items.insert(items.end(), best.begin(), best.end());
+}
+
+struct Range { int off, n; };   // a list within `items`
+
+// The build lists of every block of a generation, appended to `items`.  blk_start: [n_blk][B].  A build's row tiles run
+// straight through the block (its rows get a state too, which nothing reads: a tile more per sequence would cost more); a
+// sequence without fixed rows has none.  So a list depends on the block in its items' blk_start alone: it is planned once
+// (28 heads, 8192 tokens, 64 blocks: 3.1 ms of host time with each block planned by itself, 0.06 now).
+inline std::vector<Range> add_build_lists(std::vector<WorkItem>& items, const int32_t* cu, int B, int block_len,
+                                          const int32_t* blk_start, int n_blk, int heads, int num_sms) {
+  std::vector<WorkItem> list;
+  for (int b = 0; b < B; ++b)
+    if (cu[b + 1] - cu[b] > block_len) add_row_tiles(list, b, cu[b], cu[b + 1], TC_ROW_ITEM, cu[b], cu[b + 1], 0);
+  sort_longest_first(list, 0);
+  split_items(list, 0, heads, num_sms);
+  std::vector<Range> ranges;
+  for (int k = 0; k < n_blk; ++k) {
+    ranges.push_back({(int)items.size(), (int)list.size()});
+    for (WorkItem w : list) {
+      w.blk_start = blk_start[(size_t)k * B + w.seq];
+      items.push_back(w);
+    }
+  }
+  return ranges;
+}
+
+}  // namespace plan
+}  // namespace lacache

@@ -1,0 +1,98 @@
+"""The build's work lists (csrc/lacache_plan.h), planned on the host: every row once, the most work first, each block's list
+what planning that block alone gives -- and planned once per context, not once per block."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2607_16339_b200", "csrc")
+
+HARNESS = r"""
+#include <chrono>
+#include <cstdio>
+#include <cstdlib>
+#include "lacache_plan.h"
+using namespace lacache;
+using namespace lacache::plan;
+// argv: mode heads sms block n_blk prompt...
+int main(int argc, char** argv) {
+  const int mode = atoi(argv[1]), heads = atoi(argv[2]), sms = atoi(argv[3]), L = atoi(argv[4]), n_blk = atoi(argv[5]);
+  const int B = argc - 6;
+  std::vector<int32_t> cu(B + 1, 0), start((size_t)n_blk * B);
+  for (int b = 0; b < B; ++b) cu[b + 1] = cu[b] + atoi(argv[6 + b]) + n_blk * L;
+  for (int k = 0; k < n_blk; ++k)
+    for (int b = 0; b < B; ++b) start[(size_t)k * B + b] = cu[b] + atoi(argv[6 + b]) + k * L;
+  std::vector<WorkItem> items;
+  auto lists = [&](int k0, int n) { return add_build_lists(items, cu.data(), B, L, start.data() + (size_t)k0 * B, n, heads, sms); };
+  if (mode == 2) {   // the best of ten timings of all blocks' lists, and of one block's
+    double best[2] = {1e9, 1e9};
+    for (int r = 0; r < 10; ++r)
+      for (int one = 0; one < 2; ++one) {
+        items.clear();
+        const auto t0 = std::chrono::steady_clock::now();
+        lists(0, one ? 1 : n_blk);
+        best[one] = std::min(best[one], std::chrono::duration<double, std::micro>(std::chrono::steady_clock::now() - t0).count());
+      }
+    printf("%f %f\n", best[0], best[1]);
+    return 0;
+  }
+  std::vector<Range> ranges;
+  if (mode == 0) ranges = lists(0, n_blk);
+  else for (int k = 0; k < n_blk; ++k) ranges.push_back(lists(k, 1)[0]);
+  for (int k = 0; k < n_blk; ++k)
+    for (int i = ranges[k].off; i < ranges[k].off + ranges[k].n; ++i) {
+      const WorkItem& w = items[i];
+      printf("%d %d %d %d %d %d %d %d\n", k, w.kind, w.seq, w.row0, w.nrows, w.seq_start, w.seq_end, w.blk_start);
+    }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def harness(tmp_path_factory):
+    d = tmp_path_factory.mktemp("plan")
+    src, exe = str(d / "plan.cpp"), str(d / "plan")
+    open(src, "w").write(HARNESS)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I", CSRC, "-I", "/usr/local/cuda/include", src, "-o", exe], check=True)
+
+    def run(mode, heads, sms, block, n_blk, prompts):
+        args = [exe, str(mode), str(heads), str(sms), str(block), str(n_blk)] + [str(p) for p in prompts]
+        return subprocess.run(args, check=True, capture_output=True, text=True).stdout
+    return run
+
+
+@pytest.mark.parametrize("heads,sms,block,n_blk,prompts", [
+    (28, 148, 64, 16, (4096,)),
+    (32, 148, 32, 8, (500, 256, 798, 584, 526, 932, 396, 371)),
+    (32, 148, 32, 8, (512,)),
+    (4, 3, 16, 2, (95, 96, 97)),
+    (4, 148, 32, 1, (0, 33)),            # a sequence without fixed rows
+    (28, 148, 32, 4, (1000,) * 40),      # too many units for the search
+])
+def test_lists(harness, heads, sms, block, n_blk, prompts):
+    text = harness(0, heads, sms, block, n_blk, prompts)
+    assert text == harness(1, heads, sms, block, n_blk, prompts)
+    rows = [tuple(int(x) for x in line.split()) for line in text.splitlines()]
+    cu = [0]
+    for p in prompts:
+        cu.append(cu[-1] + p + n_blk * block)
+    for k in range(n_blk):
+        mine = [r for r in rows if r[0] == k]
+        seen = []
+        cost = []
+        for _, kind, seq, row0, nrows, lo, hi, blk in mine:
+            assert kind == 0 and 1 <= nrows <= 256 and (lo, hi) == (cu[seq], cu[seq + 1])
+            assert blk == cu[seq] + prompts[seq] + k * block
+            seen += range(row0, row0 + nrows)
+            cost.append((1.0 if nrows > 128 else 0.62) * ((hi - lo + 127) // 128) + 1.5)
+        want = [t for b in range(len(prompts)) if cu[b + 1] - cu[b] > block for t in range(cu[b], cu[b + 1])]
+        assert sorted(seen) == want
+        assert cost == sorted(cost, reverse=True)
+
+
+def test_planned_once_per_context(harness):
+    """64 blocks must not cost 64 plans: what is done per block is the copy of a list (8 times one plan is several times
+    what that takes; a plan per block takes 64)."""
+    every, one = (float(x) for x in harness(2, 28, 148, 64, 64, (4096,)).split())
+    assert every < 8 * one, (every, one)
