@@ -636,6 +636,7 @@ AttnArgs attn_args(lacache_ctx* c, int mode, lacache_ctx::ListRef list, int blk,
   a.status = c->d_status;
   a.no_pdl = c->knobs.no_pdl ? 1 : 0;
   a.split = c->split ? 1 : 0;
+  a.step_overlap = (c->engine == LACACHE_ENGINE_SIMT && !c->knobs.no_pdl && !c->knobs.no_step_overlap) ? 1 : 0;
   if (c->engine == LACACHE_ENGINE_TCGEN05) {
     // persistent grid: one CTA per SM, split between the two roles by a cost
     // estimate (units x per-unit cost, in arbitrary time units)
@@ -1183,8 +1184,9 @@ lacache_status step_impl(lacache_ctx* c, const void* q, const void* k, const voi
     c->last_launches++;
   }
   AttnArgs a = attn_args(c, MODE_STEP, c->step_list[blk], blk, c->rot, out, lse);
-  a.step_overlap = (overlap || (a.step_overlap && !inputs_just_written)) ? 1 : 0;   // (the planner's rule: steps without a producer ahead)
-  if (c->engine == LACACHE_ENGINE_SIMT) {
+  if (c->engine == LACACHE_ENGINE_TCGEN05) {
+    a.step_overlap = early_trigger(c->step_overlap != 0, a.step_overlap != 0, inputs_just_written, c->knobs.no_pdl || c->knobs.no_step_overlap) ? 1 : 0;
+  } else {
     a.n_split_items = c->g.B * ((c->g.block_len + SIMT_ROWS - 1) / SIMT_ROWS);
     a.raw_bf16 = c->cfg.dtype == LACACHE_DTYPE_BF16 ? 1 : 0;
   }

@@ -1,4 +1,5 @@
-// Work lists of the row kernel (lacache_rows.cu), planned on the host when a context is created.  Host code only.
+// Host-side planning without state: the work lists of the row kernel (lacache_rows.cu), made when a context is created, and
+// the rule of the early trigger.  Host code only.
 #pragma once
 #include <algorithm>
 #include <vector>
@@ -70,6 +71,13 @@ inline void split_items(std::vector<WorkItem>& items, size_t from, int heads, in
   }
   items.resize(from);
   items.insert(items.end(), best.begin(), best.end());
+}
+
+// Whether a step's attention kernel lets the kernels behind it be scheduled while it drains: always with the overlap of
+// consecutive steps on; else in a short step (see the caller) that no producer runs ahead of.  `off`: the knobs that ask
+// for kernels that start when the one before has ended.
+inline bool early_trigger(bool overlap_on, bool short_step, bool producer_ahead, bool off) {
+  return !off && (overlap_on || (short_step && !producer_ahead));
 }
 
 struct Range { int off, n; };   // a list within `items`

@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(THREADS, 3) simt_attn_kernel(const __grid_cons
     t = tn;
   }
 
-  grid_launch_dependents();
+  if (a.step_overlap) grid_launch_dependents();
   // this warp's partial state of its rows to shared memory (every warp has left the keys behind)
 #pragma unroll
   for (int i = 0; i < 4; ++i)

@@ -164,6 +164,7 @@ extern "C" lacache_status lacache_full_recompute_static(int dtype, int n_tokens,
   a.rot = r.dst;
   a.out = out;
   a.lse = lse;
+  a.step_overlap = 1;
   if ((e = simt_attention(g, a, g_num_sms[dev], s)) != cudaSuccess) return fail(LACACHE_ERR_CUDA, cudaGetErrorString(e));
   return LACACHE_OK;
 }

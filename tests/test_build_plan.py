@@ -1,5 +1,5 @@
-"""The build's work lists (csrc/lacache_plan.h), planned on the host: every row once, the most work first, each block's list
-what planning that block alone gives -- and planned once per context, not once per block."""
+"""Host-side planning (csrc/lacache_plan.h).  The build's work lists: every row once, the most work first, each block's list
+what planning that block alone gives -- and planned once per context, not once per block.  The rule of the early trigger."""
 import os
 import subprocess
 
@@ -25,6 +25,10 @@ int main(int argc, char** argv) {
     for (int b = 0; b < B; ++b) start[(size_t)k * B + b] = cu[b] + atoi(argv[6 + b]) + k * L;
   std::vector<WorkItem> items;
   auto lists = [&](int k0, int n) { return add_build_lists(items, cu.data(), B, L, start.data() + (size_t)k0 * B, n, heads, sms); };
+  if (mode == 3) {   // early_trigger over its four arguments, the first the lowest bit
+    for (int i = 0; i < 16; ++i) printf("%d", early_trigger(i & 1, i & 2, i & 4, i & 8) ? 1 : 0);
+    return 0;
+  }
   if (mode == 2) {   // the best of ten timings of all blocks' lists, and of one block's
     double best[2] = {1e9, 1e9};
     for (int r = 0; r < 10; ++r)
@@ -96,3 +100,12 @@ def test_planned_once_per_context(harness):
     what that takes; a plan per block takes 64)."""
     every, one = (float(x) for x in harness(2, 28, 148, 64, 64, (4096,)).split())
     assert every < 8 * one, (every, one)
+
+
+def test_early_trigger_rule(harness):
+    """On with the overlap of steps; else in short steps without a producer ahead; never with the knobs that switch it off,
+    LACACHE_NO_STEP_OVERLAP and LACACHE_NO_PDL."""
+    got = harness(3, 1, 1, 1, 1, (1,))
+    want = "".join(str(int(not off and (overlap or (short and not producer))))
+                   for off in (0, 1) for producer in (0, 1) for short in (0, 1) for overlap in (0, 1))
+    assert got == want
