@@ -44,8 +44,10 @@ __device__ __forceinline__ void store8_f16(void* plane, size_t off, const float 
 // consecutive heads of one tensor; cos and sin are loaded once for all of them (with one head per thread they are two
 // thirds of what a thread loads).  d/16 threads cover a row, a warp 32 / (d/16) consecutive rows, so that both the HPT
 // heads it reads per row and the rows it writes per head are contiguous.  blockIdx.y: group of HPT heads -- q, then k,
-// then v.  HPT = 4 from 65536 (row, head) pairs on (157 MB of bf16 rows in, as much out: 71 us with one head per thread,
-// 55 us = 5.7 TB/s with four; two and eight the same within 4 %), else 1: a block's rows are too few to fill the GPU with more per thread.
+// then v.  tcgen05 storage: HPT = 4 from 65536 (row, head) pairs on (157 MB of bf16 rows in, as much out: 71 us with one head
+// per thread, 55 us = 5.7 TB/s with four; two and eight the same within 4 %), else 1: a block's rows are too few to fill the
+// GPU with more per thread.  fp32 storage: always 1, whose rows are wide enough by themselves, while four heads' rows do
+// not fit the registers (fp32 rows of 128 features, 65544 pairs: 15.1 us against 20.7 with four; 589824: 96 against 108).
 template <bool TC, int HPT>
 __global__ void __launch_bounds__(256, HPT > 1 ? 3 : 1) rope_write_kernel(const __grid_constant__ Geometry g, const __grid_constant__ RopeArgs a) {
   // This kernel and the attention kernel behind it are launched programmatically dependent.  The attention
@@ -240,8 +242,9 @@ cudaError_t merge_chunk_states(const Geometry& g, const ChunkMergeArgs& a, cudaS
 
 template <bool TC>
 static cudaError_t rope_launch(const Geometry& g, const RopeArgs& a, cudaStream_t s) {
+  constexpr int MANY = TC ? 4 : 1;
   const bool many = (long long)a.n_src_rows * (g.Hq + 2 * g.Hkv) >= 65536;
-  const int hpt = many ? 4 : 1;
+  const int hpt = many ? MANY : 1;
   const int rows_per_cta = 256 / (g.d / 16);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)((a.n_src_rows + rows_per_cta - 1) / rows_per_cta),
@@ -253,7 +256,7 @@ static cudaError_t rope_launch(const Geometry& g, const RopeArgs& a, cudaStream_
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = a.no_pdl ? 0 : 1;
-  return many ? cudaLaunchKernelEx(&cfg, rope_write_kernel<TC, 4>, g, a) : cudaLaunchKernelEx(&cfg, rope_write_kernel<TC, 1>, g, a);
+  return many ? cudaLaunchKernelEx(&cfg, rope_write_kernel<TC, MANY>, g, a) : cudaLaunchKernelEx(&cfg, rope_write_kernel<TC, 1>, g, a);
 }
 
 cudaError_t rope_write(const Geometry& g, const RopeArgs& a, int engine, cudaStream_t s) {
