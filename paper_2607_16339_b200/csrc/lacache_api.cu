@@ -7,6 +7,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <exception>
 #include <new>
 #include <string>
 #include <vector>
@@ -227,11 +228,11 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
   g.maxN = 0;
   long long tot = 0;
   for (int b = 0; b < g.B; ++b) {
-    int n = c->prompt_lens[b] + cfg->gen_len;
+    const long long n = (long long)c->prompt_lens[b] + cfg->gen_len;
     tot += n;
     if (tot > (1ll << 30)) return fail(c, LACACHE_ERR_SHAPE, "too many tokens");
     c->cu[b + 1] = (int32_t)tot;
-    g.maxN = std::max(g.maxN, n);
+    g.maxN = std::max(g.maxN, (int)n);
   }
   g.T = (int)tot;
   g.Tp = (g.T + 127) / 128 * 128 + 128;
@@ -509,6 +510,8 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
     c->full_list = {off, (int)items.size() - off};
   }
   c->items_host = items;
+  c->step_plan.resize(g.n_blk);
+  c->allocs.reserve(128);   // (every device allocation a context may ever make)
 
   // ---- device memory ----
   if (tc) {
@@ -652,7 +655,6 @@ AttnArgs attn_args(lacache_ctx* c, int mode, lacache_ctx::ListRef list, int blk,
       int total = (int)std::min<long long>(c->num_sms, units_stream + units_merge);
       const bool deep_ok = c->g.block_len <= 32 || !c->split;   // (which variant of the merge role the step runs)
       const int deep_cap = deep_unit_cap(c);
-      if (c->step_plan.empty()) c->step_plan.resize(c->g.n_blk);
       lacache_ctx::StepPlan& plan = c->step_plan[blk];
       const bool planned = plan.deep_cap == deep_cap;
       double sum_tiles = 0;   // ragged batches mix short and long units on a CTA: cost a unit between mean and longest
@@ -839,7 +841,12 @@ lacache_status lacache_create(const lacache_config* cfg, lacache_ctx** out) {
   if (!cfg || !out) return fail(nullptr, LACACHE_ERR_INVALID_ARG, "cfg or out is NULL");
   lacache_ctx* c = new (std::nothrow) lacache_ctx();
   if (!c) return fail(nullptr, LACACHE_ERR_OOM, "host allocation failed");
-  lacache_status st = create_impl(cfg, c);
+  lacache_status st;
+  try {   // (the host's lists and tables grow with the tokens and blocks; nothing after create allocates host memory)
+    st = create_impl(cfg, c);
+  } catch (const std::exception& e) {
+    st = fail(c, LACACHE_ERR_OOM, "host allocation failed: %s", e.what());
+  }
   if (st != LACACHE_OK) {
     snprintf(g_create_err, sizeof(g_create_err), "%s", c->err);
     cudaGetLastError();

@@ -3,6 +3,8 @@
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import __graft_entry__ as entry
 from paper_2607_16339_b200 import binding
@@ -63,6 +65,30 @@ def test_create_rejects_bad_configs_without_gpu():
         assert lib.lacache_last_error(None)
     assert lib.lacache_create(None, ctypes.byref(h)) == binding.ERR_INVALID_ARG
     assert lib.lacache_build(None, 0, None, None, None, None) == binding.ERR_INVALID_ARG
+
+
+def test_create_reports_sizes_beyond_the_host_without_gpu():
+    """Nothing is thrown through the C interface: token counts that overflow 32 bits are refused, and lists or tables that
+    do not fit the host's memory give LACACHE_ERR_OOM (in a process with little address space left)."""
+    script = """
+import ctypes, resource, sys
+from paper_2607_16339_b200 import binding
+lib = binding.load()
+def create(prompt, gen, block):
+    h = ctypes.c_void_p()
+    pl = (ctypes.c_int32 * 1)(prompt)
+    c = binding.LacacheConfig(0, 0, 4, 2, 128, 1e4, 0.0, 1, pl, gen, block, 0, binding.OUT_FP32, binding.PRECISION_SPLIT, 0)
+    st = lib.lacache_create(ctypes.byref(c), ctypes.byref(h))
+    assert not h.value and lib.lacache_last_error(None)
+    return st
+assert create(2 ** 31 - 1, 32, 16) == binding.ERR_SHAPE
+assert create(2 ** 30, 32, 16) == binding.ERR_SHAPE
+used = int(open("/proc/self/statm").read().split()[0]) * 4096
+resource.setrlimit(resource.RLIMIT_AS, (used + (1 << 30), used + (1 << 30)))
+assert create(2 ** 30 - 64, 32, 16) == binding.ERR_OOM
+"""
+    r = subprocess.run([sys.executable, "-c", script], cwd=ROOT, capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, (r.returncode, r.stderr[-1000:])
 
 
 def test_producer_create_rejects_bad_configs_without_gpu():
