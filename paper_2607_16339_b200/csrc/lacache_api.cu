@@ -65,7 +65,6 @@ struct lacache_ctx {
 
   // device memory
   std::vector<void*> allocs;
-  int32_t* d_cu = nullptr;
   int32_t* d_blk_start_all = nullptr;
   int32_t* d_pos = nullptr;
   float* d_cos = nullptr;
@@ -376,7 +375,7 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
         items[i].chunk = flags;
       }
     };
-    enum { W_INIT = 1, W_SNAP = 2, W_SKIP_BLOCK = 4, W_JUMP_BLOCK = 8 };
+    enum { W_INIT = 1, W_SNAP = 2, W_JUMP_BLOCK = 8 };
     int off = (int)items.size();
     for (int b = 0; b < g.B; ++b) {
       const int cs = c->cu[b], ce = c->cu[b + 1], s0 = c->blk_start_all[(size_t)k * g.B + b], e0 = s0 + g.block_len;
@@ -521,8 +520,6 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
     CU_TRY(c, simt_prepare());
   }
 
-  CU_TRY(c, dev_alloc(c, &c->d_cu, g.B + 1));
-  CU_TRY(c, cudaMemcpy(c->d_cu, c->cu.data(), sizeof(int32_t) * (g.B + 1), cudaMemcpyHostToDevice));
   CU_TRY(c, dev_alloc(c, &c->d_blk_start_all, c->blk_start_all.size()));
   CU_TRY(c, cudaMemcpy(c->d_blk_start_all, c->blk_start_all.data(), sizeof(int32_t) * c->blk_start_all.size(), cudaMemcpyHostToDevice));
   CU_TRY(c, dev_alloc(c, &c->d_pos, g.T));
@@ -626,7 +623,6 @@ AttnArgs attn_args(lacache_ctx* c, int mode, lacache_ctx::ListRef list, int blk,
   a.mode = mode;
   a.items = c->d_items + list.off;
   a.n_items = list.n;
-  a.cu = c->d_cu;
   a.blk_start = blk >= 0 ? c->d_blk_start_all + (size_t)blk * c->g.B : nullptr;
   a.rot = rot;
   a.st = c->st;

@@ -15,10 +15,9 @@ enum ItemKind : int32_t {
   ITEM_ROWS_WINDOW = 2,  // (build) a tile of query rows x the keys [kt0, kt1) of its sequence, given as token
                          // indices; key tiles are counted from token `pad` (<= kt0, may be negative).
                          // chunk bit 0: continue from the rows' state in AttnArgs::init; bit 1: store the
-                         // state after the first key tile to AttnArgs::snap; bit 2: leave out the keys of
-                         // the block at blk_start; bit 3: the first tile ends at blk_start (pad = blk_start -
-                         // tile width) and the tiles after it are counted from the end of that block; bit 4:
-                         // the unit writes normalised rows to out / lse instead of a state
+                         // state after the first key tile to AttnArgs::snap; bit 3: the first tile ends at
+                         // blk_start (pad = blk_start - tile width) and the tiles after it are counted from the
+                         // end of that block; bit 4: the unit writes normalised rows to out / lse instead of a state
 };
 struct WorkItem {
   int32_t kind;   // ItemKind
@@ -123,7 +122,6 @@ struct AttnArgs {
   int split_ctas;            // SIMT: CTAs (one cluster) a cut unit takes; chosen by the launcher
   int step_overlap;          // let the kernels behind be scheduled while this one drains (tcgen05, steps: from its entry on;
                              // SIMT: once a CTA has left its last key tile)
-  const int32_t* cu;         // [B+1]
   const int32_t* blk_start;  // [B] absolute token index of the block's first row
   RotBuffers rot;
   StateBuffers st;

@@ -43,7 +43,7 @@ constexpr int THREADS = 384;
 constexpr int LAUNCH_REGS = 168, ROW_REGS = 208, ISSUER_REGS = 88;
 static_assert(ROW_THREADS * ROW_REGS + (THREADS - ROW_THREADS) * ISSUER_REGS <= THREADS * LAUNCH_REGS, "more registers than the block has");
 constexpr int KT = TC_ROW_KEYS;   // keys per tile
-constexpr int W_QUERIES = 8, W_MMA = 9, W_KEYS = 10, W_VALUES = 11;   // the warps with another role
+constexpr int W_QUERIES = 8, W_MMA = 9, W_KEYS = 10;   // the warps with another role (the last one, 11: values)
 
 struct RowMaps {
   CUtensorMap q;      // box {64, 128 rows, 2 halves, 1 head, planes}: a whole Q' tile
@@ -117,7 +117,6 @@ __device__ __forceinline__ Unit decode(const Geometry& g, const AttnArgs& a, int
     un.k0 = it.kt0;
     un.k1 = it.kt1;
     un.n_tiles = it.kt1 > it.pad ? (it.kt1 - it.pad + KT - 1) / KT : 0;
-    if (it.chunk & 4) { un.x0 = it.blk_start; un.x1 = it.blk_start + g.block_len; }
     if (it.chunk & 8) {   // the first tile ends where the block starts; the others start right after the block
       un.base1 = it.blk_start + g.block_len;
       un.n_tiles = 1 + (it.kt1 > un.base1 ? (it.kt1 - un.base1 + KT - 1) / KT : 0);
@@ -358,7 +357,6 @@ template <bool SPLIT>
 __device__ __forceinline__ void store_rows(const Cta& c, uint32_t o_tmem, bool have_o, float mul, float* dst32,
                                            __nv_bfloat16* dst16, size_t stride, int rows) {
   const int lane = threadIdx.x & 31;
-  uint8_t* const st = c.gen + Lay<SPLIT>::SM_ST + (threadIdx.x >> 5) * 4096;
 #pragma unroll 1
   for (int cb = 0; cb < 4; ++cb) {
     uint32_t r[32];
@@ -371,7 +369,7 @@ __device__ __forceinline__ void store_rows(const Cta& c, uint32_t o_tmem, bool h
 #pragma unroll
       for (int i = 0; i < 32; ++i) r[i] = 0u;
     }
-    if (SPLIT) {
+    if constexpr (SPLIT) {
       if (lane < rows) {
         const size_t off = (size_t)lane * stride + 32 * cb;
         if (dst16) {
@@ -390,23 +388,24 @@ __device__ __forceinline__ void store_rows(const Cta& c, uint32_t o_tmem, bool h
           for (int i = 0; i < 8; ++i) *reinterpret_cast<uint4*>(dst32 + off + 4 * i) = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
         }
       }
-      continue;
-    }
+    } else {
+      uint8_t* const st = c.gen + Lay<SPLIT>::SM_ST + (threadIdx.x >> 5) * 4096;
 #pragma unroll
-    for (int i = 0; i < 8; ++i)
-      *reinterpret_cast<uint4*>(st + lane * 128 + ((i ^ (lane & 7)) << 4)) = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
-    __syncwarp();
+      for (int i = 0; i < 8; ++i)
+        *reinterpret_cast<uint4*>(st + lane * 128 + ((i ^ (lane & 7)) << 4)) = make_uint4(r[4 * i], r[4 * i + 1], r[4 * i + 2], r[4 * i + 3]);
+      __syncwarp();
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int rr = 4 * i + (lane >> 3), ch = lane & 7;
-      if (rr < rows) {
-        const float4 v = *reinterpret_cast<const float4*>(st + rr * 128 + ((ch ^ (rr & 7)) << 4));
-        const size_t off = (size_t)rr * stride + 32 * cb + 4 * ch;
-        if (dst16) *reinterpret_cast<uint2*>(dst16 + off) = make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w));
-        else *reinterpret_cast<float4*>(dst32 + off) = v;
+      for (int i = 0; i < 8; ++i) {
+        const int rr = 4 * i + (lane >> 3), ch = lane & 7;
+        if (rr < rows) {
+          const float4 v = *reinterpret_cast<const float4*>(st + rr * 128 + ((ch ^ (rr & 7)) << 4));
+          const size_t off = (size_t)rr * stride + 32 * cb + 4 * ch;
+          if (dst16) *reinterpret_cast<uint2*>(dst16 + off) = make_uint2(pack_bf16x2(v.x, v.y), pack_bf16x2(v.z, v.w));
+          else *reinterpret_cast<float4*>(dst32 + off) = v;
+        }
       }
+      __syncwarp();
     }
-    __syncwarp();
   }
 }
 

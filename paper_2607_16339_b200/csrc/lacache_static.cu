@@ -11,7 +11,6 @@
 // fixed array that lives in the library's device image.
 #include <math.h>
 #include <stdio.h>
-#include <string.h>
 
 #include "lacache_internal.h"
 
@@ -28,7 +27,7 @@ namespace {
 constexpr size_t STATIC_MAX_PLANE_ELEMS = (size_t)4 << 20;  // T * (Hq + 2 Hkv) * d
 constexpr int STATIC_MAX_TOKENS = 4096;
 constexpr size_t STATIC_TABLE_ELEMS = (size_t)STATIC_MAX_TOKENS * 64 * 2;      // cos + sin, d/2 <= 64
-constexpr size_t STATIC_META_WORDS = STATIC_MAX_TOKENS + 16 + (STATIC_MAX_TOKENS / SIMT_ROWS + 1) * 12;
+constexpr size_t STATIC_META_WORDS = STATIC_MAX_TOKENS + (STATIC_MAX_TOKENS / SIMT_ROWS + 1) * 12;
 constexpr size_t STATIC_WORDS = STATIC_MAX_PLANE_ELEMS + STATIC_TABLE_ELEMS + STATIC_META_WORDS;
 
 static __device__ __align__(256) float g_static_scratch[STATIC_WORDS];
@@ -110,16 +109,15 @@ extern "C" lacache_status lacache_full_recompute_static(int dtype, int n_tokens,
   float* d_cos = base + STATIC_MAX_PLANE_ELEMS;
   float* d_sin = d_cos + (size_t)STATIC_MAX_TOKENS * 64;
   int32_t* d_meta = reinterpret_cast<int32_t*>(base + STATIC_MAX_PLANE_ELEMS + STATIC_TABLE_ELEMS);
-  // meta: [0, T) positions | [T, T+16) cu (padded) | work items
+  // meta: [0, T) positions | work items
   const int n_items = (n_tokens + SIMT_ROWS - 1) / SIMT_ROWS;
-  const size_t items_off = ((size_t)n_tokens + 16 + 3) & ~(size_t)3;  // 16-byte aligned
+  const size_t items_off = ((size_t)n_tokens + 3) & ~(size_t)3;  // 16-byte aligned
   Filled& filled = g_filled[dev];
   const bool refill = filled.n_tokens != n_tokens || filled.head_dim != head_dim || filled.theta != rope_theta;
   if (refill) {
     filled.n_tokens = 0;   // (until the copies below are enqueued)
     for (int t = 0; t < n_tokens; ++t) h_meta[t] = t;
-    memset(h_meta + n_tokens, 0, sizeof(int32_t) * 16);
-    h_meta[n_tokens + 1] = n_tokens;  // cu = {0, T}
+    for (size_t i = n_tokens; i < items_off; ++i) h_meta[i] = 0;
     WorkItem* items = reinterpret_cast<WorkItem*>(h_meta + items_off);
     for (int i = 0; i < n_items; ++i) {
       WorkItem w{};
@@ -159,7 +157,6 @@ extern "C" lacache_status lacache_full_recompute_static(int dtype, int n_tokens,
   a.mode = MODE_FULL;
   a.items = reinterpret_cast<const WorkItem*>(d_meta + items_off);
   a.n_items = n_items;
-  a.cu = d_meta + n_tokens;
   a.blk_start = nullptr;
   a.rot = r.dst;
   a.out = out;

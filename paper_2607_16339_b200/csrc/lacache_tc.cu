@@ -73,9 +73,6 @@ struct Tile {
   static_assert(BN % 32 == 0 && BN <= 128, "tile width");
   static_assert(KS_BOX % 1024 == 0, "swizzled boxes need 1024-byte alignment");
   static_assert(SM_V + 2 * V_STAGE <= SM_XCH, "stream-role tiles overrun");
-  // (A key tile is wider than a block, so no tile lies wholly inside the keys a build excludes: every
-  // tile in [t0, t1) is processed, excluded columns are masked by the row threads.)
-  static_assert(BN > TC_MAX_BLOCK, "a key tile could fall wholly inside the excluded block");
 };
 // The stream role stages its epilogue (128 rows x 512 B, 16-byte chunks XOR-swizzled
 // by the row so row-wise writes and row-wise reads are both conflict-free) in the
@@ -150,8 +147,8 @@ enum StreamKind : int { KIND_STEP = 1, KIND_STEP2 = 3 };
 
 struct Unit {
   int row0, nrows, h, kh, seq;
-  int key_base, t0, t1;   // key tiles [t0, t1): tile t holds keys key_base + 64 t ...
-  int k0, k1, x0, x1;     // valid keys [k0, k1) minus [x0, x1)
+  int key_base, t0, t1;   // key tiles [t0, t1): tile t holds keys key_base + BN t ...
+  int k1;                 // valid keys [key_base, k1)
   int epi, chunk, nchunks;
   int q_rows;             // rows of the Q box: 128 or 64
   int nh, rh;             // packed block queries: nh heads h, h + 1, ... of one KV group, rh lanes each (rh = 0: one head)
@@ -182,8 +179,6 @@ __device__ __forceinline__ int unit_item(const Geometry& g, const AttnArgs& a, i
 // head arithmetic: this kernel is sensitive to its code size.
 template <bool PACKED, int KIND, bool SPLIT>
 __device__ __forceinline__ Unit decode_stream(const Geometry& g, const AttnArgs& a, const WorkItem& it, int u) {
-  using TL = Tile<SPLIT>;
-  constexpr int BN = TL::BN;
   Unit un;
   // units are head-minor: unit u = item u / slots of head (or head group) u % slots (a CTA's units, a
   // fixed stride apart, then cycle through the items instead of drawing one item's heads)
@@ -205,14 +200,7 @@ __device__ __forceinline__ Unit decode_stream(const Geometry& g, const AttnArgs&
   un.row0 = it.row0;
   un.nrows = it.nrows;
   un.key_base = it.seq_start;
-  un.k0 = it.seq_start;
   un.k1 = it.seq_end;
-  un.x0 = un.x1 = 0;
-  un.t0 = 0;
-  un.t1 = (it.seq_end - it.seq_start + BN - 1) / BN;
-  un.chunk = 0;
-  un.nchunks = 1;
-  un.q_rows = BM;
   un.t0 = it.kt0;
   un.t1 = it.kt1;
   un.chunk = it.chunk;
@@ -692,21 +680,13 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
       bool o_waited = first_tile;
       if (active) {
         const int tile_lo = tile_key_row<SPLIT>(un, t);
-        const int v_lo = max(un.k0 - tile_lo, 0), v_hi = min(un.k1 - tile_lo, BN);
-        const int e_lo = un.x0 - tile_lo, e_hi = un.x1 - tile_lo;
-        const bool all_valid = v_lo == 0 && v_hi == BN && (un.x1 <= un.x0 || e_hi <= 0 || e_lo >= BN);
+        const int v_hi = min(un.k1 - tile_lo, BN);   // (a tile starts inside its sequence)
+        const bool all_valid = v_hi == BN;
         // the masks of a tile are the same for every row: one bit per column of this thread's half
         // (bit j: column mc + j takes part), built once per tile
         const int mc = HC * half;   // this thread's columns
-        auto span_bits = [](int lo, int hi) -> uint64_t {   // bits [lo, hi) of 64
-          lo = max(lo, 0);
-          hi = min(hi, 64);
-          if (hi <= lo) return 0ull;
-          return (hi - lo == 64 ? ~0ull : ((1ull << (hi - lo)) - 1ull)) << lo;
-        };
-        const uint64_t col_bits = all_valid ? ~0ull
-                                            : (span_bits(v_lo - mc, v_hi - mc) &
-                                               ~((un.x1 > un.x0) ? span_bits(e_lo - mc, e_hi - mc) : 0ull));
+        const int n_mine = v_hi - mc;
+        const uint64_t col_bits = n_mine >= 64 ? ~0ull : n_mine <= 0 ? 0ull : (1ull << n_mine) - 1ull;
         const uint32_t s_addr = tlane + TS_S + 128 * b;
         // This thread's HC scores come out of TMEM once, every load in flight before the one wait (the
         // time of these threads per tile is what bounds a build: a second pass over TMEM and a wait per
@@ -762,7 +742,7 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
             tmem_ld_wait();
 #pragma unroll
             for (int j = 0; j < 16; ++j) rr[j] = __float_as_uint(__uint_as_float(rr[j]) * alpha);
-            tmem_st16(tlane + TS_O + 64 * half + 16 * cb, rr, 0);
+            tmem_st16(tlane + TS_O + 64 * half + 16 * cb, rr);
           }
         }
         // Probabilities of this thread's columns, from the registers: P~ = 2^(S c - m) rounded to fp16 (what
@@ -1283,11 +1263,11 @@ struct Deep {
   static_assert(!WIDE || V + 2 * BOX <= DM_IO, "the Q' region's upper half");
 };
 
-struct DUnit { int row0, nrows, blk_start, h, seq; };
+struct DUnit { int row0, nrows, blk_start, h; };
 template <bool SPLIT, bool WIDE>
 __device__ __forceinline__ DUnit deep_unit(const Cta& c, int i) {
   const int4 v = *reinterpret_cast<const int4*>(c.gen + Deep<SPLIT, WIDE>::TAB + 16 * i);
-  return DUnit{v.x, v.y, v.z, v.w & 0xFFFF, v.w >> 16};
+  return DUnit{v.x, v.y, v.z, v.w};
 }
 
 template <bool SPLIT, bool WIDE>
@@ -1604,7 +1584,7 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
       // units are head-minor (unit u = row tile u / Hq of head u % Hq): a CTA's units, a
       // fixed stride apart, then cycle through the row tiles, clipped ones included
       const WorkItem w = load_item(a.items_merge + u / g.Hq);
-      *reinterpret_cast<int4*>(smem_raw + DL::TAB + 16 * i) = make_int4(w.row0, w.nrows, w.blk_start, (u % g.Hq) | (w.seq << 16));
+      *reinterpret_cast<int4*>(smem_raw + DL::TAB + 16 * i) = make_int4(w.row0, w.nrows, w.blk_start, u % g.Hq);
     }
   }
   __syncwarp();
