@@ -168,6 +168,13 @@ lacache_status alloc_rot(lacache_ctx* c, RotBuffers* r) {
   return LACACHE_OK;
 }
 
+// query heads whose block rows share a 128-row tile (1: none do)
+int heads_per_tile(const lacache_ctx* c) {
+  const int fit = 128 / (c->g.block_len <= 32 ? 32 : 64);
+  // (the packed tile's load takes `fit` heads at a time)
+  return (c->g.group >= 2 && c->g.Hq >= fit && !c->knobs.no_pack) ? std::min(fit, c->g.group) : 1;
+}
+
 lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
   c->cfg = *cfg;
   c->cfg.prompt_lens = nullptr;
@@ -414,8 +421,7 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
       const int nkt = (s0 - cs + TC_KEYS - 1) / TC_KEYS;
       // (units of all sequences: one per sequence and head, or per packed group of heads; at most eight
       // chunks, which the last one to arrive merges with every load in flight at once)
-      const int fit = 128 / (g.block_len <= 32 ? 32 : 64);
-      const int pack = (g.group >= 2 && g.Hq >= fit && !c->knobs.no_pack) ? std::min(fit, g.group) : 1;
+      const int pack = heads_per_tile(c);
       const int slots = g.B * g.Hkv * ((g.group + pack - 1) / pack);
       int chunks = std::max(1, std::min({8, nkt, c->num_sms / slots}));
       const int per = (nkt + chunks - 1) / chunks;
@@ -514,8 +520,8 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
 
   // ---- device memory ----
   if (tc) {
-    CU_TRY(c, tc_prepare(c->split));
     CU_TRY(c, rows_prepare(c->split));
+    CU_TRY(c, tc_prepare(g, c->split, heads_per_tile(c) > 1));
   } else {
     CU_TRY(c, simt_prepare());
   }
@@ -607,14 +613,10 @@ int deep_unit_cap(const lacache_ctx* c) { return c->knobs.deep_units; }
 
 // block queries of a GQA model: heads of one KV group side by side in the 128 lanes of a tile
 void set_packing(lacache_ctx* c, AttnArgs& a) {
-  if (c->g.group < 2 || c->knobs.no_pack) return;
-  const int rows = c->g.block_len <= 32 ? 32 : 64;
-  const int pack = std::min(128 / rows, c->g.group);
-  if (c->g.Hq < 128 / rows) return;   // the packed tile's load takes 128 / rows heads at a time
-  if (pack >= 2) {
-    a.pack = pack; a.pack_rows = rows;
-    a.stream_slots = c->g.Hkv * ((c->g.group + pack - 1) / pack);
-  }
+  const int pack = heads_per_tile(c);
+  if (pack < 2) return;
+  a.pack = pack; a.pack_rows = c->g.block_len <= 32 ? 32 : 64;
+  a.stream_slots = c->g.Hkv * ((c->g.group + pack - 1) / pack);
 }
 
 AttnArgs attn_args(lacache_ctx* c, int mode, lacache_ctx::ListRef list, int blk, const RotBuffers& rot,

@@ -186,7 +186,7 @@ cudaError_t simt_prepare();  // function attributes (the *_prepare functions: of
 
 struct TcMaps;  // opaque set of TMA descriptors, defined in lacache_tc.cu
 cudaError_t tc_attention(const Geometry& g, const AttnArgs& a, const TcMaps* maps, cudaStream_t s);
-cudaError_t tc_prepare(bool split);
+cudaError_t tc_prepare(const Geometry& g, bool split, bool packed);
 // row tiles over long key ranges (build, full recompute, key windows) with one-plane operands: lacache_rows.cu
 cudaError_t row_attention(const Geometry& g, const AttnArgs& a, const TcMaps* maps, cudaStream_t s);
 cudaError_t rows_prepare(bool split);

@@ -1742,18 +1742,21 @@ const void* const* kernel_table() {
       (const void*)tc_attn_kernel<false, KIND_STEP2, 1, SPLIT>};
   return t;
 }
+int step_kernel(const Geometry& g, bool packed) { return (packed ? 2 : 0) + (g.block_len <= 32 ? 1 : 0); }
+constexpr int PAIRED_KERNEL = 4;   // (unpacked heads, blocks of up to 32 rows)
 }  // namespace
 
-// A kernel is loaded on the device when it is first asked about: a context asks for those of its own operand mode only.
-// (Less to load at create, and what is loaded decides where code lies: consecutive overlapped steps of 32 heads at N = 768
-// ran at 65.1 k to 66.4 k steps/s over thirteen sets and orders of loaded kernels, 65.5 k with both modes', 66.2 k with one's.)
-cudaError_t tc_prepare(bool split) {
+// A kernel is loaded on the device when it is first asked about: a context asks for the ones it may launch and no other
+// (packed: its block queries share tiles across heads).  Less to load at create, and what is loaded decides where the code
+// lies, which moves a step by up to 2 %: overlapped steps of 32 heads at N = 768 ran at 65.1 k to 66.4 k steps/s over 42 sets
+// and orders of loaded kernels (65.8 k with this one's), eight ragged requests in 81.4 us with their own two, 84 with the
+// mode's five, 83 with all.
+cudaError_t tc_prepare(const Geometry& g, bool split, bool packed) {
   const void* const* t = split ? kernel_table<true>() : kernel_table<false>();
-  for (int i = 0; i < 5; ++i) {
-    cudaError_t e = cudaFuncSetAttribute(t[i], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(t[step_kernel(g, packed)], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
+  if (e == cudaSuccess && !packed && g.block_len <= 32)
+    e = cudaFuncSetAttribute(t[PAIRED_KERNEL], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
+  return e;
 }
 
 bool tc_set_out(TcMaps* m, const Geometry& g, float* out, bool out_bf16, char* err, int errlen) {
@@ -1822,7 +1825,7 @@ cudaError_t tc_attention(const Geometry& g, const AttnArgs& a, const TcMaps* map
   cfg.attrs = attr;
   cfg.numAttrs = n_attr;
   const void* const* t = a.split ? kernel_table<true>() : kernel_table<false>();
-  const int which = paired ? 4 : (a.pack > 1 ? 2 : 0) + (g.block_len <= 32 ? 1 : 0);
+  const int which = paired ? PAIRED_KERNEL : step_kernel(g, a.pack > 1);
   void* params[3] = {const_cast<TcMaps*>(maps), const_cast<Geometry*>(&g), const_cast<AttnArgs*>(&a)};
   return cudaLaunchKernelExC(&cfg, t[which], params);
 }

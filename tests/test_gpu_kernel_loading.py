@@ -1,4 +1,4 @@
-"""A context prepares the kernels of its own operand mode and engine only.  What a kernel was prepared for stays with the
+"""A context prepares the kernels that it may launch and no other.  What a kernel was prepared for stays with the
 process, so each order of first contexts runs in a process of its own: build, steps, full recompute and the incremental
 rebuild of every context agree with its own full recompute."""
 import os
