@@ -739,7 +739,7 @@ def run_cuda(args):
 # sampling-stage truncation: softmax over the vocabulary on the current block's rows only
 # ----------------------------------------------------------------------------
 VOCAB = {32: 126464, 28: 152064}     # vocabulary of the model a workload is shaped like, by query heads
-SAMPLER_TRAFFIC_PER_LAUNCH = {4: 66288640}   # ncu, profiles/sample_rows_kernel_cfg4_ncu_full.txt (read + write)
+SAMPLER_TRAFFIC_PER_LAUNCH = {4: 66596608}   # ncu, profiles/sample_rows_cfg4_ncu.txt (read + write)
 
 
 def sampler_leg(wl, dev, peaks, seed):
@@ -874,7 +874,7 @@ def incremental_leg(wl, dev, seed, R, precision):
 # the step fed by token ids: embedding gather + RMS norm + Q/K/V projection in front
 # ----------------------------------------------------------------------------
 D_MODEL = {32: 4096, 28: 3584}     # first-layer width of the model a workload is shaped like, by query heads
-QKV_TRAFFIC_PER_LAUNCH = {2: 104751872}   # ncu, profiles/qkv_gemm_kernel_cfg2_step_ncu_full.txt
+QKV_TRAFFIC_PER_LAUNCH = {2: 106217088}   # ncu, profiles/qkv_gemm_cfg2_step_ncu.txt
 
 
 def token_path_leg(wl, dev, peaks, seed, n_steps, precision):
@@ -968,13 +968,12 @@ def token_path_leg(wl, dev, peaks, seed, n_steps, precision):
 
 # per-launch DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of the
 # step attention kernel from the committed ncu captures
-# (profiles/tc_attn_kernel_cfg2_ncu_full.txt, tc_attn_kernel_cfg{3,4}_step_ncu_full.txt,
-# tc_attn_kernel_cfg5_{split,plain}_ncu_full.txt), bytes; None where no capture exists for the workload
+# (profiles/attention_cfg{2,4,5}_ncu.txt, attention_cfg3_split_ncu.txt), bytes; None where no capture exists for the workload
 # and precision mode.  The fp32 output (12.6 MB) is still in L2 when the
 # kernel ends, so the figure is dominated by reads.
 DEFAULT_PRECISION = {1: 1, 2: 3, 3: 1, 4: 3, 5: 3, 6: 3}   # binding.PRECISION_*: 1 = split bf16 planes, 3 = one fp16 plane
-TRAFFIC_PER_LAUNCH = {(2, 1): 48370432, (3, 1): 93736960, (4, 1): 460605952, (5, 1): 209015552, (5, 0): 161659392,
-                      (2, 3): 34980608, (4, 3): 345821952, (5, 3): 161281536}   # (config, precision mode)
+TRAFFIC_PER_LAUNCH = {(2, 1): 44727936, (3, 1): 93297536, (4, 1): 456484864, (5, 1): 208400768, (5, 0): 156070400,
+                      (2, 3): 32033663, (4, 3): 341052160, (5, 3): 156948480}   # (config, precision mode)
 
 
 # ----------------------------------------------------------------------------
