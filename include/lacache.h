@@ -189,7 +189,14 @@ lacache_status lacache_build_advance(lacache_ctx* ctx, const void* q_fin, const 
  * everything enqueued on that stream before it, and is complete, with out / lse
  * fully written, before any later operation of that stream runs: an ordinary
  * stream-ordered call.  q_blk / k_blk / v_blk must stay unchanged until the
- * call's work has completed.
+ * call's work has completed.  One thing to know for a caller who writes kernels
+ * and launches them programmatically dependent (the stream-serialization launch
+ * attribute) right behind a call of this library: the library's kernels signal
+ * griddepcontrol.launch_dependents before they end (short steps and the producer's
+ * kernels at their start, the sampler and the fp32 kernels behind their last loads),
+ * so such a kernel may be running while they still read and write, and must
+ * execute griddepcontrol.wait before it touches anything of theirs.
+ * Every other operation, ordinary kernels included, starts when they are complete.
  *
  * Optional overlap of consecutive steps, lacache_set_step_overlap(ctx, 1): two
  * lacache_step calls in a row on one stream then overlap on the device (the
@@ -218,7 +225,7 @@ lacache_status lacache_step(lacache_ctx* ctx, const void* q_blk, const void* k_b
  * (sequence-major): token = the most probable vocabulary entry (the lowest id among entries of
  * exactly equal logit), conf = its probability, lse = log sum_v exp(logit_v) (lse may be NULL).
  * conf / token / lse are DEVICE arrays [B*L_b] (fp32, int32, fp32).  A logit of -inf contributes
- * nothing.  fp32 arithmetic.  LACACHE_ERR_STATE before a build.  Allocates a small scratch on first
+ * nothing, nor does the type's lowest finite value beside any larger one.  fp32 arithmetic.  LACACHE_ERR_STATE before a build.  Allocates a small scratch on first
  * use.  Calls on one context must not overlap on the GPU (they share that scratch).
  */
 lacache_status lacache_sample_block(lacache_ctx* ctx, const void* logits, int dtype, int vocab,

@@ -464,7 +464,7 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
     // (B_r = B_c).  With [lo, hi) the tokens of the tiles that overlap the block: state is cached for the
     // rows outside [lo, hi) over the keys outside [lo, hi) (first the keys before lo, then, on top, the
     // keys from hi on); a step gives those rows the keys [lo, hi) and runs the rows of [lo, hi) over all
-    // keys.  The work items are key-window items of the build kernel.
+    // keys.  The work items are key-window items of the row kernel.
     enum { W_INIT = 1, W_OUT = 16 };
     auto window = [&](size_t from, int base, int k0, int k1, int flags) {
       for (size_t i = from; i < items.size(); ++i) {
@@ -987,8 +987,8 @@ lacache_status lacache_build_advance(lacache_ctx* c, const void* q, const void* 
   c->last_launches = 0;
   c->built_block = -1;
   c->prefix_block = -1;
-  // the finished block's rows, rotated into the cache (an ordinary launch: everything ahead in the
-  // stream, a step that still reads the cached state included, completes first)
+  // the finished block's rows, rotated into the cache (the kernel waits, before its first load, for everything ahead in
+  // the stream, a step that still reads the cached state included)
   RopeArgs r{};
   r.q = q; r.k = k; r.v = v;
   r.n_src_rows = c->g.B * c->g.block_len;
@@ -1113,7 +1113,7 @@ lacache_status lacache_build_advance_tokens(lacache_ctx* c, lacache_qkv* p, cons
   if (st != LACACHE_OK) return st;
   void *q, *k, *v;
   qkv_scratch(p, true, &q, &k, &v);
-  // (the RoPE launch of the advance is an ordinary one: it starts when the projection has completed)
+  // (the RoPE kernel of the advance waits for the projection before anything else)
   st = qkv_project_rows(p, fin_token_ids, fin_hidden, n, q, k, v, nullptr, nullptr, 0, false, stream);
   if (st != LACACHE_OK) return fail(c, st, "producer: %s", lacache_qkv_last_error(p));
   st = lacache_build_advance(c, q, k, v, stream);
@@ -1174,8 +1174,8 @@ lacache_status step_impl(lacache_ctx* c, const void* q, const void* k, const voi
   r.dst = c->rot;
   r.in_dtype = c->cfg.dtype;
   if (c->cfg.cache_granularity == LACACHE_GRANULARITY_TILE) {
-    // Algorithm 1's reuse pass at tile granularity: ordinary launches, one pass of the build kernel over
-    // key windows (rows of the overlapping tiles x all keys; every other row: cached state + the keys of
+    // Algorithm 1's reuse pass at tile granularity: no kernel reads anything before the one ahead is complete, and one pass
+    // of the row kernel over key windows (rows of the overlapping tiles x all keys; every other row: cached state + the keys of
     // the overlapping tiles), normalised output instead of state
     r.early_inputs = 0;
     CU_TRY(c, rope_write(c->g, r, c->engine, s));

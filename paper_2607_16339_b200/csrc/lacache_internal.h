@@ -1,5 +1,5 @@
-// Internal declarations shared by the host side (lacache_api.cu) and the two
-// kernel families (lacache_simt.cu: CUDA-core fp32; lacache_tc.cu: tcgen05).
+// Internal declarations shared by the host side (lacache_api.cu) and the kernel files (lacache_simt.cu: CUDA-core fp32
+// attention; lacache_tc.cu, lacache_rows.cu: tcgen05 attention; lacache_rope.cu; lacache_sample.cu).
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -8,7 +8,7 @@
 
 namespace lacache {
 
-// Work item kinds.  A launch walks a list of items; blockIdx.y is the q head.
+// Work item kinds.  A launch walks a list of items, every head of each.
 enum ItemKind : int32_t {
   ITEM_ROWS = 0,   // a tile of query rows [row0, row0 + nrows) of one sequence
   ITEM_BLOCK_CHUNK = 1,  // the block's query rows x one chunk of key tiles
@@ -187,7 +187,7 @@ cudaError_t simt_prepare();  // function attributes (the *_prepare functions: of
 struct TcMaps;  // opaque set of TMA descriptors, defined in lacache_tc.cu
 cudaError_t tc_attention(const Geometry& g, const AttnArgs& a, const TcMaps* maps, cudaStream_t s);
 cudaError_t tc_prepare(const Geometry& g, bool split, bool packed);
-// row tiles over long key ranges (build, full recompute, key windows) with one-plane operands: lacache_rows.cu
+// row tiles over long key ranges (build, full recompute, key windows): lacache_rows.cu
 cudaError_t row_attention(const Geometry& g, const AttnArgs& a, const TcMaps* maps, cudaStream_t s);
 cudaError_t rows_prepare(bool split);
 // builds TMA descriptors for a rotated buffer set; returns nullptr and fills
@@ -213,14 +213,14 @@ bool qkv_full_owner_is(const lacache_qkv* p, const void* ctx, int n_tokens);
 
 constexpr int SIMT_ROWS = 32;    // query rows per SIMT work item
 constexpr int TC_ROWS = 128;     // query rows per tcgen05 work item
-// keys per tile of the tcgen05 stream role: 96 with split operands (two stages of {K hi, K lo} and of V fit
+// keys per tile of a step's stream role: 96 with split operands (two stages of {K hi, K lo} and of V fit
 // beside the Q tile), 128 with plain ones
 constexpr int TC_KEYS_SPLIT = 96;
 constexpr int TC_KEYS_PLAIN = 128;
 inline int tc_keys(bool split) { return split ? TC_KEYS_SPLIT : TC_KEYS_PLAIN; }
 constexpr int TC_ROW_KEYS = 128;   // keys per tile of the row kernel (lacache_rows.cu)
 constexpr int TC_ROW_ITEM = 256;   // query rows per item of the row kernel (two tiles)
-constexpr int TC_MAX_BLOCK = 64;
-constexpr int TC_DEEP_MAX_UNITS = 512;  // units per CTA the pipelined merge role can tabulate // largest block length the tcgen05 merge role handles
+constexpr int TC_MAX_BLOCK = 64;   // largest block length the tcgen05 merge role handles
+constexpr int TC_DEEP_MAX_UNITS = 512;   // units per CTA the pipelined merge role can tabulate
 
 }  // namespace lacache

@@ -1,8 +1,9 @@
 // Token-wise producer in front of the first-layer attention (Sec. 3.3.2: embedding, attention norm,
 // Q/K/V projections; the rotation of Eq. 1 is applied by the kernels that consume the result).
 //
-// Two kernels:
-//   qkv_norm_kernel  one CTA per token: gathers the token's embedding row (or takes a given hidden
+// Two kernels a call (many tokens, or few heads: the second is proj_kernel of lacache_proj.cu):
+//   qkv_norm_kernel  one CTA per token, each walking several where there are more tokens than resident
+//                    CTAs: gathers the token's embedding row (or takes a given hidden
 //                    state), RMS-normalises it in fp32 and writes the bf16 operand row X^ (and, on
 //                    request, the embedding row itself: what the EmbedCache keeps).
 //   qkv_gemm_kernel  Y^T = W X^T on tcgen05: the 128 output features of one head are the M rows of the
@@ -1063,7 +1064,8 @@ lacache_status project_impl(lacache_qkv* p, const int32_t* token_ids, const void
     // closers take `per_closer` chunks each, helpers about 7/16 of a tile's chunks fewer: a helper's parts have to be
     // published and counted before a closer may fetch them, and a closer's loads speed up once the helpers are through
     // (the weights' stream as a whole is what is limited).  96 heads x 4096, 32 tokens, the whole step from token ids:
-    // 48.8 us at 8 chunks, 48.5 at 16, 48.1 at 24, 47.9 at 28, 47.8 at 32, 47.9 at 40.
+    // 48.8 us at 8 chunks, 48.5 at 16, 48.1 at 24, 47.9 at 28, 47.8 at 32, 47.9 at 40.  (Measured at this one shape; the
+    // split by role is reached with 75 to 147 heads on 148 SMs.)
     const int head_start = ga.kc * 7 / 16;
     const int n_helpers = n_ctas - ga.n_tiles;
     const long long num = ga.total_chunks + (long long)n_helpers * head_start;

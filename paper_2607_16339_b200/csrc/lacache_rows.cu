@@ -351,8 +351,8 @@ __device__ __forceinline__ uint64_t span_bits(int lo, int hi) {   // bits [lo, h
 
 // The O~ row of every thread of a warp, scaled by `mul`, to rows of global memory: state rows (fp32, `stride` D) or
 // output rows, through the warp's 4 KB of staging, 32 features at a time, so that a store instruction writes four rows'
-// 128 contiguous bytes (thread per row, it would touch 32 rows; split planes leave no room for the staging).  `rows`: how many of the warp's rows exist.  have_o: TMEM
-// holds O~ (else zeros).
+// 128 contiguous bytes (thread per row, it would touch 32 rows; split planes leave no room for the staging).  `rows`: how
+// many of the warp's rows exist.  have_o: TMEM holds O~ (else zeros).
 template <bool SPLIT>
 __device__ __forceinline__ void store_rows(const Cta& c, uint32_t o_tmem, bool have_o, float mul, float* dst32,
                                            __nv_bfloat16* dst16, size_t stride, int rows) {

@@ -19,7 +19,7 @@
 //
 // Two roles, chosen per CTA:
 //   stream role  the block queries: a tile of 128 (or 64) query rows streams key
-//                tiles of 128 keys; O~ accumulates in TMEM and is rescaled in
+//                tiles of 128 keys (96 with split planes); O~ accumulates in TMEM and is rescaled in
 //                place only when a row maximum outgrows the reference exponent
 //                (one chunk of key tiles per work unit; the last chunk to finish
 //                merges the partials).
@@ -141,8 +141,8 @@ __device__ __forceinline__ void load_v_box(uint32_t dst, const CUtensorMap* map,
 // One unit of work of the stream role, decoded identically by every warp role.
 // KIND_STEP2: a step whose block-row units all have exactly two key chunks, run by the two CTAs of a
 // thread-block cluster: the CTA with the second chunk hands its partial state to its partner through
-// distributed shared memory, and the partner writes the merged rows (one round of units, unpacked heads,
-// one-plane operands: the receiving buffer needs 32 KB that the split planes' tiles leave no room for).
+// distributed shared memory, and the partner writes the merged rows (one round of units, unpacked heads; the place of the
+// receiving buffer: see Rx).
 enum StreamKind : int { KIND_STEP = 1, KIND_STEP2 = 3 };
 
 struct Unit {
@@ -175,8 +175,8 @@ __device__ __forceinline__ int unit_item(const Geometry& g, const AttnArgs& a, i
 }
 
 // PACKED (a.pack > 1): the units are block queries of several heads side by side in one tile.  A template
-// parameter of the whole kernel, so that the kernel a build or an MHA step runs carries none of the per-row
-// head arithmetic: this kernel is sensitive to its code size.
+// parameter of the whole kernel, so that the kernel an MHA step runs carries none of the per-row head
+// arithmetic: this kernel is sensitive to its code size.
 template <bool PACKED, int KIND, bool SPLIT>
 __device__ __forceinline__ Unit decode_stream(const Geometry& g, const AttnArgs& a, const WorkItem& it, int u) {
   Unit un;
@@ -688,9 +688,8 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
         const int n_mine = v_hi - mc;
         const uint64_t col_bits = n_mine >= 64 ? ~0ull : n_mine <= 0 ? 0ull : (1ull << n_mine) - 1ull;
         const uint32_t s_addr = tlane + TS_S + 128 * b;
-        // This thread's HC scores come out of TMEM once, every load in flight before the one wait (the
-        // time of these threads per tile is what bounds a build: a second pass over TMEM and a wait per
-        // sixteen columns cost more than the registers).  Columns that take no part are set to -inf here,
+        // This thread's HC scores come out of TMEM once, every load in flight before the one wait (a second pass
+        // over TMEM and a wait per sixteen columns cost more than the registers).  Columns that take no part are set to -inf here,
         // so that the maximum and the exponentials below need no per-column tests (the common tile has none).
         uint32_t sr[HC];
 #pragma unroll
@@ -1514,8 +1513,8 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
   const int warp = tid >> 5;
   // In a step with the overlap on, the kernels behind it may be scheduled as SMs free up from here on: they read,
   // before they wait for this grid, only state that stays fixed until the next build and inputs that were
-  // complete long before.  So they may in a short step without it, where they wait first (the planner's rule).  Otherwise
-  // this kernel lets its successor start when it ends.
+  // complete long before.  So they may in a short step without it, where they wait first (the rule: early_trigger in
+  // lacache_plan.h).  Otherwise this kernel lets its successor start when it ends.
   if (a.step_overlap) grid_launch_dependents();
   if (a.span != nullptr && tid == 0) atomicMin(a.span, global_timer_ns());   // first CTA entry of this launch
   Cta c;
