@@ -13,9 +13,10 @@
 //
 // Per element: half a packed maximum, a conversion, half a multiply-add, one exponential, half an addition
 // (f32x2 arithmetic).  The multiply-add forms x log2 e - R with R the rounded m log2 e; what the rounding of R
-// did to every term alike is divided out of the segment's sum at the end.  m log2 e overflows for the lowest and the
-// largest values of the type, which is what a mask may fill in: the pass counts such entries as nothing, which they are
-// beside any other, and a segment that has no other is summed again relative to its maximum.  The index of the
+// did to every term alike is divided out of the segment's sum at the end.  That works while what it did is a factor
+// fp32 can hold: not for an m of -1e10 or the type's lowest value, which is what a mask may fill in.  The pass counts
+// entries of that size as nothing, which they are beside any smaller maximum, and a segment whose maximum is one of them
+// is summed again relative to it.  The index of the
 // maximum costs nothing per element: a thread remembers which batch of its elements raised its maximum, and
 // only the threads that hold the segment's maximum look at their batch again.  (With a compare and two
 // selects per element and CTAs per row rounded to whole slices, 64.7 MB of bf16 logits took 22.6 us; now 16.8, and 49.4 us
@@ -40,7 +41,8 @@ constexpr int WARPS = SAMPLE_THREADS / 32;
 struct Wide { static constexpr int CTAS = 4, DEPTH = 3; };
 struct Deep { static constexpr int CTAS = 3, DEPTH = 5; };
 constexpr float LOG2E = 1.4426950408889634f;
-constexpr float HUGE_LOGIT = 0x1p127f;   // from this magnitude on x log2 e may overflow, and two different values are 2^103 apart
+// Up to here the rounding of m log2 e is at most 2^5: every term and sum is off by at most 2^32, which fp32 holds.
+constexpr float HUGE_LOGIT = 0x1p29f;
 constexpr float FLOAT_MAX = 3.402823466e38f;
 constexpr float LN2F = 0.69314718055994531f;
 
@@ -119,12 +121,12 @@ struct Words<float> {
   }
 };
 
-// 1 for the maximum's equals, 0 otherwise.  (Next to never called, and the kernel's end is its tail: inlined there it took
-// 256 rows of 126464 entries from 16.85 us to 16.95, as a call it leaves 16.75.)
+// The elements i, i + 32, ... relative to a huge maximum.  (Next to never called, and the kernel's end is its tail: inlined
+// there it took 256 rows of 126464 entries from 16.85 us to 16.95, as a call it leaves 16.75.)
 template <class T>
-__device__ __noinline__ float equals_of(const T* x, int i, int hi, float M) {
+__device__ __noinline__ float sum_again(const T* x, int i, int hi, float M) {
   float s = 0.f;
-  for (; i < hi; i += 32) s += ex2f(to_float(x[i]) - M);
+  for (; i < hi; i += 32) s += ex2f((to_float(x[i]) - M) * LOG2E);
   return s;
 }
 
@@ -149,7 +151,7 @@ __global__ void __launch_bounds__(SAMPLE_THREADS, SHAPE::CTAS) sample_rows_kerne
     float m = -INFINITY, R = 0.f, s = 0.f;
     int at = ~0x7fffffff;
     auto raise = [&](float to, int where) {
-      const float Rn = fmaxf(to * LOG2E, -FLOAT_MAX);   // (a huge m: every term is 0, to either side)
+      const float Rn = fabsf(to) < HUGE_LOGIT ? to * LOG2E : INFINITY;   // (a huge m: every term is 0, and so is s)
       s *= ex2f(fminf(R - Rn, 0.f));   // (the first finite logit finds s = 0)
       m = to;
       R = Rn;
@@ -213,9 +215,9 @@ __global__ void __launch_bounds__(SAMPLE_THREADS, SHAPE::CTAS) sample_rows_kerne
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, o));
     if (fabsf(M) >= HUGE_LOGIT && fabsf(M) <= FLOAT_MAX) {   // (the same for the whole warp)
-      s = equals_of<T>(x, lo + lane, hi, M);
+      s = sum_again<T>(x, lo + lane, hi, M);
     } else {
-      s = m == -INFINITY ? 0.f : s * ex2f((m - M) * LOG2E - fmaf(m, LOG2E, -R));
+      s = m == -INFINITY ? 0.f : fabsf(m) < HUGE_LOGIT ? s * ex2f((m - M) * LOG2E - fmaf(m, LOG2E, -R)) : s;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);

@@ -123,6 +123,47 @@ def test_entries_masked_with_the_lowest_value_of_the_type(dtype, vocab):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("size", [1e8, 5e8, 6e8, 1e9, 1e10, 1e30, 1.6e38])
+def test_entries_of_any_size_as_a_mask(dtype, size):
+    """Finite masks of every size in use (the rounding of a large maximum times log2 e is itself large), and as large logits:
+    below, at and above the size from which a segment is summed relative to its maximum."""
+    vocab = 5003
+    wl = small_workload(name="samp-mask", prompt_lens=(21,), gen_len=32, block_len=16, steps=1, hq=2, hkv=2)
+    ctx, sch = _built_ctx(wl, 0)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    logits = (torch.randn(wl.total_tokens, vocab, generator=g, device="cuda") * 4).to(dtype)
+    at = sch.block_rows(0)
+    logits[at[0], : vocab // 2] = -size
+    logits[at[1], vocab // 2:] = -size
+    logits[at[2], ::2] = -size
+    logits[at[3], : vocab - 1] = -size
+    logits[at[4]] = -size
+    logits[at[5]] = -size
+    logits[at[5], vocab // 2:] = -size * 1.02
+    logits[at[6], vocab // 3] = size
+    logits[at[7], ::7] = size
+    logits[at[8], ::7] = size
+    logits[at[8], 1] = size * 1.02
+    near = torch.tensor(float(size), dtype=dtype, device="cuda")
+    for k in range(40):                               # neighbouring values of the type: their differences count
+        logits[at[9], 100 * k] = near
+        logits[at[10], 100 * k] = -near
+        near = torch.nextafter(near.float(), torch.tensor(0.0, device="cuda")).to(dtype) if dtype == torch.float32 else near * 0.99
+    n = at.shape[0]
+    conf, lse = torch.empty(n, device="cuda"), torch.empty(n, device="cuda")
+    tok = torch.empty(n, device="cuda", dtype=torch.int32)
+    ctx.sample_block(logits, conf, tok, lse)
+    torch.cuda.synchronize()
+    assert ctx.poll_status()[0] == 0
+    ref_tok, ref_conf, ref_lse = sampler.block_confidence(logits.float().cpu().numpy().astype(np.float64), at)
+    assert np.array_equal(tok.cpu().numpy().astype(np.int64), ref_tok)
+    c, l = conf.cpu().numpy().astype(np.float64), lse.cpu().numpy().astype(np.float64)
+    assert np.all(np.abs(c - ref_conf) <= 2e-5 * ref_conf), (c, ref_conf)
+    assert np.all(np.abs(l - ref_lse) <= 2e-5 * np.maximum(1.0, np.abs(ref_lse))), (l, ref_lse)
+    ctx.destroy()
+
+
 def test_full_size_block_and_vocabulary():
     """The headline configuration's block (32 rows) and the large-batch extension's (8192 rows) at a
     vocabulary of 126464 entries (bf16 logits of every token would not fit for the latter: its logits
