@@ -1,5 +1,5 @@
-// Host-side planning without state: the work lists of the row kernel (lacache_rows.cu), made when a context is created, and
-// the rule of the early trigger.  Host code only.
+// Host-side planning without state: the work lists of the row kernel (lacache_rows.cu), made when a context is created, the
+// rule of the early trigger, and the split by role of the projection (lacache_qkv.cu).  Host code only.
 #pragma once
 #include <algorithm>
 #include <vector>
@@ -102,6 +102,26 @@ inline std::vector<Range> add_build_lists(std::vector<WorkItem>& items, const in
     }
   }
   return ranges;
+}
+
+// The projection of a block's tokens, n_tiles tiles of kc chunks on n_ctas CTAs: how many chunks of every tile the helpers
+// share (the closers, one per tile, take the rest); 0: no split by role.
+// Closers take `per_closer` chunks each, helpers about 7/16 of a tile's chunks fewer: a helper's parts have to be
+// published and counted before a closer may fetch them, and a closer's loads speed up once the helpers are through
+// (the weights' stream as a whole is what is limited).  96 heads x 4096, 32 tokens, the whole step from token ids:
+// 48.8 us at 8 chunks, 48.5 at 16, 48.1 at 24, 47.9 at 28, 47.8 at 32, 47.9 at 40.  (Measured at this one shape; the
+// split by role is reached with 75 to about 100 heads on 148 SMs.)
+// A helper publishes a partial tile for every tile its range touches and has `max_parts` places for them.  With more than
+// about two tiles per helper it would need more: then there is no split by role.
+inline int helper_chunks(int n_ctas, int n_tiles, int kc, int max_parts) {
+  if (n_ctas <= n_tiles || n_ctas >= 2 * n_tiles) return 0;
+  const int head_start = kc * 7 / 16, n_helpers = n_ctas - n_tiles;
+  const long long num = (long long)n_tiles * kc + (long long)n_helpers * head_start;
+  const int hp = kc - (int)((num + n_ctas - 1) / n_ctas);
+  if (hp < 1 || (long long)n_tiles * hp < n_helpers) return 0;
+  const long long longest = ((long long)n_tiles * hp + n_helpers - 1) / n_helpers;   // a helper's range
+  if ((longest - 1 + hp - 1) / hp + 1 > max_parts) return 0;   // (one that starts in a tile's last chunk touches the most)
+  return hp;
 }
 
 }  // namespace plan

@@ -34,6 +34,7 @@
 #include <new>
 
 #include "lacache_internal.h"
+#include "lacache_plan.h"
 #include "lacache_proj.h"
 #include "lacache_ptx.h"
 
@@ -97,7 +98,7 @@ struct GemmArgs {
   int n_tokens, tn, n_ttiles, n_tiles, kc;   // kc = d_model / 64 chunks per tile
   long long total_chunks;
   // Closer / helper split (hp > 0), used when there are more CTAs than tiles and fewer than twice as
-  // many: n_tiles of the CTAs ("closers", the high block indices) own the last kc - hp chunks of one tile
+  // many (the rule: helper_chunks in lacache_plan.h): n_tiles of the CTAs ("closers", the high block indices) own the last kc - hp chunks of one tile
   // each and finish it; the other CTAs ("helpers", placed first) share the first hp chunks of all tiles
   // in equal contiguous ranges and only publish partial tiles.  Helpers start earlier and get less work
   // than closers, so their parts are published by the time a closer is through: the closer fetches them
@@ -1059,20 +1060,7 @@ lacache_status project_impl(lacache_qkv* p, const int32_t* token_ids, const void
   ga.counters = p->counters;
   ga.status = p->status;
   const int n_ctas = (int)std::min<long long>(p->num_sms, ga.total_chunks);
-  ga.hp = 0;
-  if (n_ctas > ga.n_tiles && n_ctas < 2 * ga.n_tiles && !p->plain_split) {
-    // closers take `per_closer` chunks each, helpers about 7/16 of a tile's chunks fewer: a helper's parts have to be
-    // published and counted before a closer may fetch them, and a closer's loads speed up once the helpers are through
-    // (the weights' stream as a whole is what is limited).  96 heads x 4096, 32 tokens, the whole step from token ids:
-    // 48.8 us at 8 chunks, 48.5 at 16, 48.1 at 24, 47.9 at 28, 47.8 at 32, 47.9 at 40.  (Measured at this one shape; the
-    // split by role is reached with 75 to 147 heads on 148 SMs.)
-    const int head_start = ga.kc * 7 / 16;
-    const int n_helpers = n_ctas - ga.n_tiles;
-    const long long num = ga.total_chunks + (long long)n_helpers * head_start;
-    const int per_closer = (int)((num + n_ctas - 1) / n_ctas);
-    const int hp = ga.kc - per_closer;
-    if (hp >= 1 && (long long)ga.n_tiles * hp >= n_helpers) ga.hp = hp;
-  }
+  ga.hp = p->plain_split ? 0 : plan::helper_chunks(n_ctas, ga.n_tiles, ga.kc, WS_SLOTS);
 
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(n_ctas);

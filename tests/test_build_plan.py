@@ -1,5 +1,6 @@
 """Host-side planning (csrc/lacache_plan.h).  The build's work lists: every row once, the most work first, each block's list
-what planning that block alone gives -- and planned once per context, not once per block.  The rule of the early trigger."""
+what planning that block alone gives -- and planned once per context, not once per block.  The rule of the early trigger.
+The projection's split by role: what its helpers publish fits the places they have."""
 import os
 import subprocess
 
@@ -25,6 +26,27 @@ int main(int argc, char** argv) {
     for (int b = 0; b < B; ++b) start[(size_t)k * B + b] = cu[b] + atoi(argv[6 + b]) + k * L;
   std::vector<WorkItem> items;
   auto lists = [&](int k0, int n) { return add_build_lists(items, cu.data(), B, L, start.data() + (size_t)k0 * B, n, heads, sms); };
+  if (mode == 4) {   // helper_chunks(heads = CTAs, sms = tiles, L = chunks, n_blk = places): "hp" and, where it splits, its two extremes
+    const int n_ctas = heads, places = n_blk;
+    for (int tiles = 1; tiles <= sms; ++tiles)
+      for (int kc = 1; kc <= L; ++kc) {
+        const int hp = helper_chunks(n_ctas, tiles, kc, places);
+        if (hp == 0) continue;
+        const int nh = n_ctas - tiles;
+        const long long total = (long long)tiles * hp;
+        int most_tiles = 0, most_parts = 0;
+        std::vector<int> parts(tiles, 0);
+        bool empty = false;
+        for (int j = 0; j < nh; ++j) {   // the ranges as the kernel cuts them
+          const long long a = j * total / nh, b = (j + 1) * total / nh;
+          empty |= b <= a;
+          most_tiles = std::max(most_tiles, (int)((b - 1) / hp - a / hp + 1));
+          for (long long t = a / hp; t <= (b - 1) / hp; ++t) most_parts = std::max(most_parts, ++parts[t]);
+        }
+        printf("%d %d %d %d %d %d\n", tiles, kc, hp, most_tiles, most_parts, empty ? 1 : 0);
+      }
+    return 0;
+  }
   if (mode == 3) {   // early_trigger over its four arguments, the first the lowest bit
     for (int i = 0; i < 16; ++i) printf("%d", early_trigger(i & 1, i & 2, i & 4, i & 8) ? 1 : 0);
     return 0;
@@ -109,3 +131,14 @@ def test_early_trigger_rule(harness):
     want = "".join(str(int(not off and (overlap or (short and not producer))))
                    for off in (0, 1) for producer in (0, 1) for short in (0, 1) for overlap in (0, 1))
     assert got == want
+
+
+def test_the_parts_of_a_helper_fit_its_places(harness):
+    """Every number of heads and every reduction length: a helper touches at most the three tiles it has places for, a
+    closer adds at most three parts, no helper is without work; and the width the split is made for still splits."""
+    rows = [tuple(int(x) for x in line.split()) for line in harness(4, 148, 200, 128, 3, (1,)).splitlines()]
+    for tiles, kc, hp, most_tiles, most_parts, empty in rows:
+        assert 1 <= hp < kc and most_tiles <= 3 and most_parts <= 3 and not empty, (tiles, kc, hp, most_tiles, most_parts)
+    split = {(t, kc): hp for t, kc, hp, *_ in rows}
+    assert split[(96, 64)] == 12 and (96, 32) in split and (84, 56) in split
+    assert (108, 33) not in split and (120, 64) not in split

@@ -26,3 +26,21 @@ def test_token_counts_and_head_counts(hq, hkv, d_model, n):
         assert st == binding.OK, msg
     check_qkv(tm, q, k, v, ids=ids, what="n=%d" % n)
     prod.destroy()
+
+
+@pytest.mark.parametrize("hq,hkv,d_model,n", [
+    (36, 36, 2112, 6), (36, 36, 2112, 33),       # 108 tiles on 148 SMs: more than two tiles per helper
+    (40, 40, 1024, 32), (46, 46, 512, 17),       # 120; 138
+    (32, 32, 1024, 32), (33, 33, 1024, 31),      # 96 and 99: two tiles per helper, and just above
+])
+def test_few_tokens_of_models_with_many_heads(hq, hkv, d_model, n):
+    """The projection of a block's tokens on both sides of where its work is split by role, repeatedly (parts that land in
+    another CTA's place show up now and then only)."""
+    tm = TokenModel(W.small_workload(hq=hq, hkv=hkv), d_model, 500)
+    prod = make_producer(tm, n)
+    for rep in range(4):
+        ids = np.random.default_rng(rep).integers(0, tm.vocab, n).astype(np.int32)
+        st, msg, q, k, v, _ = project(prod, tm, n, ids=ids)
+        assert st == binding.OK, msg
+        check_qkv(tm, q, k, v, ids=ids, what="rep %d" % rep)
+    prod.destroy()
