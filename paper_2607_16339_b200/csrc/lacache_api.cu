@@ -28,10 +28,10 @@ struct lacache_ctx {
   struct ListRef { int off, n; };
   std::vector<ListRef> build_list, step_list;  // per block (step_list: SIMT all items; tcgen05 block-chunk items)
   std::vector<ListRef> merge_list;             // per block: fixed-row items of a step (tcgen05)
-  // per block, tcgen05: row tiles x key windows of the incremental build (prefix state from scratch;
+  // per block, tcgen05: row tiles x key windows of the incremental build (prefix state from scratch, and on to the
   // cached state = prefix state + the keys after the block; the finished block's rows from scratch;
   // every other row advanced by the finished block's keys and completed by the keys after the block)
-  std::vector<ListRef> inc_prefix, inc_comb, inc_fresh, inc_fresh_chunks, inc_fused;
+  std::vector<ListRef> inc_build, inc_fresh, inc_fresh_chunks, inc_fused;
   // per block, tile-granular caching (Algorithm 1's overlap predicates): the build in two launches over
   // the key tiles before / after the tiles that overlap the block, the step in one
   std::vector<ListRef> tile_prefix, tile_suffix, tile_step;
@@ -39,7 +39,11 @@ struct lacache_ctx {
   float* sample_part = nullptr;   // scratch of lacache_sample_block (allocated on first use)
   int* sample_counters = nullptr;
   StateBuffers pst{};      // prefix state of every token: its keys before the current block (allocated on first use)
-  int prefix_block = -1;   // block pst is valid for
+  int prefix_block = -1;   // block the incremental build or advance last left pst for
+  // [2][B], by the block's parity: the token up to which the rows' states in pst hold the keys.  An advance adds the keys
+  // since, and stores the states again only when one key tile would no longer hold them.  On the device, so that a
+  // captured advance follows whatever was built before it.
+  int32_t* d_pst_end = nullptr;
   int num_sms = 148;
   // experiment knobs, read from the environment once at create (none is needed in normal use)
   struct Knobs {
@@ -373,36 +377,28 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
     // [cs, ce): the prefix state holds keys [cs, s); the cached state adds keys [e, ce); advancing
     // from block k - 1 adds that block's keys [s - L_b, s) to the rows outside it and computes the
     // rows inside it (whose queries changed) over [cs, s) from scratch.
-    auto window = [&](int from, int base, int k0, int k1, int flags) {
+    auto window = [&](int from, int base, int k0, int k1, int flags, int n_before = 0) {
       for (size_t i = from; i < items.size(); ++i) {
         items[i].kind = ITEM_ROWS_WINDOW;
         items[i].pad = base;
         items[i].kt0 = k0;
         items[i].kt1 = k1;
         items[i].chunk = flags;
+        items[i].n_before = n_before;
       }
     };
-    enum { W_INIT = 1, W_SNAP = 2, W_JUMP_BLOCK = 8 };
+    enum { W_INIT = 1, W_SNAP = 2, W_JUMP_BLOCK = 8, W_GROW = 32 };
     int off = (int)items.size();
     for (int b = 0; b < g.B; ++b) {
+      // the keys before the block = prefix state, stored; + the keys after it = cached state
       const int cs = c->cu[b], ce = c->cu[b + 1], s0 = c->blk_start_all[(size_t)k * g.B + b], e0 = s0 + g.block_len;
-      const int from = (int)items.size();
+      const int from = (int)items.size(), before = (s0 - cs + RI_KEYS - 1) / RI_KEYS;
       add_row_tiles(items, b, cs, s0, RI, cs, ce, s0);
       add_row_tiles(items, b, e0, ce, RI, cs, ce, s0);
-      window(from, cs, cs, s0, 0);
+      window(from, s0 - before * RI_KEYS, cs, ce > e0 ? ce : s0, W_SNAP | W_JUMP_BLOCK, before);
     }
     longest_first(off);
-    c->inc_prefix.push_back({off, (int)items.size() - off});
-    off = (int)items.size();
-    for (int b = 0; b < g.B; ++b) {
-      const int cs = c->cu[b], ce = c->cu[b + 1], s0 = c->blk_start_all[(size_t)k * g.B + b], e0 = s0 + g.block_len;
-      const int from = (int)items.size();
-      add_row_tiles(items, b, cs, s0, RI, cs, ce, s0);
-      add_row_tiles(items, b, e0, ce, RI, cs, ce, s0);
-      window(from, e0, e0, ce, W_INIT);
-    }
-    longest_first(off);
-    c->inc_comb.push_back({off, (int)items.size() - off});
+    c->inc_build.push_back({off, (int)items.size() - off});
     // advancing from block k - 1 (rows [sp, s0), blocks are consecutive), in two launches:
     off = (int)items.size();
     for (int b = 0; b < g.B && k > 0; ++b) {
@@ -443,17 +439,13 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
     off = (int)items.size();
     for (int b = 0; b < g.B && k > 0; ++b) {
       const int cs = c->cu[b], ce = c->cu[b + 1], s0 = c->blk_start_all[(size_t)k * g.B + b], e0 = s0 + g.block_len;
-      const int sp = s0 - g.block_len;
-      // every other fixed row: old prefix state + the finished block's keys (exactly the first key
-      // tile, which ends at s0) = new prefix state, stored; + the keys after block k = cached state
-      int from = (int)items.size();
-      add_row_tiles(items, b, cs, sp, RI, cs, ce, s0);
+      // stored prefix state + the keys of the blocks finished since it was stored (within the first key tile, which
+      // ends at s0; none for the rows of the block finished last) = prefix state, stored again only when the next
+      // block's keys would not fit that tile as well; + the keys after block k = cached state
+      const int from = (int)items.size();
+      add_row_tiles(items, b, cs, s0, RI, cs, ce, s0);
       add_row_tiles(items, b, e0, ce, RI, cs, ce, s0);
-      window(from, s0 - RI_KEYS, sp, ce > e0 ? ce : s0, W_INIT | W_SNAP | W_JUMP_BLOCK);
-      // the finished block's rows: their new prefix state + the keys after block k
-      from = (int)items.size();
-      add_row_tiles(items, b, sp, s0, RI, cs, ce, s0);
-      window(from, e0, e0, ce, W_INIT);
+      window(from, s0 - RI_KEYS, s0 - RI_KEYS, ce > e0 ? ce : s0, W_INIT | W_SNAP | W_JUMP_BLOCK | W_GROW, 1);
     }
     longest_first(off);
     c->inc_fused.push_back({off, (int)items.size() - off});
@@ -906,6 +898,7 @@ lacache_status ensure_prefix_state(lacache_ctx* c) {
     return fail(c, LACACHE_ERR_UNSUPPORTED, "the incremental build is token-granular only");
   if (c->pst.o) return LACACHE_OK;
   const Geometry& g = c->g;
+  CU_TRY(c, dev_alloc(c, &c->d_pst_end, (size_t)2 * g.B, true));
   CU_TRY(c, dev_alloc(c, &c->pst.m, (size_t)g.Hq * g.Tp, true));
   CU_TRY(c, dev_alloc(c, &c->pst.l, (size_t)g.Hq * g.Tp, true));
   CU_TRY(c, dev_alloc(c, &c->pst.o, (size_t)g.Hq * g.Tp * g.d, true));
@@ -939,12 +932,16 @@ lacache_status run_block_rows_to_state(lacache_ctx* c, lacache_ctx::ListRef list
 
 lacache_status run_window(lacache_ctx* c, lacache_ctx::ListRef list, int blk, const StateBuffers& init,
                           const StateBuffers& dst, const StateBuffers& snap, cudaStream_t s, float* out, float* lse) {
-  if (list.n == 0) return LACACHE_OK;
+  if (list.n == 0) return LACACHE_OK;   // (a sequence of several blocks always has fixed rows)
   AttnArgs a = attn_args(c, MODE_BUILD, list, blk, c->rot, out, lse);
   a.window = 1;
   a.init = init;
   a.st = dst;
   a.snap = snap;
+  if (snap.o) {   // an incremental build or an advance
+    a.state_end = init.o ? c->d_pst_end + (size_t)((blk - 1) & 1) * c->g.B : nullptr;
+    a.state_end_out = c->d_pst_end + (size_t)(blk & 1) * c->g.B;
+  }
   return run_attention(c, a, false, s);
 }
 }  // namespace
@@ -964,9 +961,7 @@ lacache_status lacache_build_incremental(lacache_ctx* c, int block_idx, const vo
   c->prefix_block = -1;
   st = rope_all(c, q, k, v, c->rot, s);
   if (st != LACACHE_OK) return st;
-  st = run_window(c, c->inc_prefix[block_idx], block_idx, StateBuffers{}, c->pst, StateBuffers{}, s);
-  if (st != LACACHE_OK) return st;
-  st = run_window(c, c->inc_comb[block_idx], block_idx, c->pst, c->st, StateBuffers{}, s);
+  st = run_window(c, c->inc_build[block_idx], block_idx, StateBuffers{}, c->st, c->pst, s);
   if (st != LACACHE_OK) return st;
   c->built_block = block_idx;
   c->prefix_block = block_idx;

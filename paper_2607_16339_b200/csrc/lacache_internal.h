@@ -15,9 +15,10 @@ enum ItemKind : int32_t {
   ITEM_ROWS_WINDOW = 2,  // (build) a tile of query rows x the keys [kt0, kt1) of its sequence, given as token
                          // indices; key tiles are counted from token `pad` (<= kt0, may be negative).
                          // chunk bit 0: continue from the rows' state in AttnArgs::init; bit 1: store the
-                         // state after the first key tile to AttnArgs::snap; bit 3: the first tile ends at
-                         // blk_start (pad = blk_start - tile width) and the tiles after it are counted from the
-                         // end of that block; bit 4: the unit writes normalised rows to out / lse instead of a state
+                         // state over the keys before the block to AttnArgs::snap; bit 3: the first n_before tiles
+                         // end at blk_start (pad = blk_start - n_before tiles) and the tiles after them are counted
+                         // from the end of that block; bit 4: the unit writes normalised rows to out / lse instead of a state;
+                         // bit 5: the first tile's keys are those the row's stored state lacks (AttnArgs::state_end)
 };
 struct WorkItem {
   int32_t kind;   // ItemKind
@@ -31,7 +32,7 @@ struct WorkItem {
   int32_t seq_start;  // first packed token of the sequence
   int32_t seq_end;    // one past its last token
   int32_t blk_start;  // first packed token of the sequence's current block
-  int32_t pad2;
+  int32_t n_before;   // ITEM_ROWS_WINDOW, bit 3: key tiles before the block
 };
 
 // What a launch computes for ITEM_ROWS items.
@@ -127,8 +128,10 @@ struct AttnArgs {
   StateBuffers st;
   int window;                // build: the items are ITEM_ROWS_WINDOW (the kernel instantiation that knows them)
   StateBuffers init;         // build over key windows: the state units with the init bit start from (may alias st)
-  StateBuffers snap;         // ... and where units with the snapshot bit store their state after the first key tile
-                             // (may alias init: a unit loads its rows before it stores them)
+  StateBuffers snap;         // ... and where units with the snapshot bit store their state over the keys before the
+                             // block (may alias init: a unit loads its rows before it stores them)
+  const int32_t* state_end;  // [B] bit 5 of an item: the token up to which the sequence's stored states hold the keys
+  int32_t* state_end_out;    // [B] where the launch notes that for the states it leaves (null: it does not)
   float* out; float* lse;    // token-major [T,Hq,d], [T,Hq]
   int out_bf16;              // `out` holds bf16 elements (lse stays fp32)
   // split-key partial states of block queries and their arrival counters

@@ -25,6 +25,11 @@
 // 1536 tokens x 32 heads, split planes: 84 / 76.  Bound by the row threads and by the chain probabilities -> products ->
 // scores about equally: without the exponentials 278 us, with a quarter of the products 267, with neither 170.
 //
+// Key windows (incremental build and advance, 28/4 heads x 5120 rows, one fp16 plane; before / now): the incremental build in
+// one launch, the state before the block stored on the way, 282 + 72 / 327 us; an advance, where a unit has four key tiles
+// and moves 128 KB of state each way, 85 / 70 us, 84 when it stores the prefix states again (every second block of 64 rows,
+// every fourth of 32).  Bound by the transfers of state, which every CTA makes at the same time.
+//
 // Arithmetic as in lacache_tc.cu: integer reference exponent, moved only when the row's maximum outgrows it by more
 // than RESCALE_SLACK; P~ rounded to fp16, the normaliser sums the rounded values.
 #include <algorithm>
@@ -83,10 +88,12 @@ struct Unit {
   int row0, nrows, h, kh;
   int key_base, n_tiles;  // key tile t holds keys key_base + 128 t ... (or see base1)
   int k0, k1, x0, x1;     // valid keys [k0, k1) minus [x0, x1)
-  int base1;              // >= 0: tiles after the first are counted from this token
-  bool init, snap, out;   // start from a stored state; store the state after the first tile; write normalised rows
+  int n1, base1;          // tiles from the n1-th on are counted from token base1
+  int seq, blk;           // sequence, and the first token of its current block
+  bool grow;              // the first tile adds the keys the row's stored state lacks (first_key)
+  bool init, snap, out;   // start from a stored state; store the state after n1 tiles; write normalised rows
   __device__ __forceinline__ int tiles() const { return nrows > BM ? 2 : 1; }
-  __device__ __forceinline__ int key_row(int t) const { return (base1 >= 0 && t > 0) ? base1 + (t - 1) * KT : key_base + t * KT; }
+  __device__ __forceinline__ int key_row(int t) const { return t >= n1 ? base1 + (t - n1) * KT : key_base + t * KT; }
 };
 
 // A CTA's units: the list, sorted by work, is dealt out in a snake, so that who draws first in one round draws last in
@@ -98,8 +105,7 @@ struct Walk {
 
 // units are head-minor (unit u = item u / Hq of head u % Hq): neighbours share keys in L2
 template <bool WINDOW>
-__device__ __forceinline__ Unit decode(const Geometry& g, const AttnArgs& a, int u) {
-  const WorkItem it = load_item(a.items + u / g.Hq);
+__device__ __forceinline__ Unit decode(const Geometry& g, const AttnArgs& a, int u, const WorkItem& it) {
   Unit un;
   un.h = u % g.Hq;
   un.kh = un.h / g.group;
@@ -108,8 +114,11 @@ __device__ __forceinline__ Unit decode(const Geometry& g, const AttnArgs& a, int
   un.key_base = un.k0 = it.seq_start;
   un.k1 = it.seq_end;
   un.x0 = un.x1 = 0;
-  un.base1 = -1;
-  un.init = un.snap = false;
+  un.n1 = 1 << 30;
+  un.base1 = 0;
+  un.seq = it.seq;
+  un.blk = it.blk_start;
+  un.init = un.snap = un.grow = false;
   un.out = a.mode == MODE_FULL;
   un.n_tiles = (it.seq_end - it.seq_start + KT - 1) / KT;
   if (WINDOW) {
@@ -117,18 +126,36 @@ __device__ __forceinline__ Unit decode(const Geometry& g, const AttnArgs& a, int
     un.k0 = it.kt0;
     un.k1 = it.kt1;
     un.n_tiles = it.kt1 > it.pad ? (it.kt1 - it.pad + KT - 1) / KT : 0;
-    if (it.chunk & 8) {   // the first tile ends where the block starts; the others start right after the block
+    if (it.chunk & 8) {   // the first tiles end where the block starts; the others start right after the block
+      un.n1 = it.n_before;
       un.base1 = it.blk_start + g.block_len;
-      un.n_tiles = 1 + (it.kt1 > un.base1 ? (it.kt1 - un.base1 + KT - 1) / KT : 0);
+      un.n_tiles = un.n1 + (it.kt1 > un.base1 ? (it.kt1 - un.base1 + KT - 1) / KT : 0);
     }
     un.init = it.chunk & 1;
     un.snap = (it.chunk >> 1) & 1;
     un.out = (it.chunk & 16) != 0;
+    un.grow = (it.chunk & 32) != 0;
   } else if (a.mode == MODE_BUILD) {
     un.x0 = it.blk_start;
     un.x1 = it.blk_start + g.block_len;
   }
   return un;
+}
+
+template <bool WINDOW>
+__device__ __forceinline__ Unit decode(const Geometry& g, const AttnArgs& a, int u) {
+  return decode<WINDOW>(g, a, u, load_item(a.items + u / g.Hq));
+}
+// load_item in two: the loads (here, and not where the words are first used), and the item
+__device__ __forceinline__ void ask_item(const AttnArgs& a, int i, int4 (&w)[3]) {
+  const WorkItem* p = a.items + min(i, a.n_items - 1);
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    asm volatile("ld.global.nc.v4.s32 {%0, %1, %2, %3}, [%4];" : "=r"(w[k].x), "=r"(w[k].y), "=r"(w[k].z), "=r"(w[k].w)
+                 : "l"(reinterpret_cast<const int4*>(p) + k));
+}
+__device__ __forceinline__ WorkItem as_item(const int4 (&w)[3]) {
+  return WorkItem{w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w, w[2].x, w[2].y, w[2].z, w[2].w};
 }
 
 // wait_bar without a call: a row thread has most of its registers in use where it waits
@@ -152,11 +179,30 @@ __device__ __forceinline__ bool wait_here(const Cta& c, int slot, uint32_t parit
 // ---- producers ----------------------------------------------------------------------------------------------
 // One lane each for Q' tiles, key tiles and value tiles, with blocking waits (one lane that polled all three took several
 // hundred cycles to notice a free stage, which with two stages is time the tensor core waits).
+// The stored state a unit starts from (one contiguous run of its rows), asked into L2.
+__device__ __forceinline__ void prefetch_state(const Geometry& g, const AttnArgs& a, const Unit& un) {
+  const size_t srow = (size_t)un.h * g.Tp + un.row0;
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.init.o + srow * D), "r"(un.nrows * D * 4) : "memory");
+  for (int i = 0; i < un.nrows; i += 32) {
+    prefetch_l2(a.init.m + srow + i);
+    prefetch_l2(a.init.l + srow + i);
+  }
+}
 template <bool SPLIT, bool WINDOW>
 __device__ void load_queries(const Cta& c, const RowMaps& maps, const Geometry& g, const AttnArgs& a, const Walk& wk) {
   int n0 = 0, n1 = 0;   // Q' tiles loaded, per tile slot
   for (int k_ = 0, u = wk.unit(0); u < wk.n_units; u = wk.unit(++k_)) {
     const Unit un = decode<WINDOW>(g, a, u);
+    if (WINDOW) {
+      // The state of the next unit: this one's Q' is requested when the unit before has no more scores to issue, so
+      // its rows have a unit's time to come into L2 before the row threads ask for them.
+      if (k_ == 0 && un.init) prefetch_state(g, a, un);
+      const int u2 = wk.unit(k_ + 1);
+      if (u2 < wk.n_units) {
+        const Unit nx = decode<WINDOW>(g, a, u2);
+        if (nx.init) prefetch_state(g, a, nx);
+      }
+    }
     if (un.n_tiles == 0) continue;
     for (int x = 0; x < un.tiles(); ++x) {
       const int n = x ? n1 : n0;
@@ -349,6 +395,40 @@ __device__ __forceinline__ uint64_t span_bits(int lo, int hi) {   // bits [lo, h
   return (hi - lo == 64 ? ~0ull : ((1ull << (hi - lo)) - 1ull)) << lo;
 }
 
+// Rows of a stored state (the warp's first `rows`; zeros behind them) to the warp's lanes of O~ in TMEM: all loads leave
+// together, 128 contiguous bytes of four rows each, and pass through the warp's staging (thread per row, a load would
+// touch 32 rows).  Split planes have no staging.  (Plain loads: the launch may update these rows in place.)
+template <bool SPLIT>
+__device__ __forceinline__ void load_rows(const Cta& c, uint32_t o_tmem, const float* src, int rows) {
+  const int lane = threadIdx.x & 31;
+  uint4 w[4][8];
+#pragma unroll
+  for (int cb = 0; cb < 4; ++cb)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int rr = SPLIT ? lane : 4 * i + (lane >> 3), ch = SPLIT ? i : lane & 7;
+      w[cb][i] = make_uint4(0u, 0u, 0u, 0u);
+      if (rr < rows) w[cb][i] = __ldcg(reinterpret_cast<const uint4*>(src + (size_t)rr * D + 32 * cb + 4 * ch));
+    }
+  uint8_t* const st = c.gen + Lay<false>::SM_ST + (threadIdx.x >> 5) * 4096;
+#pragma unroll
+  for (int cb = 0; cb < 4; ++cb) {
+    if constexpr (!SPLIT) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int rr = 4 * i + (lane >> 3), ch = lane & 7;
+        *reinterpret_cast<uint4*>(st + rr * 128 + ((ch ^ (rr & 7)) << 4)) = w[cb][i];
+      }
+      __syncwarp();
+#pragma unroll
+      for (int i = 0; i < 8; ++i) w[cb][i] = *reinterpret_cast<const uint4*>(st + lane * 128 + ((i ^ (lane & 7)) << 4));
+      __syncwarp();
+    }
+    tmem_st32(o_tmem + 32 * cb, *reinterpret_cast<uint32_t(*)[32]>(w[cb]));
+  }
+  tmem_st_wait();
+}
+
 // The O~ row of every thread of a warp, scaled by `mul`, to rows of global memory: state rows (fp32, `stride` D) or
 // output rows, through the warp's 4 KB of staging, 32 features at a time, so that a store instruction writes four rows'
 // 128 contiguous bytes (thread per row, it would touch 32 rows; split planes leave no room for the staging).  `rows`: how
@@ -420,10 +500,17 @@ __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, 
   const uint32_t s_tmem = tlane + TM_S(x), p_tmem = tlane + TM_S(x), o_tmem = tlane + TM_O(x);
   int n = 0, units = 0;                            // key tiles and units (with key tiles) of this tile slot so far
   bool waited = false;                             // for the grids ahead
+  // The item of the unit at hand: its words are asked for before the unit ahead of it stores its rows, and read after that
+  // (asked for where they are used, 1500 to 3000 cycles of the 35000 of an advance's unit at 5120 tokens).
+  int4 item[3];
+  ask_item(a, wk.unit(0) / g.Hq, item);
   for (int k_ = 0, u = wk.unit(0); u < wk.n_units; u = wk.unit(++k_)) {
-    const Unit un = decode<WINDOW>(g, a, u);
+    const Unit un = decode<WINDOW>(g, a, u, as_item(item));
     const int n_rows = min(un.nrows - BM * x, BM);
-    if (n_rows <= 0) continue;                     // (a unit of one tile)
+    if (n_rows <= 0) {                             // (a unit of one tile)
+      ask_item(a, wk.unit(k_ + 1) / g.Hq, item);
+      continue;
+    }
     const int warp_rows = min(n_rows - 32 * quad, 32);   // rows of this warp (<= 0: none)
     const bool valid = r < n_rows;
     const int row = un.row0 + BM * x + r;
@@ -431,36 +518,35 @@ __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, 
     float m_ref = -INFINITY, l = 0.f;
     bool have_o = false;                           // O~ in TMEM holds something
     if (WINDOW && un.init) {
-      if (!waited) { grid_dependency_wait(); waited = true; }
       // The unit continues from a stored state of its rows.  Nobody else touches this tile's O~ between units (the
       // previous unit's products are complete, and these threads have read its O~).
-      if (valid) { m_ref = a.init.m[srow]; l = a.init.l[srow]; }
+      if (!waited) { grid_dependency_wait(); waited = true; }
+      if (valid) { m_ref = __ldcg(a.init.m + srow); l = __ldcg(a.init.l + srow); }
       if (un.n_tiles > 0) {
-#pragma unroll 1
-        for (int h2 = 0; h2 < 2; ++h2) {
-          uint32_t o[64];
-#pragma unroll
-          for (int i = 0; i < 64; ++i) o[i] = 0u;
-          if (valid) {   // (plain loads: the launch may update these rows in place)
-#pragma unroll
-            for (int i = 0; i < 8; ++i) ld_global_v8(a.init.o + srow * D + 64 * h2 + 8 * i, o + 8 * i);
-          }
-          tmem_st32(o_tmem + 64 * h2, *reinterpret_cast<uint32_t(*)[32]>(o));
-          tmem_st32(o_tmem + 64 * h2 + 32, *reinterpret_cast<uint32_t(*)[32]>(o + 32));
-        }
-        tmem_st_wait();
+        if (warp_rows > 0) load_rows<SPLIT>(c, o_tmem, a.init.o + (srow - lane) * D, warp_rows);
         have_o = true;
       }
+    }
+    // The first key the row's stored state lacks.  Rows outside the blocks finished since the states were last stored have
+    // the keys before those blocks; a finished block's rows were computed anew, over their own block too.
+    int k0 = un.k0;
+    bool snap = WINDOW && un.snap;
+    if (WINDOW && un.grow) {
+      const int before = __ldcg(a.state_end + un.seq);   // where the stored states of the sequence end
+      k0 = before;
+      if (row >= before && row < un.blk) k0 += ((row - before) / g.block_len + 1) * g.block_len;
+      // stored again only when the next block's keys would no longer fit the tile
+      snap = un.blk + g.block_len - before > KT;
     }
 
     for (int j = 0; j < un.n_tiles; ++j, ++n) {
       if (!wait_here(c, B_S_FULL + x, n & 1, LOC_WAIT_S)) return;
       tc_fence_after();
-      if (WINDOW && un.snap && j == 1) {
-        // the state after the unit's first key tile (its products are complete: these scores were issued behind them)
+      if (WINDOW && snap && j == un.n1) {
+        // the state over the keys before the block (their products are complete: these scores were issued behind them)
         if (!waited) { grid_dependency_wait(); waited = true; }
         if (warp_rows > 0) {
-          store_rows<SPLIT>(c, o_tmem, true, 1.f, a.snap.o + (srow - lane) * D, nullptr, D, warp_rows);
+          store_rows<SPLIT>(c, o_tmem, have_o, 1.f, a.snap.o + (srow - lane) * D, nullptr, D, warp_rows);
           if (valid) { a.snap.m[srow] = m_ref; a.snap.l[srow] = l; }
         }
       }
@@ -471,12 +557,12 @@ __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, 
         for (int i = 0; i < KT; i += 32) tmem_ld32(s_tmem + i, *reinterpret_cast<uint32_t(*)[32]>(s + i));
         tmem_ld_wait();
         const int tile_lo = un.key_row(j);
-        if (tile_lo < un.k0 || tile_lo + KT > un.k1 || (un.x0 < tile_lo + KT && un.x1 > tile_lo)) {
+        if (tile_lo < k0 || tile_lo + KT > un.k1 || (un.x0 < tile_lo + KT && un.x1 > tile_lo)) {
           // columns that take no part: -inf (the same for every row)
 #pragma unroll
           for (int hf = 0; hf < 2; ++hf) {
             const int lo = tile_lo + 64 * hf;
-            const uint64_t bits = span_bits(un.k0 - lo, un.k1 - lo) & ~(un.x1 > un.x0 ? span_bits(un.x0 - lo, un.x1 - lo) : 0ull);
+            const uint64_t bits = span_bits(k0 - lo, un.k1 - lo) & ~(un.x1 > un.x0 ? span_bits(un.x0 - lo, un.x1 - lo) : 0ull);
 #pragma unroll
             for (int i = 0; i < 64; ++i) s[64 * hf + i] = ((bits >> i) & 1ull) ? s[64 * hf + i] : 0xff800000u;
           }
@@ -525,12 +611,12 @@ __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, 
           probabilities(0);
         }
         // (the normaliser sums the rounded probabilities)
-        float l0 = 0.f, l1 = 0.f, l2 = 0.f, l3 = 0.f;
+        float sum[4] = {0.f, 0.f, 0.f, 0.f};
         auto sums = [&]() {
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
-            if (i & 1) { l2 = add_half(l2, p[i], false); l3 = add_half(l3, p[i], true); }
-            else { l0 = add_half(l0, p[i], false); l1 = add_half(l1, p[i], true); }
+            sum[2 * (i & 1)] = add_half(sum[2 * (i & 1)], p[i], false);
+            sum[2 * (i & 1) + 1] = add_half(sum[2 * (i & 1) + 1], p[i], true);
           }
         };
         tmem_st32(p_tmem, p);
@@ -546,7 +632,7 @@ __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, 
         __syncwarp();
         if (lane == 0) mbar_arrive(c.bar(B_P_RDY + 2 * x + 1));
         sums();
-        l += (l0 + l1) + (l2 + l3);
+        l += (sum[0] + sum[1]) + (sum[2] + sum[3]);
         have_o = true;
       } else {   // a warp without rows keeps the barriers' counts (and stays in step: no arrival a phase ahead)
         if (lane == 0) {
@@ -557,6 +643,7 @@ __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, 
     }
 
     // ---- epilogue ----
+    ask_item(a, wk.unit(k_ + 1) / g.Hq, item);
     if (!waited) { grid_dependency_wait(); waited = true; }   // no global store before the grids ahead are complete
     if (un.n_tiles > 0) {
       if (!wait_here(c, B_O_FULL + x, units & 1, LOC_WAIT_O)) return;
@@ -584,7 +671,7 @@ __device__ void row_threads(const Cta& c, const Geometry& g, const AttnArgs& a, 
       } else {
         store_rows<SPLIT>(c, o_tmem, have_o, 1.f, a.st.o + (srow - lane) * D, nullptr, D, warp_rows);
         if (valid) { a.st.m[srow] = m_ref; a.st.l[srow] = l; }
-        if (WINDOW && un.snap && un.n_tiles == 1) {   // a single key tile: the state after it is the final one as well
+        if (WINDOW && snap && un.n_tiles == un.n1) {   // no keys after the block: the state before it is the final one as well
           store_rows<SPLIT>(c, o_tmem, have_o, 1.f, a.snap.o + (srow - lane) * D, nullptr, D, warp_rows);
           if (valid) { a.snap.m[srow] = m_ref; a.snap.l[srow] = l; }
         }
@@ -654,6 +741,15 @@ row_attn_kernel(const __grid_constant__ RowMaps maps, const __grid_constant__ Ge
   }
   __syncwarp();
 
+  if (a.state_end_out != nullptr && blockIdx.x == 0 && warp == W_QUERIES) {
+    // where the stored states end after this launch (read by the next one)
+    grid_dependency_wait();
+    for (int b = tid & 31; b < g.B; b += 32) {
+      const int s0 = a.blk_start[b];
+      const int before = a.state_end ? __ldcg(a.state_end + b) : s0;
+      a.state_end_out[b] = s0 + g.block_len - before > KT ? s0 : before;
+    }
+  }
   if (*c.abort_flag) {
     // A bounded wait ran out and the roles have returned where they stood: copies and products issued before that
     // get a fixed 50 us to land before shared memory and TMEM are given up.

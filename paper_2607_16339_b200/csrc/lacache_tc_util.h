@@ -94,7 +94,7 @@ __device__ __forceinline__ WorkItem load_item(const WorkItem* p) {
   WorkItem w;
   w.kind = a.x; w.seq = a.y; w.row0 = a.z; w.nrows = a.w;
   w.chunk = b.x; w.kt0 = b.y; w.kt1 = b.z; w.pad = b.w;
-  w.seq_start = c.x; w.seq_end = c.y; w.blk_start = c.z; w.pad2 = c.w;
+  w.seq_start = c.x; w.seq_end = c.y; w.blk_start = c.z; w.n_before = c.w;
   return w;
 }
 
