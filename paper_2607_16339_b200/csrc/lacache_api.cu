@@ -859,8 +859,20 @@ lacache_status run_window(lacache_ctx* c, lacache_ctx::ListRef list, int blk, co
                           float* lse = nullptr);
 }  // namespace
 
+namespace {
+lacache_status build_impl(lacache_ctx* c, int block_idx, const void* q, const void* k, const void* v, void* stream, bool rotated);
+lacache_status build_incremental_impl(lacache_ctx* c, int block_idx, const void* q, const void* k, const void* v, void* stream, bool rotated);
+lacache_status ensure_prefix_state(lacache_ctx* c);
+}  // namespace
+
 lacache_status lacache_build(lacache_ctx* c, int block_idx, const void* q, const void* k, const void* v,
                              void* stream) {
+  return build_impl(c, block_idx, q, k, v, stream, false);
+}
+
+namespace {
+// rotated: the kernel ahead in the stream has left these rows in the rotated cache already
+lacache_status build_impl(lacache_ctx* c, int block_idx, const void* q, const void* k, const void* v, void* stream, bool rotated) {
   if (!c) return LACACHE_ERR_INVALID_ARG;
   if (!q || !k || !v) return fail(c, LACACHE_ERR_INVALID_ARG, "NULL input pointer");
   if (misaligned(q) || misaligned(k) || misaligned(v)) return fail(c, LACACHE_ERR_INVALID_ARG, "input pointer not 16-byte aligned");
@@ -870,7 +882,7 @@ lacache_status lacache_build(lacache_ctx* c, int block_idx, const void* q, const
   c->last_launches = 0;
   c->built_block = -1;
   c->prefix_block = -1;
-  lacache_status st = rope_all(c, q, k, v, c->rot, s);
+  lacache_status st = rotated ? LACACHE_OK : rope_all(c, q, k, v, c->rot, s);
   if (st != LACACHE_OK) return st;
   if (c->cfg.cache_granularity == LACACHE_GRANULARITY_TILE) {
     // state of the rows outside the tiles that overlap the block: over the key tiles before them, then
@@ -889,7 +901,6 @@ lacache_status lacache_build(lacache_ctx* c, int block_idx, const void* q, const
   return LACACHE_OK;
 }
 
-namespace {
 // the prefix state's buffers, allocated when the incremental build is first used
 lacache_status ensure_prefix_state(lacache_ctx* c) {
   if (c->engine != LACACHE_ENGINE_TCGEN05)
@@ -948,6 +959,12 @@ lacache_status run_window(lacache_ctx* c, lacache_ctx::ListRef list, int blk, co
 
 lacache_status lacache_build_incremental(lacache_ctx* c, int block_idx, const void* q, const void* k, const void* v,
                                          void* stream) {
+  return build_incremental_impl(c, block_idx, q, k, v, stream, false);
+}
+
+namespace {
+lacache_status build_incremental_impl(lacache_ctx* c, int block_idx, const void* q, const void* k, const void* v, void* stream,
+                                      bool rotated) {
   if (!c) return LACACHE_ERR_INVALID_ARG;
   if (!q || !k || !v) return fail(c, LACACHE_ERR_INVALID_ARG, "NULL input pointer");
   if (misaligned(q) || misaligned(k) || misaligned(v)) return fail(c, LACACHE_ERR_INVALID_ARG, "input pointer not 16-byte aligned");
@@ -959,7 +976,7 @@ lacache_status lacache_build_incremental(lacache_ctx* c, int block_idx, const vo
   c->last_launches = 0;
   c->built_block = -1;
   c->prefix_block = -1;
-  st = rope_all(c, q, k, v, c->rot, s);
+  st = rotated ? LACACHE_OK : rope_all(c, q, k, v, c->rot, s);
   if (st != LACACHE_OK) return st;
   st = run_window(c, c->inc_build[block_idx], block_idx, StateBuffers{}, c->st, c->pst, s);
   if (st != LACACHE_OK) return st;
@@ -968,6 +985,8 @@ lacache_status lacache_build_incremental(lacache_ctx* c, int block_idx, const vo
   c->steps_since_build = 0;
   return LACACHE_OK;
 }
+
+}  // namespace
 
 lacache_status lacache_build_advance(lacache_ctx* c, const void* q, const void* k, const void* v, void* stream) {
   if (!c) return LACACHE_ERR_INVALID_ARG;
@@ -1041,6 +1060,17 @@ lacache_status check_producer(lacache_ctx* c, lacache_qkv* p, int n) {
   if (n > max_tokens) return fail(c, LACACHE_ERR_SHAPE, "%d tokens, producer max_tokens %d", n, max_tokens);
   return LACACHE_OK;
 }
+// All tokens projected into q / k / v and, where the projection can, rotated into the cache behind it.  A build that will be
+// refused (`accepted` false) leaves the cache alone.
+lacache_status project_all(lacache_ctx* c, lacache_qkv* p, const int32_t* token_ids, const void* hidden, void* q, void* k,
+                           void* v, void* stream, bool accepted, bool* rotated) {
+  const RotateTarget target{c->rot, c->d_pos, c->d_cos, c->d_sin, c->g.Tp, c->g.op_f16};
+  const bool rotate = accepted && c->engine == LACACHE_ENGINE_TCGEN05;
+  lacache_status st = qkv_project_rows(p, token_ids, hidden, c->g.T, q, k, v, nullptr, nullptr, 0, false, stream,
+                                       rotate ? &target : nullptr, rotated);
+  if (st != LACACHE_OK) return fail(c, st, "producer: %s", lacache_qkv_last_error(p));
+  return LACACHE_OK;
+}
 }  // namespace
 
 lacache_status lacache_build_tokens(lacache_ctx* c, lacache_qkv* p, int block_idx, const int32_t* token_ids,
@@ -1051,9 +1081,10 @@ lacache_status lacache_build_tokens(lacache_ctx* c, lacache_qkv* p, int block_id
   void *q, *k, *v;
   qkv_scratch(p, false, &q, &k, &v);
   qkv_set_full_owner(p, nullptr, 0);
-  st = lacache_qkv_project(p, token_ids, hidden, c->g.T, q, k, v, nullptr, stream);
-  if (st != LACACHE_OK) return fail(c, st, "producer: %s", lacache_qkv_last_error(p));
-  st = lacache_build(c, block_idx, q, k, v, stream);
+  bool rotated = false;
+  st = project_all(c, p, token_ids, hidden, q, k, v, stream, block_idx >= 0 && block_idx < c->g.n_blk, &rotated);
+  if (st != LACACHE_OK) return st;
+  st = build_impl(c, block_idx, q, k, v, stream, rotated);
   if (st != LACACHE_OK) return st;
   qkv_set_full_owner(p, c, c->g.T);
   c->last_launches += lacache_qkv_last_launch_count(p);
@@ -1091,9 +1122,11 @@ lacache_status lacache_build_tokens_incremental(lacache_ctx* c, lacache_qkv* p, 
   void *q, *k, *v;
   qkv_scratch(p, false, &q, &k, &v);
   qkv_set_full_owner(p, nullptr, 0);
-  st = lacache_qkv_project(p, token_ids, hidden, c->g.T, q, k, v, nullptr, stream);
-  if (st != LACACHE_OK) return fail(c, st, "producer: %s", lacache_qkv_last_error(p));
-  st = lacache_build_incremental(c, block_idx, q, k, v, stream);
+  bool rotated = false;
+  const bool accepted = block_idx >= 0 && block_idx < c->g.n_blk && ensure_prefix_state(c) == LACACHE_OK;
+  st = project_all(c, p, token_ids, hidden, q, k, v, stream, accepted, &rotated);
+  if (st != LACACHE_OK) return st;
+  st = build_incremental_impl(c, block_idx, q, k, v, stream, rotated);
   if (st == LACACHE_OK) c->last_launches += lacache_qkv_last_launch_count(p);
   return st;
 }

@@ -204,12 +204,22 @@ void tc_free_maps(TcMaps* m);
 // and its head configuration (returns head_dim)
 void qkv_scratch(lacache_qkv* p, bool block, void** q, void** k, void** v);
 int qkv_heads(const lacache_qkv* p, int* hq, int* hkv, int* max_tokens);
+// Where a projection leaves its rows rotated as well, in the tcgen05 engine's storage (what the RoPE kernel would make of
+// them): row t is token t of the context.
+struct RotateTarget {
+  RotBuffers dst;
+  const int32_t* pos;                 // [T] position of a token
+  const float* cos_tab; const float* sin_tab;   // [positions][64]
+  int Tp, op_f16;
+};
 // lacache_qkv_project with a scatter: input token t is written to output row dst_rows[t] (null: t)
 // early_inputs: token_ids / hidden were complete before the grid ahead in the stream was enqueued, so the
 // norm kernel may read them while that grid still runs (it waits for it at its end instead).
+// rotate: null, or where the rows go rotated too; *rotated (if rotate) says whether they did (a projection of few tokens
+// does not rotate).
 lacache_status qkv_project_rows(lacache_qkv* p, const int32_t* token_ids, const void* hidden, int n_tokens, void* q,
                                 void* k, void* v, void* h_out, const int32_t* dst_rows, int max_rows, bool early_inputs,
-                                void* stream);
+                                void* stream, const RotateTarget* rotate = nullptr, bool* rotated = nullptr);
 // which context's tokens the all-token scratch holds (set by a full projection)
 void qkv_set_full_owner(lacache_qkv* p, const void* ctx, int n_tokens);
 bool qkv_full_owner_is(const lacache_qkv* p, const void* ctx, int n_tokens);

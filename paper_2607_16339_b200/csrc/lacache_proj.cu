@@ -8,8 +8,13 @@
 // rows of one tile are stored while the next is computed.
 //   warp 0 (one lane)  producer of this CTA's operands; every load counts its bytes on the leader's barrier
 //   warp 1             (leader CTA, one elected lane) issues the pair's MMAs
-//   warps 2..5         epilogue: TMEM lane = token; bf16 rows through 4 KB of staging per warp, so that a store
-//                      instruction writes 128 contiguous bytes of each of four rows
+//   warps 2..5         epilogue: TMEM lane = token; bf16 rows through 8 KB of staging per warp, a head at a time, so that a
+//                      store instruction writes 128 contiguous bytes of each of four rows; for a build the rows also
+//                      leave rotated, in the storage of the attention kernels (a thread then holds 8 features of a row's
+//                      head and their partners, as in the RoPE kernel, whose arithmetic it uses).  The tile's 40000 cycles
+//                      of MMAs hide it; as a kernel of its own the rotation of 6411 tokens x 96 heads read the rows again
+//                      and took 61 us
+//                      of the 886 that entering a block of eight requests takes (now 828).
 // Tiles are dealt out with the token tiles running fastest: the clusters at work share few feature tiles, and both
 // operands of what they share stay in L2.
 #include <cuda.h>
@@ -20,6 +25,7 @@
 #include "lacache_internal.h"
 #include "lacache_proj.h"
 #include "lacache_ptx.h"
+#include "lacache_rope_math.h"
 
 namespace lacache {
 namespace {
@@ -32,8 +38,8 @@ constexpr int THREADS = 192;
 constexpr uint32_t HALF = 128 * BK * 2;  // 16 KB: one operand of one CTA
 constexpr uint32_t STAGE = 2 * HALF;
 constexpr int STAGES = 6;
-constexpr uint32_t SM_ST = STAGES * STAGE;            // 4 x 4 KB of staging
-constexpr uint32_t SM_BAR = SM_ST + 4 * 4096;
+constexpr uint32_t SM_ST = STAGES * STAGE;            // 4 x 8 KB of staging
+constexpr uint32_t SM_BAR = SM_ST + 4 * 8192;
 enum { B_FULL = 0, B_FREE = STAGES, B_ACC_FULL = 2 * STAGES, B_ACC_FREE = B_ACC_FULL + 2, N_BARS = B_ACC_FREE + 2 };
 constexpr uint32_t SM_TOTAL = SM_BAR + 8 * N_BARS + 16;
 static_assert(SM_TOTAL <= 232448, "exceeds the 227 KB per-CTA limit");
@@ -185,7 +191,7 @@ proj_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant__ C
     }
   } else {
     const int quad = warp & 3;                     // the TMEM lanes this warp may read
-    uint8_t* const st = smem_raw + SM_ST + (warp - 2) * 4096;
+    uint8_t* const st = smem_raw + SM_ST + (warp - 2) * 8192;
     int n = 0;
     for (int i = first; i < a.n_tiles; i += stride, ++n) {
       const Tile t = tile_of(a, i);
@@ -196,44 +202,84 @@ proj_kernel(const __grid_constant__ CUtensorMap w_map, const __grid_constant__ C
       const int rows = min(a.n_tokens - t0, 32);
       const uint32_t acc = tmem + ((uint32_t)(quad * 32) << 16) + 256u * buf;
       if (n == 0) grid_dependency_wait();   // results may overwrite rows that a grid ahead in the stream still reads
+      const int tok = t0 + lane;                     // of this lane's row
+      const int dst_row = rows > lane ? (a.dst_rows ? __ldg(a.dst_rows + tok) : tok) : -1;
+      const int pos = a.rotate && rows > lane ? __ldg(a.rot.pos + tok) : 0;
+      // (a row out of range is reported by the norm kernel)
+      const bool stored = dst_row >= 0 && (!a.dst_rows || dst_row < a.max_rows);
 #pragma unroll 1
-      for (int cb = 0; cb < 4; ++cb) {             // 64 features: half a head
-        const int head = t.nt * 2 + (cb >> 1);
-        uint32_t r[64];
-        tmem_ld32(acc + 64 * cb, *reinterpret_cast<uint32_t(*)[32]>(r));
-        tmem_ld32(acc + 64 * cb + 32, *reinterpret_cast<uint32_t(*)[32]>(r + 32));
-        tmem_ld_wait();
-        if (cb == 3) {   // the accumulator may be overwritten
+      for (int hh = 0; hh < 2; ++hh) {             // a head: [feature half][row][64]
+        const int head = t.nt * 2 + hh;
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {
+          uint32_t r[64];
+          tmem_ld32(acc + 128 * hh + 64 * half, *reinterpret_cast<uint32_t(*)[32]>(r));
+          tmem_ld32(acc + 128 * hh + 64 * half + 32, *reinterpret_cast<uint32_t(*)[32]>(r + 32));
+          tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            uint32_t p[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const __nv_bfloat162 b = __floats2bfloat162_rn(__uint_as_float(r[8 * j + 2 * e]), __uint_as_float(r[8 * j + 2 * e + 1]));
+              p[e] = *reinterpret_cast<const uint32_t*>(&b);
+            }
+            *reinterpret_cast<uint4*>(st + half * 4096 + lane * 128 + ((j ^ (lane & 7)) << 4)) = make_uint4(p[0], p[1], p[2], p[3]);
+          }
+        }
+        if (hh == 1) {   // the accumulator may be overwritten
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive_cluster(mapa_shared(c.bar(B_ACC_FREE + buf), 0));
         }
-        if (rows <= 0 || head >= a.n_heads) continue;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          uint32_t p[4];
-#pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            const __nv_bfloat162 b = __floats2bfloat162_rn(__uint_as_float(r[8 * j + 2 * e]), __uint_as_float(r[8 * j + 2 * e + 1]));
-            p[e] = *reinterpret_cast<const uint32_t*>(&b);
-          }
-          *reinterpret_cast<uint4*>(st + lane * 128 + ((j ^ (lane & 7)) << 4)) = make_uint4(p[0], p[1], p[2], p[3]);
-        }
         __syncwarp();
-        __nv_bfloat16* dst;
-        int H, h;
-        if (head < a.Hq) { dst = a.q; H = a.Hq; h = head; }
-        else if (head < a.Hq + a.Hkv) { dst = a.k; H = a.Hkv; h = head - a.Hq; }
-        else { dst = a.v; H = a.Hkv; h = head - a.Hq - a.Hkv; }
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const int rr = 4 * j + (lane >> 3), ch = lane & 7;
-          if (rr < rows) {
-            int tok = t0 + rr;
-            if (a.dst_rows) tok = __ldg(a.dst_rows + tok);
-            if (!a.dst_rows || (unsigned)tok < (unsigned)a.max_rows)   // (a row out of range is reported by the norm kernel)
-              *reinterpret_cast<uint4*>(dst + ((size_t)tok * H + h) * HD + 64 * (cb & 1) + 8 * ch) =
-                  *reinterpret_cast<const uint4*>(st + rr * 128 + ((ch ^ (rr & 7)) << 4));
+        if (rows > 0 && head < a.n_heads) {
+          __nv_bfloat16* dst;
+          int H, h, which;   // 0 q, 1 k, 2 v
+          if (head < a.Hq) { dst = a.q; H = a.Hq; h = head; which = 0; }
+          else if (head < a.Hq + a.Hkv) { dst = a.k; H = a.Hkv; h = head - a.Hq; which = 1; }
+          else { dst = a.v; H = a.Hkv; h = head - a.Hq - a.Hkv; which = 2; }
+          const int ch = lane & 7;
+#pragma unroll 4
+          for (int j = 0; j < 8; ++j) {
+            const int rr = 4 * j + (lane >> 3);
+            const uint4 u1 = *reinterpret_cast<const uint4*>(st + rr * 128 + ((ch ^ (rr & 7)) << 4));
+            const uint4 u2 = *reinterpret_cast<const uint4*>(st + 4096 + rr * 128 + ((ch ^ (rr & 7)) << 4));
+            const int drow = __shfl_sync(0xffffffffu, dst_row, rr);
+            const bool keep = __shfl_sync(0xffffffffu, (int)stored, rr) != 0;
+            if (keep) {
+              __nv_bfloat16* const p = dst + ((size_t)drow * H + h) * HD + 8 * ch;
+              *reinterpret_cast<uint4*>(p) = u1;
+              *reinterpret_cast<uint4*>(p + 64) = u2;
+            }
+            if (a.rotate) {
+              const size_t ang = (size_t)__shfl_sync(0xffffffffu, pos, rr) * 64 + 8 * ch;
+              float x1[8], x2[8], y1[8], y2[8];
+              const uint4 w1[1] = {u1}, w2[1] = {u2};
+              rope_unpack8<1>(w1, true, x1);
+              rope_unpack8<1>(w2, true, x2);
+              if (which < 2) {
+                float cs[8], sn[8];
+                *reinterpret_cast<float4*>(cs) = __ldg(reinterpret_cast<const float4*>(a.rot.cos_tab + ang));
+                *reinterpret_cast<float4*>(cs + 4) = __ldg(reinterpret_cast<const float4*>(a.rot.cos_tab + ang) + 1);
+                *reinterpret_cast<float4*>(sn) = __ldg(reinterpret_cast<const float4*>(a.rot.sin_tab + ang));
+                *reinterpret_cast<float4*>(sn + 4) = __ldg(reinterpret_cast<const float4*>(a.rot.sin_tab + ang) + 1);
+                rope_rotate8(x1, x2, cs, sn, y1, y2);
+              }
+              if (keep) {
+                const size_t o1 = ((size_t)(2 * h) * a.rot.Tp + drow) * 64 + 8 * ch, o2 = o1 + (size_t)a.rot.Tp * 64;
+                if (which == 2) {
+                  __half* const p = reinterpret_cast<__half*>(a.rot.dst.v);
+                  *reinterpret_cast<uint4*>(p + o1) = rope_half8(x1);
+                  *reinterpret_cast<uint4*>(p + o2) = rope_half8(x2);
+                } else {
+                  void* const hi = which == 0 ? a.rot.dst.q_hi : a.rot.dst.k_hi;
+                  void* const lo = which == 0 ? a.rot.dst.q_lo : a.rot.dst.k_lo;
+                  rope_store8(hi, lo, o1, y1, a.rot.op_f16 != 0);
+                  rope_store8(hi, lo, o2, y2, a.rot.op_f16 != 0);
+                }
+              }
+            }
           }
         }
         __syncwarp();

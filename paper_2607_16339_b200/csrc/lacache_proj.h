@@ -4,6 +4,8 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include "lacache_internal.h"
+
 namespace lacache {
 
 struct ProjArgs {
@@ -11,6 +13,7 @@ struct ProjArgs {
   int Hq, Hkv;
   __nv_bfloat16 *q, *k, *v;
   const int32_t* dst_rows; int max_rows;    // output row of input token t (null: t); rows outside [0, max_rows) are dropped
+  int rotate; RotateTarget rot;             // also leave the rows rotated (dst_rows null)
   int32_t* status;
   long long wait_cycles;
   int n_heads, n_ttiles, n_tiles;           // set by proj_many

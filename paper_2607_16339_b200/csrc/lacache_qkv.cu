@@ -949,17 +949,18 @@ namespace lacache {
 namespace {
 lacache_status project_impl(lacache_qkv* p, const int32_t* token_ids, const void* hidden, int n_tokens, void* q,
                             void* k, void* v, void* h_out, const int32_t* dst_rows, int max_rows, bool early_inputs,
-                            void* stream, bool without_norm);
+                            void* stream, bool without_norm, const RotateTarget* rotate = nullptr, bool* rotated = nullptr);
 }
 lacache_status qkv_project_rows(lacache_qkv* p, const int32_t* token_ids, const void* hidden, int n_tokens, void* q,
                                 void* k, void* v, void* h_out, const int32_t* dst_rows, int max_rows, bool early_inputs,
-                                void* stream) {
-  return project_impl(p, token_ids, hidden, n_tokens, q, k, v, h_out, dst_rows, max_rows, early_inputs, stream, false);
+                                void* stream, const RotateTarget* rotate, bool* rotated) {
+  if (rotated) *rotated = false;
+  return project_impl(p, token_ids, hidden, n_tokens, q, k, v, h_out, dst_rows, max_rows, early_inputs, stream, false, rotate, rotated);
 }
 namespace {
 lacache_status project_impl(lacache_qkv* p, const int32_t* token_ids, const void* hidden, int n_tokens, void* q,
                             void* k, void* v, void* h_out, const int32_t* dst_rows, int max_rows, bool early_inputs,
-                            void* stream, bool without_norm) {
+                            void* stream, bool without_norm, const RotateTarget* rotate, bool* rotated) {
   if (!p) return LACACHE_ERR_INVALID_ARG;
   if ((token_ids == nullptr) == (hidden == nullptr))
     return qfail(p, LACACHE_ERR_INVALID_ARG, "pass exactly one of token_ids and hidden");
@@ -1025,11 +1026,13 @@ lacache_status project_impl(lacache_qkv* p, const int32_t* token_ids, const void
     pa.v = reinterpret_cast<__nv_bfloat16*>(v);
     pa.dst_rows = dst_rows;
     pa.max_rows = max_rows;
+    if (rotate && !dst_rows) { pa.rotate = 1; pa.rot = *rotate; }
     pa.status = p->status;
     pa.wait_cycles = p->wait_cycles > 0 ? p->wait_cycles : Q_WAIT_CYCLES;
     const bool timed = p->ev_start && p->ev_stop;   // (an event between the two kernels: an ordinary launch)
     if (timed) QCU_TRY(p, cudaEventRecord(p->ev_start, s));
     QCU_TRY(p, proj_many(p->w_map, p->x_map[2], pa, p->num_sms, !no_pdl && !timed, s));
+    if (pa.rotate && rotated) *rotated = true;
     if (timed) QCU_TRY(p, cudaEventRecord(p->ev_stop, s));
     p->last_launches++;
     return LACACHE_OK;

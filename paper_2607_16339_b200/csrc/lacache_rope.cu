@@ -23,19 +23,6 @@ __device__ __forceinline__ void store8_f32(void* plane, size_t off, const float 
   p[1] = make_float4(y[4], y[5], y[6], y[7]);
 }
 
-__device__ __forceinline__ void store8_split(void* hi_plane, void* lo_plane, size_t off,
-                                             const float (&y)[8], bool f16) {
-  if (f16) {   // one fp16 plane: the rotated value rounded once to fp16
-    *reinterpret_cast<uint4*>(reinterpret_cast<__half*>(hi_plane) + off) = rope_half8(y);
-    return;
-  }
-  uint4 uh, ul;
-  rope_split8(y, uh, ul);
-  *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(hi_plane) + off) = uh;
-  // (plain operands keep the hi plane alone: the rotated value rounded once to bf16)
-  if (lo_plane) *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(lo_plane) + off) = ul;
-}
-
 __device__ __forceinline__ void store8_f16(void* plane, size_t off, const float (&y)[8]) {
   *reinterpret_cast<uint4*>(reinterpret_cast<__half*>(plane) + off) = rope_half8(y);
 }
@@ -122,8 +109,8 @@ __global__ void __launch_bounds__(256, HPT > 1 ? 3 : 1) rope_write_kernel(const 
       } else {
         void* const hi = which == 0 ? a.dst.q_hi : a.dst.k_hi;
         void* const lo = which == 0 ? a.dst.q_lo : a.dst.k_lo;
-        store8_split(hi, lo, o1, y1, g.op_f16 != 0);
-        store8_split(hi, lo, o2, y2, g.op_f16 != 0);
+        rope_store8(hi, lo, o1, y1, g.op_f16 != 0);
+        rope_store8(hi, lo, o2, y2, g.op_f16 != 0);
       }
     } else {
       void* const plane = which == 0 ? a.dst.q_hi : (which == 1 ? a.dst.k_hi : a.dst.v);

@@ -1,6 +1,6 @@
-// Rotation and storage-format arithmetic shared by the RoPE-on-write kernel and
-// the attention kernel's in-place rotation of a block's queries (Eq. 1): both
-// must produce the same bits, so both call these.
+// Rotation and storage-format arithmetic shared by the RoPE-on-write kernel, the
+// projection's epilogue and the attention kernel's in-place rotation of a block's
+// queries (Eq. 1): all must produce the same bits, so all call these.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -79,6 +79,19 @@ __device__ __forceinline__ uint4 rope_half8(const float (&y)[8]) {
     p[i] = __floats2half2_rn(a, b);
   }
   return u;
+}
+
+// 8 rotated values of q or k at element offset off of the tcgen05 engine's planes
+__device__ __forceinline__ void rope_store8(void* hi_plane, void* lo_plane, size_t off, const float (&y)[8], bool f16) {
+  if (f16) {   // one fp16 plane: the rotated value rounded once to fp16
+    *reinterpret_cast<uint4*>(reinterpret_cast<__half*>(hi_plane) + off) = rope_half8(y);
+    return;
+  }
+  uint4 uh, ul;
+  rope_split8(y, uh, ul);
+  *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(hi_plane) + off) = uh;
+  // (plain operands keep the hi plane alone: the rotated value rounded once to bf16)
+  if (lo_plane) *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(lo_plane) + off) = ul;
 }
 
 }  // namespace lacache

@@ -1,0 +1,56 @@
+"""A build from tokens whose projection leaves the rotated cache itself, against the build from the projected rows (RoPE
+kernel), bit for bit: token counts around the projection's 128- and 256-row tiles, odd head counts (half a tile of features),
+every operand mode; the rows a later update needs; a refused build, which leaves the cache as it was."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2607_16339_b200 import binding, workloads as W
+from paper_2607_16339_b200.workloads import TokenModel
+
+from lacache_testlib import make_ctx
+from test_gpu_tokenwise import make_producer, project
+
+pytestmark = pytest.mark.gpu
+
+
+def _cache(ctx, wl):
+    r = [torch.empty(wl.total_tokens, h, wl.head_dim, device="cuda") for h in (wl.n_q_heads, wl.n_kv_heads, wl.n_kv_heads)]
+    ctx.export_rope_cache(*r)
+    torch.cuda.synchronize()
+    assert ctx.poll_status()[0] == binding.OK
+    return r
+
+
+@pytest.mark.parametrize("prompts,hq,hkv", [((33,), 4, 4), ((64, 63), 3, 1), ((65, 63), 2, 1), ((191,), 5, 5), ((100, 300, 7), 8, 2)])
+@pytest.mark.parametrize("mode", [binding.PRECISION_PLAIN, binding.PRECISION_FP16, binding.PRECISION_SPLIT])
+@pytest.mark.parametrize("incremental", [False, True])
+def test_rotated_cache_of_a_build_from_tokens(prompts, hq, hkv, mode, incremental):
+    wl = W.small_workload(prompt_lens=prompts, gen_len=64, block_len=32, steps=1, hq=hq, hkv=hkv)
+    tm = TokenModel(wl, 192, 700)
+    prod = make_producer(tm, wl.total_tokens)
+    ids = tm.full_ids(1)
+    dev_ids = torch.from_numpy(ids).cuda()
+    a, b = make_ctx(wl, precision_mode=mode), make_ctx(wl, precision_mode=mode)
+    (a.build_tokens_incremental if incremental else a.build_tokens)(prod, 1, token_ids=dev_ids)
+    st, msg, q, k, v, _ = project(prod, tm, wl.total_tokens, ids=ids)
+    assert st == binding.OK, msg
+    (b.build_incremental if incremental else b.build)(1, q, k, v)
+    want = _cache(b, wl)
+    for x, y in zip(_cache(a, wl), want):
+        assert torch.equal(x, y)
+    with pytest.raises(binding.LacacheError):     # (no such block)
+        a.build_tokens(prod, 2, token_ids=torch.flip(dev_ids, (0,)))
+    for x, y in zip(_cache(a, wl), want):
+        assert torch.equal(x, y)
+    if not incremental:                            # an update starts from the rows of the last build from tokens
+        a.build_tokens(prod, 0, token_ids=dev_ids)
+        rows = np.arange(5, 25, dtype=np.int32)
+        new = dev_ids.clone()
+        new[5:25] = 3
+        a.build_tokens_update(prod, 1, torch.from_numpy(rows).cuda(), token_ids=new[5:25].contiguous())
+        b.build_tokens(prod, 1, token_ids=new)
+        for x, y, h in zip(_cache(a, wl), _cache(b, wl), range(3)):
+            assert torch.equal(x, y) or (x - y).abs().max().item() <= 2.0 ** -6 * y.abs().max().item(), h
+    for o in (a, b, prod):
+        o.destroy()
