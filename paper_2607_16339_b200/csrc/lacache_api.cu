@@ -693,9 +693,9 @@ AttnArgs attn_args(lacache_ctx* c, int mode, lacache_ctx::ListRef list, int blk,
         // lose 0.3 us; a step from token ids, behind which the projection's CTAs would wait on SMs, between -0.8 and 2.8.
         a.step_overlap = (a.merge_deep && !c->split && c->g.block_len <= 32 && per_cta <= 5) ? 1 : 0;
       }
-      // Two key chunks per (sequence, head), one round of block-row units, unpacked heads:
-      // the two chunks of a head run as a pair of CTAs that merge through distributed shared memory.
-      if (a.pack == 1 && (a.merge_deep || a.split_merge) && !c->knobs.no_pair && c->g.block_len <= 32 &&
+      // Two key chunks per (sequence, head), one round of block-row units: the two chunks of a head (of a group of packed heads,
+      // with one plane) run as a pair of CTAs that merge through distributed shared memory.
+      if ((a.pack == 1 ? c->g.block_len <= 32 : !c->split) && (a.merge_deep || a.split_merge) && !c->knobs.no_pair &&
           units_stream == ns && (ns % 2) == 0 && (a.n_ctas % 2) == 0) {
         if (plan.pair < 0) {
           plan.pair = 1;

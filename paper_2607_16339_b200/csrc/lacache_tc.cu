@@ -87,6 +87,10 @@ struct Rx {
   static constexpr uint32_t O = Tile<SPLIT>::SM_V + 2 * Tile<SPLIT>::V_STAGE;
   static constexpr uint32_t ML = SM_Q + 32768 + 32 * STAGE_ROW;
   static_assert(O + 32 * STAGE_ROW <= SM_XCH && ML + 32 * 8 <= SM_K, "no room for the partner's partial state");
+  // packed heads (one plane): half of a tile's rows, up to 64 of them, and their (m, l) in the upper half of the Q region, which
+  // neither the 128-row Q tile nor the rows staged over it reach
+  static constexpr uint32_t ML_PACKED = SM_Q + 32768;
+  static_assert(SPLIT || O + 64 * STAGE_ROW <= SM_XCH, "no room for half a tile of the partner's partial state");
 };
 // merge role: the 96 KB after Q hold 2 stages of the block's keys {K hi, K lo, V} of 64
 // rows, then the staging tile of the cached O~ / the output
@@ -141,8 +145,9 @@ __device__ __forceinline__ void load_v_box(uint32_t dst, const CUtensorMap* map,
 // One unit of work of the stream role, decoded identically by every warp role.
 // KIND_STEP2: a step whose block-row units all have exactly two key chunks, run by the two CTAs of a
 // thread-block cluster: the CTA with the second chunk hands its partial state to its partner through
-// distributed shared memory, and the partner writes the merged rows (one round of units, unpacked heads; the place of the
-// receiving buffer: see Rx).
+// distributed shared memory, and the partner writes the merged rows (one round of units; the place of the receiving buffer:
+// see Rx).  With packed heads, whose tiles have up to 128 rows, each CTA merges and writes half of the tile's rows and hands
+// the other half's partial states to its partner (one plane only: split planes leave no room).
 enum StreamKind : int { KIND_STEP = 1, KIND_STEP2 = 3 };
 
 struct Unit {
@@ -170,7 +175,7 @@ __device__ __forceinline__ bool unit_row_valid(const Unit& un, int r) {
 // (u / 2) % Hq of sequence (u / 2) / Hq, and u % 2 its key chunk: a sequence's two chunk items are adjacent)
 template <bool PACKED, int KIND>
 __device__ __forceinline__ int unit_item(const Geometry& g, const AttnArgs& a, int u) {
-  if (KIND == KIND_STEP2) return ((u >> 1) / g.Hq) * 2 + (u & 1);
+  if (KIND == KIND_STEP2) return ((u >> 1) / (PACKED ? a.stream_slots : g.Hq)) * 2 + (u & 1);
   return u / (PACKED ? a.stream_slots : g.Hq);
 }
 
@@ -601,6 +606,91 @@ __device__ __forceinline__ void merge_partials(const Geometry& g, const AttnArgs
   }
 }
 
+// Paired step with packed heads: rows [lo, hi) of a tile, which this CTA of the pair writes (rank 0 the first half).
+__device__ __forceinline__ void pair_half(const Unit& un, uint32_t rank, int& lo, int& hi) {
+  const int rows = un.nh * un.rh;
+  lo = rank ? rows / 2 : 0;
+  hi = rank ? rows : rows / 2;
+}
+// The partial state of the rows the partner writes goes to it -- O~ from TMEM into its receiving buffer (the layout of a
+// staging tile), m and l beside it, one arrival per thread on its barrier --, the partner's of this CTA's rows is waited for
+// (bounded), and this thread's half of its row, merged (Eq. 2-6) and normalised, goes to the row's place in the staging tile.
+// In place of partial states in global memory, a count and a merge by the last CTA to arrive, which is 20000 cycles for two heads
+// of 64 rows (cold code, one L2 round trip after another): the step of 28/4 heads x 5120 tokens 45.2 us with it, 39.2 as a pair.
+template <bool SPLIT>
+__device__ __forceinline__ bool exchange_halves(const Cta& c, const Geometry& g, const AttnArgs& a, const Unit& un, int r, int half,
+                                                uint32_t o_tmem, bool empty, float m, float l) {
+  const uint32_t rank = cluster_ctarank(), peer = rank ^ 1u;
+  int lo, hi, plo, phi;
+  pair_half(un, rank, lo, hi);
+  pair_half(un, peer, plo, phi);
+  const bool valid = unit_row_valid(un, r);
+  const bool mine = valid && r >= lo && r < hi, theirs = valid && r >= plo && r < phi;
+  uint32_t o[64];   // O~, this thread's 64 features
+  if (!empty) {
+    tmem_ld32(o_tmem, *reinterpret_cast<uint32_t(*)[32]>(o));
+    tmem_ld32(o_tmem + 32, *reinterpret_cast<uint32_t(*)[32]>(o + 32));
+    tmem_ld_wait();
+  } else {
+#pragma unroll
+    for (int i = 0; i < 64; ++i) o[i] = 0u;
+  }
+  if (theirs) {
+    const int pr = r - plo;
+    const uint32_t dst = mapa_shared(c.base + Rx<SPLIT>::O + (uint32_t)pr * STAGE_ROW, peer);
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      st_cluster_v4(dst + (((16 * half + i) ^ (pr & 7)) << 4), __uint_as_float(o[4 * i]), __uint_as_float(o[4 * i + 1]),
+                    __uint_as_float(o[4 * i + 2]), __uint_as_float(o[4 * i + 3]));
+    if (half == 0) st_cluster_v2(mapa_shared(c.base + Rx<SPLIT>::ML_PACKED + (uint32_t)pr * 8u, peer), m, l);
+  }
+  mbar_arrive_cluster(mapa_shared(c.bar(BAR_RX), peer));   // (a release: it makes the stores visible to the acquiring wait)
+  {
+    const uint32_t bar = c.bar(BAR_RX);
+    const long long t0 = clock64();
+    while (!mbar_try_acquire_cluster(bar, 0u)) {
+      if (*c.abort_flag) return false;
+      if (clock64() - t0 > WAIT_CYCLES) {
+        *c.abort_flag = 1;
+        if (atomicCAS(c.status, 0, (int)LACACHE_ERR_TIMEOUT) == 0) {
+          c.status[1] = LOC_WAIT_O; c.status[2] = blockIdx.x; c.status[3] = threadIdx.x;
+        }
+        return false;
+      }
+    }
+  }
+  if (mine) {
+    const int lr = r - lo;
+    const float2 ml = *reinterpret_cast<const float2*>(c.gen + Rx<SPLIT>::ML_PACKED + lr * 8);
+    const float M = fmaxf(m, ml.x);
+    const float w1 = (m == -INFINITY) ? 0.f : ex2(m - M);
+    const float w2 = (ml.x == -INFINITY) ? 0.f : ex2(ml.x - M);
+    const float L = fmaf(l, w1, ml.y * w2);
+    const float inv = 1.f / L, f1 = w1 * inv, f2 = w2 * inv;
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+      const uint32_t off = (uint32_t)lr * STAGE_ROW + (((16 * half + i) ^ (lr & 7)) << 4);
+      const float4 p = *reinterpret_cast<const float4*>(c.gen + Rx<SPLIT>::O + off);
+      *reinterpret_cast<float4*>(c.gen + SM_Q + off) =
+          make_float4(fmaf(p.x, f2, __uint_as_float(o[4 * i]) * f1), fmaf(p.y, f2, __uint_as_float(o[4 * i + 1]) * f1),
+                      fmaf(p.z, f2, __uint_as_float(o[4 * i + 2]) * f1), fmaf(p.w, f2, __uint_as_float(o[4 * i + 3]) * f1));
+    }
+    if (half == 0 && a.lse) a.lse[(size_t)(un.row0 + unit_row(un, r)) * g.Hq + unit_head(un, r)] = (M + log2f(L)) * 0.69314718055994530942f;
+  }
+  return true;
+}
+// The staged rows of this CTA's half to the output: every warp-wide store writes one whole row.
+__device__ __forceinline__ void store_half(const Cta& c, const Geometry& g, const AttnArgs& a, const Unit& un) {
+  int lo, hi;
+  pair_half(un, cluster_ctarank(), lo, hi);
+  for (int i = threadIdx.x - 64; i < (hi - lo) * 32; i += ROW_THREADS) {
+    const int lr = i >> 5, ch = i & 31, r = lo + lr;
+    if (!unit_row_valid(un, r)) continue;   // (lanes between a short block and the next head's rows)
+    const float4 v = *reinterpret_cast<const float4*>(c.gen + SM_Q + lr * STAGE_ROW + ((ch ^ (lr & 7)) << 4));
+    store_out4(a, ((size_t)(un.row0 + unit_row(un, r)) * g.Hq + unit_head(un, r)) * D + ch * 4, v);
+  }
+}
+
 template <bool PACKED, int KIND, bool SPLIT>
 __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, int first, int stride, int n_units,
                             WorkItem it) {
@@ -794,7 +884,17 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
     const float l_run = lx[0] + lx[1];
     float mul = (un.epi == EPI_OUT) ? 1.f / l_run : 1.f;
     float mul_rx = 0.f, lse2 = 0.f;   // paired step: weight of the partner's O~, merged log2 normaliser
-    if (KIND == KIND_STEP2) {
+    if constexpr (PACKED && KIND == KIND_STEP2) {
+      if (!exchange_halves<SPLIT>(c, g, a, un, r, half, tlane + TS_O + 64 * half, first_tile, m_ref, l_run)) return;
+      tc_fence_before();
+      mbar_arrive(c.bar(BAR_O_FREE));   // (one unit per CTA; kept for the barrier's phase count)
+      if (!epi_sync(c, epi_phase)) return;
+      store_half(c, g, a, un);
+      if (!epi_sync(c, epi_phase)) return;
+      if (threadIdx.x == 64) mbar_arrive(c.bar(BAR_Q_FREE));
+      continue;
+    }
+    if constexpr (!PACKED && KIND == KIND_STEP2) {
       const uint32_t rx_row = Rx<SPLIT>::O + (uint32_t)r * STAGE_ROW;
       if (un.epi == EPI_SEND) {
         // Second key chunk of its (sequence, head): O~ of the block's rows from TMEM into the partner CTA's
@@ -1732,17 +1832,20 @@ bool make_v_map(CUtensorMap* m, void* base, int H, int Tp, int box_rows, char* e
 
 namespace {
 // The step of an MHA and of a GQA model, each for blocks of more than 32 rows (the pipelined merge role for wide blocks, with
-// split planes the one with a single staging tile) and of up to 32; the paired step.
+// split planes the one with a single staging tile) and of up to 32; the paired steps (packed heads: one plane only).
 template <bool SPLIT>
 const void* const* kernel_table() {
-  static const void* const t[5] = {
+  static const void* const t[7] = {
       (const void*)tc_attn_kernel<false, KIND_STEP, SPLIT ? 0 : 2, SPLIT>, (const void*)tc_attn_kernel<false, KIND_STEP, 1, SPLIT>,
       (const void*)tc_attn_kernel<true, KIND_STEP, SPLIT ? 0 : 2, SPLIT>,  (const void*)tc_attn_kernel<true, KIND_STEP, 1, SPLIT>,
-      (const void*)tc_attn_kernel<false, KIND_STEP2, 1, SPLIT>};
+      (const void*)tc_attn_kernel<false, KIND_STEP2, 1, SPLIT>,
+      SPLIT ? nullptr : (const void*)tc_attn_kernel<true, KIND_STEP2, 2, false>,
+      SPLIT ? nullptr : (const void*)tc_attn_kernel<true, KIND_STEP2, 1, false>};
   return t;
 }
 int step_kernel(const Geometry& g, bool packed) { return (packed ? 2 : 0) + (g.block_len <= 32 ? 1 : 0); }
-constexpr int PAIRED_KERNEL = 4;   // (unpacked heads, blocks of up to 32 rows)
+// (unpacked heads: blocks of up to 32 rows; packed ones: one plane)
+int paired_kernel(const Geometry& g, bool packed) { return !packed ? 4 : g.block_len <= 32 ? 6 : 5; }
 }  // namespace
 
 // A kernel is loaded on the device when it is first asked about: a context asks for the ones it may launch and no other
@@ -1753,8 +1856,8 @@ constexpr int PAIRED_KERNEL = 4;   // (unpacked heads, blocks of up to 32 rows)
 cudaError_t tc_prepare(const Geometry& g, bool split, bool packed) {
   const void* const* t = split ? kernel_table<true>() : kernel_table<false>();
   cudaError_t e = cudaFuncSetAttribute(t[step_kernel(g, packed)], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
-  if (e == cudaSuccess && !packed && g.block_len <= 32)
-    e = cudaFuncSetAttribute(t[PAIRED_KERNEL], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
+  if (e == cudaSuccess && (packed ? !split : g.block_len <= 32))
+    e = cudaFuncSetAttribute(t[paired_kernel(g, packed)], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
   return e;
 }
 
@@ -1824,7 +1927,7 @@ cudaError_t tc_attention(const Geometry& g, const AttnArgs& a, const TcMaps* map
   cfg.attrs = attr;
   cfg.numAttrs = n_attr;
   const void* const* t = a.split ? kernel_table<true>() : kernel_table<false>();
-  const int which = paired ? PAIRED_KERNEL : step_kernel(g, a.pack > 1);
+  const int which = paired ? paired_kernel(g, a.pack > 1) : step_kernel(g, a.pack > 1);
   void* params[3] = {const_cast<TcMaps*>(maps), const_cast<Geometry*>(&g), const_cast<AttnArgs*>(&a)};
   return cudaLaunchKernelExC(&cfg, t[which], params);
 }

@@ -1,0 +1,51 @@
+"""A step of a model with grouped heads whose block rows have two key chunks, as pairs of CTAs that each merge half of a tile
+of packed heads: block lengths that fill a head's lanes and that do not, groups that leave the last tile with one to four heads,
+both output types -- against the oracle, and against the same step with its partial states merged through global memory."""
+import pytest
+import torch
+
+from paper_2607_16339_b200 import binding
+from paper_2607_16339_b200.workloads import SyntheticSchedule, small_workload
+
+from lacache_testlib import advance_to_block, check_against_oracle, make_ctx, new_outputs, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("block_len,hq,hkv", [(16, 7, 1), (24, 6, 2), (32, 8, 2), (32, 14, 2), (40, 6, 2), (48, 4, 2), (64, 7, 1), (64, 2, 1)])
+@pytest.mark.parametrize("mode", [binding.PRECISION_FP16, binding.PRECISION_PLAIN])
+def test_pairs_of_packed_heads(block_len, hq, hkv, mode, monkeypatch):
+    kw = dict(scale_mode="inv_sqrt_d") if mode == binding.PRECISION_PLAIN else {}
+    # (two key tiles of 128 in every sequence)
+    wl = small_workload(name="pairs", prompt_lens=(200 - 2 * block_len, 256 - 2 * block_len, 130 - block_len), gen_len=2 * block_len,
+                        block_len=block_len, steps=1, hq=hq, hkv=hkv, **kw)
+    pack = 4 if block_len <= 32 else 2
+    units = wl.batch * 2 * hkv * -(-(hq // hkv) // pack)
+    monkeypatch.setenv("LACACHE_STREAM_CTAS", str(units))
+    outs = {}
+    for pair in (True, False):
+        if not pair:
+            monkeypatch.setenv("LACACHE_NO_PAIR", "1")
+        sch = SyntheticSchedule(wl, seed=4)
+        q, k, v = (to_dev(a, wl) for a in advance_to_block(sch, 1))
+        step = [to_dev(a, wl) for a in sch.draw_step(1, 1)]
+        ctx = make_ctx(wl, engine=binding.ENGINE_TCGEN05, precision_mode=mode, sc_tiles_per_chunk=1)
+        ctx.build(1, q, k, v)
+        for _ in range(2):
+            out, lse = new_outputs(wl)
+            ctx.step(*step, out, lse)
+        torch.cuda.synchronize()
+        assert ctx.poll_status()[0] == 0
+        check_against_oracle(wl, sch, out, lse, None, "pair %d" % pair)
+        outs[pair] = (out, lse)
+        ctx.destroy()
+        bf = make_ctx(wl, engine=binding.ENGINE_TCGEN05, precision_mode=mode, sc_tiles_per_chunk=1, out_dtype=binding.OUT_BF16)
+        bf.build(1, q, k, v)
+        out16, lse16 = out.to(torch.bfloat16).fill_(float("nan")), torch.empty_like(lse)
+        bf.step(*step, out16, lse16)
+        torch.cuda.synchronize()
+        assert bf.poll_status()[0] == 0
+        assert torch.equal(out16, out.to(torch.bfloat16)) and torch.equal(lse16, lse)
+        bf.destroy()
+    assert (outs[True][0] - outs[False][0]).abs().max().item() <= 1e-5
+    assert (outs[True][1] - outs[False][1]).abs().max().item() <= 1e-5
