@@ -179,6 +179,18 @@ int heads_per_tile(const lacache_ctx* c) {
   return (c->g.group >= 2 && c->g.Hq >= fit && !c->knobs.no_pack) ? std::min(fit, c->g.group) : 1;
 }
 
+// units a step's block rows of one sequence and key chunk make
+int step_slots(const lacache_ctx* c) {
+  const int pack = heads_per_tile(c);
+  return c->g.Hkv * ((c->g.group + pack - 1) / pack);
+}
+StepShape step_shape(const lacache_ctx* c, double units_merge) {
+  const int pack = heads_per_tile(c), len = c->g.block_len;
+  const bool deep = len <= 32 || !c->split;
+  const bool pairs = (pack == 1 ? len <= 32 : !c->split) && !c->knobs.no_pair;
+  return StepShape{pack == 1 ? len : pack * (len <= 32 ? 32 : 64), pairs, units_merge, deep, c->knobs.deep_units, c->num_sms};
+}
+
 lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
   c->cfg = *cfg;
   c->cfg.prompt_lens = nullptr;
@@ -276,13 +288,8 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
   // builds, full recomputes and key windows run the row kernel: items of two row tiles, 128-key tiles
   const int RI = tc ? TC_ROW_ITEM : R, RI_KEYS = tc ? TC_ROW_KEYS : TC_KEYS;
   std::vector<WorkItem> items;
-  // Block-query units: the keys of each (sequence, head) are cut into balanced
-  // chunks of `tpc` tiles.  Unless the caller fixes it, pick the chunk size and
-  // the role split together from a small cost model (times in microseconds,
-  // measured on B200: a stream unit costs ~3 + 1.6 per key tile, plus ~2 + 0.8
-  // per chunk when partial states have to be merged; a merge unit ~2.6
-  // (pipelined variant, block_len <= 32, few units per CTA) or ~3.4 after a ~4 us cold start),
-  // at most 16 chunks per sequence.
+  // Block-query units: the keys of each (sequence, head) are cut into balanced chunks of `tpc` tiles, at most 16 per sequence.
+  // Unless the caller fixes it, the chunk size and the role split are picked together (step_us, lacache_plan.h).
   int tpc = cfg->sc_tiles_per_chunk;
   if (c->knobs.sc_tiles > 0) tpc = c->knobs.sc_tiles;
   if (tc && tpc <= 0) {
@@ -293,14 +300,15 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
       int n_u = c->cu[b + 1] - c->cu[b] - g.block_len;
       rows_u += (n_u + TC_ROWS - 1) / TC_ROWS + 1;
     }
-    const int sms = c->num_sms;
-    const double units_m = (double)rows_u * g.Hq;
+    const int sms = c->num_sms, slots = step_slots(c);
+    const StepShape shape = step_shape(c, (double)rows_u * g.Hq);
     double best = 1e30;
     for (int cand = 1; cand <= max_nkt; ++cand) {
       // the chunks this candidate would produce (balanced within a sequence, as below); a CTA
       // draws short and long units alike, so a unit is costed between the mean and the longest
       double units_s = 0, sum_t = 0;
       int max_ch = 1, max_t = 1;
+      bool all_two = true;
       for (int b = 0; b < g.B; ++b) {
         int nkt = (c->cu[b + 1] - c->cu[b] + TC_KEYS - 1) / TC_KEYS;
         int ch = std::min(16, (nkt + cand - 1) / cand);
@@ -308,19 +316,17 @@ lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {
         ch = (nkt + per - 1) / per;
         max_ch = std::max(max_ch, ch);
         max_t = std::max(max_t, per);
-        units_s += ch * (double)g.Hq;
+        all_two = all_two && ch == 2;
+        units_s += ch * (double)slots;
         sum_t += nkt;
       }
-      const double eff_tiles = 0.5 * (sum_t * g.Hq / units_s + max_t);
-      const double merge_cost = max_ch > 1 ? 2.0 + 0.8 * max_ch : 0.0;
-      for (int ns = std::min(8, std::max(1, sms / 4)); ns <= std::max(1, sms - 8); ns += 4) {
-        double ts = ceil(units_s / ns) * (3.0 + 1.6 * eff_tiles + merge_cost);
-        // (a CTA with many merge units runs in the HBM-saturated regime, where a unit costs more)
-        const double per_cta = ceil(units_m / (sms - ns));
-        double tm = 4.0 + per_cta * (((g.block_len <= 32 || !c->split) && per_cta <= 8) ? 2.6 : 3.4);
-        double t = std::max(ts, tm);
+      const double eff_tiles = 0.5 * (sum_t * slots / units_s + max_t);
+      auto consider = [&](int ns) {
+        const double t = step_us(shape, units_s, ns, eff_tiles, max_ch, all_two);
         if (t < best - 1e-9) { best = t; tpc = cand; }
-      }
+      };
+      if (units_s <= sms - 8) consider((int)units_s);
+      for (int ns = std::min(8, std::max(1, sms / 4)); ns <= std::max(1, sms - 8) && ns <= units_s; ns += 4) consider(ns);
     }
   }
   if (tpc <= 0) tpc = 2;
@@ -649,24 +655,19 @@ AttnArgs attn_args(lacache_ctx* c, int mode, lacache_ctx::ListRef list, int blk,
       const bool planned = plan.deep_cap == deep_cap;
       double sum_tiles = 0;   // ragged batches mix short and long units on a CTA: cost a unit between mean and longest
       int longest = 1;
+      bool all_two = true;
       for (int i = 0; i < list.n && !planned; ++i) {
         const WorkItem& w = c->items_host[list.off + i];
         sum_tiles += w.kt1 - w.kt0;
         longest = std::max(longest, w.kt1 - w.kt0);
+        all_two = all_two && w.pad == 2;
       }
       const double max_tiles = list.n > 0 ? 0.5 * (sum_tiles / list.n + longest) : 1.0;
       int ns = planned ? plan.ns : 1;
       double best = 1e30;
-      for (int cand = 1; cand < total && !planned; ++cand) {
-        double ts = ceil((double)units_stream / cand) * (3.0 + 1.6 * max_tiles + (c->max_chunks > 1 ? 2.0 + 0.8 * c->max_chunks : 0.0));
-        double per_cta = ceil((double)units_merge / (total - cand));
-        double rest = 0.0;   // merge units beyond what one launch of the pipelined variant takes: further launches, all SMs
-        if (deep_ok && per_cta > deep_cap) {
-          rest = (double)units_merge - (double)deep_cap * (total - cand);
-          per_cta = deep_cap;
-        }
-        double tm = 4.0 + per_cta * ((deep_ok && per_cta <= 8) ? 2.6 : 3.4);
-        double t = std::max(ts, tm) + (rest > 0 ? 4.0 + ceil(rest / c->num_sms) * 3.4 : 0.0);
+      const StepShape shape = step_shape(c, (double)units_merge);
+      for (int cand = 1; cand < total && cand <= units_stream && !planned; ++cand) {
+        const double t = step_us(shape, (double)units_stream, cand, max_tiles, c->max_chunks, all_two);
         if (t < best - 1e-9) { best = t; ns = cand; }
       }
       if (c->knobs.stream_ctas > 0) ns = c->knobs.stream_ctas;

@@ -1,6 +1,8 @@
 // Host-side planning without state: the work lists of the row kernel (lacache_rows.cu), made when a context is created, the
 // rule of the early trigger, and the split by role of the projection (lacache_qkv.cu).  Host code only.
 #pragma once
+#include <math.h>
+
 #include <algorithm>
 #include <vector>
 
@@ -78,6 +80,40 @@ inline void split_items(std::vector<WorkItem>& items, size_t from, int heads, in
 // for kernels that start when the one before has ended.
 inline bool early_trigger(bool overlap_on, bool short_step, bool producer_ahead, bool off) {
   return !off && (overlap_on || (short_step && !producer_ahead));
+}
+
+// What a step takes with its block-row units on ns of the SMs and its fixed-row tiles on the others, in microseconds: the
+// longer of the two roles, a little of the shorter one.  A round of block-row units is a chain of key tiles (one-plane tiles of
+// 128 keys and split ones of 96 take about the same), and with several key chunks the last CTA to arrive merges the
+// partial states of the tile's rows (`rows`: of all heads that share it): 4 us for one head of 32 rows, 10 to 12 for 128 rows;
+// more than four chunks go through the slow path.  A pair of CTAs merges in place.  Fitted to 12/2, 28/4, 32/8, 16/16 and
+// 32/32 heads, 60 to 4096 + 1024 tokens, blocks of 16 to 64 rows, 1 to 8 sequences, both operand layouts; the plan it picks
+// is within 4 % of the best one of a grid over chunks and SMs (a model that counted a unit per head, and 2.8 to 5.2 us for any
+// merge, was up to 2.3 times off it: 12/2 heads x 1212 tokens 54.0 us, now 18.4; 28/4 x 456 with split planes 23.5, now 16.0;
+// 32/8 x 5120 62.5, now 49.7).
+struct StepShape {
+  int rows;              // block rows of a tile
+  bool pairs;            // two key chunks of every unit may run as a pair of CTAs
+  double units_merge;    // fixed-row tiles, all heads
+  bool deep; int deep_cap;   // pipelined merge role, and the tiles a CTA takes in one launch of it
+  int sms;
+};
+inline double step_us(const StepShape& s, double units, int ns, double tiles, int chunks, bool all_two) {
+  double merge = 0.0;
+  if (chunks > 1) {
+    if (all_two && s.pairs && units == ns && ns % 2 == 0) merge = s.rows > 64 ? 2.5 : 1.5;
+    else if (chunks <= 4) merge = 1.0 + 0.07 * s.rows + 0.01 * s.rows * (chunks - 2);
+    else merge = 0.35 * s.rows;
+  }
+  const double ts = 9.0 + (ceil(units / ns) - 1.0) * 5.0 + ceil(units / ns) * (1.35 * tiles + merge);
+  double per_cta = s.units_merge > 0 ? ceil(s.units_merge / std::max(1, s.sms - ns)) : 0.0, rest = 0.0;
+  if (s.deep && per_cta > s.deep_cap) {   // further launches, all SMs
+    rest = s.units_merge - (double)s.deep_cap * (s.sms - ns);
+    per_cta = s.deep_cap;
+  }
+  // (a CTA with many tiles runs in the HBM-saturated regime, where a tile costs more)
+  const double tm = 8.0 + per_cta * ((s.deep && per_cta <= 8) ? 2.6 : 3.4) + (rest > 0 ? 4.0 + ceil(rest / s.sms) * 3.4 : 0.0);
+  return std::max(ts, tm) + 0.1 * std::min(ts, tm);
 }
 
 struct Range { int off, n; };   // a list within `items`
