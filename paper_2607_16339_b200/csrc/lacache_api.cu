@@ -187,7 +187,7 @@ int step_slots(const lacache_ctx* c) {
 StepShape step_shape(const lacache_ctx* c, double units_merge) {
   const int pack = heads_per_tile(c), len = c->g.block_len;
   const bool deep = len <= 32 || !c->split;
-  const bool pairs = (pack == 1 ? len <= 32 : !c->split) && !c->knobs.no_pair;
+  const bool pairs = (pack > 1 || len <= 32) && !c->knobs.no_pair;
   return StepShape{pack == 1 ? len : pack * (len <= 32 ? 32 : 64), pairs, units_merge, deep, c->knobs.deep_units, c->num_sms};
 }
 
@@ -694,9 +694,9 @@ AttnArgs attn_args(lacache_ctx* c, int mode, lacache_ctx::ListRef list, int blk,
         // lose 0.3 us; a step from token ids, behind which the projection's CTAs would wait on SMs, between -0.8 and 2.8.
         a.step_overlap = (a.merge_deep && !c->split && c->g.block_len <= 32 && per_cta <= 5) ? 1 : 0;
       }
-      // Two key chunks per (sequence, head), one round of block-row units: the two chunks of a head (of a group of packed heads,
-      // with one plane) run as a pair of CTAs that merge through distributed shared memory.
-      if ((a.pack == 1 ? c->g.block_len <= 32 : !c->split) && (a.merge_deep || a.split_merge) && !c->knobs.no_pair &&
+      // Two key chunks per (sequence, head), one round of block-row units: the two chunks of a head (of a group of packed heads)
+      // run as a pair of CTAs that merge through distributed shared memory.
+      if (shape.pairs && (a.merge_deep || a.split_merge || !deep_ok) &&
           units_stream == ns && (ns % 2) == 0 && (a.n_ctas % 2) == 0) {
         if (plan.pair < 0) {
           plan.pair = 1;

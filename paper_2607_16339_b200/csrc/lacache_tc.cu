@@ -87,9 +87,11 @@ struct Rx {
   static constexpr uint32_t O = Tile<SPLIT>::SM_V + 2 * Tile<SPLIT>::V_STAGE;
   static constexpr uint32_t ML = SM_Q + 32768 + 32 * STAGE_ROW;
   static_assert(O + 32 * STAGE_ROW <= SM_XCH && ML + 32 * 8 <= SM_K, "no room for the partner's partial state");
-  // packed heads (one plane): half of a tile's rows, up to 64 of them, and their (m, l) in the upper half of the Q region, which
-  // neither the 128-row Q tile nor the rows staged over it reach
-  static constexpr uint32_t ML_PACKED = SM_Q + 32768;
+  // packed heads: half of a tile's rows, up to 64 of them.  One plane: in the same place, and (m, l) in the upper half of the Q
+  // region, which neither the 128-row Q tile nor the rows staged over it reach.  Split planes: over the key stages, once
+  // the CTA's last products are done (BAR_RX_READY).
+  static constexpr uint32_t O_PACKED = SPLIT ? SM_K : O;
+  static constexpr uint32_t ML_PACKED = SPLIT ? SM_K + 64 * STAGE_ROW : SM_Q + 32768;
   static_assert(SPLIT || O + 64 * STAGE_ROW <= SM_XCH, "no room for half a tile of the partner's partial state");
 };
 // merge role: the 96 KB after Q hold 2 stages of the block's keys {K hi, K lo, V} of 64
@@ -130,6 +132,7 @@ enum {
   BAR_IO_FULL1, BAR_OUT_RDY, BAR_OUT_RDY1,  // pipelined merge role: second staging tile; output tile b is complete
   BAR_PAIR,  // 4 barriers: the two warps that share a TMEM lane quadrant
   N_BARS = BAR_PAIR + 4,
+  BAR_RX_READY = BAR_OUT_RDY,  // ... packed heads, split planes: the partner's key stages may be written
   BAR_RX = BAR_IO_FULL,  // stream role of a paired step (it has no staging-tile barriers): the partner's partial state has arrived
 };
 
@@ -147,7 +150,7 @@ __device__ __forceinline__ void load_v_box(uint32_t dst, const CUtensorMap* map,
 // thread-block cluster: the CTA with the second chunk hands its partial state to its partner through
 // distributed shared memory, and the partner writes the merged rows (one round of units; the place of the receiving buffer:
 // see Rx).  With packed heads, whose tiles have up to 128 rows, each CTA merges and writes half of the tile's rows and hands
-// the other half's partial states to its partner (one plane only: split planes leave no room).
+// the other half's partial states to its partner.
 enum StreamKind : int { KIND_STEP = 1, KIND_STEP2 = 3 };
 
 struct Unit {
@@ -635,18 +638,9 @@ __device__ __forceinline__ bool exchange_halves(const Cta& c, const Geometry& g,
 #pragma unroll
     for (int i = 0; i < 64; ++i) o[i] = 0u;
   }
-  if (theirs) {
-    const int pr = r - plo;
-    const uint32_t dst = mapa_shared(c.base + Rx<SPLIT>::O + (uint32_t)pr * STAGE_ROW, peer);
-#pragma unroll
-    for (int i = 0; i < 16; ++i)
-      st_cluster_v4(dst + (((16 * half + i) ^ (pr & 7)) << 4), __uint_as_float(o[4 * i]), __uint_as_float(o[4 * i + 1]),
-                    __uint_as_float(o[4 * i + 2]), __uint_as_float(o[4 * i + 3]));
-    if (half == 0) st_cluster_v2(mapa_shared(c.base + Rx<SPLIT>::ML_PACKED + (uint32_t)pr * 8u, peer), m, l);
-  }
-  mbar_arrive_cluster(mapa_shared(c.bar(BAR_RX), peer));   // (a release: it makes the stores visible to the acquiring wait)
-  {
-    const uint32_t bar = c.bar(BAR_RX);
+  // (`which`: a barrier the partner arrives on, waited for with its stores acquired)
+  auto wait_partner = [&](int which) -> bool {
+    const uint32_t bar = c.bar(which);
     const long long t0 = clock64();
     while (!mbar_try_acquire_cluster(bar, 0u)) {
       if (*c.abort_flag) return false;
@@ -658,7 +652,24 @@ __device__ __forceinline__ bool exchange_halves(const Cta& c, const Geometry& g,
         return false;
       }
     }
+    return true;
+  };
+  if constexpr (SPLIT) {
+    // (every row thread of this CTA has seen its last products complete: the caller's rendezvous)
+    if (threadIdx.x == 64) mbar_arrive_cluster(mapa_shared(c.bar(BAR_RX_READY), peer));
+    if (!wait_partner(BAR_RX_READY)) return false;
   }
+  if (theirs) {
+    const int pr = r - plo;
+    const uint32_t dst = mapa_shared(c.base + Rx<SPLIT>::O_PACKED + (uint32_t)pr * STAGE_ROW, peer);
+#pragma unroll
+    for (int i = 0; i < 16; ++i)
+      st_cluster_v4(dst + (((16 * half + i) ^ (pr & 7)) << 4), __uint_as_float(o[4 * i]), __uint_as_float(o[4 * i + 1]),
+                    __uint_as_float(o[4 * i + 2]), __uint_as_float(o[4 * i + 3]));
+    if (half == 0) st_cluster_v2(mapa_shared(c.base + Rx<SPLIT>::ML_PACKED + (uint32_t)pr * 8u, peer), m, l);
+  }
+  mbar_arrive_cluster(mapa_shared(c.bar(BAR_RX), peer));   // (a release: it makes the stores visible to the acquiring wait)
+  if (!wait_partner(BAR_RX)) return false;
   if (mine) {
     const int lr = r - lo;
     const float2 ml = *reinterpret_cast<const float2*>(c.gen + Rx<SPLIT>::ML_PACKED + lr * 8);
@@ -670,7 +681,7 @@ __device__ __forceinline__ bool exchange_halves(const Cta& c, const Geometry& g,
 #pragma unroll
     for (int i = 0; i < 16; ++i) {
       const uint32_t off = (uint32_t)lr * STAGE_ROW + (((16 * half + i) ^ (lr & 7)) << 4);
-      const float4 p = *reinterpret_cast<const float4*>(c.gen + Rx<SPLIT>::O + off);
+      const float4 p = *reinterpret_cast<const float4*>(c.gen + Rx<SPLIT>::O_PACKED + off);
       *reinterpret_cast<float4*>(c.gen + SM_Q + off) =
           make_float4(fmaf(p.x, f2, __uint_as_float(o[4 * i]) * f1), fmaf(p.y, f2, __uint_as_float(o[4 * i + 1]) * f1),
                       fmaf(p.z, f2, __uint_as_float(o[4 * i + 2]) * f1), fmaf(p.w, f2, __uint_as_float(o[4 * i + 3]) * f1));
@@ -1668,6 +1679,7 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
       if (i == BAR_DONE) count = THREADS;
       if (i == BAR_Q_FREE && stream) count = 2;  // score MMAs done + epilogue staging read
       if (KIND == KIND_STEP2 && i == BAR_RX && stream) count = ROW_THREADS;  // the partner's row threads
+      if (PACKED && KIND == KIND_STEP2 && SPLIT && i == BAR_RX_READY && stream) count = 1;
       if (i >= BAR_PAIR) count = 64;
       mbar_init(c.bar(i), count);
     }
@@ -1832,19 +1844,18 @@ bool make_v_map(CUtensorMap* m, void* base, int H, int Tp, int box_rows, char* e
 
 namespace {
 // The step of an MHA and of a GQA model, each for blocks of more than 32 rows (the pipelined merge role for wide blocks, with
-// split planes the one with a single staging tile) and of up to 32; the paired steps (packed heads: one plane only).
+// split planes the one with a single staging tile) and of up to 32; the paired steps.
 template <bool SPLIT>
 const void* const* kernel_table() {
   static const void* const t[7] = {
       (const void*)tc_attn_kernel<false, KIND_STEP, SPLIT ? 0 : 2, SPLIT>, (const void*)tc_attn_kernel<false, KIND_STEP, 1, SPLIT>,
       (const void*)tc_attn_kernel<true, KIND_STEP, SPLIT ? 0 : 2, SPLIT>,  (const void*)tc_attn_kernel<true, KIND_STEP, 1, SPLIT>,
       (const void*)tc_attn_kernel<false, KIND_STEP2, 1, SPLIT>,
-      SPLIT ? nullptr : (const void*)tc_attn_kernel<true, KIND_STEP2, 2, false>,
-      SPLIT ? nullptr : (const void*)tc_attn_kernel<true, KIND_STEP2, 1, false>};
+      (const void*)tc_attn_kernel<true, KIND_STEP2, SPLIT ? 0 : 2, SPLIT>, (const void*)tc_attn_kernel<true, KIND_STEP2, 1, SPLIT>};
   return t;
 }
 int step_kernel(const Geometry& g, bool packed) { return (packed ? 2 : 0) + (g.block_len <= 32 ? 1 : 0); }
-// (unpacked heads: blocks of up to 32 rows; packed ones: one plane)
+// (unpacked heads: blocks of up to 32 rows)
 int paired_kernel(const Geometry& g, bool packed) { return !packed ? 4 : g.block_len <= 32 ? 6 : 5; }
 }  // namespace
 
@@ -1856,7 +1867,7 @@ int paired_kernel(const Geometry& g, bool packed) { return !packed ? 4 : g.block
 cudaError_t tc_prepare(const Geometry& g, bool split, bool packed) {
   const void* const* t = split ? kernel_table<true>() : kernel_table<false>();
   cudaError_t e = cudaFuncSetAttribute(t[step_kernel(g, packed)], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
-  if (e == cudaSuccess && (packed ? !split : g.block_len <= 32))
+  if (e == cudaSuccess && (packed || g.block_len <= 32))
     e = cudaFuncSetAttribute(t[paired_kernel(g, packed)], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
   return e;
 }

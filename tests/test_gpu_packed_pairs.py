@@ -13,11 +13,12 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("block_len,hq,hkv", [(16, 7, 1), (24, 6, 2), (32, 8, 2), (32, 14, 2), (40, 6, 2), (48, 4, 2), (64, 7, 1), (64, 2, 1)])
-@pytest.mark.parametrize("mode", [binding.PRECISION_FP16, binding.PRECISION_PLAIN])
+@pytest.mark.parametrize("mode", [binding.PRECISION_FP16, binding.PRECISION_PLAIN, binding.PRECISION_SPLIT])
 def test_pairs_of_packed_heads(block_len, hq, hkv, mode, monkeypatch):
     kw = dict(scale_mode="inv_sqrt_d") if mode == binding.PRECISION_PLAIN else {}
-    # (two key tiles of 128 in every sequence)
-    wl = small_workload(name="pairs", prompt_lens=(200 - 2 * block_len, 256 - 2 * block_len, 130 - block_len), gen_len=2 * block_len,
+    # (two key tiles in every sequence, of 128 keys, or 96 with split planes)
+    lens = (180, 192, 100) if mode == binding.PRECISION_SPLIT else (200, 256, 130)
+    wl = small_workload(name="pairs", prompt_lens=tuple(max(1, n - 2 * block_len) for n in lens), gen_len=2 * block_len,
                         block_len=block_len, steps=1, hq=hq, hkv=hkv, **kw)
     pack = 4 if block_len <= 32 else 2
     units = wl.batch * 2 * hkv * -(-(hq // hkv) // pack)
