@@ -187,7 +187,7 @@ int step_slots(const lacache_ctx* c) {
 StepShape step_shape(const lacache_ctx* c, double units_merge) {
   const int pack = heads_per_tile(c), len = c->g.block_len;
   const bool deep = len <= 32 || !c->split;
-  const bool pairs = (pack > 1 || len <= 32) && !c->knobs.no_pair;
+  const bool pairs = (pack > 1 || len <= 32 || !c->split) && !c->knobs.no_pair;
   return StepShape{pack == 1 ? len : pack * (len <= 32 ? 32 : 64), pairs, units_merge, deep, c->knobs.deep_units, c->num_sms};
 }
 

@@ -87,7 +87,7 @@ struct Rx {
   static constexpr uint32_t O = Tile<SPLIT>::SM_V + 2 * Tile<SPLIT>::V_STAGE;
   static constexpr uint32_t ML = SM_Q + 32768 + 32 * STAGE_ROW;
   static_assert(O + 32 * STAGE_ROW <= SM_XCH && ML + 32 * 8 <= SM_K, "no room for the partner's partial state");
-  // packed heads: half of a tile's rows, up to 64 of them.  One plane: in the same place, and (m, l) in the upper half of the Q
+  // half of a tile's rows, up to 64 of them.  One plane: in the same place, and (m, l) in the upper half of the Q
   // region, which neither the 128-row Q tile nor the rows staged over it reach.  Split planes: over the key stages, once
   // the CTA's last products are done (BAR_RX_READY).
   static constexpr uint32_t O_PACKED = SPLIT ? SM_K : O;
@@ -149,9 +149,10 @@ __device__ __forceinline__ void load_v_box(uint32_t dst, const CUtensorMap* map,
 // KIND_STEP2: a step whose block-row units all have exactly two key chunks, run by the two CTAs of a
 // thread-block cluster: the CTA with the second chunk hands its partial state to its partner through
 // distributed shared memory, and the partner writes the merged rows (one round of units; the place of the receiving buffer:
-// see Rx).  With packed heads, whose tiles have up to 128 rows, each CTA merges and writes half of the tile's rows and hands
-// the other half's partial states to its partner.
-enum StreamKind : int { KIND_STEP = 1, KIND_STEP2 = 3 };
+// see Rx).  KIND_STEP2X: likewise, but each CTA merges and writes half of the tile's rows and hands the other half's partial
+// states to its partner -- packed heads, whose tiles have up to 128 rows, and blocks of 33 to 64 rows.  (For one head of 32 rows
+// the one-way hand-over is the faster: 19.8 us against 20.1 for 32 heads x 768 tokens with split planes.)
+enum StreamKind : int { KIND_STEP = 1, KIND_STEP2 = 3, KIND_STEP2X = 5 };
 
 struct Unit {
   int row0, nrows, h, kh, seq;
@@ -178,7 +179,7 @@ __device__ __forceinline__ bool unit_row_valid(const Unit& un, int r) {
 // (u / 2) % Hq of sequence (u / 2) / Hq, and u % 2 its key chunk: a sequence's two chunk items are adjacent)
 template <bool PACKED, int KIND>
 __device__ __forceinline__ int unit_item(const Geometry& g, const AttnArgs& a, int u) {
-  if (KIND == KIND_STEP2) return ((u >> 1) / (PACKED ? a.stream_slots : g.Hq)) * 2 + (u & 1);
+  if (KIND != KIND_STEP) return ((u >> 1) / (PACKED ? a.stream_slots : g.Hq)) * 2 + (u & 1);
   return u / (PACKED ? a.stream_slots : g.Hq);
 }
 
@@ -190,7 +191,7 @@ __device__ __forceinline__ Unit decode_stream(const Geometry& g, const AttnArgs&
   Unit un;
   // units are head-minor: unit u = item u / slots of head (or head group) u % slots (a CTA's units, a
   // fixed stride apart, then cycle through the items instead of drawing one item's heads)
-  const int slot = (KIND == KIND_STEP2 ? (u >> 1) : u) % (PACKED ? a.stream_slots : g.Hq);
+  const int slot = (KIND != KIND_STEP ? (u >> 1) : u) % (PACKED ? a.stream_slots : g.Hq);
   if (PACKED) {
     const int per_kv = (g.group + a.pack - 1) / a.pack;
     un.kh = slot / per_kv;
@@ -609,9 +610,9 @@ __device__ __forceinline__ void merge_partials(const Geometry& g, const AttnArgs
   }
 }
 
-// Paired step with packed heads: rows [lo, hi) of a tile, which this CTA of the pair writes (rank 0 the first half).
+// Paired step: rows [lo, hi) of a tile, which this CTA of the pair writes (rank 0 the first half).
 __device__ __forceinline__ void pair_half(const Unit& un, uint32_t rank, int& lo, int& hi) {
-  const int rows = un.nh * un.rh;
+  const int rows = un.rh ? un.nh * un.rh : un.nrows;
   lo = rank ? rows / 2 : 0;
   hi = rank ? rows : rows / 2;
 }
@@ -895,17 +896,17 @@ __device__ void stream_rows(const Cta& c, const Geometry& g, const AttnArgs& a, 
     const float l_run = lx[0] + lx[1];
     float mul = (un.epi == EPI_OUT) ? 1.f / l_run : 1.f;
     float mul_rx = 0.f, lse2 = 0.f;   // paired step: weight of the partner's O~, merged log2 normaliser
-    if constexpr (PACKED && KIND == KIND_STEP2) {
+    if constexpr (KIND == KIND_STEP2X) {
       if (!exchange_halves<SPLIT>(c, g, a, un, r, half, tlane + TS_O + 64 * half, first_tile, m_ref, l_run)) return;
       tc_fence_before();
       mbar_arrive(c.bar(BAR_O_FREE));   // (one unit per CTA; kept for the barrier's phase count)
       if (!epi_sync(c, epi_phase)) return;
       store_half(c, g, a, un);
       if (!epi_sync(c, epi_phase)) return;
-      if (threadIdx.x == 64) mbar_arrive(c.bar(BAR_Q_FREE));
+      if (un.q_rows == BM && threadIdx.x == 64) mbar_arrive(c.bar(BAR_Q_FREE));
       continue;
     }
-    if constexpr (!PACKED && KIND == KIND_STEP2) {
+    if constexpr (KIND == KIND_STEP2) {
       const uint32_t rx_row = Rx<SPLIT>::O + (uint32_t)r * STAGE_ROW;
       if (un.epi == EPI_SEND) {
         // Second key chunk of its (sequence, head): O~ of the block's rows from TMEM into the partner CTA's
@@ -1678,8 +1679,8 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
         count = ROW_THREADS;
       if (i == BAR_DONE) count = THREADS;
       if (i == BAR_Q_FREE && stream) count = 2;  // score MMAs done + epilogue staging read
-      if (KIND == KIND_STEP2 && i == BAR_RX && stream) count = ROW_THREADS;  // the partner's row threads
-      if (PACKED && KIND == KIND_STEP2 && SPLIT && i == BAR_RX_READY && stream) count = 1;
+      if (KIND != KIND_STEP && i == BAR_RX && stream) count = ROW_THREADS;  // the partner's row threads
+      if (KIND == KIND_STEP2X && SPLIT && i == BAR_RX_READY && stream) count = 1;
       if (i >= BAR_PAIR) count = 64;
       mbar_init(c.bar(i), count);
     }
@@ -1711,7 +1712,7 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
   c.tmem = words[0];
   // (paired step: nobody writes into the partner's shared memory or arrives on its barrier before the
   // partner has initialised them)
-  if (KIND == KIND_STEP2) cluster_sync_all();
+  if (KIND != KIND_STEP) cluster_sync_all();
 
   if (warp == 0) {
     if (stream) {
@@ -1847,16 +1848,17 @@ namespace {
 // split planes the one with a single staging tile) and of up to 32; the paired steps.
 template <bool SPLIT>
 const void* const* kernel_table() {
-  static const void* const t[7] = {
+  static const void* const t[8] = {
       (const void*)tc_attn_kernel<false, KIND_STEP, SPLIT ? 0 : 2, SPLIT>, (const void*)tc_attn_kernel<false, KIND_STEP, 1, SPLIT>,
       (const void*)tc_attn_kernel<true, KIND_STEP, SPLIT ? 0 : 2, SPLIT>,  (const void*)tc_attn_kernel<true, KIND_STEP, 1, SPLIT>,
       (const void*)tc_attn_kernel<false, KIND_STEP2, 1, SPLIT>,
-      (const void*)tc_attn_kernel<true, KIND_STEP2, SPLIT ? 0 : 2, SPLIT>, (const void*)tc_attn_kernel<true, KIND_STEP2, 1, SPLIT>};
+      (const void*)tc_attn_kernel<true, KIND_STEP2X, SPLIT ? 0 : 2, SPLIT>, (const void*)tc_attn_kernel<true, KIND_STEP2X, 1, SPLIT>,
+      SPLIT ? nullptr : (const void*)tc_attn_kernel<false, KIND_STEP2X, 2, false>};
   return t;
 }
 int step_kernel(const Geometry& g, bool packed) { return (packed ? 2 : 0) + (g.block_len <= 32 ? 1 : 0); }
-// (unpacked heads: blocks of up to 32 rows)
-int paired_kernel(const Geometry& g, bool packed) { return !packed ? 4 : g.block_len <= 32 ? 6 : 5; }
+// (unpacked heads, blocks of more than 32 rows: one plane; with split planes no faster, 45.9 us against 45.7 at 32 heads x 2512 tokens)
+int paired_kernel(const Geometry& g, bool packed) { return packed ? (g.block_len <= 32 ? 6 : 5) : (g.block_len <= 32 ? 4 : 7); }
 }  // namespace
 
 // A kernel is loaded on the device when it is first asked about: a context asks for the ones it may launch and no other
@@ -1867,7 +1869,7 @@ int paired_kernel(const Geometry& g, bool packed) { return !packed ? 4 : g.block
 cudaError_t tc_prepare(const Geometry& g, bool split, bool packed) {
   const void* const* t = split ? kernel_table<true>() : kernel_table<false>();
   cudaError_t e = cudaFuncSetAttribute(t[step_kernel(g, packed)], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
-  if (e == cudaSuccess && (packed || g.block_len <= 32))
+  if (e == cudaSuccess && (packed || g.block_len <= 32 || !split))
     e = cudaFuncSetAttribute(t[paired_kernel(g, packed)], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM_TOTAL);
   return e;
 }

@@ -1,6 +1,6 @@
-"""A step of a model with grouped heads whose block rows have two key chunks, as pairs of CTAs that each merge half of a tile
-of packed heads: block lengths that fill a head's lanes and that do not, groups that leave the last tile with one to four heads,
-both output types -- against the oracle, and against the same step with its partial states merged through global memory."""
+"""A step whose block rows have two key chunks, as pairs of CTAs that each merge half of a tile -- of one head, or of packed ones:
+block lengths that fill a head's lanes and that do not, odd ones, groups that leave the last tile with one to four heads, both
+output types -- against the oracle, and against the same step with its partial states merged through global memory."""
 import pytest
 import torch
 
@@ -12,7 +12,8 @@ from lacache_testlib import advance_to_block, check_against_oracle, make_ctx, ne
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("block_len,hq,hkv", [(16, 7, 1), (24, 6, 2), (32, 8, 2), (32, 14, 2), (40, 6, 2), (48, 4, 2), (64, 7, 1), (64, 2, 1)])
+@pytest.mark.parametrize("block_len,hq,hkv", [(16, 7, 1), (24, 6, 2), (32, 8, 2), (32, 14, 2), (40, 6, 2), (48, 4, 2), (64, 7, 1), (64, 2, 1),
+                                              (16, 2, 2), (17, 2, 2), (32, 3, 3), (40, 2, 2), (63, 2, 2), (64, 3, 3)])
 @pytest.mark.parametrize("mode", [binding.PRECISION_FP16, binding.PRECISION_PLAIN, binding.PRECISION_SPLIT])
 def test_pairs_of_packed_heads(block_len, hq, hkv, mode, monkeypatch):
     kw = dict(scale_mode="inv_sqrt_d") if mode == binding.PRECISION_PLAIN else {}
@@ -21,7 +22,7 @@ def test_pairs_of_packed_heads(block_len, hq, hkv, mode, monkeypatch):
     wl = small_workload(name="pairs", prompt_lens=tuple(max(1, n - 2 * block_len) for n in lens), gen_len=2 * block_len,
                         block_len=block_len, steps=1, hq=hq, hkv=hkv, **kw)
     pack = 4 if block_len <= 32 else 2
-    units = wl.batch * 2 * hkv * -(-(hq // hkv) // pack)
+    units = wl.batch * 2 * (hq if hq == hkv else hkv * -(-(hq // hkv) // pack))
     monkeypatch.setenv("LACACHE_STREAM_CTAS", str(units))
     outs = {}
     for pair in (True, False):
