@@ -511,19 +511,47 @@ cudaError_t simt_prepare() {
                               (int)Smem<64>::bytes);
 }
 
+namespace {
+
+// The CTAs a unit is cut over.  A step's block queries are few and its chain: as many parts as leave three CTAs to an SM, the
+// fixed rows' included (8 heads, two sequences: 34 fixed-row tiles and blocks of 32 rows 24.0 us cut in 5, 20.2 in 8; blocks of 64
+// 44.7 in 8, 36.6 in 5).
+int split_of_step(long long units, long long rest, int max_tiles, int num_sms) {
+  int S = 1;
+  while (S < MAX_SPLIT && S < max_tiles && units * (S + 1) + rest <= 3ll * num_sms) ++S;
+  return std::max(S, std::min(2, max_tiles));
+}
+// Builds and full recomputes: every part costs its prologue and merge again, long parts end unevenly.  A part's time with n
+// CTAs on its SM (four fit) is tiles x max(3.6, 2.2 n) + 2.5 n + 3 us at 128 features; rounds of four to an SM, then the rest of
+// them, unevenly placed where the RoPE kernel ahead still holds SMs.  (Cuts in 3, 5 and 7 pack badly.)  672 units of 20 tiles:
+// 314 us cut in 8, as before, 238 in 2; 472 of 20: 229 and 192 (in 4; 180 in 2); 152 of 10: 52 in 5, and in 4.
+int split_of_rows(long long units, int max_tiles, int d, int num_sms) {
+  if (max_tiles < 4) return units < num_sms ? max_tiles : std::max(1, max_tiles / 2);
+  int S = 2;
+  double best = 1e30;
+  for (int c = 2; c <= std::min(MAX_SPLIT, max_tiles / 2); c += 2) {
+    const double tiles = (double)max_tiles / c * d / 128;
+    auto part = [&](double n) { return tiles * std::max(3.6, 2.2 * n) + 2.5 * n + 3.0; };
+    const long long ctas = units * c, rounds = ctas / (4ll * num_sms), left = ctas % (4ll * num_sms);
+    const double t = rounds * part(4) + (left > 0 ? part((double)std::min(4ll, (left + num_sms - 1) / num_sms + 1)) : 0.0);
+    if (t < best - 1e-9) { best = t; S = c; }
+  }
+  return S;
+}
+
+}  // namespace
+
 cudaError_t simt_attention(const Geometry& g, const AttnArgs& args, int num_sms, cudaStream_t s) {
   AttnArgs a = args;
   if (a.n_items == 0) return cudaSuccess;
-  // Units with the long key range: the block queries of a step (its first items), every unit otherwise.  They
-  // are cut into parts of at least two tiles; of one where even that leaves SMs without a CTA, because a
-  // part's chain of tiles is then all the launch takes.
+  // Units with the long key range: the block queries of a step (its first items), every unit otherwise.
   const bool step = a.mode == MODE_STEP;
   if (!step) a.n_split_items = a.n_items;
   const int rest = a.n_items - a.n_split_items;
   const int max_tiles = (g.maxN + KT - 1) / KT;
-  int S = std::min(MAX_SPLIT, std::max(1, max_tiles / 2));
-  if ((long long)(a.n_split_items * S + rest) * g.Hq < num_sms) S = std::min(MAX_SPLIT, max_tiles);
-  a.split_ctas = S;
+  a.split_ctas = step ? split_of_step((long long)a.n_split_items * g.Hq, (long long)rest * g.Hq, max_tiles, num_sms)
+                      : split_of_rows((long long)a.n_items * g.Hq, max_tiles, g.d, num_sms);
+  const int S = a.split_ctas;
   const int n_ctas = a.n_split_items * S + (rest + S - 1) / S * S;
   return g.d == 128 ? launch<128>(g, a, n_ctas, s) : launch<64>(g, a, n_ctas, s);
 }
