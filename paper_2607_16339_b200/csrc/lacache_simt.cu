@@ -119,10 +119,6 @@ __global__ void __launch_bounds__(THREADS, 3) simt_attn_kernel(const __grid_cons
   constexpr int DPL = D / 32;        // output features per lane (P.V)
   extern __shared__ __align__(16) float sm[];
 
-  // Launched programmatically dependent: nothing is touched before the grids ahead have completed, but this
-  // grid's launch overlaps their end.
-  grid_dependency_wait();
-
   // the first n_split_items items are cut over the `split` CTAs of a cluster, the others take one CTA each
   const int S = a.split_ctas;
   int item = (int)blockIdx.x, part = 0, n_parts = 1;
@@ -140,6 +136,9 @@ __global__ void __launch_bounds__(THREADS, 3) simt_attn_kernel(const __grid_cons
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int bs = a.blk_start ? a.blk_start[it.seq] : 0;
   const int be = bs + g.block_len;
+  // Launched programmatically dependent: but for the lists above, which nothing writes, nothing is touched before the grids
+  // ahead have completed; this grid's launch and those two round trips to L2 overlap their end.
+  grid_dependency_wait();
 
   int k0 = it.seq_start, k1 = it.seq_end, x0 = 0, x1 = 0;
   bool from_state = false, to_state = false;
