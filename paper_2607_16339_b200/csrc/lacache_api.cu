@@ -188,7 +188,8 @@ StepShape step_shape(const lacache_ctx* c, double units_merge) {
   const int pack = heads_per_tile(c), len = c->g.block_len;
   const bool deep = len <= 32 || !c->split;
   const bool pairs = (pack > 1 || len <= 32 || !c->split) && !c->knobs.no_pair;
-  return StepShape{pack == 1 ? len : pack * (len <= 32 ? 32 : 64), pairs, units_merge, deep, c->knobs.deep_units, c->num_sms};
+  // (not the knob that makes small steps go out in several launches: their plan, and so their bits, are those of one launch)
+  return StepShape{pack == 1 ? len : pack * (len <= 32 ? 32 : 64), pairs, units_merge, deep, TC_DEEP_MAX_UNITS, c->num_sms};
 }
 
 lacache_status create_impl(const lacache_config* cfg, lacache_ctx* c) {

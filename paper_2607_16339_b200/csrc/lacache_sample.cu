@@ -138,13 +138,13 @@ __global__ void __launch_bounds__(SAMPLE_THREADS, SHAPE::CTAS) sample_rows_kerne
   constexpr int DEPTH = SHAPE::DEPTH;               // batches of a lane in flight, the one in hand included
   const int lane = threadIdx.x & 31;
   const int warp = (int)blockIdx.x * WARPS + (int)(threadIdx.x >> 5);
-  // launched programmatically dependent: nothing is touched before the grids ahead have completed
+  const int r = warp / a.segments, seg = warp - r * a.segments;
+  const int row = r < a.n_rows ? a.rows[r] : 0;   // (the context's own list, which nothing writes)
+  // launched programmatically dependent: nothing else is touched before the grids ahead have completed
   grid_dependency_wait();
 
-  const int r = warp / a.segments, seg = warp - r * a.segments;
   if (r < a.n_rows) {
     const int lo = seg * a.quota, hi = min(lo + a.quota, a.vocab);
-    const int row = a.rows[r];
     const bool bad = row < 0 || row >= a.n_tokens;
     // s: the sum of 2^(x log2 e - R); R = m log2 e, rounded (0 before any finite logit).
     // `at`: where m was first seen -- >= 0: a batch of vectors that starts there; < 0: element ~at
