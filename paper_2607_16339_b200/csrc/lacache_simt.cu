@@ -9,14 +9,13 @@
 // Mapping: a CTA of 4 warps owns 32 query rows of one (sequence, q head), 8 rows a
 // warp, and walks key tiles of 32.  A unit with many keys is cut over the S <= 8
 // CTAs of a thread-block cluster, whose online-softmax states are merged through
-// distributed shared memory.  What bounds this kernel at the sizes it serves is
-// not arithmetic but too few warps, each waiting for its own shared-memory loads
-// (a small model has about as many row tiles as the GPU has SMs), and the last
-// CTAs of an uneven wave: hence small CTAs, four to an SM, and many of them.
+// distributed shared memory (how many: split_of_rows, split_of_step).  A tile is bound by the shared-memory pipe, which a 16-byte
+// load holds for four cycles: a tile's scores take 3118 cycles on an SM of their own, as six loads per step, 32 steps and
+// four warps say, P.V 2000.  Around the tiles it is latency (4000 to 7000 cycles from the wait for the grids ahead to the
+// queries in place) and the last CTAs of an uneven wave: hence small CTAs, four to an SM, and many of them.
 // Per tile, a warp computes its 8 x 32 scores with 4 rows x 2 keys per lane and
 // its 8 x d part of P.V with 8 rows x d/32 features per lane: 32 products per 6
-// to 8 shared-memory wavefronts, which keeps the FMA pipe and the shared-memory
-// pipe about equally busy (one key and one row at a time, as this kernel once
+// to 8 shared-memory loads (one key and one row at a time, as this kernel once
 // did, read 9 words per 4 products).  Values stream in while the scores are
 // computed and the next keys while P.V is (cp.async, one buffer of each).
 //
