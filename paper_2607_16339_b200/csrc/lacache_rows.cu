@@ -179,30 +179,11 @@ __device__ __forceinline__ bool wait_here(const Cta& c, int slot, uint32_t parit
 // ---- producers ----------------------------------------------------------------------------------------------
 // One lane each for Q' tiles, key tiles and value tiles, with blocking waits (one lane that polled all three took several
 // hundred cycles to notice a free stage, which with two stages is time the tensor core waits).
-// The stored state a unit starts from (one contiguous run of its rows), asked into L2.
-__device__ __forceinline__ void prefetch_state(const Geometry& g, const AttnArgs& a, const Unit& un) {
-  const size_t srow = (size_t)un.h * g.Tp + un.row0;
-  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.init.o + srow * D), "r"(un.nrows * D * 4) : "memory");
-  for (int i = 0; i < un.nrows; i += 32) {
-    prefetch_l2(a.init.m + srow + i);
-    prefetch_l2(a.init.l + srow + i);
-  }
-}
 template <bool SPLIT, bool WINDOW>
 __device__ void load_queries(const Cta& c, const RowMaps& maps, const Geometry& g, const AttnArgs& a, const Walk& wk) {
   int n0 = 0, n1 = 0;   // Q' tiles loaded, per tile slot
   for (int k_ = 0, u = wk.unit(0); u < wk.n_units; u = wk.unit(++k_)) {
     const Unit un = decode<WINDOW>(g, a, u);
-    if (WINDOW) {
-      // The state of the next unit: this one's Q' is requested when the unit before has no more scores to issue, so
-      // its rows have a unit's time to come into L2 before the row threads ask for them.
-      if (k_ == 0 && un.init) prefetch_state(g, a, un);
-      const int u2 = wk.unit(k_ + 1);
-      if (u2 < wk.n_units) {
-        const Unit nx = decode<WINDOW>(g, a, u2);
-        if (nx.init) prefetch_state(g, a, nx);
-      }
-    }
     if (un.n_tiles == 0) continue;
     for (int x = 0; x < un.tiles(); ++x) {
       const int n = x ? n1 : n0;
@@ -397,33 +378,47 @@ __device__ __forceinline__ uint64_t span_bits(int lo, int hi) {   // bits [lo, h
 
 // Rows of a stored state (the warp's first `rows`; zeros behind them) to the warp's lanes of O~ in TMEM: all loads leave
 // together, 128 contiguous bytes of four rows each, and pass through the warp's staging (thread per row, a load would
-// touch 32 rows).  Split planes have no staging.  (Plain loads: the launch may update these rows in place.)
+// touch 32 rows).  Split planes have no staging: thread per row.  (Plain loads: the launch may update these rows in place.)
 template <bool SPLIT>
 __device__ __forceinline__ void load_rows(const Cta& c, uint32_t o_tmem, const float* src, int rows) {
   const int lane = threadIdx.x & 31;
+  if constexpr (SPLIT) {   // 32 bytes of a row per load, half a row at a time
+#pragma unroll 1
+    for (int h2 = 0; h2 < 2; ++h2) {
+      uint32_t o[64];
+#pragma unroll
+      for (int i = 0; i < 64; ++i) o[i] = 0u;
+      if (lane < rows) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) ld_global_v8(src + (size_t)lane * D + 64 * h2 + 8 * i, o + 8 * i);
+      }
+      tmem_st32(o_tmem + 64 * h2, *reinterpret_cast<uint32_t(*)[32]>(o));
+      tmem_st32(o_tmem + 64 * h2 + 32, *reinterpret_cast<uint32_t(*)[32]>(o + 32));
+    }
+    tmem_st_wait();
+    return;
+  }
   uint4 w[4][8];
 #pragma unroll
   for (int cb = 0; cb < 4; ++cb)
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      const int rr = SPLIT ? lane : 4 * i + (lane >> 3), ch = SPLIT ? i : lane & 7;
+      const int rr = 4 * i + (lane >> 3), ch = lane & 7;
       w[cb][i] = make_uint4(0u, 0u, 0u, 0u);
       if (rr < rows) w[cb][i] = __ldcg(reinterpret_cast<const uint4*>(src + (size_t)rr * D + 32 * cb + 4 * ch));
     }
   uint8_t* const st = c.gen + Lay<false>::SM_ST + (threadIdx.x >> 5) * 4096;
 #pragma unroll
   for (int cb = 0; cb < 4; ++cb) {
-    if constexpr (!SPLIT) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int rr = 4 * i + (lane >> 3), ch = lane & 7;
-        *reinterpret_cast<uint4*>(st + rr * 128 + ((ch ^ (rr & 7)) << 4)) = w[cb][i];
-      }
-      __syncwarp();
-#pragma unroll
-      for (int i = 0; i < 8; ++i) w[cb][i] = *reinterpret_cast<const uint4*>(st + lane * 128 + ((i ^ (lane & 7)) << 4));
-      __syncwarp();
+    for (int i = 0; i < 8; ++i) {
+      const int rr = 4 * i + (lane >> 3), ch = lane & 7;
+      *reinterpret_cast<uint4*>(st + rr * 128 + ((ch ^ (rr & 7)) << 4)) = w[cb][i];
     }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[cb][i] = *reinterpret_cast<const uint4*>(st + lane * 128 + ((i ^ (lane & 7)) << 4));
+    __syncwarp();
     tmem_st32(o_tmem + 32 * cb, *reinterpret_cast<uint32_t(*)[32]>(w[cb]));
   }
   tmem_st_wait();
