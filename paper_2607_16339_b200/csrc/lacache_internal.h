@@ -1,4 +1,4 @@
-// Internal declarations shared by the host side (lacache_api.cu) and the kernel files (lacache_simt.cu: CUDA-core fp32
+// Internal declarations shared by the host side (lacache_api.cu) and the kernel files (lacache_simt.cu: fp32
 // attention; lacache_tc.cu, lacache_rows.cu: tcgen05 attention; lacache_rope.cu; lacache_sample.cu).
 #pragma once
 #include <cuda_runtime.h>
@@ -72,6 +72,12 @@ struct RotBuffers {
   void* k_hi; void* k_lo;
   void* v;
 };
+
+// fp32 planes (SIMT engine): feature c of token tok's row lies at c ^ swizzle.  Rows are 16-byte chunks; the fp32 attention
+// kernel reads four neighbouring chunks of adjacent rows of q and k at once (odd rows: the halves of 32 features change places),
+// and two chunks of every other row of v (pairs of rows: rotated by eight features).
+__host__ __device__ inline int simt_swz_qk(int tok) { return (tok & 1) << 4; }
+__host__ __device__ inline int simt_swz_v(int tok) { return ((tok >> 1) & 3) << 3; }
 
 struct StateBuffers {       // head-major: m,l [Hq][Tp]; o [Hq][Tp][d]
   float* m; float* l; float* o;   // m in log2 units (reference exponent)

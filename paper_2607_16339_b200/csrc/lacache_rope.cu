@@ -114,7 +114,7 @@ __global__ void __launch_bounds__(256, HPT > 1 ? 3 : 1) rope_write_kernel(const 
       }
     } else {
       void* const plane = which == 0 ? a.dst.q_hi : (which == 1 ? a.dst.k_hi : a.dst.v);
-      const size_t doff = ((size_t)h * g.Tp + tok) * g.d + c0;
+      const size_t doff = ((size_t)h * g.Tp + tok) * g.d + (c0 ^ (which == 2 ? simt_swz_v(tok) : simt_swz_qk(tok)));
       store8_f32(plane, doff, y1);
       store8_f32(plane, doff + half, y2);
     }
@@ -142,8 +142,10 @@ __global__ void __launch_bounds__(256) export_kernel(Geometry g, ExportArgs a) {
   int h = (int)(t % g.Hq);
   int tok = (int)(t / g.Hq);
   const size_t srow = ((size_t)h * g.Tp + tok) * g.d + c;   // state: [head][Tp][d]
-  // rotated planes: the tcgen05 engine stores [head][feature half][Tp][64]
-  const size_t src = TC ? ((size_t)(2 * h + c / 64) * g.Tp + tok) * 64 + c % 64 : srow;
+  // rotated planes: the tcgen05 engine stores [head][feature half][Tp][64], the other [head][Tp][d] with swizzled rows
+  const size_t row = ((size_t)h * g.Tp + tok) * g.d;
+  const size_t src = TC ? ((size_t)(2 * h + c / 64) * g.Tp + tok) * 64 + c % 64 : row + (c ^ simt_swz_qk(tok));
+  const size_t src_v = TC ? src : row + (c ^ simt_swz_v(tok));
   const float LN2 = 0.69314718055994530942f;
   if (a.o) a.o[idx] = a.st.o[srow];
   if (c == 0) {
@@ -155,8 +157,8 @@ __global__ void __launch_bounds__(256) export_kernel(Geometry g, ExportArgs a) {
     size_t dst = ((size_t)tok * g.Hkv + h) * g.d + c;
     if (a.k_rot) a.k_rot[dst] = read_rot<TC>(a.rot.k_hi, a.rot.k_lo, src, g.op_f16 != 0);
     if (a.v) {
-      a.v[dst] = TC ? __half2float(reinterpret_cast<const __half*>(a.rot.v)[src])
-                    : reinterpret_cast<const float*>(a.rot.v)[src];
+      a.v[dst] = TC ? __half2float(reinterpret_cast<const __half*>(a.rot.v)[src_v])
+                    : reinterpret_cast<const float*>(a.rot.v)[src_v];
     }
   }
 }

@@ -1,30 +1,34 @@
-// CUDA-core fp32 attention kernels (the fp32 dtype path, and any shape the
-// tcgen05 path does not cover).  One generic kernel runs every mode:
+// fp32 attention kernels (the fp32 dtype path, and any shape the tcgen05 path does not cover).
+// One generic kernel runs every mode:
 //   build : fixed queries x fixed keys            -> cached (m, l, O~)
 //   step  : fixed queries x block keys, merged with the cached state
 //           (Algorithm 1 reuse pass); block queries x all keys
 //   full  : all queries x all keys (no cache)
 // following the online-softmax recurrence of Eq. 2-6 with key tiles of 32.
 //
-// Mapping: a CTA of 4 warps owns 32 query rows of one (sequence, q head), 8 rows a
-// warp, and walks key tiles of 32.  A unit with many keys is cut over the S <= 8
-// CTAs of a thread-block cluster, whose online-softmax states are merged through
-// distributed shared memory (how many: simt_row_parts, simt_step_parts).  A tile is bound by the shared-memory pipe, which a 16-byte
-// load holds for four cycles: a tile's scores take 3118 cycles on an SM of their own, as six loads per step, 32 steps and
-// four warps say, P.V 2000.  Around the tiles it is latency (4000 to 7000 cycles from the wait for the grids ahead to the
-// queries in place) and the last CTAs of an uneven wave: hence small CTAs, three to an SM (168 registers a thread),
-// and many of them.
-// Per tile, a warp computes its 8 x 32 scores with 4 rows x 2 keys per lane and
-// its 8 x d part of P.V with 8 rows x d/32 features per lane: 32 products per 6
-// to 8 shared-memory loads (one key and one row at a time, as this kernel once
-// did, read 9 words per 4 products).  Values stream in while the scores are
-// computed and the next keys while P.V is (cp.async, one buffer of each).
+// Mapping: a CTA of 4 warps owns 32 query rows of one (sequence, q head) and walks key tiles of 32; a warp has 16 of the rows
+// and 16 keys of every tile, its own maxima and sums, and merges with the warp of the other 16 keys at the end.  A unit with
+// many keys is cut over the S <= 8 CTAs of a thread-block cluster, whose online-softmax states are merged through distributed
+// shared memory (how many: simt_row_parts, simt_step_parts).
+//
+// Products run on the tensor cores with fp32 accuracy: an operand is split in two tf32 parts, x = hi + lo, and a product is
+// hi.hi + hi.lo + lo.hi (what is left out is 2^-22 of it).  The tensor cores cut a sum off where an fp32 addition rounds, so
+// sums go over few steps there (32 features, 16 keys) and are then added up in fp32.  Error of the output against fp64 (2-norm, 24
+// models of 90 to 650 tokens): 1.1e-7, and 3.6e-7 where scores are of order 50; chains of fp32 products on the CUDA cores, which
+// this replaced, 1.35e-7 and 4.6e-7.
+//
+// What bounds it: a tile of 128 features is 768 tensor-core instructions of 2 cycles, 1536 on an SM (on the CUDA cores it took 5100,
+// the shared-memory pipe's: every thread read its operands 16 bytes for 32 products).  Two CTAs to an SM (254 registers a thread, 82 KB)
+// keep it fed; alone a CTA takes about 4000 a tile.  Around the tiles it is latency: item and lists, the first tile's way, the merge
+// of the parts, about 10000 cycles a CTA.  Build with its RoPE launch, before and now: 152 units x 11 tiles 48.5 -> 36.5 us, 660 x 21
+// 233 -> 172, 560 x 71 660 -> 450; step of 4 heads x 5120 tokens 102 -> 78.
 //
 // In a step the kernel rotates the block's rows itself, wherever it needs them,
 // and leaves them in the rotated cache: one launch, no kernel in front of it.
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "lacache_internal.h"
 #include "lacache_plan.h"
@@ -37,33 +41,39 @@ namespace {
 using namespace ptx;
 
 constexpr int KT = 32;       // keys per tile
-constexpr int RPW = 8;       // rows per warp
-constexpr int WARPS = SIMT_ROWS / RPW;
-constexpr int THREADS = WARPS * 32;
-constexpr int MAX_SPLIT = 8;  // CTAs of a cluster (the portable limit)
+constexpr int THREADS = 128; // warp w: rows 16 (w & 1) .. of the unit, keys 16 (w >> 1) .. of each tile
 
-// Shared memory, in floats: queries [32][D + 4] and keys [32][D + 4] (rows 16 bytes apart in the banks:
-// lanes read rows), values [32][D], per warp probabilities [32 keys][8 rows].  After the last tile the keys'
-// place holds the CTA's partial O~ [32][D], ML the partial (m, l).
+// Shared memory, in floats: queries, keys and values [32][D] as they lie in the rotated cache, whose rows are swizzled so
+// that the reads below meet no bank twice (simt_swz_qk, simt_swz_v).  After the last tile the first values' place holds the
+// CTA's partial O~ [32][D], ML the partial (m, l); the first keys' place, what half of the warps hand to the others.
 template <int D>
 struct Smem {
-  static constexpr int QS = D + 4, KS = D + 4;
   static constexpr int Q = 0;
-  static constexpr int K = Q + SIMT_ROWS * QS;
-  static constexpr int V = K + KT * KS;
-  static constexpr int P = V + KT * D;
-  static constexpr int ML = P + WARPS * KT * RPW;
-  static constexpr int TOTAL = ML + SIMT_ROWS * 2;
+  static constexpr int TILE = KT * D;
+  static constexpr int K = Q + SIMT_ROWS * D;          // two buffers of keys, two of values
+  static constexpr int V = K + 2 * TILE;
+  static constexpr int ML = V + 2 * TILE;
+  static constexpr int BAR = ML + 2 * SIMT_ROWS * 2;   // barriers: queries, keys 0 and 1, values 0 and 1 in place
+  static constexpr int TOTAL = BAR + 12;
   static constexpr size_t bytes = TOTAL * sizeof(float);
+  static_assert(SIMT_ROWS == KT, "the partial O~ over the values");
 };
 
-__device__ __forceinline__ void cp_async16(float* dst, const float* src, bool valid) {
-  const int n = valid ? 16 : 0;   // 0: zero-fill
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(n) : "memory");
+__device__ __forceinline__ void bulk_load(float* dst, const float* src, uint32_t bytes, uint32_t bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
+               "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+// Bounded wait (~2 s) for the bulk loads of a phase; one that runs out is reported and the values are whatever is there.
+__device__ __forceinline__ void wait_loads(uint32_t bar, uint32_t parity, int32_t* status, int loc) {
+  if (mbar_try(bar, parity)) return;
+  const long long t0 = clock64();
+  while (!mbar_try(bar, parity)) {
+    if (clock64() - t0 > 4000000000ll) {
+      if (status && atomicCAS(status, 0, (int)LACACHE_ERR_TIMEOUT) == 0) { status[1] = loc; status[2] = blockIdx.x; status[3] = threadIdx.x; }
+      return;
+    }
+  }
+}
 __device__ __forceinline__ float4 ld_cluster_v4(uint32_t addr) {
   float4 v;
   asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
@@ -75,26 +85,16 @@ __device__ __forceinline__ float2 ld_cluster_v2(uint32_t addr) {
   asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
   return v;
 }
-// two fp32 products-and-sums in one instruction (the same roundings as two fmaf)
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
+// D += A B on the warp's tensor core, 16 x 8 x 8, operands as tf32 (the low 13 bits are not read), fp32 sums
+__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t pack2(float a, float b) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ float2 unpack2(uint64_t v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
+// x = hi + lo: hi the nearest tf32 value, lo the rest, of which a product reads the first 11 bits (all but the last bit of x
+// at most)
+__device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
+  hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
+  lo = __float_as_uint(x - __uint_as_float(hi));
 }
 __device__ __forceinline__ float4 load4(const void* base, size_t off, bool bf16) {
   if (!bf16) return *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(base) + off);
@@ -113,11 +113,10 @@ __device__ __forceinline__ void rotate4(float4 x1, float4 x2, float4 cs, float4 
 }
 
 template <int D>
-__global__ void __launch_bounds__(THREADS, 3) simt_attn_kernel(const __grid_constant__ Geometry g,
+__global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(const __grid_constant__ Geometry g,
                                                               const __grid_constant__ AttnArgs a) {
   using SM = Smem<D>;
   constexpr int D4 = D / 4;          // 16-byte columns of a row
-  constexpr int DPL = D / 32;        // output features per lane (P.V)
   extern __shared__ __align__(16) float sm[];
 
   // the first n_split_items items are cut over the `split` CTAs of a cluster, the others take one CTA each
@@ -137,6 +136,11 @@ __global__ void __launch_bounds__(THREADS, 3) simt_attn_kernel(const __grid_cons
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int bs = a.blk_start ? a.blk_start[it.seq] : 0;
   const int be = bs + g.block_len;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < 5; ++i) mbar_init(smem_u32(sm + SM::BAR) + 8 * i, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  __syncthreads();
   // Launched programmatically dependent: but for the lists above, which nothing writes, nothing is touched before the grids
   // ahead have completed; this grid's launch and those two round trips to L2 overlap their end.
   grid_dependency_wait();
@@ -170,319 +174,484 @@ __global__ void __launch_bounds__(THREADS, 3) simt_attn_kernel(const __grid_cons
   float* const Vs = sm + SM::V;
   const bool writes_cache = q_raw && it.row0 == bs && h % g.group == 0;   // leaves the block's keys and values in the cache
 
-  // (a tile that holds block rows of a step: the loads of a batch of raw rows leave together, then they are
-  // rotated and stored)
-  auto load_keys = [&](int t) {
+  // Tiles, and the rows of fixed queries, are contiguous in the cache: a bulk copy each, the next tile's under way while a tile
+  // is computed (two buffers).  (Rows past the key range are other rows of the cache: their scores are masked.)
+  const uint32_t bar_q = smem_u32(sm + SM::BAR), bar_k = bar_q + 8, bar_v = bar_q + 24;
+  auto issue = [&](float* dst, const float* src, uint32_t bar) {
+    mbar_expect_tx(bar, KT * D * 4);
+    bulk_load(dst, src, KT * D * 4, bar);
+  };
+  auto issue_tile = [&](int t, int buf) {
+    if (threadIdx.x != 0) return;
+    fence_async_smem();   // (a tile that the threads stored may have been there)
+    issue(Ks + buf * SM::TILE, kr + (size_t)(k0 + t * KT) * D, bar_k + 8 * buf);
+    issue(Vs + buf * SM::TILE, vr + (size_t)(k0 + t * KT) * D, bar_v + 8 * buf);
+  };
+  // A tile that holds block rows of a step is loaded by all threads, who rotate the block's rows (BATCH raw rows' loads leave
+  // together) and take the others from the cache.
+  auto is_mixed = [&](int t) { return raw && k0 + t * KT < be && k0 + t * KT + KT > bs; };
+  auto load_keys = [&](auto batch, int t, float* Kb) {
     const int kt = k0 + t * KT;
-    constexpr int N = KT * (D4 / 2) / THREADS, BATCH = 2;
+    constexpr int N = KT * (D4 / 2) / THREADS, BATCH = decltype(batch)::value < N ? decltype(batch)::value : N;
     static_assert(N % BATCH == 0, "whole batches");
-    const bool mixed = raw && kt < be && kt + KT > bs;
-    if (!mixed && kt + KT <= k1) {   // the common tile: one address, constant offsets
-      const int r = threadIdx.x / (D4 / 2), c = (threadIdx.x % (D4 / 2)) * 4;
-      const float* src = kr + (size_t)(kt + r) * D + c;
-      float* dst = Ks + r * SM::KS + c;
-      constexpr int RS = THREADS / (D4 / 2);   // rows per pass of the CTA
-#pragma unroll
-      for (int j = 0; j < N; ++j) {
-        cp_async16(dst + j * RS * SM::KS, src + j * RS * D, true);
-        cp_async16(dst + j * RS * SM::KS + D / 2, src + j * RS * D + D / 2, true);
-      }
-      cp_async_commit();
-      return;
-    }
 #pragma unroll 1
     for (int b = 0; b < N; b += BATCH) {
       float4 x1[BATCH], x2[BATCH], cs[BATCH], sn[BATCH];
-      if (mixed) {
 #pragma unroll
-        for (int j = 0; j < BATCH; ++j) {
-          const int i = threadIdx.x + (b + j) * THREADS, c = (i % (D4 / 2)) * 4, key = kt + i / (D4 / 2);
-          const size_t row = blk_row0 + (min(max(key, bs), be - 1) - bs);
+      for (int j = 0; j < BATCH; ++j) {
+        const int i = threadIdx.x + (b + j) * THREADS, c = (i % (D4 / 2)) * 4, key = kt + i / (D4 / 2);
+        if (raw && key >= bs && key < be) {
+          const size_t row = blk_row0 + (key - bs);
           x1[j] = load4(a.k_raw, (row * g.Hkv + kh) * D + c, a.raw_bf16);
           x2[j] = load4(a.k_raw, (row * g.Hkv + kh) * D + c + D / 2, a.raw_bf16);
           cs[j] = *reinterpret_cast<const float4*>(a.row_cos + row * (D / 2) + c);
           sn[j] = *reinterpret_cast<const float4*>(a.row_sin + row * (D / 2) + c);
+        } else {
+          const float* src = kr + (size_t)key * D + (c ^ simt_swz_qk(key));
+          x1[j] = *reinterpret_cast<const float4*>(src);
+          x2[j] = *reinterpret_cast<const float4*>(src + D / 2);
         }
       }
 #pragma unroll
       for (int j = 0; j < BATCH; ++j) {
         const int i = threadIdx.x + (b + j) * THREADS, r = i / (D4 / 2), c = (i % (D4 / 2)) * 4, key = kt + r;
-        float* dst = Ks + r * SM::KS + c;
-        if (mixed && key >= bs && key < be) {
-          float4 y1, y2;
+        const int cz = c ^ simt_swz_qk(key);   // (as rows lie in the cache)
+        float4 y1 = x1[j], y2 = x2[j];
+        if (raw && key >= bs && key < be) {
           rotate4(x1[j], x2[j], cs[j], sn[j], y1, y2);
-          *reinterpret_cast<float4*>(dst) = y1;
-          *reinterpret_cast<float4*>(dst + D / 2) = y2;
           if (writes_cache) {
-            *reinterpret_cast<float4*>(kr + (size_t)key * D + c) = y1;
-            *reinterpret_cast<float4*>(kr + (size_t)key * D + c + D / 2) = y2;
+            *reinterpret_cast<float4*>(kr + (size_t)key * D + cz) = y1;
+            *reinterpret_cast<float4*>(kr + (size_t)key * D + cz + D / 2) = y2;
           }
-        } else {
-          const float* src = kr + (size_t)(key < k1 ? key : k0) * D + c;
-          cp_async16(dst, src, key < k1);
-          cp_async16(dst + D / 2, src + D / 2, key < k1);
         }
+        *reinterpret_cast<float4*>(Kb + r * D + cz) = y1;
+        *reinterpret_cast<float4*>(Kb + r * D + cz + D / 2) = y2;
       }
     }
-    cp_async_commit();
   };
-  auto load_values = [&](int t) {
+  auto load_values = [&](auto batch, int t, float* Vb) {
     const int kt = k0 + t * KT;
-    constexpr int N = KT * D4 / THREADS, BATCH = 4;
+    constexpr int N = KT * D4 / THREADS, BATCH = decltype(batch)::value < N ? decltype(batch)::value : N;
     static_assert(N % BATCH == 0, "whole batches");
-    const bool mixed = raw && kt < be && kt + KT > bs;
-    if (!mixed && kt + KT <= k1) {   // (a tile of values is one contiguous run)
-      const float* src = vr + (size_t)kt * D + threadIdx.x * 4;
-#pragma unroll
-      for (int j = 0; j < N; ++j) cp_async16(Vs + (threadIdx.x + j * THREADS) * 4, src + j * THREADS * 4, true);
-      cp_async_commit();
-      return;
-    }
 #pragma unroll 1
     for (int b = 0; b < N; b += BATCH) {
       float4 v[BATCH];
-      if (mixed) {
 #pragma unroll
-        for (int j = 0; j < BATCH; ++j) {
-          const int i = threadIdx.x + (b + j) * THREADS, c = (i % D4) * 4, key = kt + i / D4;
-          v[j] = load4(a.v_raw, ((blk_row0 + (min(max(key, bs), be - 1) - bs)) * g.Hkv + kh) * D + c, a.raw_bf16);
-        }
+      for (int j = 0; j < BATCH; ++j) {
+        const int i = threadIdx.x + (b + j) * THREADS, c = (i % D4) * 4, key = kt + i / D4;
+        v[j] = raw && key >= bs && key < be ? load4(a.v_raw, ((blk_row0 + (key - bs)) * g.Hkv + kh) * D + c, a.raw_bf16)
+                                            : *reinterpret_cast<const float4*>(vr + (size_t)key * D + (c ^ simt_swz_v(key)));
       }
 #pragma unroll
       for (int j = 0; j < BATCH; ++j) {
         const int i = threadIdx.x + (b + j) * THREADS, r = i / D4, c = (i % D4) * 4, key = kt + r;
-        if (mixed && key >= bs && key < be) {
-          *reinterpret_cast<float4*>(Vs + r * D + c) = v[j];
-          if (writes_cache) *reinterpret_cast<float4*>(vr + (size_t)key * D + c) = v[j];
-        } else {
-          cp_async16(Vs + r * D + c, vr + (size_t)(key < k1 ? key : k0) * D + c, key < k1);
-        }
+        const int cz = c ^ simt_swz_v(key);
+        *reinterpret_cast<float4*>(Vb + r * D + cz) = v[j];
+        if (writes_cache && key >= bs && key < be) *reinterpret_cast<float4*>(vr + (size_t)key * D + cz) = v[j];
       }
     }
-    cp_async_commit();
   };
+  using Few = std::integral_constant<int, 2>;     // (beside the accumulators)
+  using Many = std::integral_constant<int, 8>;
 
   // the cached state merged at the end is asked into L2 now
   if (from_state)
     for (int i = threadIdx.x; i < it.nrows * (D / 32); i += THREADS)
       prefetch_l2(a.st.o + ((size_t)h * g.Tp + it.row0 + i / (D / 32)) * D + (i % (D / 32)) * 32);
   int t = next_tile(t_begin);
-  if (t < t_end) {
-    load_keys(t);
-    load_values(t);
-  }
-  // queries (rows past the tile's end are zero)
+  if (t < t_end && !is_mixed(t)) issue_tile(t, 0);
+  // queries (what rows past the tile's end hold is not used)
+  if (!q_raw) {
+    if (threadIdx.x == 0) issue(sm + SM::Q, qr + (size_t)it.row0 * D, bar_q);
+  } else {
+    constexpr int N = SIMT_ROWS * (D4 / 2) / THREADS;
+    float4 x1[N], x2[N], cs[N], sn[N];
 #pragma unroll
-  for (int j = 0; j < SIMT_ROWS * (D4 / 2) / THREADS; ++j) {
-    const int i = threadIdx.x + j * THREADS, r = i / (D4 / 2), c = (i % (D4 / 2)) * 4;
-    float4 y1 = make_float4(0.f, 0.f, 0.f, 0.f), y2 = y1;
-    if (r < it.nrows) {
-      const size_t tok = (size_t)(it.row0 + r);
-      if (q_raw) {
-        const size_t row = blk_row0 + (it.row0 - bs) + r, off = (row * g.Hq + h) * D + c, tab = row * (D / 2) + c;
-        rotate4(load4(a.q_raw, off, a.raw_bf16), load4(a.q_raw, off + D / 2, a.raw_bf16),
-                *reinterpret_cast<const float4*>(a.row_cos + tab), *reinterpret_cast<const float4*>(a.row_sin + tab), y1, y2);
-        if (part == 0) {
-          *reinterpret_cast<float4*>(qr + tok * D + c) = y1;
-          *reinterpret_cast<float4*>(qr + tok * D + c + D / 2) = y2;
-        }
-      } else {
-        y1 = *reinterpret_cast<const float4*>(qr + tok * D + c);
-        y2 = *reinterpret_cast<const float4*>(qr + tok * D + c + D / 2);
-      }
+    for (int j = 0; j < N; ++j) {
+      const int i = threadIdx.x + j * THREADS, r = min(i / (D4 / 2), it.nrows - 1), c = (i % (D4 / 2)) * 4;
+      const size_t row = blk_row0 + (it.row0 - bs) + r, off = (row * g.Hq + h) * D + c, tab = row * (D / 2) + c;
+      x1[j] = load4(a.q_raw, off, a.raw_bf16);
+      x2[j] = load4(a.q_raw, off + D / 2, a.raw_bf16);
+      cs[j] = *reinterpret_cast<const float4*>(a.row_cos + tab);
+      sn[j] = *reinterpret_cast<const float4*>(a.row_sin + tab);
     }
-    *reinterpret_cast<float4*>(sm + SM::Q + r * SM::QS + c) = y1;
-    *reinterpret_cast<float4*>(sm + SM::Q + r * SM::QS + c + D / 2) = y2;
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const int i = threadIdx.x + j * THREADS, r = i / (D4 / 2), c = (i % (D4 / 2)) * 4;
+      float4 y1, y2;
+      rotate4(x1[j], x2[j], cs[j], sn[j], y1, y2);
+      const int cz = c ^ simt_swz_qk(it.row0 + r);
+      if (part == 0 && r < it.nrows) {
+        *reinterpret_cast<float4*>(qr + (size_t)(it.row0 + r) * D + cz) = y1;
+        *reinterpret_cast<float4*>(qr + (size_t)(it.row0 + r) * D + cz + D / 2) = y2;
+      }
+      *reinterpret_cast<float4*>(sm + SM::Q + r * D + cz) = y1;
+      *reinterpret_cast<float4*>(sm + SM::Q + r * D + cz + D / 2) = y2;
+    }
   }
-  __syncthreads();   // the queries are in place
+  if (t < t_end && is_mixed(t)) {
+    load_keys(Many(), t, Ks);
+    load_values(Many(), t, Vs);
+  }
+  if (!q_raw) wait_loads(bar_q, 0u, a.status, LOC_WAIT_Q);
 
-  // scores: lane = keys kp and kp + 16 x rows 4 rh .. 4 rh + 3 of the warp's eight
-  const int kp = lane & 15, rh = lane >> 4;
-  float m[4], l[4];
-  uint64_t o[RPW / 2][DPL];   // O~ of rows 2 i and 2 i + 1 of the warp, feature DPL * lane + c
+  // The warp's 16 rows x 16 keys of a tile, as the tensor cores lay them out: this thread has rows g and g + 8, keys 2 t and
+  // 2 t + 1 of either eight (scores: n columns; P.V: k index t <-> key 2 t, t + 4 <-> key 2 t + 1, so that a thread's
+  // probabilities are its operand), and features 32 q + 8 t .. + 7 of O~.
+  const int g8 = lane >> 2, t4 = lane & 3, rw = warp & 1, kw = warp >> 1;
+  const bool rows = 16 * rw < it.nrows;   // this warp has rows (the others only help loading)
+  // (where the thread's first 16 bytes of a row lie, the rows' parity and pairs counted from the cache's first row: tiles are
+  // 32 rows apart, so it is the same place in every tile)
+  const float* const qp = sm + SM::Q + (16 * rw + g8) * D + ((4 * t4) ^ simt_swz_qk(it.row0 + g8));
+  const float* const kp0 = Ks + (16 * kw + g8) * D + ((4 * t4) ^ simt_swz_qk(k0 + g8));
+  const float* const vpa = Vs + (16 * kw + 2 * t4) * D + ((4 * g8) ^ simt_swz_v(k0 + 2 * t4));
+  const float* const vpb = Vs + (16 * kw + 2 * t4 + 1) * D + ((4 * g8) ^ simt_swz_v(k0 + 2 * t4 + 1));
+  const int qflip = simt_swz_qk(it.row0 + g8) ? -16 : 16, kflip = simt_swz_qk(k0 + g8) ? -16 : 16;   // to the next 16 features
+  float m[2], l[2];
+  float o[D / 8][4];   // [4 q + j]: {row g: features 8 t + j, 8 t + 4 + j; row g + 8: likewise} of the 32 from 32 q
 #pragma unroll
-  for (int i = 0; i < 4; ++i) { m[i] = -INFINITY; l[i] = 0.f; }
+  for (int i = 0; i < 2; ++i) { m[i] = -INFINITY; l[i] = 0.f; }
 #pragma unroll
-  for (int i = 0; i < RPW / 2; ++i)
+  for (int i = 0; i < D / 8; ++i)
 #pragma unroll
-    for (int c = 0; c < DPL; ++c) o[i][c] = 0ull;
-  const bool rows = warp * RPW < it.nrows;   // this warp has rows (the others only help loading)
-  float* const Pw = sm + SM::P + warp * KT * RPW;
-  const float* const qw = sm + SM::Q + (warp * RPW + 4 * rh) * SM::QS;
-
-  while (t < t_end) {
+    for (int c = 0; c < 4; ++c) o[i][c] = 0.f;
+  uint32_t phases = 0;   // bit b: phase of buffer b's barriers
+  for (int buf = 0; t < t_end; buf ^= 1) {
     const int tn = next_tile(t + 1);
-    cp_async_wait<1>();        // this tile's keys
-    __syncthreads();
-    // (each score in two halves: the even and the odd features)
-    uint64_t s0[4] = {0ull, 0ull, 0ull, 0ull}, s1[4] = {0ull, 0ull, 0ull, 0ull};
-    if (rows) {
-      const float* ka = Ks + kp * SM::KS;
-      const float* kb = ka + 16 * SM::KS;
-#pragma unroll 4
-      for (int c = 0; c < D; c += 4) {
-        const ulonglong2 va = *reinterpret_cast<const ulonglong2*>(ka + c), vb = *reinterpret_cast<const ulonglong2*>(kb + c);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const ulonglong2 q = *reinterpret_cast<const ulonglong2*>(qw + i * SM::QS + c);
-          s0[i] = fma2(q.x, va.x, s0[i]); s1[i] = fma2(q.x, vb.x, s1[i]);
-          s0[i] = fma2(q.y, va.y, s0[i]); s1[i] = fma2(q.y, vb.y, s1[i]);
-        }
+    __syncthreads();   // every warp is done with the tile before (and what the threads stored of this one is there)
+    if (tn < t_end) {
+      if (!is_mixed(tn)) {
+        issue_tile(tn, buf ^ 1);
+      } else {
+        load_keys(Few(), tn, Ks + (buf ^ 1) * SM::TILE);
+        load_values(Few(), tn, Vs + (buf ^ 1) * SM::TILE);
       }
     }
-    cp_async_wait<0>();        // this tile's values
-    __syncthreads();            // (and every warp has read the keys)
-    if (tn < t_end) load_keys(tn);
+    const bool bulk = !is_mixed(t);
+    const uint32_t phase = (phases >> buf) & 1u;
+    if (bulk) {
+      wait_loads(bar_k + 8 * buf, phase, a.status, LOC_WAIT_K);
+      phases ^= 1u << buf;
+    }
+    const float* const kp = kp0 + buf * SM::TILE;
+    const float* const vp0 = vpa + buf * SM::TILE;
+    const float* const vp1 = vpb + buf * SM::TILE;
+    float s[2][4];
     if (rows) {
-      const int key0 = k0 + t * KT + kp, key1 = key0 + 16;
-      const bool ok0 = key0 < k1 && !(key0 >= x0 && key0 < x1), ok1 = key1 < k1 && !(key1 >= x0 && key1 < x1);
-      float alpha[4];
-      float4 p0, p1;
+      // Every product as hi.hi + (lo.hi + hi.lo), the small ones in sums of their own; the tensor cores cut sums off
+      // instead of rounding them, so the large ones go over four steps and are then added with rounding.
+      float small[2][4], big[2][4];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const float2 h0 = unpack2(s0[i]), h1 = unpack2(s1[i]);
-        const float a0 = ok0 ? (h0.x + h0.y) * g.scale_log2 : -INFINITY, a1 = ok1 ? (h1.x + h1.y) * g.scale_log2 : -INFINITY;
-        float mx = fmaxf(a0, a1);
+      for (int n = 0; n < 2; ++n)
 #pragma unroll
-        for (int x = 8; x > 0; x >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, x));
+        for (int c = 0; c < 4; ++c) { s[n][c] = 0.f; small[n][c] = 0.f; }
+#pragma unroll 2
+      for (int c0 = 0; c0 < D; c0 += 32) {
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) big[n][c] = 0.f;
+#pragma unroll
+        for (int cc = 0; cc < 2; ++cc) {
+          uint32_t qh[2][4], ql[2][4];   // [step][operand register]
+          {
+            const float* const qc = qp + c0 + (cc ? qflip : 0);
+            const float4 qa = *reinterpret_cast<const float4*>(qc), qb = *reinterpret_cast<const float4*>(qc + 8 * D);
+            split_tf32(qa.x, qh[0][0], ql[0][0]); split_tf32(qb.x, qh[0][1], ql[0][1]);
+            split_tf32(qa.y, qh[0][2], ql[0][2]); split_tf32(qb.y, qh[0][3], ql[0][3]);
+            split_tf32(qa.z, qh[1][0], ql[1][0]); split_tf32(qb.z, qh[1][1], ql[1][1]);
+            split_tf32(qa.w, qh[1][2], ql[1][2]); split_tf32(qb.w, qh[1][3], ql[1][3]);
+          }
+#pragma unroll
+          for (int n = 0; n < 2; ++n) {
+            const float4 k4 = *reinterpret_cast<const float4*>(kp + 8 * n * D + c0 + (cc ? kflip : 0));
+            uint32_t kh[4], kl[4];
+            split_tf32(k4.x, kh[0], kl[0]); split_tf32(k4.y, kh[1], kl[1]);
+            split_tf32(k4.z, kh[2], kl[2]); split_tf32(k4.w, kh[3], kl[3]);
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              mma_tf32(big[n], qh[e], kh[2 * e], kh[2 * e + 1]);
+              mma_tf32(small[n], ql[e], kh[2 * e], kh[2 * e + 1]);
+              mma_tf32(small[n], qh[e], kl[2 * e], kl[2 * e + 1]);
+            }
+          }
+        }
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) s[n][c] += big[n][c];
+      }
+#pragma unroll
+      for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) s[n][c] += small[n][c];
+    }
+    if (bulk) wait_loads(bar_v + 8 * buf, phase, a.status, LOC_WAIT_V);
+    if (rows) {
+      float alpha[2];
+      bool ok[2][2];
+#pragma unroll
+      for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int key = k0 + t * KT + 16 * kw + 8 * n + 2 * t4 + e;
+          ok[n][e] = key < k1 && !(key >= x0 && key < x1);
+        }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {   // rows g and g + 8
+        float a[2][2], mx = -INFINITY;
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            a[n][e] = ok[n][e] ? s[n][2 * i + e] * g.scale_log2 : -INFINITY;
+            mx = fmaxf(mx, a[n][e]);
+          }
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
         const float m_new = fmaxf(m[i], mx);
         const float m_use = m_new == -INFINITY ? 0.f : m_new;
         alpha[i] = m[i] == -INFINITY ? 0.f : exp2f(m[i] - m_new);
         m[i] = m_new;
-        const float e0 = ok0 ? exp2f(a0 - m_use) : 0.f, e1 = ok1 ? exp2f(a1 - m_use) : 0.f;
-        l[i] = l[i] * alpha[i] + (e0 + e1);
-        (&p0.x)[i] = e0;
-        (&p1.x)[i] = e1;
+        float sum = 0.f;
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            s[n][2 * i + e] = ok[n][e] ? exp2f(a[n][e] - m_use) : 0.f;
+            sum += s[n][2 * i + e];
+          }
+        l[i] = l[i] * alpha[i] + sum;
       }
-      *reinterpret_cast<float4*>(Pw + kp * RPW + 4 * rh) = p0;
-      *reinterpret_cast<float4*>(Pw + (kp + 16) * RPW + 4 * rh) = p1;
-      if (__any_sync(0xffffffffu, alpha[0] != 1.f || alpha[1] != 1.f || alpha[2] != 1.f || alpha[3] != 1.f)) {
+      uint32_t ph[2][4], pl[2][4];
 #pragma unroll
-        for (int i = 0; i < RPW / 2; ++i) {
-          const int src = (i >> 1) * 16;   // the lanes of rows 0..3 / 4..7
-          const uint64_t al = pack2(__shfl_sync(0xffffffffu, alpha[(2 * i) & 3], src), __shfl_sync(0xffffffffu, alpha[(2 * i + 1) & 3], src));
-#pragma unroll
-          for (int c = 0; c < DPL; ++c) o[i][c] = mul2(o[i][c], al);
-        }
+      for (int n = 0; n < 2; ++n) {
+        split_tf32(s[n][0], ph[n][0], pl[n][0]); split_tf32(s[n][2], ph[n][1], pl[n][1]);
+        split_tf32(s[n][1], ph[n][2], pl[n][2]); split_tf32(s[n][3], ph[n][3], pl[n][3]);
       }
-      __syncwarp();
-      // O~ += P~ V: lane = features DPL * lane .. of the warp's eight rows
-      const float* vl = Vs + lane * DPL;
-#pragma unroll 4
-      for (int j = 0; j < KT; ++j) {
-        const ulonglong2 pa = *reinterpret_cast<const ulonglong2*>(Pw + j * RPW), pb = *reinterpret_cast<const ulonglong2*>(Pw + j * RPW + 4);
-        float v[DPL];
-        if (DPL == 4) *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(vl + j * D);
-        else *reinterpret_cast<float2*>(v) = *reinterpret_cast<const float2*>(vl + j * D);
 #pragma unroll
-        for (int c = 0; c < DPL; ++c) {
-          const uint64_t vv = pack2(v[c], v[c]);
-          o[0][c] = fma2(pa.x, vv, o[0][c]); o[1][c] = fma2(pa.y, vv, o[1][c]);
-          o[2][c] = fma2(pb.x, vv, o[2][c]); o[3][c] = fma2(pb.y, vv, o[3][c]);
+      for (int q = 0; q < D / 32; ++q) {
+        // (the small products first: a sum is cut off at the size it has reached)
+        float pv[4][4] = {};
+        uint32_t vh[2][2][4], vl[2][2][4];   // [step][key][feature]
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const float4 v4 = *reinterpret_cast<const float4*>((e ? vp1 : vp0) + 8 * n * D + 32 * q);
+            split_tf32(v4.x, vh[n][e][0], vl[n][e][0]); split_tf32(v4.y, vh[n][e][1], vl[n][e][1]);
+            split_tf32(v4.z, vh[n][e][2], vl[n][e][2]); split_tf32(v4.w, vh[n][e][3], vl[n][e][3]);
+          }
+#pragma unroll
+        for (int n = 0; n < 2; ++n) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) mma_tf32(pv[j], pl[n], vh[n][0][j], vh[n][1][j]);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) mma_tf32(pv[j], ph[n], vl[n][0][j], vl[n][1][j]);
         }
+#pragma unroll
+        for (int n = 0; n < 2; ++n)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) mma_tf32(pv[j], ph[n], vh[n][0][j], vh[n][1][j]);
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) o[4 * q + j][c] = fmaf(o[4 * q + j][c], alpha[c >> 1], pv[j][c]);
       }
     }
-    __syncthreads();            // every warp has read the values
-    if (tn < t_end) load_values(tn);
     t = tn;
   }
-
-  if (a.step_overlap) grid_launch_dependents();
-  // this warp's partial state of its rows to shared memory (every warp has left the keys behind)
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int x = 8; x > 0; x >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], x);
+  // Values that two tf32 parts do not hold (infinities, NaN, the last few below the largest) leave a NaN or an infinity behind:
+  // the unit is then done once more with plain products and sums, where they give what they give.
+  bool bad = false;
   if (rows) {
 #pragma unroll
-    for (int i = 0; i < RPW / 2; ++i) {
-      float* dst = Ks + (warp * RPW + 2 * i) * D + lane * DPL;
-      float2 h[DPL];
+    for (int i = 0; i < 2; ++i) {
+      float z = l[i] * 0.f;
 #pragma unroll
-      for (int c = 0; c < DPL; ++c) h[c] = unpack2(o[i][c]);
-      if (DPL == 4) {
-        *reinterpret_cast<float4*>(dst) = make_float4(h[0].x, h[1].x, h[2 % DPL].x, h[3 % DPL].x);
-        *reinterpret_cast<float4*>(dst + D) = make_float4(h[0].y, h[1].y, h[2 % DPL].y, h[3 % DPL].y);
-      } else {
-        *reinterpret_cast<float2*>(dst) = make_float2(h[0].x, h[1].x);
-        *reinterpret_cast<float2*>(dst + D) = make_float2(h[0].y, h[1].y);
-      }
-    }
-    if (kp == 0) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        *reinterpret_cast<float2*>(sm + SM::ML + (warp * RPW + 4 * rh + i) * 2) = make_float2(m[i], l[i]);
+      for (int f = 0; f < D / 8; ++f) z = fmaf(o[f][2 * i], 0.f, fmaf(o[f][2 * i + 1], 0.f, z));
+      bad = bad || (16 * rw + g8 + 8 * i < it.nrows && !(z == 0.f));
     }
   }
-  // the partial states of a row -- one of every CTA of the cluster, and the cached state -- merged (Eq. 2-6),
-  // 16 bytes of a row per thread; a split unit's rows are dealt out over its CTAs
+  const bool plain = __syncthreads_or(bad);   // (every warp has left the keys and values behind)
+
+  if (a.step_overlap) grid_launch_dependents();
+  // the partial states of the rows to shared memory
+  if (plain) {   // thread = a row and a quarter of its features
+    const int r = threadIdx.x >> 2, f0 = (threadIdx.x & 3) * (D / 4);
+    const float* const qrow = sm + SM::Q + r * D;
+    const int zq = simt_swz_qk(it.row0 + r);
+    float M = -INFINITY, L = 0.f, acc[D / 4];
+#pragma unroll
+    for (int f = 0; f < D / 4; ++f) acc[f] = 0.f;
+    for (t = next_tile(t_begin); t < t_end; t = next_tile(t + 1)) {
+      load_keys(Few(), t, Ks);
+      load_values(Few(), t, Vs);
+      __syncthreads();
+      for (int j = 0; j < KT; ++j) {
+        const int key = k0 + t * KT + j;
+        if (key >= k1 || (key >= x0 && key < x1)) continue;
+        const int zk = simt_swz_qk(key), zv = simt_swz_v(key);
+        float sc = 0.f;
+#pragma unroll 4
+        for (int f = 0; f < D; ++f) sc = fmaf(qrow[f ^ zq], Ks[j * D + (f ^ zk)], sc);
+        sc *= g.scale_log2;
+        const float m_new = fmaxf(M, sc);
+        const float al = M == -INFINITY ? 0.f : exp2f(M - m_new), p = exp2f(sc - (m_new == -INFINITY ? 0.f : m_new));
+        M = m_new;
+        L = L * al + p;
+#pragma unroll
+        for (int f = 0; f < D / 4; ++f) acc[f] = fmaf(p, Vs[j * D + ((f0 + f) ^ zv)], acc[f] * al);
+      }
+      __syncthreads();
+    }
+    for (int f = 0; f < D / 4; ++f) Vs[r * D + f0 + f] = acc[f];
+    if (f0 == 0) *reinterpret_cast<float2*>(sm + SM::ML + r * 2) = make_float2(M, L);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int x = 1; x < 4; x <<= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], x);
+    // the warps of the upper 16 keys hand theirs to those of the lower 16, who hold the same rows and features
+    float4* const hand = reinterpret_cast<float4*>(Ks) + rw * (D / 8) * 32 + lane;
+    float* const ml = sm + SM::ML;
+    const int r0 = 16 * rw + g8;
+    if (kw == 1 && rows) {
+#pragma unroll
+      for (int f = 0; f < D / 8; ++f) hand[f * 32] = make_float4(o[f][0], o[f][1], o[f][2], o[f][3]);
+      if (t4 == 0)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) *reinterpret_cast<float2*>(ml + (SIMT_ROWS + r0 + 8 * i) * 2) = make_float2(m[i], l[i]);
+    }
+    __syncthreads();
+    if (kw == 0 && rows) {
+      float w0[2], w1[2];
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const float2 other = *reinterpret_cast<const float2*>(ml + (SIMT_ROWS + r0 + 8 * i) * 2);
+        const float M = fmaxf(m[i], other.x);
+        w0[i] = m[i] == -INFINITY ? 0.f : exp2f(m[i] - M);
+        w1[i] = other.x == -INFINITY ? 0.f : exp2f(other.x - M);
+        if (t4 == 0) *reinterpret_cast<float2*>(ml + (r0 + 8 * i) * 2) = make_float2(M, fmaf(other.y, w1[i], l[i] * w0[i]));
+      }
+#pragma unroll
+      for (int f = 0; f < D / 8; ++f) {
+        const float4 x = hand[f * 32];
+        o[f][0] = fmaf(x.x, w1[0], o[f][0] * w0[0]); o[f][1] = fmaf(x.y, w1[0], o[f][1] * w0[0]);
+        o[f][2] = fmaf(x.z, w1[1], o[f][2] * w0[1]); o[f][3] = fmaf(x.w, w1[1], o[f][3] * w0[1]);
+      }
+      float* const dst = Vs + r0 * D + 8 * t4;
+#pragma unroll
+      for (int q = 0; q < D / 32; ++q)
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+          float* const d = dst + 8 * i * D + 32 * q;
+          *reinterpret_cast<float4*>(d) = make_float4(o[4 * q][2 * i], o[4 * q + 1][2 * i], o[4 * q + 2][2 * i], o[4 * q + 3][2 * i]);
+          *reinterpret_cast<float4*>(d + 4) = make_float4(o[4 * q][2 * i + 1], o[4 * q + 1][2 * i + 1], o[4 * q + 2][2 * i + 1], o[4 * q + 3][2 * i + 1]);
+        }
+    }
+  }
+  // the partial states of a row -- one of every CTA of the cluster, and the cached state -- merged (Eq. 2-6), 16 bytes of a row
+  // per thread and ITEMS of them at a time, PARTS partial states' loads in flight; a split unit's rows are dealt out over its CTAs
   if (n_parts > 1) cluster_sync_all();
   else __syncthreads();
-  const float LN2 = 0.69314718055994530942f;
   const uint32_t sm_base = smem_u32(sm);
-  const int my_rows = (it.nrows - part + n_parts - 1) / n_parts;
-  for (int i = threadIdx.x; i < my_rows * D4; i += THREADS) {
-    const int r = part + (i / D4) * n_parts, c4 = i % D4;
-    const int tok = it.row0 + r;
-    const size_t srow = (size_t)h * g.Tp + tok;
-    float M = -INFINITY, L = 0.f;
-    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (from_state) {
-      M = a.st.m[srow];
-      L = a.st.l[srow];
-      acc = *reinterpret_cast<const float4*>(a.st.o + srow * D + c4 * 4);
-    }
-    for (int p0 = 0; p0 < n_parts; p0 += 4) {
-      float2 ml[4];
-      float4 v[4];
+  const int n_out = (it.nrows - part + n_parts - 1) / n_parts * D4;
+  auto merge = [&](auto items, auto parts) {
+    constexpr int ITEMS = decltype(items)::value, PARTS = decltype(parts)::value;
+    const float LN2 = 0.69314718055994530942f;
+#pragma unroll 1
+    for (int i0 = threadIdx.x; i0 < n_out; i0 += ITEMS * THREADS) {
+      float M[ITEMS], L[ITEMS];
+      float4 acc[ITEMS];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {   // (the loads of four parts leave together)
-        const uint32_t base = n_parts > 1 ? mapa_shared(sm_base, (uint32_t)min(p0 + k, n_parts - 1)) : sm_base;
-        ml[k] = ld_cluster_v2(base + (SM::ML + r * 2) * 4);
-        v[k] = ld_cluster_v4(base + (SM::K + r * D + c4 * 4) * 4);
+      for (int b = 0; b < ITEMS; ++b) {
+        M[b] = -INFINITY; L[b] = 0.f;
+        acc[b] = make_float4(0.f, 0.f, 0.f, 0.f);
+        const int i = min(i0 + b * THREADS, n_out - 1);
+        const size_t srow = (size_t)h * g.Tp + it.row0 + part + (i / D4) * n_parts;
+        if (from_state) {
+          M[b] = a.st.m[srow];
+          L[b] = a.st.l[srow];
+          acc[b] = *reinterpret_cast<const float4*>(a.st.o + srow * D + (i % D4) * 4);
+        }
       }
-      float Mn = M;
+#pragma unroll 1
+      for (int p0 = 0; p0 < n_parts; p0 += PARTS) {
+        float2 ml[ITEMS][PARTS];
+        float4 v[ITEMS][PARTS];
 #pragma unroll
-      for (int k = 0; k < 4; ++k) Mn = fmaxf(Mn, ml[k].x);
-      const float w0 = M == -INFINITY ? 0.f : exp2f(M - Mn);
-      L *= w0; acc.x *= w0; acc.y *= w0; acc.z *= w0; acc.w *= w0;
+        for (int k = 0; k < PARTS; ++k) {
+          const uint32_t base = n_parts > 1 ? mapa_shared(sm_base, (uint32_t)min(p0 + k, n_parts - 1)) : sm_base;
 #pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const float w = (p0 + k >= n_parts || ml[k].x == -INFINITY) ? 0.f : exp2f(ml[k].x - Mn);
-        L = fmaf(ml[k].y, w, L);
-        acc.x = fmaf(v[k].x, w, acc.x); acc.y = fmaf(v[k].y, w, acc.y);
-        acc.z = fmaf(v[k].z, w, acc.z); acc.w = fmaf(v[k].w, w, acc.w);
+          for (int b = 0; b < ITEMS; ++b) {
+            const int i = min(i0 + b * THREADS, n_out - 1), r = part + (i / D4) * n_parts;
+            ml[b][k] = ld_cluster_v2(base + (SM::ML + r * 2) * 4);
+            v[b][k] = ld_cluster_v4(base + (SM::V + r * D + (i % D4) * 4) * 4);
+          }
+        }
+#pragma unroll
+        for (int b = 0; b < ITEMS; ++b) {
+          float Mn = M[b];
+#pragma unroll
+          for (int k = 0; k < PARTS; ++k) Mn = fmaxf(Mn, ml[b][k].x);
+          const float w0 = M[b] == -INFINITY ? 0.f : exp2f(M[b] - Mn);
+          L[b] *= w0; acc[b].x *= w0; acc[b].y *= w0; acc[b].z *= w0; acc[b].w *= w0;
+#pragma unroll
+          for (int k = 0; k < PARTS; ++k) {
+            const float w = (p0 + k >= n_parts || ml[b][k].x == -INFINITY) ? 0.f : exp2f(ml[b][k].x - Mn);
+            L[b] = fmaf(ml[b][k].y, w, L[b]);
+            acc[b].x = fmaf(v[b][k].x, w, acc[b].x); acc[b].y = fmaf(v[b][k].y, w, acc[b].y);
+            acc[b].z = fmaf(v[b][k].z, w, acc[b].z); acc[b].w = fmaf(v[b][k].w, w, acc[b].w);
+          }
+          M[b] = Mn;
+        }
       }
-      M = Mn;
-    }
-    if (to_state) {
-      if (c4 == 0) { a.st.m[srow] = M; a.st.l[srow] = L; }
-      *reinterpret_cast<float4*>(a.st.o + srow * D + c4 * 4) = acc;
-    } else {
-      const float inv = 1.f / L;
-      const size_t orow = (size_t)tok * g.Hq + h;
-      acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
-      if (a.out_bf16) {
-        const __nv_bfloat162 b0 = __floats2bfloat162_rn(acc.x, acc.y), b1 = __floats2bfloat162_rn(acc.z, acc.w);
-        uint2 u;
-        u.x = *reinterpret_cast<const uint32_t*>(&b0);
-        u.y = *reinterpret_cast<const uint32_t*>(&b1);
-        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.out) + orow * D + c4 * 4) = u;
-      } else {
-        *reinterpret_cast<float4*>(a.out + orow * D + c4 * 4) = acc;
+#pragma unroll
+      for (int b = 0; b < ITEMS; ++b) {
+        const int i = i0 + b * THREADS;
+        if (i >= n_out) break;
+        const int tok = it.row0 + part + (i / D4) * n_parts, c4 = i % D4;
+        if (to_state) {
+          const size_t srow = (size_t)h * g.Tp + tok;
+          if (c4 == 0) { a.st.m[srow] = M[b]; a.st.l[srow] = L[b]; }
+          *reinterpret_cast<float4*>(a.st.o + srow * D + c4 * 4) = acc[b];
+        } else {
+          const float inv = 1.f / L[b];
+          const size_t orow = (size_t)tok * g.Hq + h;
+          const float4 y = make_float4(acc[b].x * inv, acc[b].y * inv, acc[b].z * inv, acc[b].w * inv);
+          if (a.out_bf16) {
+            const __nv_bfloat162 b0 = __floats2bfloat162_rn(y.x, y.y), b1 = __floats2bfloat162_rn(y.z, y.w);
+            uint2 u;
+            u.x = *reinterpret_cast<const uint32_t*>(&b0);
+            u.y = *reinterpret_cast<const uint32_t*>(&b1);
+            *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(a.out) + orow * D + c4 * 4) = u;
+          } else {
+            *reinterpret_cast<float4*>(a.out + orow * D + c4 * 4) = y;
+          }
+          if (a.lse && c4 == 0) a.lse[orow] = (M[b] + log2f(L[b])) * LN2;
+        }
       }
-      if (a.lse && c4 == 0) a.lse[orow] = (M + log2f(L)) * LN2;
     }
-  }
+  };
+  if (n_parts <= 2) merge(std::integral_constant<int, 4>(), std::integral_constant<int, 2>());
+  else merge(std::integral_constant<int, 2>(), std::integral_constant<int, 4>());
   if (n_parts > 1) cluster_sync_all();   // the partner CTAs may still read this one's shared memory
 }
 
+constexpr size_t SMEM_ALONE = 116 * 1024, SMEM_TWO = 78 * 1024;   // one CTA to an SM, two
+
 template <int D>
-cudaError_t launch(const Geometry& g, const AttnArgs& a, int n_ctas, cudaStream_t s) {
+cudaError_t launch(const Geometry& g, const AttnArgs& a, int n_ctas, int num_sms, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)n_ctas, (unsigned)g.Hq);
   cfg.blockDim = dim3(THREADS);
-  cfg.dynamicSmemBytes = Smem<D>::bytes;
+  // The kernel ahead still holds SMs when CTAs of this one are placed, and they pile up on the others: where all would find an
+  // SM of their own, or one with one other, they ask for so much shared memory that they do.  (A cluster lies within a group
+  // of at least 16 SMs, and fills seven eighths of the places that are left there.)
+  const int S = a.split_ctas, group = S > 1 ? 14 / S * S : 16;
+  const long long total = (long long)n_ctas * g.Hq * 16, places = (long long)num_sms * group;
+  cfg.dynamicSmemBytes = std::max(Smem<D>::bytes, total <= places ? SMEM_ALONE : total <= 2 * places ? SMEM_TWO : (size_t)0);
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   int n_attr = 0;
@@ -505,10 +674,10 @@ cudaError_t launch(const Geometry& g, const AttnArgs& a, int n_ctas, cudaStream_
 
 cudaError_t simt_prepare() {
   cudaError_t e = cudaFuncSetAttribute(simt_attn_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)Smem<128>::bytes);
+                                       (int)SMEM_ALONE);
   if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(simt_attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)Smem<64>::bytes);
+                              (int)SMEM_ALONE);
 }
 
 cudaError_t simt_attention(const Geometry& g, const AttnArgs& args, int num_sms, cudaStream_t s) {
@@ -519,11 +688,11 @@ cudaError_t simt_attention(const Geometry& g, const AttnArgs& args, int num_sms,
   if (!step) a.n_split_items = a.n_items;
   const int rest = a.n_items - a.n_split_items;
   const int max_tiles = (g.maxN + KT - 1) / KT;
-  a.split_ctas = step ? plan::simt_step_parts(a.n_split_items, rest, g.Hq, max_tiles, g.d, num_sms)
-                      : plan::simt_row_parts((long long)a.n_items * g.Hq, max_tiles, g.d, num_sms);
+  a.split_ctas = step ? plan::simt_step_parts(a.n_split_items, rest, g.Hq, max_tiles, g.d, num_sms, plan::SIMT_TENSOR_CORES)
+                      : plan::simt_row_parts((long long)a.n_items * g.Hq, max_tiles, g.d, num_sms, plan::SIMT_TENSOR_CORES);
   const int S = a.split_ctas;
   const int n_ctas = a.n_split_items * S + (rest + S - 1) / S * S;
-  return g.d == 128 ? launch<128>(g, a, n_ctas, s) : launch<64>(g, a, n_ctas, s);
+  return g.d == 128 ? launch<128>(g, a, n_ctas, num_sms, s) : launch<64>(g, a, n_ctas, num_sms, s);
 }
 
 }  // namespace lacache

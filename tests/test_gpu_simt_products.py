@@ -1,0 +1,80 @@
+"""The fp32 engine's products, which run as three tf32 products each: values that two tf32 parts do not hold (infinities, NaN,
+the largest finite ones) give what fp32 arithmetic gives, in the rows and features they reach and in no other; the range is that of
+fp32; and the results stay as close to fp64 as fp32 sums are, at sizes around a tile of 32 rows or keys."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2607_16339_b200 import binding
+from paper_2607_16339_b200.workloads import SyntheticSchedule, small_workload
+
+from lacache_testlib import make_ctx, new_outputs, to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(wl, q, k, v, blk=None):
+    """full recompute; and build + step of block 0 with the block's own rows"""
+    ctx = make_ctx(wl)
+    assert ctx.engine == binding.ENGINE_SIMT
+    got = [new_outputs(wl), new_outputs(wl)]
+    dq, dk, dv = (to_dev(a, wl) for a in (q, k, v))
+    ctx.full_recompute(dq, dk, dv, *got[0])
+    rows = torch.from_numpy(SyntheticSchedule(wl).block_rows(0)).cuda().long()
+    ctx.build(0, dq, dk, dv)
+    ctx.step(dq[rows].contiguous(), dk[rows].contiguous(), dv[rows].contiguous(), *got[1])
+    torch.cuda.synchronize()
+    assert ctx.poll_status()[0] == 0
+    ctx.destroy()
+    return [(o.cpu().numpy().astype(np.float64), l.cpu().numpy().astype(np.float64)) for o, l in got]
+
+
+@pytest.mark.parametrize("value", [np.inf, -np.inf, np.nan, 3.4028235e38, -3.4e38])
+@pytest.mark.parametrize("d", [64, 128])
+def test_values_that_two_parts_do_not_hold(value, d):
+    wl = small_workload(name="products", dtype="fp32", prompt_lens=(45, 30), gen_len=64, block_len=32, steps=2, hq=4, hkv=2, d=d,
+                        scale_mode="inv_sqrt_d")
+    sch = SyntheticSchedule(wl, seed=4)
+    q, k, v = (np.array(a) for a in sch.begin_block(0))
+    want, wlse = oracle.attention(q, k, v, wl.cu_seqlens, wl.rope_theta, d ** -0.5)
+    tok, kh, f = 7, 1, 5                                   # a prompt token of the first sequence
+    v[tok, kh, f] = value
+    for out, lse in _run(wl, q, k, v):
+        assert np.abs(lse - wlse).max() <= 1e-5
+        hit = np.zeros(out.shape, bool)
+        hit[wl.cu_seqlens[0]:wl.cu_seqlens[1], 2 * kh:2 * kh + 2, f] = True
+        assert np.abs(out - want)[~hit].max() <= 1e-5       # every other row and feature: as without it
+        if np.isnan(value):
+            assert np.isnan(out[hit]).all()
+        elif np.isinf(value):
+            assert (out[hit] == value).all()
+        else:                                               # p / l of the largest value: the weights are about 1 / n
+            n = wl.cu_seqlens[1] - wl.cu_seqlens[0]
+            assert (np.abs(out[hit] / value * n - 1) < 0.2).all()
+
+
+def test_the_range_is_that_of_fp32():
+    """q and k scaled by powers of two that cancel: the same bits."""
+    wl = small_workload(name="products", dtype="fp32", prompt_lens=(45, 30), gen_len=64, block_len=32, steps=2, hq=4, hkv=4, d=128,
+                        scale_mode="inv_sqrt_d")
+    q, k, v = (np.array(a) for a in SyntheticSchedule(wl, seed=5).begin_block(0))
+    a = _run(wl, q, k, v)
+    b = _run(wl, q * np.float32(2.0 ** -90), k * np.float32(2.0 ** 90), v)
+    for (o0, l0), (o1, l1) in zip(a, b):
+        assert np.array_equal(o0, o1) and np.array_equal(l0, l1)
+
+
+@pytest.mark.parametrize("prompts,gen,block", [((1,), 32, 32), ((31, 33), 32, 16), ((95, 64, 7), 64, 64), ((260,), 96, 48)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_as_close_to_fp64_as_fp32_sums(prompts, gen, block, d):
+    """Relative error (2-norm) of the output.  A sum of n fp32 products in a chain is off by about 2^-24 sqrt(n / 6) of itself, 4e-7 at 350
+    keys; here a product is cut at 2^-22 (2^-24 in the mean) and sums are cut off over two steps at a time: 1.4e-7 measured, for
+    chains on the CUDA cores 1.35e-7; the bound leaves three times that."""
+    wl = small_workload(name="products", dtype="fp32", prompt_lens=prompts, gen_len=gen, block_len=block, steps=2, hq=4, hkv=2, d=d,
+                        scale_mode="inv_sqrt_d")
+    q, k, v = (np.array(a) for a in SyntheticSchedule(wl, seed=6).begin_block(0))
+    want, wlse = oracle.attention(q, k, v, wl.cu_seqlens, wl.rope_theta, d ** -0.5)
+    for out, lse in _run(wl, q, k, v):
+        assert np.linalg.norm(out - want) <= 4.5e-7 * np.linalg.norm(want)
+        assert np.abs(lse - wlse).max() <= 2e-6
