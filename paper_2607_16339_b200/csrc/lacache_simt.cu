@@ -53,7 +53,8 @@ struct Smem {
   static constexpr int K = Q + SIMT_ROWS * D;          // two buffers of keys, two of values
   static constexpr int V = K + 2 * TILE;
   static constexpr int ML = V + 2 * TILE;
-  static constexpr int BAR = ML + 2 * SIMT_ROWS * 2;   // barriers: queries, keys 0 and 1, values 0 and 1 in place
+  static constexpr int ST = ML + 2 * SIMT_ROWS * 2;    // (m, l) of the rows' cached state
+  static constexpr int BAR = ST + SIMT_ROWS * 2;       // barriers: queries, keys 0 and 1, values 0 and 1 in place
   static constexpr int TOTAL = BAR + 12;
   static constexpr size_t bytes = TOTAL * sizeof(float);
   static_assert(SIMT_ROWS == KT, "the partial O~ over the values");
@@ -141,10 +142,6 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  // Launched programmatically dependent: but for the lists above, which nothing writes, nothing is touched before the grids
-  // ahead have completed; this grid's launch and those two round trips to L2 overlap their end.
-  grid_dependency_wait();
-
   int k0 = it.seq_start, k1 = it.seq_end, x0 = 0, x1 = 0;
   bool from_state = false, to_state = false;
   if (a.mode == MODE_BUILD) {
@@ -190,75 +187,67 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
   // A tile that holds block rows of a step is loaded by all threads, who rotate the block's rows (BATCH raw rows' loads leave
   // together) and take the others from the cache.
   auto is_mixed = [&](int t) { return raw && k0 + t * KT < be && k0 + t * KT + KT > bs; };
-  auto load_keys = [&](auto batch, int t, float* Kb) {
+  auto load_mixed = [&](auto batch, int t, float* Kb, float* Vb) {
     const int kt = k0 + t * KT;
-    constexpr int N = KT * (D4 / 2) / THREADS, BATCH = decltype(batch)::value < N ? decltype(batch)::value : N;
+    constexpr int N = KT * (D4 / 2) / THREADS, BATCH = decltype(batch)::value < N ? decltype(batch)::value : N;   // a key's two halves, its values'
     static_assert(N % BATCH == 0, "whole batches");
 #pragma unroll 1
     for (int b = 0; b < N; b += BATCH) {
-      float4 x1[BATCH], x2[BATCH], cs[BATCH], sn[BATCH];
+      float4 x1[BATCH], x2[BATCH], cs[BATCH], sn[BATCH], v1[BATCH], v2[BATCH];
 #pragma unroll
       for (int j = 0; j < BATCH; ++j) {
         const int i = threadIdx.x + (b + j) * THREADS, c = (i % (D4 / 2)) * 4, key = kt + i / (D4 / 2);
         if (raw && key >= bs && key < be) {
-          const size_t row = blk_row0 + (key - bs);
-          x1[j] = load4(a.k_raw, (row * g.Hkv + kh) * D + c, a.raw_bf16);
-          x2[j] = load4(a.k_raw, (row * g.Hkv + kh) * D + c + D / 2, a.raw_bf16);
+          const size_t row = blk_row0 + (key - bs), off = (row * g.Hkv + kh) * D + c;
+          x1[j] = load4(a.k_raw, off, a.raw_bf16);
+          x2[j] = load4(a.k_raw, off + D / 2, a.raw_bf16);
           cs[j] = *reinterpret_cast<const float4*>(a.row_cos + row * (D / 2) + c);
           sn[j] = *reinterpret_cast<const float4*>(a.row_sin + row * (D / 2) + c);
+          v1[j] = load4(a.v_raw, off, a.raw_bf16);
+          v2[j] = load4(a.v_raw, off + D / 2, a.raw_bf16);
         } else {
           const float* src = kr + (size_t)key * D + (c ^ simt_swz_qk(key));
           x1[j] = *reinterpret_cast<const float4*>(src);
           x2[j] = *reinterpret_cast<const float4*>(src + D / 2);
+          src = vr + (size_t)key * D + (c ^ simt_swz_v(key));
+          v1[j] = *reinterpret_cast<const float4*>(src);
+          v2[j] = *reinterpret_cast<const float4*>(src + D / 2);
         }
       }
 #pragma unroll
       for (int j = 0; j < BATCH; ++j) {
         const int i = threadIdx.x + (b + j) * THREADS, r = i / (D4 / 2), c = (i % (D4 / 2)) * 4, key = kt + r;
-        const int cz = c ^ simt_swz_qk(key);   // (as rows lie in the cache)
+        const int ck = c ^ simt_swz_qk(key), cv = c ^ simt_swz_v(key);   // (as rows lie in the cache)
         float4 y1 = x1[j], y2 = x2[j];
         if (raw && key >= bs && key < be) {
           rotate4(x1[j], x2[j], cs[j], sn[j], y1, y2);
           if (writes_cache) {
-            *reinterpret_cast<float4*>(kr + (size_t)key * D + cz) = y1;
-            *reinterpret_cast<float4*>(kr + (size_t)key * D + cz + D / 2) = y2;
+            *reinterpret_cast<float4*>(kr + (size_t)key * D + ck) = y1;
+            *reinterpret_cast<float4*>(kr + (size_t)key * D + ck + D / 2) = y2;
+            *reinterpret_cast<float4*>(vr + (size_t)key * D + cv) = v1[j];
+            *reinterpret_cast<float4*>(vr + (size_t)key * D + cv + D / 2) = v2[j];
           }
         }
-        *reinterpret_cast<float4*>(Kb + r * D + cz) = y1;
-        *reinterpret_cast<float4*>(Kb + r * D + cz + D / 2) = y2;
+        *reinterpret_cast<float4*>(Kb + r * D + ck) = y1;
+        *reinterpret_cast<float4*>(Kb + r * D + ck + D / 2) = y2;
+        *reinterpret_cast<float4*>(Vb + r * D + cv) = v1[j];
+        *reinterpret_cast<float4*>(Vb + r * D + cv + D / 2) = v2[j];
       }
     }
   };
-  auto load_values = [&](auto batch, int t, float* Vb) {
-    const int kt = k0 + t * KT;
-    constexpr int N = KT * D4 / THREADS, BATCH = decltype(batch)::value < N ? decltype(batch)::value : N;
-    static_assert(N % BATCH == 0, "whole batches");
-#pragma unroll 1
-    for (int b = 0; b < N; b += BATCH) {
-      float4 v[BATCH];
-#pragma unroll
-      for (int j = 0; j < BATCH; ++j) {
-        const int i = threadIdx.x + (b + j) * THREADS, c = (i % D4) * 4, key = kt + i / D4;
-        v[j] = raw && key >= bs && key < be ? load4(a.v_raw, ((blk_row0 + (key - bs)) * g.Hkv + kh) * D + c, a.raw_bf16)
-                                            : *reinterpret_cast<const float4*>(vr + (size_t)key * D + (c ^ simt_swz_v(key)));
-      }
-#pragma unroll
-      for (int j = 0; j < BATCH; ++j) {
-        const int i = threadIdx.x + (b + j) * THREADS, r = i / D4, c = (i % D4) * 4, key = kt + r;
-        const int cz = c ^ simt_swz_v(key);
-        *reinterpret_cast<float4*>(Vb + r * D + cz) = v[j];
-        if (writes_cache && key >= bs && key < be) *reinterpret_cast<float4*>(vr + (size_t)key * D + cz) = v[j];
-      }
-    }
-  };
-  using Few = std::integral_constant<int, 2>;     // (beside the accumulators)
-  using Many = std::integral_constant<int, 8>;
+  using Few = std::integral_constant<int, 1>;     // (beside the accumulators)
+  using Many = std::integral_constant<int, 4>;
 
-  // the cached state merged at the end is asked into L2 now
-  if (from_state)
-    for (int i = threadIdx.x; i < it.nrows * (D / 32); i += THREADS)
-      prefetch_l2(a.st.o + ((size_t)h * g.Tp + it.row0 + i / (D / 32)) * D + (i % (D / 32)) * 32);
   int t = next_tile(t_begin);
+  // Launched programmatically dependent: but for the lists above, which nothing writes, nothing is touched before the grids
+  // ahead have completed; this grid's launch and those two round trips to L2 overlap their end.
+  grid_dependency_wait();
+  // (the cached state of a step's fixed rows: m and l now, O~ behind the last tile's keys)
+  float m_st = -INFINITY, l_st = 0.f;
+  if (from_state && warp == 3 && lane < it.nrows) {
+    m_st = a.st.m[(size_t)h * g.Tp + it.row0 + lane];
+    l_st = a.st.l[(size_t)h * g.Tp + it.row0 + lane];
+  }
   if (t < t_end && !is_mixed(t)) issue_tile(t, 0);
   // queries (what rows past the tile's end hold is not used)
   if (!q_raw) {
@@ -290,8 +279,7 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
     }
   }
   if (t < t_end && is_mixed(t)) {
-    load_keys(Many(), t, Ks);
-    load_values(Many(), t, Vs);
+    load_mixed(Many(), t, Ks, Vs);
   }
   if (!q_raw) wait_loads(bar_q, 0u, a.status, LOC_WAIT_Q);
 
@@ -316,16 +304,20 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
 #pragma unroll
     for (int c = 0; c < 4; ++c) o[i][c] = 0.f;
   uint32_t phases = 0;   // bit b: phase of buffer b's barriers
-  for (int buf = 0; t < t_end; buf ^= 1) {
+  int buf = 0;
+  for (; t < t_end; buf ^= 1) {
     const int tn = next_tile(t + 1);
     __syncthreads();   // every warp is done with the tile before (and what the threads stored of this one is there)
     if (tn < t_end) {
       if (!is_mixed(tn)) {
         issue_tile(tn, buf ^ 1);
       } else {
-        load_keys(Few(), tn, Ks + (buf ^ 1) * SM::TILE);
-        load_values(Few(), tn, Vs + (buf ^ 1) * SM::TILE);
+        load_mixed(Few(), tn, Ks + (buf ^ 1) * SM::TILE, Vs + (buf ^ 1) * SM::TILE);
       }
+    }
+    if (from_state && tn >= t_end && threadIdx.x == 0) {   // the rows' cached O~, into the buffer that no further keys need
+      fence_async_smem();
+      issue(Ks + (buf ^ 1) * SM::TILE, a.st.o + ((size_t)h * g.Tp + it.row0) * D, bar_k + 8 * (buf ^ 1));
     }
     const bool bulk = !is_mixed(t);
     const uint32_t phase = (phases >> buf) & 1u;
@@ -474,6 +466,7 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
     }
   }
   const bool plain = __syncthreads_or(bad);   // (every warp has left the keys and values behind)
+  float* const Kl = Ks + (buf ^ 1) * SM::TILE;   // the last tile's keys' place; the cached O~ is in the other one
 
   if (a.step_overlap) grid_launch_dependents();
   // the partial states of the rows to shared memory
@@ -485,8 +478,7 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
 #pragma unroll
     for (int f = 0; f < D / 4; ++f) acc[f] = 0.f;
     for (t = next_tile(t_begin); t < t_end; t = next_tile(t + 1)) {
-      load_keys(Few(), t, Ks);
-      load_values(Few(), t, Vs);
+      load_mixed(Few(), t, Kl, Vs);
       __syncthreads();
       for (int j = 0; j < KT; ++j) {
         const int key = k0 + t * KT + j;
@@ -494,7 +486,7 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
         const int zk = simt_swz_qk(key), zv = simt_swz_v(key);
         float sc = 0.f;
 #pragma unroll 4
-        for (int f = 0; f < D; ++f) sc = fmaf(qrow[f ^ zq], Ks[j * D + (f ^ zk)], sc);
+        for (int f = 0; f < D; ++f) sc = fmaf(qrow[f ^ zq], Kl[j * D + (f ^ zk)], sc);
         sc *= g.scale_log2;
         const float m_new = fmaxf(M, sc);
         const float al = M == -INFINITY ? 0.f : exp2f(M - m_new), p = exp2f(sc - (m_new == -INFINITY ? 0.f : m_new));
@@ -513,7 +505,7 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
 #pragma unroll
       for (int x = 1; x < 4; x <<= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], x);
     // the warps of the upper 16 keys hand theirs to those of the lower 16, who hold the same rows and features
-    float4* const hand = reinterpret_cast<float4*>(Ks) + rw * (D / 8) * 32 + lane;
+    float4* const hand = reinterpret_cast<float4*>(Kl) + rw * (D / 8) * 32 + lane;
     float* const ml = sm + SM::ML;
     const int r0 = 16 * rw + g8;
     if (kw == 1 && rows) {
@@ -553,8 +545,11 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
   }
   // the partial states of a row -- one of every CTA of the cluster, and the cached state -- merged (Eq. 2-6), 16 bytes of a row
   // per thread and ITEMS of them at a time, PARTS partial states' loads in flight; a split unit's rows are dealt out over its CTAs
+  if (from_state && warp == 3) *reinterpret_cast<float2*>(sm + SM::ST + lane * 2) = make_float2(m_st, l_st);
   if (n_parts > 1) cluster_sync_all();
   else __syncthreads();
+  if (from_state) wait_loads(bar_k + 8 * buf, (phases >> buf) & 1u, a.status, LOC_WAIT_O);
+  const float* const o_st = Ks + buf * SM::TILE;
   const uint32_t sm_base = smem_u32(sm);
   const int n_out = (it.nrows - part + n_parts - 1) / n_parts * D4;
   auto merge = [&](auto items, auto parts) {
@@ -568,12 +563,12 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
       for (int b = 0; b < ITEMS; ++b) {
         M[b] = -INFINITY; L[b] = 0.f;
         acc[b] = make_float4(0.f, 0.f, 0.f, 0.f);
-        const int i = min(i0 + b * THREADS, n_out - 1);
-        const size_t srow = (size_t)h * g.Tp + it.row0 + part + (i / D4) * n_parts;
-        if (from_state) {
-          M[b] = a.st.m[srow];
-          L[b] = a.st.l[srow];
-          acc[b] = *reinterpret_cast<const float4*>(a.st.o + srow * D + (i % D4) * 4);
+        if (from_state) {   // (a unit that is not cut)
+          const int i = min(i0 + b * THREADS, n_out - 1);
+          const float2 ml = *reinterpret_cast<const float2*>(sm + SM::ST + (i / D4) * 2);
+          M[b] = ml.x;
+          L[b] = ml.y;
+          acc[b] = *reinterpret_cast<const float4*>(o_st + i * 4);
         }
       }
 #pragma unroll 1
