@@ -129,7 +129,6 @@ struct AttnArgs {
   int split_ctas;            // SIMT: CTAs (one cluster) a cut unit takes; chosen by the launcher
   int step_overlap;          // let the kernels behind be scheduled while this one drains (tcgen05, steps: 1 from its entry on, 2 once a
                              // CTA has asked for its last tiles; SIMT: once a CTA has left its last key tile)
-  int trigger_late;          // host only: a step for which step_overlap = 2 is worth it
   const int32_t* blk_start;  // [B] absolute token index of the block's first row
   RotBuffers rot;
   StateBuffers st;

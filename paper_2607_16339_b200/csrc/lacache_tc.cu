@@ -1630,7 +1630,7 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
   // before they wait for this grid, only state that stays fixed until the next build and inputs that were
   // complete long before.  So they may in a short step without it, where they wait first (the rule: early_trigger in
   // lacache_plan.h).  Otherwise this kernel lets its successor start when it ends.
-  if (a.step_overlap == 1) grid_launch_dependents();
+  if (SPLIT ? a.step_overlap == 1 : a.step_overlap) grid_launch_dependents();
   if (a.span != nullptr && tid == 0) atomicMin(a.span, global_timer_ns());   // first CTA entry of this launch
   Cta c;
   c.base = smem_u32(smem_raw);
