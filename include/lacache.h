@@ -61,7 +61,7 @@ typedef enum {
 
 enum { LACACHE_DTYPE_BF16 = 0, LACACHE_DTYPE_FP32 = 1 };
 /* which kernel family runs the attention: AUTO picks tcgen05 for bf16 with
- * head_dim 128 and the fp32 CUDA-core kernels otherwise */
+ * head_dim 128 and the fp32 kernels otherwise */
 enum { LACACHE_ENGINE_AUTO = 0, LACACHE_ENGINE_SIMT = 1, LACACHE_ENGINE_TCGEN05 = 2 };
 /* element type of `out` (lse is always fp32) */
 enum { LACACHE_OUT_BF16 = 0, LACACHE_OUT_FP32 = 1 };
@@ -83,7 +83,7 @@ enum { LACACHE_OUT_BF16 = 0, LACACHE_OUT_FP32 = 1 };
  *          about two in hand on the maximum and four on the mean (measured against the fp64 evaluation
  *          on the LLaDA-shaped configurations, outlier keys included); SPLIT has a factor of twenty.
  *          Rotated values beyond the fp16 range (|x| > 65504) saturate: inputs of that size need SPLIT.
- * The fp32 CUDA-core engine ignores the mode (its operands are fp32).
+ * The fp32 engine ignores the mode (its operands are fp32).
  */
 enum { LACACHE_PRECISION_PLAIN = 0, LACACHE_PRECISION_SPLIT = 1, LACACHE_PRECISION_FP16 = 3 };
 /* (2 is reserved: split planes plus split probabilities, which this library does not offer) */
@@ -283,7 +283,7 @@ lacache_status lacache_full_recompute(lacache_ctx* ctx, const void* q_pre, const
  *     call overwrites what it reads, and the previous call's contents are
  *     simply left behind.  Two calls that overlap on the GPU (different
  *     streams, or different host threads) race on it: serialise them.
- *   - Runs the fp32 CUDA-core kernels (any dtype).
+ *   - Runs the fp32 kernels (any dtype).
  */
 lacache_status lacache_full_recompute_static(int dtype, int n_tokens, int n_q_heads, int n_kv_heads,
                                              int head_dim, float rope_theta, float softmax_scale,
