@@ -18,7 +18,7 @@
 // this replaced, 1.35e-7 and 4.6e-7.
 //
 // What bounds it: a tile of 128 features is 768 tensor-core instructions of 2 cycles, 1536 on an SM (on the CUDA cores it took 5100,
-// the shared-memory pipe's: every thread read its operands 16 bytes for 32 products).  Two CTAs to an SM (254 registers a thread, 82 KB)
+// the shared-memory pipe's: every thread read its operands 16 bytes for 32 products).  Two CTAs to an SM (226 and 246 registers a thread, 82 KB)
 // keep it fed; alone a CTA takes about 4000 a tile.  Around the tiles it is latency: item and lists, the first tile's way, the merge
 // of the parts, about 10000 cycles a CTA.  Build with its RoPE launch, before and now: 152 units x 11 tiles 48.5 -> 36.5 us, 660 x 21
 // 233 -> 172, 560 x 71 660 -> 450; step of 4 heads x 5120 tokens 102 -> 78.
@@ -113,7 +113,10 @@ __device__ __forceinline__ void rotate4(float4 x1, float4 x2, float4 cs, float4 
   y2 = make_float4(hi(x1.x, x2.x, cs.x, sn.x), hi(x1.y, x2.y, cs.y, sn.y), hi(x1.z, x2.z, cs.z, sn.z), hi(x1.w, x2.w, cs.w, sn.w));
 }
 
-template <int D>
+// STEP: a launch of a step.  What only steps do, the rows they rotate and the state they start from, is code that a build's CTAs would
+// fetch around, and the other way: one instantiation for both took a small build and step 55.8 us (now 53.0), the tiny model's step
+// 6.05 (5.62).
+template <int D, bool STEP>
 __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(const __grid_constant__ Geometry g,
                                                               const __grid_constant__ AttnArgs a) {
   using SM = Smem<D>;
@@ -144,12 +147,12 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
   __syncthreads();
   int k0 = it.seq_start, k1 = it.seq_end, x0 = 0, x1 = 0;
   bool from_state = false, to_state = false;
-  if (a.mode == MODE_BUILD) {
+  if (!STEP && a.mode == MODE_BUILD) {
     x0 = bs; x1 = be; to_state = true;
-  } else if (a.mode == MODE_STEP && it.kind == ITEM_ROWS) {
+  } else if (STEP && it.kind == ITEM_ROWS) {
     k0 = bs; k1 = be; from_state = true;
   }
-  const bool raw = a.k_raw != nullptr;                    // a step that rotates the block's rows here
+  const bool raw = STEP && a.k_raw != nullptr;                    // a step that rotates the block's rows here
   const bool q_raw = raw && it.kind == ITEM_BLOCK_CHUNK;  // (these rows' queries are the block's)
   const size_t blk_row0 = (size_t)it.seq * g.block_len;   // the sequence's first row of the block's inputs
 
@@ -662,17 +665,19 @@ cudaError_t launch(const Geometry& g, const AttnArgs& a, int n_ctas, int num_sms
   }
   cfg.attrs = attr;
   cfg.numAttrs = n_attr;
-  return cudaLaunchKernelEx(&cfg, simt_attn_kernel<D>, g, a);
+  return a.mode == MODE_STEP ? cudaLaunchKernelEx(&cfg, simt_attn_kernel<D, true>, g, a) : cudaLaunchKernelEx(&cfg, simt_attn_kernel<D, false>, g, a);
 }
 
 }  // namespace
 
 cudaError_t simt_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(simt_attn_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)SMEM_ALONE);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(simt_attn_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)SMEM_ALONE);
+  const void* const kernels[4] = {(const void*)simt_attn_kernel<128, false>, (const void*)simt_attn_kernel<128, true>,
+                                  (const void*)simt_attn_kernel<64, false>, (const void*)simt_attn_kernel<64, true>};
+  for (const void* k : kernels) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_ALONE);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t simt_attention(const Geometry& g, const AttnArgs& args, int num_sms, cudaStream_t s) {
