@@ -456,16 +456,23 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
     }
     t = tn;
   }
-  // Values that two tf32 parts do not hold (infinities, NaN, the last few below the largest) leave a NaN or an infinity behind:
-  // the unit is then done once more with plain products and sums, where they give what they give.
+  // Values that two tf32 parts do not hold (infinities, NaN, the last few below the largest) leave a NaN or an infinity behind, and
+  // the low parts of values below 2^-115 are subnormal, which the tensor cores drop: the unit is then done once more with plain
+  // products and sums, where they give what they give.
   bool bad = false;
   if (rows) {
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
       float z = l[i] * 0.f;
+      float least = INFINITY;   // of the magnitudes that are not zero
 #pragma unroll
-      for (int f = 0; f < D / 8; ++f) z = fmaf(o[f][2 * i], 0.f, fmaf(o[f][2 * i + 1], 0.f, z));
-      bad = bad || (16 * rw + g8 + 8 * i < it.nrows && !(z == 0.f));
+      for (int f = 0; f < D / 8; ++f)
+#pragma unroll
+        for (int e = 2 * i; e < 2 * i + 2; ++e) {
+          z = fmaf(o[f][e], 0.f, z);
+          least = fminf(least, o[f][e] == 0.f ? INFINITY : fabsf(o[f][e]));
+        }
+      bad = bad || (16 * rw + g8 + 8 * i < it.nrows && (least < 0x1p-100f || !(z == 0.f)));
     }
   }
   const bool plain = __syncthreads_or(bad);   // (every warp has left the keys and values behind)

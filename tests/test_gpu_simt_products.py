@@ -65,6 +65,19 @@ def test_the_range_is_that_of_fp32():
         assert np.array_equal(o0, o1) and np.array_equal(l0, l1)
 
 
+@pytest.mark.parametrize("exponent", [60, 108, 116, 122])
+def test_tiny_values_keep_their_bits(exponent):
+    """v scaled by a power of two down to where the low part of a split value is subnormal: the result scales with it, within the
+    rounding of sums taken in another order (and of subnormal results, at most 2^-149 a value of 2^-125)."""
+    wl = small_workload(name="products", dtype="fp32", prompt_lens=(45, 30), gen_len=64, block_len=32, steps=2, hq=4, hkv=4, d=128,
+                        scale_mode="inv_sqrt_d")
+    q, k, v = (np.array(a) for a in SyntheticSchedule(wl, seed=5).begin_block(0))
+    s = 2.0 ** -exponent
+    for (o0, l0), (o1, l1) in zip(_run(wl, q, k, v), _run(wl, q, k, v * np.float32(s))):
+        assert np.linalg.norm(o1 / s - o0) <= 1e-6 * np.linalg.norm(o0)
+        assert np.abs(l1 - l0).max() <= 2e-6      # (the order of the sums)
+
+
 @pytest.mark.parametrize("prompts,gen,block", [((1,), 32, 32), ((31, 33), 32, 16), ((95, 64, 7), 64, 64), ((260,), 96, 48)])
 @pytest.mark.parametrize("d", [64, 128])
 def test_as_close_to_fp64_as_fp32_sums(prompts, gen, block, d):
