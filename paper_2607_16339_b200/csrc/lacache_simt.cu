@@ -480,35 +480,102 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
 
   if (a.step_overlap) grid_launch_dependents();
   // the partial states of the rows to shared memory
-  if (plain) {   // thread = a row and a quarter of its features
-    const int r = threadIdx.x >> 2, f0 = (threadIdx.x & 3) * (D / 4);
-    const float* const qrow = sm + SM::Q + r * D;
-    const int zq = simt_swz_qk(it.row0 + r);
-    float M = -INFINITY, L = 0.f, acc[D / 4];
+  if (plain) {
+    // Eight threads for two rows, each with every eighth 16 bytes of their features: they read a key's and a value's row side by side,
+    // and share a score's sum; four keys at a time.  What bounds it is the shared-memory pipe, four cycles for the 16 bytes that
+    // serve eight products.  Build of 4 heads x 2564 tokens whose units are all done again: 1306 us, without 325; one of 32/8 heads x
+    // 664 tokens 689 (177); its step 68 (53).  (Four threads a row, a value of theirs at a time, a key at a time: 10900, 5400 and 270.)
+    const int r = threadIdx.x >> 3, c0 = (threadIdx.x & 7) * 4;
+    constexpr int NC = D / 32;
+    float4 qv[2][NC], acc[2][NC];
+    float M[2] = {-INFINITY, -INFINITY}, L[2] = {0.f, 0.f};
 #pragma unroll
-    for (int f = 0; f < D / 4; ++f) acc[f] = 0.f;
+    for (int e = 0; e < 2; ++e) {
+      const int tok = it.row0 + min(r + 16 * e, it.nrows - 1);
+      if (q_raw) {
+        const size_t row = blk_row0 + (tok - bs), off = (row * g.Hq + h) * D + c0, tab = row * (D / 2) + c0;
+#pragma unroll
+        for (int i = 0; i < NC / 2; ++i)
+          rotate4(load4(a.q_raw, off + 32 * i, a.raw_bf16), load4(a.q_raw, off + 32 * i + D / 2, a.raw_bf16),
+                  *reinterpret_cast<const float4*>(a.row_cos + tab + 32 * i), *reinterpret_cast<const float4*>(a.row_sin + tab + 32 * i),
+                  qv[e][i], qv[e][i + NC / 2]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < NC; ++i) qv[e][i] = *reinterpret_cast<const float4*>(qr + (size_t)tok * D + ((c0 + 32 * i) ^ simt_swz_qk(tok)));
+      }
+#pragma unroll
+      for (int i = 0; i < NC; ++i) acc[e][i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll 1
     for (t = next_tile(t_begin); t < t_end; t = next_tile(t + 1)) {
-      load_mixed(Few(), t, Kl, Vs);
+      load_mixed(Many(), t, Kl, Vs);
       __syncthreads();
-      for (int j = 0; j < KT; ++j) {
-        const int key = k0 + t * KT + j;
-        if (key >= k1 || (key >= x0 && key < x1)) continue;
-        const int zk = simt_swz_qk(key), zv = simt_swz_v(key);
-        float sc = 0.f;
-#pragma unroll 4
-        for (int f = 0; f < D; ++f) sc = fmaf(qrow[f ^ zq], Kl[j * D + (f ^ zk)], sc);
-        sc *= g.scale_log2;
-        const float m_new = fmaxf(M, sc);
-        const float al = M == -INFINITY ? 0.f : exp2f(M - m_new), p = exp2f(sc - (m_new == -INFINITY ? 0.f : m_new));
-        M = m_new;
-        L = L * al + p;
+#pragma unroll 1
+      for (int j0 = 0; j0 < KT; j0 += 4) {
+        const int key0 = k0 + t * KT + j0;
+        auto counts = [&](int j) { return key0 + j < k1 && !(key0 + j >= x0 && key0 + j < x1); };   // (the same in every thread)
+        float sc[2][4];
 #pragma unroll
-        for (int f = 0; f < D / 4; ++f) acc[f] = fmaf(p, Vs[j * D + ((f0 + f) ^ zv)], acc[f] * al);
+        for (int j = 0; j < 4; ++j) {
+          float4 s4[2] = {};
+#pragma unroll
+          for (int i = 0; i < NC; ++i) {
+            const float4 k4 = *reinterpret_cast<const float4*>(Kl + (j0 + j) * D + ((c0 + 32 * i) ^ simt_swz_qk(key0 + j)));
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              s4[e].x = fmaf(qv[e][i].x, k4.x, s4[e].x); s4[e].y = fmaf(qv[e][i].y, k4.y, s4[e].y);
+              s4[e].z = fmaf(qv[e][i].z, k4.z, s4[e].z); s4[e].w = fmaf(qv[e][i].w, k4.w, s4[e].w);
+            }
+          }
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            sc[e][j] = (s4[e].x + s4[e].y) + (s4[e].z + s4[e].w);
+#pragma unroll
+            for (int x = 1; x < 8; x <<= 1) sc[e][j] += __shfl_xor_sync(0xffffffffu, sc[e][j], x);
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          float m_new = M[e];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            sc[e][j] = counts(j) ? sc[e][j] * g.scale_log2 : -INFINITY;
+            m_new = fmaxf(m_new, sc[e][j]);
+          }
+          const float al = M[e] == -INFINITY ? 0.f : exp2f(M[e] - m_new), m_use = m_new == -INFINITY ? 0.f : m_new;
+          M[e] = m_new;
+          L[e] *= al;
+#pragma unroll
+          for (int i = 0; i < NC; ++i) { acc[e][i].x *= al; acc[e][i].y *= al; acc[e][i].z *= al; acc[e][i].w *= al; }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            sc[e][j] = exp2f(sc[e][j] - m_use);
+            if (counts(j)) L[e] += sc[e][j];
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          if (!counts(j)) continue;   // (its value may be anything)
+#pragma unroll
+          for (int i = 0; i < NC; ++i) {
+            const float4 v4 = *reinterpret_cast<const float4*>(Vs + (j0 + j) * D + ((c0 + 32 * i) ^ simt_swz_v(key0 + j)));
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              const float p = sc[e][j];
+              acc[e][i].x = fmaf(p, v4.x, acc[e][i].x); acc[e][i].y = fmaf(p, v4.y, acc[e][i].y);
+              acc[e][i].z = fmaf(p, v4.z, acc[e][i].z); acc[e][i].w = fmaf(p, v4.w, acc[e][i].w);
+            }
+          }
+        }
       }
       __syncthreads();
     }
-    for (int f = 0; f < D / 4; ++f) Vs[r * D + f0 + f] = acc[f];
-    if (f0 == 0) *reinterpret_cast<float2*>(sm + SM::ML + r * 2) = make_float2(M, L);
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+#pragma unroll
+      for (int i = 0; i < NC; ++i) *reinterpret_cast<float4*>(Vs + (r + 16 * e) * D + c0 + 32 * i) = acc[e][i];
+      if (c0 == 0) *reinterpret_cast<float2*>(sm + SM::ML + (r + 16 * e) * 2) = make_float2(M[e], L[e]);
+    }
   } else {
 #pragma unroll
     for (int i = 0; i < 2; ++i)
