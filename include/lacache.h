@@ -83,7 +83,8 @@ enum { LACACHE_OUT_BF16 = 0, LACACHE_OUT_FP32 = 1 };
  *          about two in hand on the maximum and four on the mean (measured against the fp64 evaluation
  *          on the LLaDA-shaped configurations, outlier keys included); SPLIT has a factor of twenty.
  *          Rotated values beyond the fp16 range (|x| > 65504) saturate: inputs of that size need SPLIT.
- * The fp32 engine ignores the mode (its operands are fp32).
+ * The fp32 engine ignores the mode: its operands are fp32, multiplied as sums of three bf16 parts that hold
+ * all their bits, and summed in fp32.
  */
 enum { LACACHE_PRECISION_PLAIN = 0, LACACHE_PRECISION_SPLIT = 1, LACACHE_PRECISION_FP16 = 3 };
 /* (2 is reserved: split planes plus split probabilities, which this library does not offer) */

@@ -11,17 +11,21 @@
 // many keys is cut over the S <= 8 CTAs of a thread-block cluster, whose online-softmax states are merged through distributed
 // shared memory (how many: simt_row_parts, simt_step_parts).
 //
-// Products run on the tensor cores with fp32 accuracy: an operand is split in two tf32 parts, x = hi + lo, and a product is
-// hi.hi + hi.lo + lo.hi (what is left out is 2^-22 of it).  The tensor cores cut a sum off where an fp32 addition rounds, so
-// sums go over few steps there (32 features, 16 keys) and are then added up in fp32.  Error of the output against fp64 (2-norm, 24
-// models of 90 to 650 tokens): 1.1e-7, and 3.6e-7 where scores are of order 50; chains of fp32 products on the CUDA cores, which
-// this replaced, 1.35e-7 and 4.6e-7.
+// Products run on the tensor cores with fp32 accuracy: an operand is split in three bf16 parts that hold all its bits, x = hi + mid + lo,
+// and a product is hi.hi + hi.mid + mid.hi + mid.mid + hi.lo + lo.hi (what is left out is 2^-24 of it at most and 2^-27 in the mean).
+// The tensor cores cut a sum off where an fp32 addition rounds.  Of hi.hi, products of 16 bits, sixteen are added there, which seldom needs
+// more than the 24 bits there are, and those sums in fp32; the others are 2^-8 of a product and less.  Error of the output against fp64
+// (2-norm, 24 models of 90 to 650 tokens): 0.86e-7, and 3.0e-7 where scores are of order 50; chains of fp32 products on the CUDA cores
+// 1.35e-7 and 4.6e-7.  Scores that one feature dominates: 0.43 to 0.6 of the chains' error, and 1.2 of it where the chains meet that feature
+// last (one large channel, the last).  (Two tf32 parts, three products: 1.1e-7 and 3.6e-7, but operands of 22 bits: twice the chains' error
+// where a score is one feature's product, and a row with one key does not return that key's value.)
 //
-// What bounds it: a tile of 128 features is 768 tensor-core instructions of 2 cycles, 1536 on an SM (on the CUDA cores it took 5100,
-// the shared-memory pipe's: every thread read its operands 16 bytes for 32 products).  Two CTAs to an SM (226 and 246 registers a thread, 82 KB)
-// keep it fed; alone a CTA takes about 4000 a tile.  Around the tiles it is latency: item and lists, the first tile's way, the merge
-// of the parts, about 10000 cycles a CTA.  Build with its RoPE launch, before and now: 152 units x 11 tiles 48.5 -> 36.5 us, 660 x 21
-// 233 -> 172, 560 x 71 660 -> 450; step of 4 heads x 5120 tokens 102 -> 78.
+// What bounds it: a tile of 128 features is 768 tensor-core instructions of 2 cycles, 1536 on an SM, and as many cycles of splitting (on
+// the CUDA cores it took 5100, the shared-memory pipe's: every thread read its operands 16 bytes for 32 products).  Two CTAs to an SM (255
+// registers a thread, 91 KB) are eight warps, whose instructions wait for the ones before: 3500 a tile.  Around the tiles it is latency:
+// item and lists, the first tile's way, the merge of the parts, about 10000 cycles a CTA.  Builds with their RoPE launch, on the CUDA cores and now:
+// 4 heads x 2564 tokens 482 -> 331 us, 32/8 x 664 243 -> 179, 16 x 1256 424 -> 300 (two tf32 parts 316, 170 and 284); steps of the
+// same 48.8 -> 42.6, 52.0 -> 50.5, 55.0 -> 50.4 (40.4, 46.0, 45.9).
 //
 // In a step the kernel rotates the block's rows itself, wherever it needs them,
 // and leaves them in the rotated cache: one launch, no kernel in front of it.
@@ -43,19 +47,20 @@ using namespace ptx;
 constexpr int KT = 32;       // keys per tile
 constexpr int THREADS = 128; // warp w: rows 16 (w & 1) .. of the unit, keys 16 (w >> 1) .. of each tile
 
-// Shared memory, in floats: queries, keys and values [32][D] as they lie in the rotated cache, whose rows are swizzled so
-// that the reads below meet no bank twice (simt_swz_qk, simt_swz_v).  After the last tile the first values' place holds the
-// CTA's partial O~ [32][D], ML the partial (m, l); the first keys' place, what half of the warps hand to the others.
+// Shared memory, in floats: the queries as operands of the tensor cores, [16 rows][16 features][part][lane][4], and keys and
+// values [32][D] as they lie in the rotated cache, whose rows are swizzled so that the reads below meet no bank twice
+// (simt_swz_qk, simt_swz_v).  After the last tile the first values' place holds the CTA's partial O~ [32][D], ML the partial
+// (m, l); the first keys' place, what half of the warps hand to the others.
 template <int D>
 struct Smem {
   static constexpr int Q = 0;
   static constexpr int TILE = KT * D;
-  static constexpr int K = Q + SIMT_ROWS * D;          // two buffers of keys, two of values
+  static constexpr int K = Q + SIMT_ROWS * D * 3 / 2;  // two buffers of keys, two of values
   static constexpr int V = K + 2 * TILE;
   static constexpr int ML = V + 2 * TILE;
   static constexpr int ST = ML + 2 * SIMT_ROWS * 2;    // (m, l) of the rows' cached state
-  static constexpr int BAR = ST + SIMT_ROWS * 2;       // barriers: queries, keys 0 and 1, values 0 and 1 in place
-  static constexpr int TOTAL = BAR + 12;
+  static constexpr int BAR = ST + SIMT_ROWS * 2;       // barriers: keys 0 and 1, values 0 and 1 in place
+  static constexpr int TOTAL = BAR + 8;
   static constexpr size_t bytes = TOTAL * sizeof(float);
   static_assert(SIMT_ROWS == KT, "the partial O~ over the values");
 };
@@ -86,16 +91,60 @@ __device__ __forceinline__ float2 ld_cluster_v2(uint32_t addr) {
   asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
   return v;
 }
-// D += A B on the warp's tensor core, 16 x 8 x 8, operands as tf32 (the low 13 bits are not read), fp32 sums
-__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+// D += A B on the warp's tensor core, 16 x 8 x 16, operands as bf16, fp32 sums
+__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// x = hi + lo: hi the nearest tf32 value, lo the rest, of which a product reads the first 11 bits (all but the last bit of x
-// at most)
-__device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) {
-  hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
-  lo = __float_as_uint(x - __uint_as_float(hi));
+// x = hi + mid + lo of a pair of values (x0 in the lower halves): each the nearest bf16 value of what is left, so that the three
+// hold all 24 bits of x (unless the last lie below the smallest bf16 value)
+__device__ __forceinline__ uint32_t nearest_bf16(float x0, float x1) {
+  uint32_t r;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(x1), "f"(x0));
+  return r;
+}
+// two fp32 values in one register pair: one instruction for both
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ float2 scaled2(float a, float b, float by) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pack2(a, b)), "l"(pack2(by, by)));
+  return unpack2(d);
+}
+__device__ __forceinline__ float bf16_lower(uint32_t p) { return __uint_as_float(p << 16); }
+__device__ __forceinline__ float bf16_upper(uint32_t p) { return __uint_as_float(p & 0xffff0000u); }
+__device__ __forceinline__ float2 less2(float2 x, float h0, float h1) { return unpack2(fma2(pack2(h0, h1), pack2(-1.f, -1.f), pack2(x.x, x.y))); }
+__device__ __forceinline__ void split3(float x0, float x1, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+  float2 x = make_float2(x0, x1);
+  hi = nearest_bf16(x.x, x.y);
+  x = less2(x, bf16_lower(hi), bf16_upper(hi));
+  mid = nearest_bf16(x.x, x.y);
+  x = less2(x, bf16_lower(mid), bf16_upper(mid));
+  lo = nearest_bf16(x.x, x.y);
+}
+// ... of two values each of two rows, a and b, paired across the rows
+__device__ __forceinline__ void split3_across(float2 a, float2 b, uint32_t (&x)[3], uint32_t (&y)[3]) {
+#pragma unroll
+  for (int p = 0; p < 3; ++p) {
+    x[p] = nearest_bf16(a.x, b.x);
+    y[p] = nearest_bf16(a.y, b.y);
+    if (p == 2) break;
+    a = less2(a, bf16_lower(x[p]), bf16_lower(y[p]));
+    b = less2(b, bf16_upper(x[p]), bf16_upper(y[p]));
+  }
 }
 __device__ __forceinline__ float4 load4(const void* base, size_t off, bool bf16) {
   if (!bf16) return *reinterpret_cast<const float4*>(reinterpret_cast<const float*>(base) + off);
@@ -141,7 +190,7 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
   const int bs = a.blk_start ? a.blk_start[it.seq] : 0;
   const int be = bs + g.block_len;
   if (threadIdx.x == 0) {
-    for (int i = 0; i < 5; ++i) mbar_init(smem_u32(sm + SM::BAR) + 8 * i, 1);
+    for (int i = 0; i < 4; ++i) mbar_init(smem_u32(sm + SM::BAR) + 8 * i, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
@@ -174,9 +223,9 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
   float* const Vs = sm + SM::V;
   const bool writes_cache = q_raw && it.row0 == bs && h % g.group == 0;   // leaves the block's keys and values in the cache
 
-  // Tiles, and the rows of fixed queries, are contiguous in the cache: a bulk copy each, the next tile's under way while a tile
+  // Tiles are contiguous in the cache: a bulk copy each, the next tile's under way while a tile
   // is computed (two buffers).  (Rows past the key range are other rows of the cache: their scores are masked.)
-  const uint32_t bar_q = smem_u32(sm + SM::BAR), bar_k = bar_q + 8, bar_v = bar_q + 24;
+  const uint32_t bar_k = smem_u32(sm + SM::BAR), bar_v = bar_k + 16;
   auto issue = [&](float* dst, const float* src, uint32_t bar) {
     mbar_expect_tx(bar, KT * D * 4);
     bulk_load(dst, src, KT * D * 4, bar);
@@ -252,39 +301,65 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
     l_st = a.st.l[(size_t)h * g.Tp + it.row0 + lane];
   }
   if (t < t_end && !is_mixed(t)) issue_tile(t, 0);
-  // queries (what rows past the tile's end hold is not used)
-  if (!q_raw) {
-    if (threadIdx.x == 0) issue(sm + SM::Q, qr + (size_t)it.row0 * D, bar_q);
-  } else {
-    constexpr int N = SIMT_ROWS * (D4 / 2) / THREADS;
-    float4 x1[N], x2[N], cs[N], sn[N];
+  // The queries, as operands: a thread takes rows g and g + 8 of a warp's sixteen, and of both four features of a step and their
+  // partners (registers 0 and 2: row g, features 0 1 and 2 3).  Times 2^24, so that the parts of small ones are bf16 values too.
+  bool bad = false;   // the unit is to be done with plain products (below)
+  {
+    // (what a key loses where its parts are smaller than any bf16 value is nothing beside a score, unless the query is huge)
+    const float q_most = fminf(0x1p80f / fabsf(g.scale_log2), 0x1p100f);
+    constexpr int STEPS = D / 16, N = STEPS / (THREADS / 32);
+    uint4* const qf = reinterpret_cast<uint4*>(sm + SM::Q);
+    float4 x1[N][2], x2[N][2], cs[N][2], sn[N][2];
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-      const int i = threadIdx.x + j * THREADS, r = min(i / (D4 / 2), it.nrows - 1), c = (i % (D4 / 2)) * 4;
-      const size_t row = blk_row0 + (it.row0 - bs) + r, off = (row * g.Hq + h) * D + c, tab = row * (D / 2) + c;
-      x1[j] = load4(a.q_raw, off, a.raw_bf16);
-      x2[j] = load4(a.q_raw, off + D / 2, a.raw_bf16);
-      cs[j] = *reinterpret_cast<const float4*>(a.row_cos + tab);
-      sn[j] = *reinterpret_cast<const float4*>(a.row_sin + tab);
-    }
+      const int i = warp + j * (THREADS / 32), c = 16 * (i % (STEPS / 2)) + (lane & 3) * 4;
 #pragma unroll
-    for (int j = 0; j < N; ++j) {
-      const int i = threadIdx.x + j * THREADS, r = i / (D4 / 2), c = (i % (D4 / 2)) * 4;
-      float4 y1, y2;
-      rotate4(x1[j], x2[j], cs[j], sn[j], y1, y2);
-      const int cz = c ^ simt_swz_qk(it.row0 + r);
-      if (part == 0 && r < it.nrows) {
-        *reinterpret_cast<float4*>(qr + (size_t)(it.row0 + r) * D + cz) = y1;
-        *reinterpret_cast<float4*>(qr + (size_t)(it.row0 + r) * D + cz + D / 2) = y2;
+      for (int e = 0; e < 2; ++e) {
+        const int r = min(16 * (i / (STEPS / 2)) + (lane >> 2) + 8 * e, it.nrows - 1);
+        if (q_raw) {
+          const size_t row = blk_row0 + (it.row0 - bs) + r, off = (row * g.Hq + h) * D + c, tab = row * (D / 2) + c;
+          x1[j][e] = load4(a.q_raw, off, a.raw_bf16);
+          x2[j][e] = load4(a.q_raw, off + D / 2, a.raw_bf16);
+          cs[j][e] = *reinterpret_cast<const float4*>(a.row_cos + tab);
+          sn[j][e] = *reinterpret_cast<const float4*>(a.row_sin + tab);
+        } else {
+          const float* const src = qr + (size_t)(it.row0 + r) * D + (c ^ simt_swz_qk(it.row0 + r));
+          x1[j][e] = *reinterpret_cast<const float4*>(src);
+          x2[j][e] = *reinterpret_cast<const float4*>(src + D / 2);
+        }
       }
-      *reinterpret_cast<float4*>(sm + SM::Q + r * D + cz) = y1;
-      *reinterpret_cast<float4*>(sm + SM::Q + r * D + cz + D / 2) = y2;
+    }
+    if (t < t_end && is_mixed(t)) load_mixed(Many(), t, Ks, Vs);
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+      const int i = warp + j * (THREADS / 32), rw = i / (STEPS / 2), step = i % (STEPS / 2);
+      if (q_raw) {
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const int r = 16 * rw + (lane >> 2) + 8 * e;
+          rotate4(x1[j][e], x2[j][e], cs[j][e], sn[j][e], x1[j][e], x2[j][e]);
+          if (part == 0 && r < it.nrows) {
+            float* const dst = qr + (size_t)(it.row0 + r) * D + ((16 * step + (lane & 3) * 4) ^ simt_swz_qk(it.row0 + r));
+            *reinterpret_cast<float4*>(dst) = x1[j][e];
+            *reinterpret_cast<float4*>(dst + D / 2) = x2[j][e];
+          }
+        }
+      }
+#pragma unroll
+      for (int f = 0; f < 2; ++f) {
+        uint32_t p[3][4];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          const float4 x = f ? x2[j][e] : x1[j][e];
+          bad = bad || !(fmaxf(fmaxf(fabsf(x.x), fabsf(x.y)), fmaxf(fabsf(x.z), fabsf(x.w))) <= q_most);
+          split3(x.x * 0x1p24f, x.y * 0x1p24f, p[0][e], p[1][e], p[2][e]);
+          split3(x.z * 0x1p24f, x.w * 0x1p24f, p[0][2 + e], p[1][2 + e], p[2][2 + e]);
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) qf[((rw * STEPS + step + f * (STEPS / 2)) * 3 + k) * 32 + lane] = make_uint4(p[k][0], p[k][1], p[k][2], p[k][3]);
+      }
     }
   }
-  if (t < t_end && is_mixed(t)) {
-    load_mixed(Many(), t, Ks, Vs);
-  }
-  if (!q_raw) wait_loads(bar_q, 0u, a.status, LOC_WAIT_Q);
 
   // The warp's 16 rows x 16 keys of a tile, as the tensor cores lay them out: this thread has rows g and g + 8, keys 2 t and
   // 2 t + 1 of either eight (scores: n columns; P.V: k index t <-> key 2 t, t + 4 <-> key 2 t + 1, so that a thread's
@@ -293,12 +368,12 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
   const bool rows = 16 * rw < it.nrows;   // this warp has rows (the others only help loading)
   // (where the thread's first 16 bytes of a row lie, the rows' parity and pairs counted from the cache's first row: tiles are
   // 32 rows apart, so it is the same place in every tile)
-  const float* const qp = sm + SM::Q + (16 * rw + g8) * D + ((4 * t4) ^ simt_swz_qk(it.row0 + g8));
+  const uint4* const qp = reinterpret_cast<const uint4*>(sm + SM::Q) + rw * (D / 16) * 3 * 32 + lane;
   const float* const kp0 = Ks + (16 * kw + g8) * D + ((4 * t4) ^ simt_swz_qk(k0 + g8));
   const float* const vpa = Vs + (16 * kw + 2 * t4) * D + ((4 * g8) ^ simt_swz_v(k0 + 2 * t4));
   const float* const vpb = Vs + (16 * kw + 2 * t4 + 1) * D + ((4 * g8) ^ simt_swz_v(k0 + 2 * t4 + 1));
-  const int qflip = simt_swz_qk(it.row0 + g8) ? -16 : 16, kflip = simt_swz_qk(k0 + g8) ? -16 : 16;   // to the next 16 features
-  float m[2], l[2];
+  const int kflip = simt_swz_qk(k0 + g8) ? -16 : 16;   // to the next 16 features
+  float m[2], l[2], past = 0.f;
   float o[D / 8][4];   // [4 q + j]: {row g: features 8 t + j, 8 t + 4 + j; row g + 8: likewise} of the 32 from 32 q
 #pragma unroll
   for (int i = 0; i < 2; ++i) { m[i] = -INFINITY; l[i] = 0.f; }
@@ -333,53 +408,45 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
     const float* const vp1 = vpb + buf * SM::TILE;
     float s[2][4];
     if (rows) {
-      // Every product as hi.hi + (lo.hi + hi.lo), the small ones in sums of their own; the tensor cores cut sums off
-      // instead of rounding them, so the large ones go over four steps and are then added with rounding.
-      float small[2][4], big[2][4];
+      // Every product but lo.lo (2^-34 of it): hi.hi, whose 16 bits leave room for a sum of sixteen, over one step at a time and then
+      // added with rounding, for the tensor cores cut sums off; the others, 2^-8 and less of it, in two sums of their own.
+      float small[2][2][4];
 #pragma unroll
       for (int n = 0; n < 2; ++n)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) { s[n][c] = 0.f; small[n][c] = 0.f; }
-#pragma unroll 2
+        for (int c = 0; c < 4; ++c) { s[n][c] = 0.f; small[n][0][c] = 0.f; small[n][1][c] = 0.f; }
+#pragma unroll
       for (int c0 = 0; c0 < D; c0 += 32) {
 #pragma unroll
-        for (int n = 0; n < 2; ++n)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) big[n][c] = 0.f;
-#pragma unroll
         for (int cc = 0; cc < 2; ++cc) {
-          uint32_t qh[2][4], ql[2][4];   // [step][operand register]
-          {
-            const float* const qc = qp + c0 + (cc ? qflip : 0);
-            const float4 qa = *reinterpret_cast<const float4*>(qc), qb = *reinterpret_cast<const float4*>(qc + 8 * D);
-            split_tf32(qa.x, qh[0][0], ql[0][0]); split_tf32(qb.x, qh[0][1], ql[0][1]);
-            split_tf32(qa.y, qh[0][2], ql[0][2]); split_tf32(qb.y, qh[0][3], ql[0][3]);
-            split_tf32(qa.z, qh[1][0], ql[1][0]); split_tf32(qb.z, qh[1][1], ql[1][1]);
-            split_tf32(qa.w, qh[1][2], ql[1][2]); split_tf32(qb.w, qh[1][3], ql[1][3]);
+          uint32_t qx[3][4];   // [part][operand register]
+#pragma unroll
+          for (int j = 0; j < 3; ++j) {
+            const uint4 u = qp[((c0 / 16 + cc) * 3 + j) * 32];
+            qx[j][0] = u.x; qx[j][1] = u.y; qx[j][2] = u.z; qx[j][3] = u.w;
           }
 #pragma unroll
           for (int n = 0; n < 2; ++n) {
             const float4 k4 = *reinterpret_cast<const float4*>(kp + 8 * n * D + c0 + (cc ? kflip : 0));
-            uint32_t kh[4], kl[4];
-            split_tf32(k4.x, kh[0], kl[0]); split_tf32(k4.y, kh[1], kl[1]);
-            split_tf32(k4.z, kh[2], kl[2]); split_tf32(k4.w, kh[3], kl[3]);
+            uint32_t kx[3][2];
+            split3(k4.x, k4.y, kx[0][0], kx[1][0], kx[2][0]);
+            split3(k4.z, k4.w, kx[0][1], kx[1][1], kx[2][1]);
+            float big[4] = {0.f, 0.f, 0.f, 0.f};
+            mma_bf16(big, qx[0], kx[0][0], kx[0][1]);
+            mma_bf16(small[n][0], qx[1], kx[0][0], kx[0][1]);
+            mma_bf16(small[n][1], qx[2], kx[0][0], kx[0][1]);
+            mma_bf16(small[n][0], qx[0], kx[1][0], kx[1][1]);
+            mma_bf16(small[n][1], qx[1], kx[1][0], kx[1][1]);
+            mma_bf16(small[n][1], qx[0], kx[2][0], kx[2][1]);
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-              mma_tf32(big[n], qh[e], kh[2 * e], kh[2 * e + 1]);
-              mma_tf32(small[n], ql[e], kh[2 * e], kh[2 * e + 1]);
-              mma_tf32(small[n], qh[e], kl[2 * e], kl[2 * e + 1]);
-            }
+            for (int c = 0; c < 4; ++c) s[n][c] += big[c];
           }
         }
-#pragma unroll
-        for (int n = 0; n < 2; ++n)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) s[n][c] += big[n][c];
       }
 #pragma unroll
       for (int n = 0; n < 2; ++n)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) s[n][c] += small[n][c];
+        for (int c = 0; c < 4; ++c) s[n][c] += small[n][0][c] + small[n][1][c];
     }
     if (bulk) wait_loads(bar_v + 8 * buf, phase, a.status, LOC_WAIT_V);
     if (rows) {
@@ -399,7 +466,8 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
         for (int n = 0; n < 2; ++n)
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
-            a[n][e] = ok[n][e] ? s[n][2 * i + e] * g.scale_log2 : -INFINITY;
+            if (ok[n][e]) past = fmaf(s[n][2 * i + e], 0.f, past);   // (NaN from a score that is none)
+            a[n][e] = ok[n][e] ? s[n][2 * i + e] * 0x1p-24f * g.scale_log2 : -INFINITY;
             mx = fmaxf(mx, a[n][e]);
           }
         mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
@@ -408,71 +476,59 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
         const float m_use = m_new == -INFINITY ? 0.f : m_new;
         alpha[i] = m[i] == -INFINITY ? 0.f : exp2f(m[i] - m_new);
         m[i] = m_new;
-        float sum = 0.f;
 #pragma unroll
         for (int n = 0; n < 2; ++n)
 #pragma unroll
           for (int e = 0; e < 2; ++e) {
             s[n][2 * i + e] = ok[n][e] ? exp2f(a[n][e] - m_use) : 0.f;
-            sum += s[n][2 * i + e];
           }
-        l[i] = l[i] * alpha[i] + sum;
+        l[i] = l[i] * alpha[i] + ((s[0][2 * i] + s[0][2 * i + 1]) + (s[1][2 * i] + s[1][2 * i + 1]));
       }
-      uint32_t ph[2][4], pl[2][4];
+      uint32_t px[3][4];   // (times 2^24, as the values below: all parts of all fp32 values are bf16 values)
 #pragma unroll
-      for (int n = 0; n < 2; ++n) {
-        split_tf32(s[n][0], ph[n][0], pl[n][0]); split_tf32(s[n][2], ph[n][1], pl[n][1]);
-        split_tf32(s[n][1], ph[n][2], pl[n][2]); split_tf32(s[n][3], ph[n][3], pl[n][3]);
-      }
+      for (int n = 0; n < 2; ++n)
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+          split3(s[n][2 * i] * 0x1p24f, s[n][2 * i + 1] * 0x1p24f, px[0][2 * n + i], px[1][2 * n + i], px[2][2 * n + i]);
 #pragma unroll
       for (int q = 0; q < D / 32; ++q) {
-        // (the small products first: a sum is cut off at the size it has reached)
-        float pv[4][4] = {};
-        uint32_t vh[2][2][4], vl[2][2][4];   // [step][key][feature]
-#pragma unroll
-        for (int n = 0; n < 2; ++n)
-#pragma unroll
-          for (int e = 0; e < 2; ++e) {
-            const float4 v4 = *reinterpret_cast<const float4*>((e ? vp1 : vp0) + 8 * n * D + 32 * q);
-            split_tf32(v4.x, vh[n][e][0], vl[n][e][0]); split_tf32(v4.y, vh[n][e][1], vl[n][e][1]);
-            split_tf32(v4.z, vh[n][e][2], vl[n][e][2]); split_tf32(v4.w, vh[n][e][3], vl[n][e][3]);
-          }
+        uint32_t vx[2][4][3];   // [operand register: keys 2 t and 2 t + 1 of either eight][feature][part]
 #pragma unroll
         for (int n = 0; n < 2; ++n) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) mma_tf32(pv[j], pl[n], vh[n][0][j], vh[n][1][j]);
-#pragma unroll
-          for (int j = 0; j < 4; ++j) mma_tf32(pv[j], ph[n], vl[n][0][j], vl[n][1][j]);
+          const float4 va = *reinterpret_cast<const float4*>(vp0 + 8 * n * D + 32 * q);
+          const float4 vb = *reinterpret_cast<const float4*>(vp1 + 8 * n * D + 32 * q);
+          split3_across(scaled2(va.x, va.y, 0x1p24f), scaled2(vb.x, vb.y, 0x1p24f), vx[n][0], vx[n][1]);
+          split3_across(scaled2(va.z, va.w, 0x1p24f), scaled2(vb.z, vb.w, 0x1p24f), vx[n][2], vx[n][3]);
         }
+        float pv[4][4] = {}, small[4][4] = {};
+        auto all = [&](float (&d)[4][4], int x, int y) {
 #pragma unroll
-        for (int n = 0; n < 2; ++n)
-#pragma unroll
-          for (int j = 0; j < 4; ++j) mma_tf32(pv[j], ph[n], vh[n][0][j], vh[n][1][j]);
+          for (int j = 0; j < 4; ++j) mma_bf16(d[j], px[x], vx[0][j][y], vx[1][j][y]);
+        };
+        all(pv, 0, 0);
+        all(small, 1, 1); all(small, 2, 0); all(small, 0, 2); all(small, 1, 0); all(small, 0, 1);
 #pragma unroll
         for (int j = 0; j < 4; ++j)
 #pragma unroll
-          for (int c = 0; c < 4; ++c) o[4 * q + j][c] = fmaf(o[4 * q + j][c], alpha[c >> 1], pv[j][c]);
+          for (int c = 0; c < 4; ++c) o[4 * q + j][c] = fmaf(o[4 * q + j][c], alpha[c >> 1], pv[j][c] + small[j][c]);
       }
     }
     t = tn;
   }
-  // Values that two tf32 parts do not hold (infinities, NaN, the last few below the largest) leave a NaN or an infinity behind, and
-  // the low parts of values below 2^-115 are subnormal, which the tensor cores drop: the unit is then done once more with plain
-  // products and sums, where they give what they give.
-  bool bad = false;
+  // Infinities, NaN and values of 2^80 and more leave a sum behind that is none, or were seen in the queries: the unit is then done
+  // once more with plain products and sums, where they give what they give.
   if (rows) {
 #pragma unroll
     for (int i = 0; i < 2; ++i) {
-      float z = l[i] * 0.f;
-      float least = INFINITY;   // of the magnitudes that are not zero
+      float z = fmaf(l[i], 0.f, past);
 #pragma unroll
       for (int f = 0; f < D / 8; ++f)
 #pragma unroll
         for (int e = 2 * i; e < 2 * i + 2; ++e) {
           z = fmaf(o[f][e], 0.f, z);
-          least = fminf(least, o[f][e] == 0.f ? INFINITY : fabsf(o[f][e]));
+          o[f][e] *= 0x1p-48f;
         }
-      bad = bad || (16 * rw + g8 + 8 * i < it.nrows && (least < 0x1p-100f || !(z == 0.f)));
+      bad = bad || (16 * rw + g8 + 8 * i < it.nrows && !(z == 0.f));
     }
   }
   const bool plain = __syncthreads_or(bad);   // (every warp has left the keys and values behind)

@@ -1,6 +1,6 @@
-"""The fp32 engine's products, which run as three tf32 products each: values that two tf32 parts do not hold (infinities, NaN,
-the largest finite ones) give what fp32 arithmetic gives, in the rows and features they reach and in no other; the range is that of
-fp32; and the results stay as close to fp64 as fp32 sums are, at sizes around a tile of 32 rows or keys."""
+"""The fp32 engine's products, which run as products of bf16 parts that hold all bits of their operands: values that three parts do
+not hold (infinities, NaN, the largest finite ones) give what fp32 arithmetic gives, in the rows and features they reach and in no other;
+the range is that of fp32; and the results stay as close to fp64 as fp32 sums are, at sizes around a tile of 32 rows or keys."""
 import numpy as np
 import pytest
 import torch
@@ -123,6 +123,147 @@ def test_the_range_is_that_of_fp32():
     b = _run(wl, q * np.float32(2.0 ** -90), k * np.float32(2.0 ** 90), v)
     for (o0, l0), (o1, l1) in zip(a, b):
         assert np.array_equal(o0, o1) and np.array_equal(l0, l1)
+
+
+def _rotated32(x, wl):
+    """rows rotated as the fp32 engine does it, every product and sum rounded: what is left of an output's error is the attention's"""
+    half = wl.head_dim // 2
+    f = np.array([wl.rope_theta ** (-2.0 * c / wl.head_dim) for c in range(half)])
+    y = np.empty_like(x)
+    for lo, hi in zip(wl.cu_seqlens, wl.cu_seqlens[1:]):
+        c, s = (fn(np.arange(hi - lo)[:, None] * f).astype(np.float32)[:, None] for fn in (np.cos, np.sin))
+        a, b = x[lo:hi, :, :half], x[lo:hi, :, half:]
+        y[lo:hi] = np.concatenate([a * c - b * s, b * c + a * s], -1)
+    return y
+
+
+def _attention64(q, k, v, wl):
+    """output and log-sum-exp of rotated rows in fp64"""
+    g, outs, lses = wl.n_q_heads // wl.n_kv_heads, [], []
+    for lo, hi in zip(wl.cu_seqlens, wl.cu_seqlens[1:]):
+        qq, kk, vv = (x[lo:hi].astype(np.float64) for x in (q, k, v))
+        sc = np.einsum("ihd,jhd->hij", qq, np.repeat(kk, g, 1)) * wl.head_dim ** -0.5
+        m = sc.max(-1, keepdims=True)
+        p = np.exp(sc - m)
+        outs.append(np.einsum("hij,jhd->ihd", p / p.sum(-1, keepdims=True), np.repeat(vv, g, 1)))
+        lses.append((m[..., 0] + np.log(p.sum(-1))).T)
+    return np.concatenate(outs), np.concatenate(lses)
+
+
+def _gauss(wl, seed):
+    rng = np.random.default_rng(seed)
+    return [rng.standard_normal((wl.total_tokens, h, wl.head_dim)).astype(np.float32) for h in (wl.n_q_heads, wl.n_kv_heads, wl.n_kv_heads)]
+
+
+def _model(d, prompts=(137, 61)):
+    return small_workload(name="products", dtype="fp32", prompt_lens=prompts, gen_len=64, block_len=32, steps=2, hq=4, hkv=2, d=d,
+                          scale_mode="inv_sqrt_d")
+
+
+def _error_of_rounded_scores(q, k, v, wl):
+    """What an output is off by, relative and in the mean, where every score is rounded four times: as the sum of two features' products
+    (twice), with the scale, and as the difference to the row's maximum.  A rounding to 24 bits is off by 2^-24 / sqrt(3) of the power of two
+    below the value; a score's error moves the output by its weight times its value's distance from the output."""
+    g, err, norm = wl.n_q_heads // wl.n_kv_heads, 0.0, 0.0
+    def rounding(x):
+        return np.exp2(np.floor(np.log2(np.maximum(np.abs(x), 1e-300)))) * 2.0 ** -24 / 3 ** 0.5
+    for lo, hi in zip(wl.cu_seqlens, wl.cu_seqlens[1:]):
+        qq, kk, vv = (x[lo:hi].astype(np.float64) for x in (q, k, v))
+        vv = np.repeat(vv, g, 1).transpose(1, 0, 2)
+        sc = np.einsum("ihd,jhd->hij", qq, np.repeat(kk, g, 1)) * wl.head_dim ** -0.5 / np.log(2)
+        top = sc.max(-1, keepdims=True)
+        p = np.exp2(sc - top)
+        p /= p.sum(-1, keepdims=True)
+        out = p @ vv
+        w = p ** 2 * (3 * rounding(sc) ** 2 + rounding(sc - top) ** 2) * np.log(2) ** 2
+        err += (w.sum(-1) * (out ** 2).sum(-1) + np.einsum("hij,hj->hi", w, (vv ** 2).sum(-1)) - 2 * ((w @ vv) * out).sum(-1)).sum()
+        norm += (out ** 2).sum()
+    return (err / norm) ** 0.5
+
+
+@pytest.mark.parametrize("where", ["first", "middle", "last"])
+@pytest.mark.parametrize("d", [64, 128])
+def test_scores_of_one_feature(where, d):
+    """A score of which one feature (and the one it turns with) is all there is: every rounding of a product shows.  Operands of 22 bits
+    are off by twice the sum's own roundings; the bound leaves three tenths for what else is rounded (weights, sums over keys)."""
+    wl = _model(d)
+    f = {"first": 0, "middle": d // 2 - 1, "last": d - 1}[where]
+    for seed in range(4):
+        q, k, v = _gauss(wl, seed)
+        for x in (q, k):
+            x[..., :f], x[..., f + 1:] = 0, 0
+            x *= 8
+        qr, kr = _rotated32(q, wl), _rotated32(k, wl)
+        want, _ = _attention64(qr, kr, v, wl)
+        most = 1.3 * _error_of_rounded_scores(qr, kr, v, wl)
+        for out, _ in _run(wl, q, k, v):
+            print(where, d, np.linalg.norm(out - want) / np.linalg.norm(want) / most)
+            assert np.linalg.norm(out - want) <= most * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_one_key_gives_its_value(d):
+    """A row whose weight is all one key's returns that key's value, to the last bit."""
+    wl = _model(d)
+    q, k, v = _gauss(wl, 9)
+    q[:], k[:] = 0, 0
+    q[..., d - 1] = 64
+    k[..., d - 1] = -64                                     # scores of -512 and less, but
+    for lo in wl.cu_seqlens[:-1]:
+        k[lo + 5, :, d - 1] = 64                            # one of +512 and less (the last feature turns by 1e-2 at most)
+    for out, lse in _run(wl, q, k, v):
+        for lo, hi in zip(wl.cu_seqlens, wl.cu_seqlens[1:]):
+            assert np.array_equal(out[lo:hi], np.repeat(np.repeat(v[lo + 5:lo + 6], 2, 1), hi - lo, 0).astype(np.float64))
+
+
+@pytest.mark.parametrize("eq,ek", [(-120, 120), (-126, 120), (-100, 60), (90, -110), (120, -120)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_scores_of_tiny_and_huge_rows(eq, ek, d):
+    """queries and keys scaled apart by powers of two, down to where parts of a split value, or the value, are subnormal: the error
+    stays that of fp32 sums (the bound of the test at the end of this file), but for what the smaller side's values, which are
+    multiples of 2^-149, lose themselves: the reference has the scaled values."""
+    wl = _model(d, (45, 30))
+    q, k, v = _gauss(wl, 5)
+    q, k = q * np.float32(d ** -0.5 * 2.0 ** (-(eq + ek) // 2)), k * np.float32(d ** -0.5 * 2.0 ** ((eq + ek) // 2 - (eq + ek)))
+    q, k = np.ldexp(q, eq), np.ldexp(k, ek)
+    want, wlse = _attention64(_rotated32(q, wl), _rotated32(k, wl), v, wl)
+    for out, lse in _run(wl, q, k, v):
+        assert np.linalg.norm(out - want) <= 4.5e-7 * np.linalg.norm(want)
+        assert np.abs(lse - wlse).max() <= 2e-6
+
+
+@pytest.mark.parametrize("exponent", [126, 130, 140])
+@pytest.mark.parametrize("d", [64, 128])
+def test_subnormal_values(exponent, d):
+    """values that are subnormal themselves: as close as fp32 sums, and within four roundings of a subnormal result (the two halves of a
+    tile's keys, the parts of a unit, the cached state, the division: half of 2^-149 each at most)."""
+    wl = _model(d, (45, 30))
+    q, k, v = _gauss(wl, 6)
+    q, k, v = q * np.float32(d ** -0.5), k * np.float32(d ** -0.5), np.ldexp(v, -exponent)
+    want, _ = _attention64(_rotated32(q, wl), _rotated32(k, wl), v, wl)
+    assert np.abs(want).max() > 2.0 ** -149
+    for out, _ in _run(wl, q, k, v):
+        assert (np.abs(out - want) <= 4 * 2.0 ** -149 + 2e-6 * np.abs(want).max()).all()
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_tiny_probabilities(d):
+    """Weights of about 2^-125 beside one of 1 whose value is zero: the result is theirs alone.  Their scores, 125 in the exponent's
+    units, are rounded to 2^-17 at worst three times (the feature's product, the scale, the difference to the maximum), a weight by 2^-18.5
+    ln 2 a time in the mean; the bound leaves three times that."""
+    wl = _model(d, (45, 30))
+    q, k, v = _gauss(wl, 7)
+    q[:], k[:] = 0, 0
+    q[..., d - 1] = 1
+    rng = np.random.default_rng(8)
+    k[..., d - 1] = -(86 + 0.5 * rng.random(k.shape[:2])) * d ** 0.5
+    v = np.ldexp(v, 100)
+    for lo in wl.cu_seqlens[:-1]:
+        k[lo + 5, :, d - 1] = 0
+        v[lo + 5] = 0
+    want, _ = _attention64(_rotated32(q, wl), _rotated32(k, wl), v, wl)
+    for out, _ in _run(wl, q, k, v):
+        assert np.linalg.norm(out - want) <= 3 * 3 ** 0.5 * 2.0 ** -18.5 * np.log(2) * np.linalg.norm(want)
 
 
 @pytest.mark.parametrize("exponent", [60, 108, 116, 122])
