@@ -223,18 +223,21 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
   float* const Vs = sm + SM::V;
   const bool writes_cache = q_raw && it.row0 == bs && h % g.group == 0;   // leaves the block's keys and values in the cache
 
-  // Tiles are contiguous in the cache: a bulk copy each, the next tile's under way while a tile
-  // is computed (two buffers).  (Rows past the key range are other rows of the cache: their scores are masked.)
+  // Tiles are contiguous in the cache: a bulk copy each, the next tile's under way while a tile is computed (two buffers).  Only the
+  // sequence's own rows are read (those behind are another's, which another CTA may be writing): the values that miss are zero, as
+  // their weights are, and the scores are masked, whatever the keys' place holds.
   const uint32_t bar_k = smem_u32(sm + SM::BAR), bar_v = bar_k + 16;
-  auto issue = [&](float* dst, const float* src, uint32_t bar) {
-    mbar_expect_tx(bar, KT * D * 4);
-    bulk_load(dst, src, KT * D * 4, bar);
-  };
   auto issue_tile = [&](int t, int buf) {
+    const int kt = k0 + t * KT, n = min(KT, k1 - kt);
+    float* const Vb = Vs + buf * SM::TILE;
+#pragma unroll 1
+    for (int i = n * D4 + threadIdx.x; i < KT * D4; i += THREADS) *reinterpret_cast<float4*>(Vb + i * 4) = make_float4(0.f, 0.f, 0.f, 0.f);
     if (threadIdx.x != 0) return;
     fence_async_smem();   // (a tile that the threads stored may have been there)
-    issue(Ks + buf * SM::TILE, kr + (size_t)(k0 + t * KT) * D, bar_k + 8 * buf);
-    issue(Vs + buf * SM::TILE, vr + (size_t)(k0 + t * KT) * D, bar_v + 8 * buf);
+    mbar_expect_tx(bar_k + 8 * buf, n * D * 4);
+    bulk_load(Ks + buf * SM::TILE, kr + (size_t)kt * D, n * D * 4, bar_k + 8 * buf);
+    mbar_expect_tx(bar_v + 8 * buf, n * D * 4);
+    bulk_load(Vb, vr + (size_t)kt * D, n * D * 4, bar_v + 8 * buf);
   };
   // A tile that holds block rows of a step is loaded by all threads, who rotate the block's rows (BATCH raw rows' loads leave
   // together) and take the others from the cache.
@@ -257,6 +260,8 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
           sn[j] = *reinterpret_cast<const float4*>(a.row_sin + row * (D / 2) + c);
           v1[j] = load4(a.v_raw, off, a.raw_bf16);
           v2[j] = load4(a.v_raw, off + D / 2, a.raw_bf16);
+        } else if (key >= k1) {
+          x1[j] = x2[j] = v1[j] = v2[j] = make_float4(0.f, 0.f, 0.f, 0.f);   // (as above)
         } else {
           const float* src = kr + (size_t)key * D + (c ^ simt_swz_qk(key));
           x1[j] = *reinterpret_cast<const float4*>(src);
@@ -395,7 +400,9 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
     }
     if (from_state && tn >= t_end && threadIdx.x == 0) {   // the rows' cached O~, into the buffer that no further keys need
       fence_async_smem();
-      issue(Ks + (buf ^ 1) * SM::TILE, a.st.o + ((size_t)h * g.Tp + it.row0) * D, bar_k + 8 * (buf ^ 1));
+      const uint32_t bytes = it.nrows * D * 4;
+      mbar_expect_tx(bar_k + 8 * (buf ^ 1), bytes);
+      bulk_load(Ks + (buf ^ 1) * SM::TILE, a.st.o + ((size_t)h * g.Tp + it.row0) * D, bytes, bar_k + 8 * (buf ^ 1));
     }
     const bool bulk = !is_mixed(t);
     const uint32_t phase = (phases >> buf) & 1u;

@@ -87,6 +87,66 @@ def test_queries_and_keys_that_two_parts_do_not_hold(value, which, d):
             assert np.nanmax(np.abs(out - want)) <= 1e-5
 
 
+@pytest.mark.parametrize("value", [np.nan, np.inf])
+@pytest.mark.parametrize("prompts,block", [((50, 1), 32), ((45, 30), 32), ((3, 40), 16), ((33, 70), 64)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_rows_of_another_sequence(prompts, block, value, d):
+    """A sequence's rows, whatever they hold, reach no other: its last key tile ends where the next one's rows (in a step, rows that are just
+    being written) begin, and its results are the same bits whether those are numbers or not."""
+    wl = small_workload(name="products", dtype="fp32", prompt_lens=prompts, gen_len=64, block_len=block, steps=2, hq=4, hkv=2, d=d,
+                        scale_mode="inv_sqrt_d")
+    q, k, v = (np.array(a) for a in SyntheticSchedule(wl, seed=4).begin_block(0))
+    n = wl.cu_seqlens[1]
+    clean = _run(wl, q, k, v)
+    q[n:], k[n:], v[n:] = value, value, value
+    for (o0, l0), (o1, l1) in zip(clean, _run(wl, q, k, v)):
+        assert np.array_equal(o0[:n], o1[:n]) and np.array_equal(l0[:n], l1[:n])
+        assert np.isnan(o1[n:]).all()
+
+
+@pytest.mark.parametrize("first,block", [(0, 32), (1, 32), (0, 16), (0, 64)])
+@pytest.mark.parametrize("d", [64, 128])
+def test_rows_of_the_excluded_block(first, block, d):
+    """A build leaves the block's own rows out: what it is given for them reaches neither the cached state nor the steps."""
+    wl = small_workload(name="products", dtype="fp32", prompt_lens=(45, 30), gen_len=64, block_len=block, steps=2, hq=4, hkv=2, d=d,
+                        scale_mode="inv_sqrt_d")
+    if (first + 1) * block > 64:
+        pytest.skip("no such block")
+    q, k, v = (np.array(a) for a in SyntheticSchedule(wl, seed=4).begin_block(0))
+    rows = torch.from_numpy(SyntheticSchedule(wl).block_rows(first)).cuda().long()
+    blk = [to_dev(x, wl)[rows].contiguous() for x in (q, k, v)]
+    got = []
+    for value in (0.0, np.nan):
+        for x in (q, k, v):
+            x[rows.cpu().numpy()] = value
+        ctx, (out, lse) = make_ctx(wl), new_outputs(wl)
+        ctx.build(first, *(to_dev(x, wl) for x in (q, k, v)))
+        ctx.step(*blk, out, lse)
+        got.append((out.cpu().numpy(), lse.cpu().numpy()))
+        ctx.destroy()
+    assert np.isfinite(got[0][0]).all()
+    assert np.abs(got[0][0] - got[1][0]).max() <= 1e-5 and np.abs(got[0][1] - got[1][1]).max() <= 1e-5
+
+
+@pytest.mark.parametrize("n", [33, 70])
+def test_words_left_by_an_earlier_call(n):
+    """The static call reads none of its scratch that it has not written: the same bits before and after a longer call of NaN."""
+    g = torch.Generator().manual_seed(3)
+    q, k, v = (torch.randn(200, 2, 64, generator=g).cuda() for _ in range(3))
+    out, lse = torch.empty(200, 2, 64, device="cuda"), torch.empty(200, 2, device="cuda")
+
+    def call(m, *rows):
+        binding.full_recompute_static(binding.DTYPE_FP32, 2, 2, 64, 1e4, *(x[:m].contiguous() for x in rows), out[:m], lse[:m])
+        torch.cuda.synchronize()
+        return out[:m].clone(), lse[:m].clone()
+    call(200, *(torch.zeros_like(x) for x in (q, k, v)))
+    before = call(n, q, k, v)
+    call(200, *(torch.full_like(x, float("nan")) for x in (q, k, v)))
+    after = call(n, q, k, v)
+    assert torch.isfinite(before[0]).all()
+    assert torch.equal(before[0], after[0]) and torch.equal(before[1], after[1])
+
+
 def test_cost_of_plain_products():
     """Units that are done once more with plain products: a build and a step where all of them are take no more than a few times as long
     (1306 us for 325 and 102 for 47 measured; 10900 and 684 where every thread took its values one at a time)."""
