@@ -697,12 +697,10 @@ AttnArgs attn_args(lacache_ctx* c, int mode, lacache_ctx::ListRef list, int blk,
         // Few tiles per CTA end together; with more, the kernels behind crowd the SMs that are idle first and run there.
         // Steps of 32 heads with one plane: 17.1 -> 16.2 us at 768 tokens, 23.6 -> 22.8 at 1536; of 28/4 heads 31.0 -> 29.3
         // at 1280 tokens (per_cta 3 to 5), but 31.1 -> 31.8 for four sequences (7) and 45 -> 49 at 5120 tokens.  Split planes
-        // lose 0.3 us; a step from token ids, behind which the projection's CTAs would wait on SMs, between -0.8 and 2.8.
+        // lose 0.3 us, and let in once a CTA has asked for its last tiles 0.952 to 1.095 of the time without (43 shapes of up to 12 units a
+        // CTA, 1.00 in the mean; nothing in their sizes tells which); a step from token ids, behind which the projection's CTAs would wait
+        // on SMs, between -0.8 and 2.8.
         a.step_overlap = (a.merge_deep && !c->split && c->g.block_len <= 32 && per_cta <= 5) ? 1 : 0;
-        // With split planes, said when a CTA has asked for its last tiles, it gains: 19.7 -> 19.0 us at 32 heads x 768 tokens (per_cta
-        // 3), 30.7 -> 29.8 at 16 x 3266 (6), 38.0 -> 35.8 at 28/4 x 11 short sequences (8), 52.3 -> 51.1 at 32 x 3638 (12); 20.7 -> 21.1 at
-        // 16 x 8 x 190 (4); and loses with many: 115 -> 125 at 32 x 8 x 900 (27).  (With one plane it loses from 7 on, 78 -> 83.)
-        if (a.merge_deep && c->split && per_cta <= 12) a.step_overlap = 2;
       }
       // Two key chunks per (sequence, head), one round of block-row units: the two chunks of a head (of a group of packed heads)
       // run as a pair of CTAs that merge through distributed shared memory.
@@ -1235,12 +1233,7 @@ lacache_status step_impl(lacache_ctx* c, const void* q, const void* k, const voi
   }
   AttnArgs a = attn_args(c, MODE_STEP, c->step_list[blk], blk, c->rot, out, lse);
   if (c->engine == LACACHE_ENGINE_TCGEN05) {
-    const bool off = c->knobs.no_pdl || c->knobs.no_step_overlap;
-    // (a late trigger not in a block's first step: what comes next may be a build, whose RoPE kernel's many CTAs crowd the SMs that
-    // are idle first; 126.5 -> 127.6 us for entering a block at 32 heads x 1536 tokens)
-    const int rule = a.step_overlap;   // (attn_args)
-    a.step_overlap = early_trigger(c->step_overlap != 0, rule == 1, inputs_just_written, off) ? 1
-                     : rule == 2 && c->steps_since_build > 1 && !inputs_just_written && !off  ? 2 : 0;
+    a.step_overlap = early_trigger(c->step_overlap != 0, a.step_overlap != 0, inputs_just_written, c->knobs.no_pdl || c->knobs.no_step_overlap) ? 1 : 0;
   } else {
     a.n_split_items = c->g.B * ((c->g.block_len + SIMT_ROWS - 1) / SIMT_ROWS);
     a.raw_bf16 = c->cfg.dtype == LACACHE_DTYPE_BF16 ? 1 : 0;

@@ -127,8 +127,8 @@ struct AttnArgs {
   int raw_bf16;
   int n_split_items;         // SIMT step: the block-query items, first in the list (their key range may be cut over CTAs)
   int split_ctas;            // SIMT: CTAs (one cluster) a cut unit takes; chosen by the launcher
-  int step_overlap;          // let the kernels behind be scheduled while this one drains (tcgen05, steps: 1 from its entry on, 2 once a
-                             // CTA has asked for its last tiles; SIMT: once a CTA has left its last key tile)
+  int step_overlap;          // let the kernels behind be scheduled while this one drains (tcgen05, steps: from its entry on;
+                             // SIMT: once a CTA has left its last key tile)
   const int32_t* blk_start;  // [B] absolute token index of the block's first row
   RotBuffers rot;
   StateBuffers st;

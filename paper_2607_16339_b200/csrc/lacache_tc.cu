@@ -408,7 +408,6 @@ __device__ void stream_producer(const Cta& c, const TcMaps& maps, const Geometry
     }
   }
   // (a CTA without units never touches memory the RoPE kernel writes)
-  if (SPLIT && a.step_overlap == 2) grid_launch_dependents();
 }
 
 // Two threads issue the stream role's MMAs, each a fixed pipeline with blocking (bounded) waits: one
@@ -1383,7 +1382,7 @@ __device__ __forceinline__ DUnit deep_unit(const Cta& c, int i) {
 }
 
 template <bool SPLIT, bool WIDE>
-__device__ void deep_producer(const Cta& c, const TcMaps& maps, const Geometry& g, int n_my, bool out_bf16, bool trigger_late) {
+__device__ void deep_producer(const Cta& c, const TcMaps& maps, const Geometry& g, int n_my, bool out_bf16) {
   using DL = Deep<SPLIT, WIDE>;
   if (n_my == 0) return;
   auto load_q = [&](int i) {
@@ -1425,7 +1424,6 @@ __device__ void deep_producer(const Cta& c, const TcMaps& maps, const Geometry& 
   grid_dependency_wait();
   load_k(0);
   load_v(0);
-  if (SPLIT && trigger_late && n_my == 1) grid_launch_dependents();
   int qu = 1, ku = 1, vu = 1, iu = 1, su = 0;
   bool pending_read = false;  // an output store may still be reading its staging tile
   long long t_idle = 0;
@@ -1451,7 +1449,6 @@ __device__ void deep_producer(const Cta& c, const TcMaps& maps, const Geometry& 
       if (pending_read) { bulk_wait_read(); pending_read = false; }
       load_io(iu);
       ++iu;
-      if (SPLIT && trigger_late && iu == n_my) grid_launch_dependents();   // (its last loads but for keys and values are under way)
       did = true;
     }
     if (did) {
@@ -1630,7 +1627,7 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
   // before they wait for this grid, only state that stays fixed until the next build and inputs that were
   // complete long before.  So they may in a short step without it, where they wait first (the rule: early_trigger in
   // lacache_plan.h).  Otherwise this kernel lets its successor start when it ends.
-  if (SPLIT ? a.step_overlap == 1 : a.step_overlap) grid_launch_dependents();
+  if (a.step_overlap) grid_launch_dependents();
   if (a.span != nullptr && tid == 0) atomicMin(a.span, global_timer_ns());   // first CTA entry of this launch
   Cta c;
   c.base = smem_u32(smem_raw);
@@ -1721,7 +1718,7 @@ tc_attn_kernel(const __grid_constant__ TcMaps maps, const Geometry g, const Attn
     if (stream) {
       if (tid == 0) stream_producer<PACKED, KIND, SPLIT>(c, maps, g, a, first, stride, n_units, it0);
     } else if (deep) {
-      if (tid == 0) deep_producer<SPLIT, WIDE>(c, maps, g, n_my, a.out_bf16 != 0, a.step_overlap == 2);
+      if (tid == 0) deep_producer<SPLIT, WIDE>(c, maps, g, n_my, a.out_bf16 != 0);
     } else {
       if (tid == 0) merge_producer<SPLIT>(c, maps, g, a, first, stride, n_units, it0);
     }
