@@ -825,8 +825,8 @@ cudaError_t simt_attention(const Geometry& g, const AttnArgs& args, int num_sms,
   if (!step) a.n_split_items = a.n_items;
   const int rest = a.n_items - a.n_split_items;
   const int max_tiles = (g.maxN + KT - 1) / KT;
-  a.split_ctas = step ? plan::simt_step_parts(a.n_split_items, rest, g.Hq, max_tiles, g.d, num_sms, plan::SIMT_TENSOR_CORES)
-                      : plan::simt_row_parts((long long)a.n_items * g.Hq, max_tiles, g.d, num_sms, plan::SIMT_TENSOR_CORES);
+  a.split_ctas = step ? plan::simt_step_parts(a.n_split_items, rest, g.Hq, max_tiles, g.d, num_sms)
+                      : plan::simt_row_parts((long long)a.n_items * g.Hq, max_tiles, g.d, num_sms);
   const int S = a.split_ctas;
   const int n_ctas = a.n_split_items * S + (rest + S - 1) / S * S;
   return g.d == 128 ? launch<128>(g, a, n_ctas, num_sms, s) : launch<64>(g, a, n_ctas, num_sms, s);
