@@ -22,10 +22,10 @@
 //
 // What bounds it: a tile of 128 features is 768 tensor-core instructions of 2 cycles, 1536 on an SM, and as many cycles of splitting (on
 // the CUDA cores it took 5100, the shared-memory pipe's: every thread read its operands 16 bytes for 32 products).  Two CTAs to an SM (255
-// registers a thread, 91 KB) are eight warps, whose instructions wait for the ones before: 3500 a tile.  Around the tiles it is latency:
+// registers a thread, 91 KB) are eight warps, whose instructions wait for the ones before: 3600 a tile.  Around the tiles it is latency:
 // item and lists, the first tile's way, the merge of the parts, about 10000 cycles a CTA.  Builds with their RoPE launch, on the CUDA cores and now:
-// 4 heads x 2564 tokens 482 -> 331 us, 32/8 x 664 243 -> 179, 16 x 1256 424 -> 300 (two tf32 parts 316, 170 and 284); steps of the
-// same 48.8 -> 42.6, 52.0 -> 50.5, 55.0 -> 50.4 (40.4, 46.0, 45.9).
+// 4 heads x 2564 tokens 480 -> 336 us, 32/8 x 664 242 -> 181, 16 x 1256 423 -> 304 (two tf32 parts 316, 170 and 285); steps of the
+// same 50.0 -> 42.7, 51.7 -> 50.4, 54.8 -> 50.2 (40.5, 46.3, 46.0); of 28 drawn models 0.60 to 1.03 of the time on the CUDA cores (0.55 to 0.95).
 //
 // In a step the kernel rotates the block's rows itself, wherever it needs them,
 // and leaves them in the rotated cache: one launch, no kernel in front of it.
@@ -163,8 +163,8 @@ __device__ __forceinline__ void rotate4(float4 x1, float4 x2, float4 cs, float4 
 }
 
 // STEP: a launch of a step.  What only steps do, the rows they rotate and the state they start from, is code that a build's CTAs would
-// fetch around, and the other way: one instantiation for both took a small build and step 55.8 us (now 53.0), the tiny model's step
-// 6.05 (5.62).
+// fetch around, and the other way: with two tf32 parts one instantiation for both took a small build and step 55.8 us (two 53.3), the
+// tiny model's step 6.05 (5.65).
 template <int D, bool STEP>
 __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(const __grid_constant__ Geometry g,
                                                               const __grid_constant__ AttnArgs a) {
@@ -546,8 +546,8 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
   if (plain) {
     // Eight threads for two rows, each with every eighth 16 bytes of their features: they read a key's and a value's row side by side,
     // and share a score's sum; four keys at a time.  What bounds it is the shared-memory pipe, four cycles for the 16 bytes that
-    // serve eight products.  Build of 4 heads x 2564 tokens whose units are all done again: 1306 us, without 325; one of 32/8 heads x
-    // 664 tokens 689 (177); its step 68 (53).  (Four threads a row, a value of theirs at a time, a key at a time: 10900, 5400 and 270.)
+    // serve eight products.  Build of 4 heads x 2564 tokens whose units are all done again: 1351 us, without 343; one of 32/8 heads x
+    // 664 tokens 710 (189); its step 74 (57).  (Four threads a row, a value of theirs at a time, a key at a time: 10900, 5400 and 270.)
     const int r = threadIdx.x >> 3, c0 = (threadIdx.x & 7) * 4;
     constexpr int NC = D / 32;
     float4 qv[2][NC], acc[2][NC];

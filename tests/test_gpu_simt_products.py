@@ -149,7 +149,7 @@ def test_words_left_by_an_earlier_call(n):
 
 def test_cost_of_plain_products():
     """Units that are done once more with plain products: a build and a step where all of them are take no more than a few times as long
-    (1306 us for 325 and 102 for 47 measured; 10900 and 684 where every thread took its values one at a time)."""
+    (1351 us for 343 and 107 for 49 measured; 10900 and 684 where every thread took its values one at a time)."""
     wl = small_workload(name="products", dtype="fp32", prompt_lens=(2500,), gen_len=64, block_len=32, steps=2, hq=4, hkv=4, d=128,
                         scale_mode="inv_sqrt_d")
     q, k, v = (np.array(a) for a in SyntheticSchedule(wl, seed=4).begin_block(0))
