@@ -96,8 +96,7 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
   asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3]) : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-// x = hi + mid + lo of a pair of values (x0 in the lower halves): each the nearest bf16 value of what is left, so that the three
-// hold all 24 bits of x (unless the last lie below the smallest bf16 value)
+// (x0 in the lower half)
 __device__ __forceinline__ uint32_t nearest_bf16(float x0, float x1) {
   uint32_t r;
   asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(x1), "f"(x0));
@@ -127,6 +126,8 @@ __device__ __forceinline__ float2 scaled2(float a, float b, float by) {
 __device__ __forceinline__ float bf16_lower(uint32_t p) { return __uint_as_float(p << 16); }
 __device__ __forceinline__ float bf16_upper(uint32_t p) { return __uint_as_float(p & 0xffff0000u); }
 __device__ __forceinline__ float2 less2(float2 x, float h0, float h1) { return unpack2(fma2(pack2(h0, h1), pack2(-1.f, -1.f), pack2(x.x, x.y))); }
+// x = hi + mid + lo of a pair of values (x0 in the lower halves): each the nearest bf16 value of what is left, so that the three
+// hold all 24 bits of x (unless the last lie below the smallest bf16 value)
 __device__ __forceinline__ void split3(float x0, float x1, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
   float2 x = make_float2(x0, x1);
   hi = nearest_bf16(x.x, x.y);
@@ -367,8 +368,8 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
   }
 
   // The warp's 16 rows x 16 keys of a tile, as the tensor cores lay them out: this thread has rows g and g + 8, keys 2 t and
-  // 2 t + 1 of either eight (scores: n columns; P.V: k index t <-> key 2 t, t + 4 <-> key 2 t + 1, so that a thread's
-  // probabilities are its operand), and features 32 q + 8 t .. + 7 of O~.
+  // 2 t + 1 of either eight (of the scores as of P.V's operand, so that a thread's probabilities are its operand), and features
+  // 32 q + 8 t .. + 7 of O~.  A step of the scores is 16 features, of which this thread has 4 t .. + 3 (k index 2 t, 2 t + 1, 2 t + 8, 2 t + 9).
   const int g8 = lane >> 2, t4 = lane & 3, rw = warp & 1, kw = warp >> 1;
   const bool rows = 16 * rw < it.nrows;   // this warp has rows (the others only help loading)
   // (where the thread's first 16 bytes of a row lie, the rows' parity and pairs counted from the cache's first row: tiles are
@@ -415,8 +416,8 @@ __global__ void __launch_bounds__(THREADS, D == 128 ? 2 : 3) simt_attn_kernel(co
     const float* const vp1 = vpb + buf * SM::TILE;
     float s[2][4];
     if (rows) {
-      // Every product but lo.lo (2^-34 of it): hi.hi, whose 16 bits leave room for a sum of sixteen, over one step at a time and then
-      // added with rounding, for the tensor cores cut sums off; the others, 2^-8 and less of it, in two sums of their own.
+      // Six products: hi.hi, whose 16 bits leave room for a sum of sixteen, over one step at a time and then added with rounding, for
+      // the tensor cores cut sums off; the others, 2^-8 and less of it, in two sums of their own.
       float small[2][2][4];
 #pragma unroll
       for (int n = 0; n < 2; ++n)
